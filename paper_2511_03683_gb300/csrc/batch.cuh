@@ -22,13 +22,12 @@
 // part of f (tiles32.cuh): df/dt within about 1e-6 of Eq. 2.
 //
 // Symmetric tiles (precision 1 and 2, every instance's channel list verified closed under
-// reversal): each instance takes a run of 64-state blocks of one padded state space, and the
-// upper block triangle of every instance is stored as 64 x 64 tiles (zero where a state pair
-// has no channel), so each unordered state pair is streamed once for both of its directions,
-// as in the single-system sweeps (half the bytes of the rows).  One launch
-// of the single-system tile kernel sweeps every instance's tiles; the partial of a state and a
-// partner block sits in the slot of that block's index within its instance, so a state's
-// partials are its instance's blocks only.  The epilogues map each state to its padded row.
+// reversal): each instance takes a run of 64-state blocks of one padded state space, its states in
+// energy order, and the tiles of its upper block triangle within reach of a phonon are stored as
+// 64 x 64 tiles (zero where a state pair has no channel), as in the single-system sweeps, so each
+// unordered state pair is streamed once for both of its directions and the pairs whose coefficients
+// are zero by their distance in energy are not streamed at all.  One launch of the single-system
+// tile kernel sweeps every instance's tiles; the epilogues map each state to its padded row.
 
 namespace pb {
 namespace dev {
@@ -274,17 +273,14 @@ struct pb_batch {
   float2 *pC = nullptr;  // precision 2: rounded FP32 (P_in, P_out) per entry
   uint32_t *pidx = nullptr;
   double *Rg = nullptr;
-  // symmetric tiles (precision >= 1): padded state space of nsp states in nblk blocks,
-  // tnt tiles; partial slots per state tnb (the largest instance's blocks); launch shape
-  // tshape (float-float: CTAs per SM of the half-tile ring, 2 or 3; FP32 pairs: the C32
-  // shape number 2..8)
+  // symmetric tiles (precision >= 1; TilePlan): tnt tiles; launch shape tshape (float-float: CTAs
+  // per SM of the half-tile ring, 2 or 3; FP32 pairs: the C32 shape number 2..8)
   bool tiles = false;
-  int64_t nsp = 0;
-  int nblk = 0, tnb = 0, tnt = 0, tshape = 0;
+  int tnt = 0, tshape = 0;
   int rev = 0;  // the next tile sweep takes the tile list from its end (alternating RK4 stages)
-  int2 *tl = nullptr;
-  int *lblk = nullptr, *pmap = nullptr;
-  int4 *binfo = nullptr;
+  pb::dev::TileD *tl = nullptr;
+  int *pmap = nullptr;
+  int2 *prow = nullptr, *tbase = nullptr;
   long long *srp = nullptr;
   void *tc = nullptr, *tp = nullptr;
   int *err = nullptr;
@@ -434,34 +430,40 @@ std::vector<int64_t> batch_pair_lenp(const pb_channels *const *chs, int32_t n) {
 // P_in and P_out swapped) and the tiles stream at most 0.7 of the rows' bytes (the row stream
 // runs closer to the copy bandwidth; sparse rows, or many instances much smaller than a
 // 64-state block, fill the tiles with zeros).
-struct BatchTiles {
+struct BatchTiles : TilePlan {
   bool on = false;
-  int64_t nsp = 0;
-  int nblk = 0, nbmax = 0, nt = 0;
 };
-BatchTiles batch_tiles_for(const pb_channels *const *chs, int32_t n, int prec, int layout, int64_t nent) {
+// nent: the padded pair entries of all rows; lenp: those of every row (batch_pair_lenp)
+BatchTiles batch_tiles_for(const pb_channels *const *chs, int32_t n, int prec, int layout,
+                           const std::vector<int64_t> &lenp) {
   BatchTiles T;
   if (prec < 1 || layout == 1) return T;
-  int64_t nt = 0;
-  for (int i = 0; i < n; ++i) {
+  int64_t nent = 0, so = 0;
+  for (const int64_t l : lenp) nent += l;
+  for (int i = 0; i < n; ++i)
     if (!chs[i]->closed) return T;
-    const int64_t B = (chs[i]->nstate + dev::kTile - 1) / dev::kTile;
-    T.nblk += (int)B;
-    T.nbmax = std::max<int>(T.nbmax, (int)B);
-    nt += B * (B + 1) / 2;
+  for (int i = 0; i < n; ++i) {
+    const pb_channels *ch = chs[i];
+    // rows as long as complete ones (up to the padding): the reach alone bounds the tiles
+    bool complete = true;
+    const int64_t full = (ch->nstate + kRowPad - 1) / kRowPad * kRowPad;
+    for (int64_t r = 0; r < ch->nstate; ++r) complete = complete && lenp[so + r] == full;
+    so += ch->nstate;
+    double gmax = 0.0;
+    for (const double g : ch->g2) gmax = std::max(gmax, g);
+    tile_plan_add(ch, complete, energy_reach(ch, gmax), T);
   }
-  if (nt == 0 || nt >= INT32_MAX / 2) return T;
+  const int64_t nt = (int64_t)T.tiles.size();
+  if (nt == 0 || nt >= INT32_MAX / 2 || T.npart >= INT32_MAX) return T;
   const double tile_bytes = (double)nt * dev::kTile * dev::kTile * (prec == 2 ? 8.0 : 16.0);
   const double row_bytes = (double)nent * (prec == 2 ? 12.0 : 20.0);
-  T.nt = (int)nt;
-  T.nsp = (int64_t)T.nblk * dev::kTile;
   T.on = layout == 2 || tile_bytes <= 0.7 * row_bytes;
   return T;
 }
 
 struct BatchLayoutFF {
   size_t items, item_inst, item_ptr, pA, pB, pC, pidx, Rg, yff, part, acc, y, tcol, tg2, tcA, tcB, titems, titem_ptr,
-      tpart, tR, tpcst, tpcnt, omega_tmp, tab_tmp, eps_tmp, kc_tmp, srp, tl, lblk, binfo, pmap, tc, tp, err, total;
+      tpart, tR, tpcst, tpcnt, omega_tmp, tab_tmp, eps_tmp, kc_tmp, srp, tl, pmap, prow, tbase, tc, tp, err, total;
 };
 
 constexpr int kBatchSetupItem = 2048;  // channels per work item of the per-instance coefficient setup
@@ -523,12 +525,12 @@ BatchLayoutFF batch_layout_ff(const pb_channels *const *chs, int n, int64_t ns, 
   L.kc_tmp = take(sizeof(short4) * maxs);
   const size_t te = c32 ? sizeof(float2) : sizeof(float4), pe = c32 ? sizeof(float) : sizeof(float4);
   L.srp = take(T.on ? sizeof(int64_t) * (ns + 1) : 0);
-  L.tl = take(T.on ? sizeof(int2) * T.nt : 0);
-  L.lblk = take(T.on ? sizeof(int32_t) * T.nblk : 0);
-  L.binfo = take(T.on ? sizeof(int4) * T.nblk : 0);
+  L.tl = take(T.on ? sizeof(dev::TileD) * T.tiles.size() : 0);
   L.pmap = take(T.on ? sizeof(int32_t) * ns : 0);
-  L.tc = take(T.on ? te * T.nt * dev::kTile * dev::kTile : 0);
-  L.tp = take(T.on ? pe * T.nsp * T.nbmax : 0);
+  L.prow = take(T.on ? sizeof(int2) * ns : 0);
+  L.tbase = take(T.on ? sizeof(int2) * T.nb : 0);
+  L.tc = take(T.on ? te * (size_t)T.nt_full * dev::kTile * dev::kTile : 0);
+  L.tp = take(T.on ? pe * (size_t)T.nsp * T.nb_max : 0);
   L.err = take(sizeof(int));
   L.total = o;
   return L;
@@ -578,7 +580,7 @@ int batch_upload_plan(pb_batch *b, int item_ch, cudaStream_t st, bool csr = fals
 
 // the tile sweep of every instance in one launch (the single-system kernels, with the slot map)
 int batch_sweep_tiles(pb_batch *b, cudaStream_t st) {
-  const int nsp = (int)b->nsp, nt = b->tnt;
+  const int nt = b->tnt;
   if (b->prec == 2) {
     with_c32_shape(b->tshape, [&](auto nst, auto cps, auto half) {
       const int gs = (int)std::max<int64_t>(1, std::min<int64_t>(nt, (int64_t)b->sm_count * cps()));
@@ -586,10 +588,10 @@ int batch_sweep_tiles(pb_batch *b, cudaStream_t st) {
       float *tp = (float *)b->tp;
       if constexpr (decltype(half)::value)
         dev::k_stream_c32_half<dev::MODE_COLL, nst(), cps()><<<gs, dev::kC32Threads, dev::c32_half_smem<nst()>(), st>>>(
-            b->tl, nt, tc, b->yff, nsp, b->tnb, tp, b->err, b->lblk, b->rev);
+            b->tl, nt, tc, b->yff, tp, b->err, b->rev);
       else
         dev::k_stream_c32<dev::MODE_COLL, nst(), cps()><<<gs, dev::kC32Threads, dev::c32_smem<nst()>(), st>>>(
-            b->tl, nt, tc, b->yff, nsp, b->tnb, tp, b->err, b->lblk, b->rev);
+            b->tl, nt, tc, b->yff, tp, b->err, b->rev);
     });
     PB_LAUNCHED("k_stream_c32 (batch tiles)");
     return PB_OK;
@@ -598,11 +600,9 @@ int batch_sweep_tiles(pb_batch *b, cudaStream_t st) {
   float4 *tp = (float4 *)b->tp;
   const int gs = (int)std::max<int64_t>(1, std::min<int64_t>(nt, (int64_t)b->sm_count * b->tshape));
   if (b->tshape == 3)
-    dev::k_stream_sym_half<2, 3><<<gs, dev::kSymThreads, dev::half_smem<2>(), st>>>(b->tl, nt, tc, b->yff, nsp, b->tnb,
-                                                                                    tp, b->err, b->lblk, b->rev);
+    dev::k_stream_sym_half<2, 3><<<gs, dev::kSymThreads, dev::half_smem<2>(), st>>>(b->tl, nt, tc, b->yff, tp, b->err, b->rev);
   else
-    dev::k_stream_sym_half<3, 2><<<gs, dev::kSymThreads, dev::half_smem<3>(), st>>>(b->tl, nt, tc, b->yff, nsp, b->tnb,
-                                                                                    tp, b->err, b->lblk, b->rev);
+    dev::k_stream_sym_half<3, 2><<<gs, dev::kSymThreads, dev::half_smem<3>(), st>>>(b->tl, nt, tc, b->yff, tp, b->err, b->rev);
   PB_LAUNCHED("k_stream_sym_half (batch tiles)");
   return PB_OK;
 }
@@ -648,13 +648,11 @@ int batch_fin(pb_batch *b, double *out, double *f, double dt, cudaStream_t st, c
     // outputs, their padded rows the partials and the next stage's float-float input
     const int ns = (int)b->ns;
     if (b->prec == 2) {
-      dev::k_fin_c32<STAGE><<<(ns + 31) / 32, 256, 0, st>>>((const float *)b->tp, b->tnb, ns, ns, 1.0, src, out, f,
-                                                            b->acc, b->y, b->yff, dt, b->pmap, b->binfo);
+      dev::k_fin_c32<STAGE><<<(ns + 31) / 32, 256, 0, st>>>((const float *)b->tp, b->prow, b->pmap, ns, 1.0, src,
+                                                            out, f, b->acc, b->y, b->yff, dt);
       PB_LAUNCHED("k_fin_c32 (batch tiles)");
     } else {
-      dev::TileSrc ts{(const float4 *)b->tp, b->tnb, ns};
-      ts.pmap = b->pmap;
-      ts.binfo = b->binfo;
+      const dev::TileSrc ts{(const float4 *)b->tp, b->prow, b->pmap};
       dev::k_fin_tiles<STAGE><<<(ns + 31) / 32, 256, 0, st>>>(ts, ns, 1.0, b->Rg, src, out, f, b->acc, b->y, b->yff,
                                                               dt);
       PB_LAUNCHED("k_fin_tiles (batch tiles)");
@@ -859,44 +857,25 @@ int batch_tile_cps(const pb_batch *b) {
   return c;
 }
 
-// The tile form: block table, tile list and state map on the host, then the tiles zeroed and
-// every stored pair scattered into them from the instances' branch-merged pair rows
-// (prefactors folded in).
-int batch_setup_tiles(pb_batch *b, const pb_channels *const *chs, int n, cudaStream_t st) {
+// The tile form: the plan's tables uploaded, then the tiles zeroed and every stored pair scattered
+// into them from the instances' branch-merged pair rows (prefactors folded in).
+int batch_setup_tiles(pb_batch *b, const TilePlan &T, cudaStream_t st) {
   std::vector<long long> srp((size_t)b->ns + 1, 0);
   for (int64_t r = 0; r < b->ns; ++r) srp[r + 1] = srp[r] + b->lenp[r];
-  std::vector<int2> tl;
-  std::vector<int32_t> lblk, pmap((size_t)b->ns);
-  std::vector<int4> binfo;
-  tl.reserve((size_t)b->tnt);
-  int G0 = 0;
-  for (int i = 0; i < n; ++i) {
-    const int ns_i = (int)chs[i]->nstate, B = (ns_i + dev::kTile - 1) / dev::kTile;
-    const int tbase = (int)tl.size();
-    for (int I = 0; I < B; ++I)
-      for (int J = I; J < B; ++J) tl.push_back(make_int2(G0 + I, G0 + J));
-    for (int g = 0; g < B; ++g) {
-      lblk.push_back(g);
-      binfo.push_back(make_int4(G0, tbase, ns_i, B));
-    }
-    for (int s = 0; s < ns_i; ++s) pmap[b->soff[i] + s] = G0 * dev::kTile + s;
-    G0 += B;
-  }
-  if ((int)tl.size() != b->tnt || G0 != b->nblk) return set_error(PB_EINVAL, "pb_batch_create: tile plan mismatch");
   PB_CUDA(cudaMemcpyAsync(b->srp, srp.data(), sizeof(long long) * srp.size(), cudaMemcpyHostToDevice, st));
-  PB_CUDA(cudaMemcpyAsync(b->tl, tl.data(), sizeof(int2) * tl.size(), cudaMemcpyHostToDevice, st));
-  PB_CUDA(cudaMemcpyAsync(b->lblk, lblk.data(), sizeof(int32_t) * lblk.size(), cudaMemcpyHostToDevice, st));
-  PB_CUDA(cudaMemcpyAsync(b->binfo, binfo.data(), sizeof(int4) * binfo.size(), cudaMemcpyHostToDevice, st));
-  PB_CUDA(cudaMemcpyAsync(b->pmap, pmap.data(), sizeof(int32_t) * pmap.size(), cudaMemcpyHostToDevice, st));
+  PB_CUDA(cudaMemcpyAsync(b->tl, T.tiles.data(), sizeof(dev::TileD) * T.tiles.size(), cudaMemcpyHostToDevice, st));
+  PB_CUDA(cudaMemcpyAsync(b->pmap, T.pmap.data(), sizeof(int32_t) * T.pmap.size(), cudaMemcpyHostToDevice, st));
+  PB_CUDA(cudaMemcpyAsync(b->prow, T.prow.data(), sizeof(int2) * T.prow.size(), cudaMemcpyHostToDevice, st));
+  PB_CUDA(cudaMemcpyAsync(b->tbase, T.tbase.data(), sizeof(int2) * T.tbase.size(), cudaMemcpyHostToDevice, st));
   const size_t tbytes = (size_t)b->tnt * dev::kTile * dev::kTile * (b->prec == 2 ? sizeof(float2) : sizeof(float4));
   PB_CUDA(cudaMemsetAsync(b->tc, 0, tbytes, st));
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((b->ns * 32 + 255) / 256, (int64_t)b->sm_count * 8));
   if (b->prec == 2)
     dev::k_tiles_scatter<true, uint32_t><<<grid, 256, 0, st>>>(b->srp, (int)b->ns, b->pidx, b->pA, b->pB, b->pmap,
-                                                               b->binfo, 0, b->tc);
+                                                               b->tbase, b->tc);
   else
     dev::k_tiles_scatter<false, uint32_t><<<grid, 256, 0, st>>>(b->srp, (int)b->ns, b->pidx, b->pA, b->pB, b->pmap,
-                                                                b->binfo, 0, b->tc);
+                                                                b->tbase, b->tc);
   PB_LAUNCHED("k_tiles_scatter (batch)");
   PB_CUDA(cudaStreamSynchronize(st));  // the host tables are released on return
   // dynamic shared memory of every launch shape the autotuner may pick
@@ -941,7 +920,7 @@ extern "C" int pb_batch_arena_bytes(const pb_channels *const *chs, int32_t n, co
       const std::vector<int64_t> lenp = batch_pair_lenp(chs, n);
       int64_t nent = 0;
       for (int64_t l : lenp) nent += l;
-      const BatchTiles T = batch_tiles_for(chs, n, prec, opts ? opts->layout : 0, nent);
+      const BatchTiles T = batch_tiles_for(chs, n, prec, opts ? opts->layout : 0, lenp);
       *bytes = batch_layout_ff(chs, n, ns, nent, batch_items_count(lenp, kBatchMinItem), prec == 2, T, lenp).total;
     } else {
       pb_batch_opts o{};
@@ -1007,7 +986,7 @@ extern "C" int pb_batch_create(const pb_channels *const *chs, int32_t n, const p
     if (b->prec >= 1) {
       int64_t nent = 0;
       for (int64_t l : b->lenp) nent += l;
-      const BatchTiles T = batch_tiles_for(chs, n, b->prec, o.layout, nent);
+      const BatchTiles T = batch_tiles_for(chs, n, b->prec, o.layout, b->lenp);
       const BatchLayoutFF LF = batch_layout_ff(chs, n, ns, nent, b->nitems_cap, b->prec == 2, T, b->lenp);
       if (bytes < LF.total) {
         delete b;
@@ -1032,30 +1011,24 @@ extern "C" int pb_batch_create(const pb_channels *const *chs, int32_t n, const p
       b->err = (int *)(A + LF.err);
       if (T.on) {
         b->tiles = true;
-        b->nsp = T.nsp;
-        b->nblk = T.nblk;
-        b->tnb = T.nbmax;
-        b->tnt = T.nt;
+        b->tnt = (int)T.tiles.size();
         b->tshape = b->prec == 2 ? 2 : 3;  // 2 stages x 3 CTAs per SM for both
         b->srp = (long long *)(A + LF.srp);
-        b->tl = (int2 *)(A + LF.tl);
-        b->lblk = (int32_t *)(A + LF.lblk);
-        b->binfo = (int4 *)(A + LF.binfo);
+        b->tl = (dev::TileD *)(A + LF.tl);
         b->pmap = (int32_t *)(A + LF.pmap);
+        b->prow = (int2 *)(A + LF.prow);
+        b->tbase = (int2 *)(A + LF.tbase);
         b->tc = A + LF.tc;
         b->tp = A + LF.tp;
       }
       {
-        // the error word; the padding of the stage input and the partial slots no instance
-        // writes stay zero
+        // the error word; the padding of the stage input stays zero
         cudaError_t e = cudaMemsetAsync(b->err, 0, sizeof(int), st);
         if (e == cudaSuccess && T.on) e = cudaMemsetAsync(b->yff, 0, sizeof(float2) * (size_t)T.nsp, st);
-        if (e == cudaSuccess && T.on)
-          e = cudaMemsetAsync(b->tp, 0, (b->prec == 2 ? sizeof(float) : sizeof(float4)) * (size_t)T.nsp * T.nbmax, st);
         if (e != cudaSuccess) status = cuda_fail(e, "pb_batch_create: clear");
       }
       if (status == PB_OK) status = batch_setup_ff(b, chs, n, LF, st);
-      if (status == PB_OK && b->tiles) status = batch_setup_tiles(b, chs, n, st);
+      if (status == PB_OK && b->tiles) status = batch_setup_tiles(b, T, st);
       if (status == PB_OK && !b->tiles && b->prec == 2 && nent > 0) {
         dev::k_pairs_c32<<<(int)std::min<int64_t>((nent + 255) / 256, 8192), 256, 0, st>>>(b->pA, b->pB,
                                                                                            (long long)nent, b->pC);

@@ -9,6 +9,7 @@
 #include <memory>
 #include <mutex>
 #include <new>
+#include <numeric>
 #include <type_traits>
 #include <vector>
 
@@ -51,7 +52,7 @@ struct Layout {
   size_t rp, item_ptr, items, col, coefA, coefB, g2, wt, eps, kc, R, omega, tab, part, acc, y, yff, fstage, Fa, Fb,
       Fff, tau, invtau, red, scal, obs, g2lo, gstate, tab32, col16, rp_real, vjpG, g2tab, vecs, hcol, hg2, hA, hB, sc,
       entries, hitems, titems, t_item_ptr, err, citems, citem_ptr, cpart, ccoefA, ccoefB, sidx16, sidx32, pcstart,
-      pcnt, srp, gitems, tiles, tcoef, tpart, g2d, gditems, gdptr, gacc, gaccg, trptr, trpart, total;
+      pcnt, srp, gitems, tiles, tcoef, tpart, pmap, prow, tbase, g2d, gditems, gdptr, gacc, gaccg, trptr, trpart, total;
 };
 
 struct Plan {
@@ -204,21 +205,116 @@ int64_t grad_chunks(const std::vector<int64_t> &rp) {
   return (int64_t)it.size();
 }
 
-// symmetric tiles of the complete-row FF sweep: nb blocks of kTile states, nt = nb(nb+1)/2 tiles
-struct TileDims {
-  int nb = 0, nt = 0, nsp = 0;
-};
-TileDims tile_dims(int64_t ns) {
-  TileDims t;
-  t.nb = (int)((ns + dev::kTile - 1) / dev::kTile);
-  t.nt = t.nb * (t.nb + 1) / 2;
-  t.nsp = t.nb * dev::kTile;
-  return t;
+// The energy distance beyond which a channel's float-float coefficients are exact zeros.  With
+// |eps_s - eps_p| > E both Gaussians of Eq. 2 have arguments beyond z = (E - max hbar omega) / sigma
+// widths, so G_a (N+1) + G_e N and G_e - G_a are at most norm (2 N_max + 1) exp(-z^2 / 2); z is
+// chosen to bring that times scale (the largest factor multiplied in before the coefficient is
+// rounded: 1 for the forms stored without |g|^2, else the largest |g|^2) below 2^-150, half the
+// smallest FP32 number, where the high part rounds to zero and with it the low part.  About 15
+// sigma; at the 40^3 window (sigma 8 meV, phonons to 60 meV) E = 0.18 eV of the 1.6 eV it spans.
+double energy_reach(const pb_channels *ch, double scale) {
+  double wmax = 0.0, wmin = INFINITY;
+  for (const double w : ch->omega)
+    if (w > 0.0) {
+      wmax = std::max(wmax, w);
+      wmin = std::min(wmin, w);
+    }
+  if (!(wmax > 0.0)) return 0.0;  // no phonon, no channel
+  const double nmax = 1.0 / std::expm1(wmin / (kBoltz * ch->T));
+  const double top = std::log(std::max(scale, 1.0)) + std::log((2.0 * nmax + 1.0) / (std::sqrt(2.0 * kPi) * ch->sigma));
+  const double z = std::sqrt(2.0 * std::max(0.0, 150.0 * std::log(2.0) + top));
+  const double e = (wmax + z * ch->sigma) * (1.0 + 1e-9);
+  return std::isfinite(e) ? e : INFINITY;
 }
 
-// tile_entry: bytes per pair of the symmetric tiles (16 float-float, 8 for the FP32 tiles of C32)
+// The symmetric tiles of one system or of a batch's systems one after the other: each system's
+// states in energy order, padded to whole blocks of kTile, and the tiles of its upper block
+// triangle within reach of each other (kernels.cuh).
+struct TilePlan {
+  int nb = 0;                     // blocks
+  int64_t nsp = 0, npart = 0;     // padded states; partial slots
+  int64_t nt_full = 0;            // tiles of the whole triangles, and the blocks of the largest system:
+  int nb_max = 0;                 // what the arena reserves, whatever the reach
+  std::vector<int32_t> pmap;      // [states] row in the padded energy order
+  std::vector<int2> prow;         // [states] first partial slot, slots
+  std::vector<int2> tbase;        // [blocks] index of tile (I, I), last block column of block row I
+  std::vector<dev::TileD> tiles;  // block rows in order, columns ascending
+};
+
+// complete: every row holds every state (the reach alone decides); else the stored channels within
+// reach do.  In energy order the columns that meet block row I are I .. hi(I), hi made monotone, so
+// that the rows that meet block column J are a contiguous range too.
+void tile_plan_add(const pb_channels *ch, bool complete, double reach, TilePlan &T) {
+  const int64_t ns = ch->nstate;
+  const double *eps = ch->eps.data();
+  std::vector<int32_t> ord((size_t)ns), pos((size_t)ns);
+  std::iota(ord.begin(), ord.end(), 0);
+  std::stable_sort(ord.begin(), ord.end(), [&](int32_t a, int32_t b) { return eps[a] < eps[b]; });
+  for (int64_t i = 0; i < ns; ++i) pos[ord[i]] = (int32_t)i;
+  const int nb = (int)((ns + dev::kTile - 1) / dev::kTile);
+  std::vector<int32_t> top((size_t)ns);  // last position in reach of each position
+  if (complete) {
+    for (int64_t i = 0, j = 0; i < ns; ++i) {
+      j = std::max(j, i);
+      while (j + 1 < ns && eps[ord[j + 1]] - eps[ord[i]] <= reach) ++j;
+      top[i] = (int32_t)j;
+    }
+  } else {
+#pragma omp parallel for schedule(dynamic, 16)
+    for (int64_t r = 0; r < ns; ++r) {
+      int32_t t = pos[r];
+      for (int64_t c = ch->row_ptr[r]; c < ch->row_ptr[r + 1]; ++c) {
+        const int32_t p = ch->col[c];
+        if (pos[p] > t && eps[p] - eps[r] <= reach) t = pos[p];
+      }
+      top[pos[r]] = t;
+    }
+  }
+  std::vector<int32_t> hi((size_t)nb), lo((size_t)nb);
+  for (int I = 0; I < nb; ++I) {
+    int32_t h = I > 0 ? std::max(hi[I - 1], I) : I;
+    for (int64_t i = (int64_t)I * dev::kTile; i < std::min<int64_t>(ns, (int64_t)(I + 1) * dev::kTile); ++i)
+      h = std::max(h, top[i] / dev::kTile);
+    hi[I] = h;
+  }
+  for (int J = 0, I = 0; J < nb; ++J) {
+    while (hi[I] < J) ++I;
+    lo[J] = I;
+  }
+  // slots of the states of block K: its partner blocks lo(K) .. hi(K)
+  std::vector<int64_t> first((size_t)nb);
+  for (int K = 0; K < nb; ++K) {
+    first[K] = T.npart;
+    T.npart += (int64_t)(hi[K] - lo[K] + 1) * dev::kTile;
+  }
+  for (int I = 0; I < nb; ++I) {
+    T.tbase.push_back(make_int2((int)T.tiles.size(), T.nb + hi[I]));
+    for (int J = I; J <= hi[I]; ++J) {
+      dev::TileD D{};
+      D.I = T.nb + I;
+      D.J = T.nb + J;
+      D.rb = (int)(first[I] + (J - lo[I]));
+      D.rs = hi[I] - lo[I] + 1;
+      D.cb = (int)(first[J] + (I - lo[J]));
+      D.cs = hi[J] - lo[J] + 1;
+      T.tiles.push_back(D);
+    }
+  }
+  for (int64_t r = 0; r < ns; ++r) {
+    const int K = pos[r] / dev::kTile, n = hi[K] - lo[K] + 1;
+    T.pmap.push_back((int32_t)((int64_t)T.nb * dev::kTile + pos[r]));
+    T.prow.push_back(make_int2((int)(first[K] + (int64_t)(pos[r] % dev::kTile) * n), n));
+  }
+  T.nb += nb;
+  T.nt_full += (int64_t)nb * (nb + 1) / 2;
+  T.nb_max = std::max(T.nb_max, nb);
+  T.nsp = (int64_t)T.nb * dev::kTile;
+}
+
+// tp: the symmetric tiles (null: none); tile_entry: their bytes per pair (16 float-float, 8 for the
+// FP32 tiles of C32)
 Layout make_layout(const pb_channels *ch, const Plan &P, const Plan *S, int variant, bool transport,
-                   int nfin_blocks, bool sym = false, const GDense &gd = GDense(), bool gacc = false,
+                   int nfin_blocks, const TilePlan *tp = nullptr, const GDense &gd = GDense(), bool gacc = false,
                    size_t tile_entry = sizeof(float4), int tr_nseg = 0) {
   Layout L{};
   size_t o = 0;
@@ -250,10 +346,12 @@ Layout make_layout(const pb_channels *ch, const Plan &P, const Plan *S, int vari
   L.gitems = take(S ? sizeof(Item) * (size_t)grad_chunks(S->rp) : 0);
   L.gacc = take(S && gacc && variant == PB_VARIANT_FF ? sizeof(float4) * nsw : 0);
   L.gaccg = take(gacc && (variant == PB_VARIANT_G32 || variant == PB_VARIANT_G16 || variant == PB_VARIANT_H16) ? 3 * sizeof(double) * (size_t)ns * (size_t)ns : 0);
-  const TileDims td = tile_dims((int64_t)ns);
-  L.tiles = take(sym ? sizeof(int2) * td.nt : 0);
-  L.tcoef = take(sym ? tile_entry * (size_t)td.nt * dev::kTile * dev::kTile : 0);
-  L.tpart = take(sym ? sizeof(float4) * (size_t)td.nb * td.nsp : 0);
+  L.tiles = take(tp ? sizeof(dev::TileD) * tp->tiles.size() : 0);
+  L.tcoef = take(tp ? tile_entry * (size_t)tp->nt_full * dev::kTile * dev::kTile : 0);
+  L.tpart = take(tp ? sizeof(float4) * (size_t)tp->nb_max * (size_t)tp->nsp : 0);
+  L.pmap = take(tp ? sizeof(int32_t) * ns : 0);
+  L.prow = take(tp ? sizeof(int2) * ns : 0);
+  L.tbase = take(tp ? sizeof(int2) * tp->nb : 0);
   L.wt = take(transport ? sizeof(float2) * nsw : 0);
   L.eps = take(sizeof(double) * ns);
   L.kc = take(sizeof(short4) * ns);
@@ -262,7 +360,7 @@ Layout make_layout(const pb_channels *ch, const Plan &P, const Plan *S, int vari
   L.tab = take(sizeof(double2) * (size_t)ch->nq * ch->nmodes);
   L.acc = take(sizeof(double) * ns);
   L.y = take(sizeof(double) * ns);
-  L.yff = take(sizeof(float2) * ns);
+  L.yff = take(sizeof(float2) * (tp ? std::max<size_t>((size_t)tp->nsp, ns) : ns));
   L.fstage = take(sizeof(double) * ns);
   L.Fa = take(transport ? sizeof(double) * 3 * ns : 0);
   L.Fb = take(transport ? sizeof(double) * 3 * ns : 0);
@@ -475,17 +573,20 @@ struct pb_dev {
   // triangle of the pair matrix once and add each tile to its rows and to its columns
   bool sym = false;
   int sym_nt = 0;  // threads of the bulk-copy tile sweep's CTA (0: the global-load tile sweep)
-  TileDims td;
-  int2 *tiles = nullptr;
+  int tnt = 0;            // stored tiles
+  int64_t nsp = 0;        // padded states of their energy order
+  dev::TileD *tiles = nullptr;
   float4 *tcoef = nullptr;
   float4 *tpart = nullptr;
+  int32_t *pmap = nullptr;  // as TilePlan
+  int2 *prow = nullptr, *tbase = nullptr;
+  dev::TileSrc tile_src() const { return dev::TileSrc{tpart, prow, pmap}; }
   // PB_VARIANT_C32: the FF device whose tiles hold FP32 (P_in, P_out) (tiles32.cuh); its
-  // partials in tpart are (N, Bd, L, Ld) per (state, block)
+  // partials in tpart are one FP32 value per (state, block)
   bool sym_half = false;  // the float-float tile sweep in half-tiles (tile_sweep 3)
   int half_cps = 3;       // its resident CTAs per SM: 3 (two stages each) or 2 (three stages)
   bool c32 = false;
   int c32_shape = 2;  // pb_dev_opts.tile_sweep: the launch shape (with_c32_shape)
-  bool complete = false;  // every row holds every state (tiles filled by position, else scattered)
   // the next tile sweep takes the tile list from its end (the RK4 stages alternate, so that each
   // sweep starts on the tiles the previous one left in L2)
   int rev = 0;
@@ -643,12 +744,11 @@ bool merge_for(const pb_dev_opts &o) {
   return (o.variant == PB_VARIANT_FF || o.variant == PB_VARIANT_F64) && o.merge_branches != 2;
 }
 
-// whether the symmetric tiles of ns states stream at most 0.7 of the bytes of a branch-merged
-// row stream of nsw entries (float-float P_in and D and a 16- or 32-bit partner index): rows
-// that miss some partners, but not many
-bool tiles_pay(int64_t ns, int64_t nsw) {
-  const double nb = (double)((ns + dev::kTile - 1) / dev::kTile);
-  const double tile_bytes = nb * (nb + 1) / 2 * dev::kTile * dev::kTile * 16.0;
+// whether nt symmetric tiles stream at most 0.7 of the bytes of a branch-merged row stream of nsw
+// entries (float-float P_in and D and a 16- or 32-bit partner index): rows that hold most of the
+// partners within reach
+bool tiles_pay(int64_t nt, int64_t ns, int64_t nsw) {
+  const double tile_bytes = (double)nt * dev::kTile * dev::kTile * 16.0;
   const double row_bytes = (double)nsw * (16.0 + (ns <= 65536 ? 2.0 : 4.0));
   return tile_bytes <= 0.7 * row_bytes;
 }
@@ -656,9 +756,13 @@ bool tiles_pay(int64_t ns, int64_t nsw) {
 // symmetric tiles: FF, branch-merged, a list verified closed under reversal (the entry of (s, p)
 // serves (p, s) with P_in and P_out swapped); dense_rows 3, or automatic (0) on complete rows or
 // when the tiles stream fewer bytes than the rows (pays)
-bool sym_for(const pb_dev_opts &o, bool merged, bool complete, bool closed, bool pays) {
-  if (!(merged && closed && o.variant == PB_VARIANT_FF && o.stream_mode != 2)) return false;
-  return o.dense_rows == 3 || (o.dense_rows == 0 && (complete || pays));
+// T: the tile plan, filled in when they may be taken.
+bool sym_for(const pb_channels *ch, const pb_dev_opts &o, bool merged, bool complete, int64_t nsw, TilePlan &T) {
+  if (!(merged && ch->closed && o.variant == PB_VARIANT_FF && o.stream_mode != 2)) return false;
+  if (o.dense_rows != 3 && o.dense_rows != 0) return false;
+  tile_plan_add(ch, complete, energy_reach(ch, 1.0), T);
+  if (T.tiles.size() >= (size_t)INT32_MAX / 2 || T.npart >= INT32_MAX) return false;
+  return o.dense_rows == 3 || complete || tiles_pay((int64_t)T.tiles.size(), ch->nstate, nsw);
 }
 
 // work-item size of the branch-merged sweep: the caller's, the bulk ring's, or the default
@@ -815,12 +919,13 @@ extern "C" int pb_dev_arena_bytes(const pb_channels *ch, const pb_dev_opts *opts
     bool complete = false;
     const bool merged = make_plans(ch, opts, o, sm, P, S, &complete);
     const int nfin = (int)((P.ns + kFinBlock - 1) / kFinBlock);
-    const bool sym = sym_for(o, merged, complete, ch->closed, merged && tiles_pay(S.ns, S.nchp));
+    TilePlan T;
+    const bool sym = sym_for(ch, o, merged, complete, S.nchp, T);
     if (c32 && !sym)
       return set_error(PB_EINVAL, "pb_dev: the FP32 coefficient tiles (C32) need the symmetric tiles: a "
                                   "closure-checked list whose rows are complete or miss few partners (or dense_rows 3)");
     const TrRows tr = tr_rows_for(P.ns, sm, o.transport != 0, merged, complete, o.variant, o);
-    *bytes = make_layout(ch, P, merged ? &S : nullptr, o.variant, o.transport != 0, nfin, sym,
+    *bytes = make_layout(ch, P, merged ? &S : nullptr, o.variant, o.transport != 0, nfin, sym ? &T : nullptr,
                          gdense_for(ch, o, sm), o.adjoint != 0, c32 ? sizeof(float2) : sizeof(float4), tr.nseg)
                  .total;
   } catch (const std::bad_alloc &) {
@@ -853,9 +958,11 @@ extern "C" int pb_dev_create(const pb_channels *ch, const pb_dev_opts *opts, voi
   pb_dev *d = new (std::nothrow) pb_dev();
   if (!d) return set_error(PB_ENOMEM, "pb_dev_create: out of host memory");
   Plan P, S;
-  bool merged = false, complete = false;
+  TilePlan T;
+  bool merged = false, complete = false, sym = false;
   try {
     merged = make_plans(ch, opts, o, sm, P, S, &complete);
+    sym = sym_for(ch, o, merged, complete, S.nchp, T);
   } catch (const std::bad_alloc &) {
     delete d;
     return set_error(PB_ENOMEM, "pb_dev_create: out of host memory");
@@ -892,8 +999,7 @@ extern "C" int pb_dev_create(const pb_channels *ch, const pb_dev_opts *opts, voi
   d->item_ch = o.item_channels;
   d->transport = o.transport != 0;
   d->nfin_blocks = (int)((d->ns + kFinBlock - 1) / kFinBlock);
-  d->sym = sym_for(o, merged, complete, ch->closed, merged && tiles_pay(S.ns, S.nchp));
-  d->complete = complete;
+  d->sym = sym;
   if (c32 && !d->sym) {
     delete d;
     return set_error(PB_EINVAL, "pb_dev: the FP32 coefficient tiles (C32) need the symmetric tiles: a "
@@ -904,7 +1010,8 @@ extern "C" int pb_dev_create(const pb_channels *ch, const pb_dev_opts *opts, voi
   d->sym_nt = d->sym && (o.tile_sweep == 2 || (o.tile_sweep == 3 && !c32)) ? dev::kSymThreads : 0;
   d->sym_half = d->sym && o.tile_sweep == 3 && !c32;
   d->half_cps = (opts && opts->ctas_per_sm == 2) ? 2 : 3;
-  d->td = tile_dims(d->ns);
+  d->tnt = (int)T.tiles.size();
+  d->nsp = T.nsp;
   const GDense gd = gdense_for(ch, o, sm);
   d->gdense = gd.on;
   d->gd_npp = gd.npp;
@@ -913,7 +1020,7 @@ extern "C" int pb_dev_create(const pb_channels *ch, const pb_dev_opts *opts, voi
   const TrRows trr = tr_rows_for(d->ns, sm, d->transport, merged, complete, o.variant, o);
   d->tr_nseg = trr.nseg;
   d->tr_seglen = trr.seglen;
-  d->L = make_layout(ch, P, merged ? &S : nullptr, o.variant, d->transport, d->nfin_blocks, d->sym, gd,
+  d->L = make_layout(ch, P, merged ? &S : nullptr, o.variant, d->transport, d->nfin_blocks, sym ? &T : nullptr, gd,
                      o.adjoint != 0, c32 ? sizeof(float2) : sizeof(float4), trr.nseg);
   if (arena_bytes < d->L.total) {
     const size_t need = d->L.total;
@@ -992,10 +1099,13 @@ extern "C" int pb_dev_create(const pb_channels *ch, const pb_dev_opts *opts, voi
     d->gitems = (Item *)(A + L.gitems);
     if (d->variant == PB_VARIANT_FF && o.adjoint) d->gacc = (float4 *)(A + L.gacc);
     if (d->sym) {
-      d->tiles = (int2 *)(A + L.tiles);
+      d->tiles = (dev::TileD *)(A + L.tiles);
       d->tcoef = (float4 *)(A + L.tcoef);
       d->tc32 = (float2 *)(A + L.tcoef);
       d->tpart = (float4 *)(A + L.tpart);
+      d->pmap = (int32_t *)(A + L.pmap);
+      d->prow = (int2 *)(A + L.prow);
+      d->tbase = (int2 *)(A + L.tbase);
     }
   } else {
     d->citems = d->items;
@@ -1130,9 +1240,9 @@ extern "C" int pb_dev_create(const pb_channels *ch, const pb_dev_opts *opts, voi
           status = cuda_fail(e_, "clear error word");
           break;
         }
-        // the tile sweeps copy the float-float f of a ragged last block rounded up to 16 bytes:
-        // the padding after the nstate values must hold zeros (it multiplies zero coefficients)
-        e_ = cudaMemsetAsync(d->yff, 0, align_up(sizeof(float2) * (size_t)d->ns), st);
+        // the tile sweeps read f in whole blocks: its padding must hold zeros (it multiplies zero
+        // coefficients)
+        e_ = cudaMemsetAsync(d->yff, 0, sizeof(float2) * (size_t)std::max<int64_t>(d->sym ? d->nsp : 0, d->ns), st);
         if (e_ != cudaSuccess) {
           status = cuda_fail(e_, "clear the stage input");
           break;
@@ -1220,15 +1330,10 @@ extern "C" int pb_dev_create(const pb_channels *ch, const pb_dev_opts *opts, voi
           UP(d->gitems, gi.data(), sizeof(Item) * gi.size());
         }
         if (d->sym) {
-          std::vector<int2> tl;
-          for (int I = 0; I < d->td.nb; ++I)
-            for (int J = I; J < d->td.nb; ++J) tl.push_back(make_int2(I, J));
-          UP(d->tiles, tl.data(), sizeof(int2) * tl.size());
-          cudaError_t e2 = cudaStreamSynchronize(st);
-          if (e2 != cudaSuccess) {
-            status = cuda_fail(e2, "upload");
-            break;
-          }
+          UP(d->tiles, T.tiles.data(), sizeof(dev::TileD) * T.tiles.size());
+          UP(d->pmap, T.pmap.data(), sizeof(int32_t) * T.pmap.size());
+          UP(d->prow, T.prow.data(), sizeof(int2) * T.prow.size());
+          UP(d->tbase, T.tbase.data(), sizeof(int2) * T.tbase.size());
         }
         cudaError_t e_ = cudaStreamSynchronize(st);  // pageable sources above go out of scope
         if (e_ != cudaSuccess) {
@@ -1407,7 +1512,7 @@ extern "C" int pb_dev_get_info(const pb_dev *d, pb_dev_info *info) {
     // streamed bytes per physical channel: per sweep entry (state pair when branch-merged)
     case PB_VARIANT_FF:
       if (d->sym)
-        info->bytes_per_channel = (double)(d->c32 ? sizeof(float2) : sizeof(float4)) * d->td.nt * dev::kTile *
+        info->bytes_per_channel = (double)(d->c32 ? sizeof(float2) : sizeof(float4)) * d->tnt * dev::kTile *
                                   dev::kTile / (double)d->nch;
       else
         info->bytes_per_channel = (2 * sizeof(float2) + (d->dense ? 0 : d->sidx16 ? 2 : 4)) *
@@ -1452,43 +1557,43 @@ int launch_stream_t(pb_dev *d, int mode, const double *fd, const float2 *fff, co
     // FP32 coefficient tiles through the bulk-copy ring (tiles32.cuh)
     float *tp = (float *)d->tpart;
     with_c32_shape(d->c32_shape, [&](auto nst, auto cps, auto half) {
-      const int gs = (int)std::max<int64_t>(1, std::min<int64_t>(d->td.nt, (int64_t)d->sm_count * cps()));
+      const int gs = (int)std::max<int64_t>(1, std::min<int64_t>(d->tnt, (int64_t)d->sm_count * cps()));
       if constexpr (decltype(half)::value) {
         const size_t sm32 = dev::c32_half_smem<nst()>();
         if (coll)
           dev::k_stream_c32_half<dev::MODE_COLL, nst(), cps()><<<gs, dev::kC32Threads, sm32, st>>>(
-              d->tiles, d->td.nt, d->tc32, fff, ns, d->td.nb, tp, d->err, nullptr, d->rev);
+              d->tiles, d->tnt, d->tc32, fff, tp, d->err, d->rev);
         else
           dev::k_stream_c32_half<dev::MODE_RATE, nst(), cps()><<<gs, dev::kC32Threads, sm32, st>>>(
-              d->tiles, d->td.nt, d->tc32, fff, ns, d->td.nb, tp, d->err, nullptr, d->rev);
+              d->tiles, d->tnt, d->tc32, fff, tp, d->err, d->rev);
       } else {
         const size_t sm32 = dev::c32_smem<nst()>();
         if (coll)
           dev::k_stream_c32<dev::MODE_COLL, nst(), cps()><<<gs, dev::kC32Threads, sm32, st>>>(
-              d->tiles, d->td.nt, d->tc32, fff, ns, d->td.nb, tp, d->err, nullptr, d->rev);
+              d->tiles, d->tnt, d->tc32, fff, tp, d->err, d->rev);
         else
           dev::k_stream_c32<dev::MODE_RATE, nst(), cps()><<<gs, dev::kC32Threads, sm32, st>>>(
-              d->tiles, d->td.nt, d->tc32, fff, ns, d->td.nb, tp, d->err, nullptr, d->rev);
+              d->tiles, d->tnt, d->tc32, fff, tp, d->err, d->rev);
       }
     });
   } else if (d->variant == PB_VARIANT_FF && d->sym && !d->c32 && part == d->part) {
     // symmetric tiles; the rate mode needs the same (A, B) partials
     if (d->sym_half && fff == d->yff) {
       const int cps = d->half_cps;
-      const int gs = (int)std::max<int64_t>(1, std::min<int64_t>(d->td.nt, (int64_t)d->sm_count * cps));
+      const int gs = (int)std::max<int64_t>(1, std::min<int64_t>(d->tnt, (int64_t)d->sm_count * cps));
       if (cps == 3)
         dev::k_stream_sym_half<2, 3><<<gs, dev::kSymThreads, dev::half_smem<2>(), st>>>(
-            d->tiles, d->td.nt, d->tcoef, fff, ns, d->td.nb, d->tpart, d->err, nullptr, d->rev);
+            d->tiles, d->tnt, d->tcoef, fff, d->tpart, d->err, d->rev);
       else
         dev::k_stream_sym_half<3, 2><<<gs, dev::kSymThreads, dev::half_smem<3>(), st>>>(
-            d->tiles, d->td.nt, d->tcoef, fff, ns, d->td.nb, d->tpart, d->err, nullptr, d->rev);
+            d->tiles, d->tnt, d->tcoef, fff, d->tpart, d->err, d->rev);
     } else if (d->sym_nt && fff == d->yff) {  // the bulk copies read f from this padded arena buffer
-      const int gs = (int)std::max<int64_t>(1, std::min<int64_t>(d->td.nt, (int64_t)d->sm_count));
-      dev::k_stream_sym_bulk<<<gs, dev::kSymThreads, dev::kSymBulkSmem, st>>>(d->tiles, d->td.nt, d->tcoef, fff, ns,
-                                                                              d->td.nb, d->tpart, d->err);
+      const int gs = (int)std::max<int64_t>(1, std::min<int64_t>(d->tnt, (int64_t)d->sm_count));
+      dev::k_stream_sym_bulk<<<gs, dev::kSymThreads, dev::kSymBulkSmem, st>>>(d->tiles, d->tnt, d->tcoef, fff,
+                                                                              d->tpart, d->err);
     } else {
-      const int gs = (int)std::max<int64_t>(1, std::min<int64_t>(d->td.nt, (int64_t)d->sm_count * 3));
-      dev::k_stream_sym<<<gs, 256, 0, st>>>(d->tiles, d->td.nt, d->tcoef, fff, ns, d->td.nb, d->tpart);
+      const int gs = (int)std::max<int64_t>(1, std::min<int64_t>(d->tnt, (int64_t)d->sm_count * 3));
+      dev::k_stream_sym<<<gs, 256, 0, st>>>(d->tiles, d->tnt, d->tcoef, fff, d->tpart);
     }
   } else if (d->variant == PB_VARIANT_FF) {
     const float4 *A4 = (const float4 *)d->coefA, *B4 = (const float4 *)d->coefB;
@@ -1587,17 +1692,17 @@ void launch_fin(pb_dev *d, const double *ysrc, double *out, double *f, double dt
   else if (d->sym && d->c32)
     if (fin_small(d))
       dev::k_fin_c32<STAGE, false, 8><<<(int)((d->ns + 7) / 8), 256, 0, st>>>(
-          (const float *)d->tpart, d->td.nb, d->td.nsp, (int)d->ns, d->c, ysrc, out, f, d->acc, y, d->yff, dt);
+          (const float *)d->tpart, d->prow, d->pmap, (int)d->ns, d->c, ysrc, out, f, d->acc, y, d->yff, dt);
     else
       dev::k_fin_c32<STAGE><<<(int)((d->ns + 31) / 32), 256, 0, st>>>(
-          (const float *)d->tpart, d->td.nb, d->td.nsp, (int)d->ns, d->c, ysrc, out, f, d->acc, y, d->yff, dt);
+          (const float *)d->tpart, d->prow, d->pmap, (int)d->ns, d->c, ysrc, out, f, d->acc, y, d->yff, dt);
   else if (d->sym)
     if (fin_small(d))
       dev::k_fin_tiles<STAGE, false, 8><<<(int)((d->ns + 7) / 8), 256, 0, st>>>(
-          dev::TileSrc{d->tpart, d->td.nb, d->td.nsp}, (int)d->ns, d->c, d->R, ysrc, out, f, d->acc, y, d->yff, dt);
+          d->tile_src(), (int)d->ns, d->c, d->R, ysrc, out, f, d->acc, y, d->yff, dt);
     else
       dev::k_fin_tiles<STAGE><<<(int)((d->ns + 31) / 32), 256, 0, st>>>(
-          dev::TileSrc{d->tpart, d->td.nb, d->td.nsp}, (int)d->ns, d->c, d->R, ysrc, out, f, d->acc, y, d->yff, dt);
+          d->tile_src(), (int)d->ns, d->c, d->R, ysrc, out, f, d->acc, y, d->yff, dt);
   else
     dev::k_fin_coll<false, STAGE><<<fin_grid(d), kFinBlock, 0, st>>>(dev::ItemSrc{d->item_ptr, d->part}, (int)d->ns, d->c, d->R, ysrc,
                                                                      out, f, d->acc, y, d->yff, dt);
@@ -1613,6 +1718,12 @@ int to_ff(pb_dev *d, const double *x, int64_t n, float2 *out, cudaStream_t st) {
 // Stage-input conversion the streaming kernel of this variant reads (once per call: splitting
 // f inside every CTA of the sweep instead costs more, FP64 being slow on this part).
 int stage_input(pb_dev *d, const double *f, cudaStream_t st) {
+  if (d->variant == PB_VARIANT_FF && d->sym) {  // in the tiles' energy order
+    dev::k_to_ff_map<<<(int)std::max<int64_t>(1, std::min<int64_t>((d->ns + 255) / 256, 1024)), 256, 0, st>>>(
+        f, (int)d->ns, d->pmap, d->yff);
+    PB_LAUNCHED("k_to_ff_map");
+    return PB_OK;
+  }
   if (d->variant == PB_VARIANT_FF || d->variant == PB_VARIANT_PAPER) return to_ff(d, f, d->ns, d->yff, st);
   if (d->mixed()) {
     dev::k_gstate_f<<<(int)((d->ns + 255) / 256), 256, 0, st>>>(f, (int)d->ns, d->gstate);
@@ -1918,20 +2029,20 @@ int rates_seq(pb_dev *d, const double *f, double *inv_tau, cudaStream_t st) {
     dev::k_fin_rate<true><<<fin_grid(d), kFinBlock, 0, st>>>(dev::ItemSrc{d->fwd_item_ptr(), d->part}, (int)d->ns,
                                                              d->mixed() ? d->gscale() : d->c, d->R, inv_tau);
   else if (d->sym && d->c32 && fin_small(d))
-    dev::k_fin_c32<-1, true, 8><<<(int)((d->ns + 7) / 8), 256, 0, st>>>((const float *)d->tpart, d->td.nb, d->td.nsp,
+    dev::k_fin_c32<-1, true, 8><<<(int)((d->ns + 7) / 8), 256, 0, st>>>((const float *)d->tpart, d->prow, d->pmap,
                                                                        (int)d->ns, d->c, nullptr, inv_tau, nullptr,
                                                                        nullptr, nullptr, nullptr, 0.0);
   else if (d->sym && d->c32)
-    dev::k_fin_c32<-1, true><<<(int)((d->ns + 31) / 32), 256, 0, st>>>((const float *)d->tpart, d->td.nb, d->td.nsp,
+    dev::k_fin_c32<-1, true><<<(int)((d->ns + 31) / 32), 256, 0, st>>>((const float *)d->tpart, d->prow, d->pmap,
                                                                        (int)d->ns, d->c, nullptr, inv_tau, nullptr,
                                                                        nullptr, nullptr, nullptr, 0.0);
   else if (d->sym && fin_small(d))
     dev::k_fin_tiles<-1, true, 8><<<(int)((d->ns + 7) / 8), 256, 0, st>>>(
-        dev::TileSrc{d->tpart, d->td.nb, d->td.nsp}, (int)d->ns, d->c, d->R, nullptr, inv_tau, nullptr, nullptr, nullptr,
+        d->tile_src(), (int)d->ns, d->c, d->R, nullptr, inv_tau, nullptr, nullptr, nullptr,
         nullptr, 0.0);
   else if (d->sym)
     dev::k_fin_tiles<-1, true><<<(int)((d->ns + 31) / 32), 256, 0, st>>>(
-        dev::TileSrc{d->tpart, d->td.nb, d->td.nsp}, (int)d->ns, d->c, d->R, nullptr, inv_tau, nullptr, nullptr, nullptr,
+        d->tile_src(), (int)d->ns, d->c, d->R, nullptr, inv_tau, nullptr, nullptr, nullptr,
         nullptr, 0.0);
   else
     dev::k_fin_rate<false><<<fin_grid(d), kFinBlock, 0, st>>>(dev::ItemSrc{d->item_ptr, d->part}, (int)d->ns, d->c, d->R, inv_tau);
@@ -2132,36 +2243,24 @@ int coef_setup(pb_dev *d, cudaStream_t st) {
       else    dev::k_pair_coef<false><<<pg, 256, 0, st>>>(cs, d->pcnt, (long long)d->nsw, d->ccoefA, d->ccoefB, d->coefA, d->coefB, 1.0, d->g2);
       PB_LAUNCHED("k_pair_coef");
     }
-    if (d->sym && !d->complete) {
-      // rows that miss some partners: the tiles zeroed, then every stored pair scattered in
-      const size_t tb = (size_t)d->td.nt * dev::kTile * dev::kTile * (d->c32 ? sizeof(float2) : sizeof(float4));
+    if (d->sym) {
+      // the tiles zeroed, then every stored pair scattered in
+      const size_t tb = (size_t)d->tnt * dev::kTile * dev::kTile * (d->c32 ? sizeof(float2) : sizeof(float4));
       void *tc = d->c32 ? (void *)d->tc32 : (void *)d->tcoef;
       PB_CUDA(cudaMemsetAsync(tc, 0, tb, st));
       const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((d->ns * 32 + 255) / 256, (int64_t)d->sm_count * 8));
       const long long *srp = (const long long *)d->srp;
       const float2 *cA = (const float2 *)d->coefA, *cB = (const float2 *)d->coefB;
-      const int ns = (int)d->ns, nb = d->td.nb;
+      const int ns = (int)d->ns;
       if (d->c32 && d->sidx16)
-        dev::k_tiles_scatter<true, uint16_t><<<grid, 256, 0, st>>>(srp, ns, d->sidx16, cA, cB, nullptr, nullptr, nb, tc);
+        dev::k_tiles_scatter<true, uint16_t><<<grid, 256, 0, st>>>(srp, ns, d->sidx16, cA, cB, d->pmap, d->tbase, tc);
       else if (d->c32)
-        dev::k_tiles_scatter<true, uint32_t><<<grid, 256, 0, st>>>(srp, ns, d->sidx32, cA, cB, nullptr, nullptr, nb, tc);
+        dev::k_tiles_scatter<true, uint32_t><<<grid, 256, 0, st>>>(srp, ns, d->sidx32, cA, cB, d->pmap, d->tbase, tc);
       else if (d->sidx16)
-        dev::k_tiles_scatter<false, uint16_t><<<grid, 256, 0, st>>>(srp, ns, d->sidx16, cA, cB, nullptr, nullptr, nb, tc);
+        dev::k_tiles_scatter<false, uint16_t><<<grid, 256, 0, st>>>(srp, ns, d->sidx16, cA, cB, d->pmap, d->tbase, tc);
       else
-        dev::k_tiles_scatter<false, uint32_t><<<grid, 256, 0, st>>>(srp, ns, d->sidx32, cA, cB, nullptr, nullptr, nb, tc);
+        dev::k_tiles_scatter<false, uint32_t><<<grid, 256, 0, st>>>(srp, ns, d->sidx32, cA, cB, d->pmap, d->tbase, tc);
       PB_LAUNCHED("k_tiles_scatter");
-    } else if (d->sym) {
-      const long long n = (long long)d->td.nt * dev::kTile * dev::kTile;
-      const int grid = (int)std::min<long long>((n + 255) / 256, 8192);
-      if (d->c32)
-        dev::k_tiles_fill_c32<<<grid, 256, 0, st>>>(d->tiles, d->td.nt, (const float2 *)d->coefA,
-                                                    (const float2 *)d->coefB, (const long long *)d->srp, (int)d->ns,
-                                                    d->tc32);
-      else
-        dev::k_tiles_fill<<<grid, 256, 0, st>>>(d->tiles, d->td.nt, (const float2 *)d->coefA,
-                                                (const float2 *)d->coefB, (const long long *)d->srp, (int)d->ns,
-                                                d->tcoef);
-      PB_LAUNCHED("k_tiles_fill");
     }
   }
   if (d->mixed()) {

@@ -181,7 +181,7 @@ __global__ void k_to_ff(const double *__restrict__ x, long long n, float2 *__res
     out[i] = ff_split(x[i]);
 }
 
-// the same into a padded state space: out[pmap[i]] (the padding keeps its zeros)
+// the same into the tiles' padded energy order: out[pmap[i]] (the padding keeps its zeros)
 __global__ void k_to_ff_map(const double *__restrict__ x, int n, const int *__restrict__ pmap,
                             float2 *__restrict__ out) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) out[pmap[i]] = ff_split(x[i]);
@@ -2149,61 +2149,57 @@ __global__ void __launch_bounds__(kBlock) k_paper_gather(const Item *__restrict_
   }
 }
 
-// ------------------------------------------------------------ symmetric tiles (complete rows)
+// ------------------------------------------------------------ symmetric tiles
 //
-// When every row holds every window state, the branch-merged pair matrix is dense, and the
-// reverse channels fix its transpose: P_in(p,s) = P_out(s,p) and P_out(p,s) = P_in(s,p). It is
-// stored as 64 x 64 tiles of its upper block triangle, (P_in hi, P_in lo, P_out hi, P_out lo)
-// per entry. Each off-diagonal tile adds to its rows (partners = its columns) and to its
-// columns (partners = its rows):
+// The reverse channels fix the transpose of the branch-merged pair matrix: P_in(p,s) = P_out(s,p)
+// and P_out(p,s) = P_in(s,p).  It is stored as 64 x 64 tiles of its upper block triangle,
+// (P_in hi, P_in lo, P_out hi, P_out lo) per entry, zero where a pair has no channel.  Each
+// off-diagonal tile adds to its rows (partners = its columns) and to its columns (partners = its
+// rows):
 //   row s:  A += f_p P_in(s,p),   C += f_p P_out(s,p)
 //   col p:  A += f_s P_out(s,p),  C += f_s P_in(s,p)
-// so each state gets B = C - A = sum f D, as in the row stream. Diagonal tiles hold all
-// 64 x 64 entries and add to their rows only. Every tile writes one (A, B) per row and per
-// column into tp[state][partner block], so each state receives exactly one partial per block
-// of partner states, stored contiguously; the epilogue adds them in block order (no atomics).
+// so each state gets B = C - A = sum f D, as in the row stream.  Diagonal tiles hold all
+// 64 x 64 entries and add to their rows only.
+//
+// Energy order.  The tiles index the states sorted by energy, each system's states padded to
+// whole blocks.  A pair further apart in energy than the largest phonon energy plus 15 or so
+// widths of the delta function has coefficients below the smallest FP32 number, stored as exact
+// zeros (the host derives the distance, energy_reach), so in energy order the nonzero part of the
+// matrix is a band along the diagonal, and only the tiles that meet it are stored and streamed:
+// 1017 of the 2850 tiles of the 40^3 window (66.6 MB instead of 187 MB, so that the sweeps of an
+// RK4 step find them in the 129 MB L2), with the same sums.
+//
+// Every tile writes one (A, C) per row and per column into tp; the slots of a state are one per
+// stored tile of its block row, contiguous, so each state receives exactly one partial per block
+// of partner states; the epilogue adds them in block order (no atomics).
 
 constexpr int kTile = 64;
 
-// tc[t][i][j] from the branch-merged coefficients of complete rows (entry (s, p) of row s is
-// at srp[s] + p); zero outside the nstate states.
-__global__ void k_tiles_fill(const int2 *__restrict__ tiles, int nt, const float2 *__restrict__ coefA,
-                             const float2 *__restrict__ coefB, const long long *__restrict__ srp, int ns,
-                             float4 *__restrict__ tc) {
-  const long long n = (long long)nt * kTile * kTile;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-    const int t = (int)(e / (kTile * kTile)), k = (int)(e % (kTile * kTile));
-    const int2 IJ = tiles[t];
-    const int s = IJ.x * kTile + k / kTile, p = IJ.y * kTile + k % kTile;
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (s < ns && p < ns) {
-      const long long c = srp[s] + p;
-      const float2 a = coefA[c], b = coefB[c];
-      const double pin = ff_to_double(a.x, a.y), pout = pin + ff_to_double(b.x, b.y);
-      const float2 x = ff_split(pin), y = ff_split(pout);
-      v = make_float4(x.x, x.y, y.x, y.y);
-    }
-    tc[e] = v;
-  }
+// One stored tile: its block row I and block column J, and where its partials go: state i of
+// block I has its slot at rb + i * rs, state j of block J at cb + j * cs.
+struct alignas(16) TileD {
+  int I, J, rb, rs, cb, cs, pad0, pad1;
+};
+__device__ __forceinline__ TileD load_tile(const TileD *__restrict__ tiles, int t) {
+  const int4 a = reinterpret_cast<const int4 *>(tiles + t)[0], b = reinterpret_cast<const int4 *>(tiles + t)[1];
+  return TileD{a.x, a.y, a.z, a.w, b.x, b.y, 0, 0};
 }
 
 // One tile per CTA trip (grid-stride over tiles); thread (ti, tj) takes rows 4ti..4ti+3 and
 // columns 4tj..4tj+3 of the tile, so a warp reads two 1 KB row segments per step.  The four
 // terms a thread adds per row (per column) use lazily renormalised float-float sums; the 16
 // thread partials of a row (column) are then added with full float-float additions.
-__global__ void __launch_bounds__(256, 3) k_stream_sym(const int2 *__restrict__ tiles, int nt,
+__global__ void __launch_bounds__(256, 3) k_stream_sym(const TileD *__restrict__ tiles, int nt,
                                                        const float4 *__restrict__ tc,
-                                                       const float2 *__restrict__ fg, int ns, int nb,
-                                                       float4 *__restrict__ tp) {
+                                                       const float2 *__restrict__ fg, float4 *__restrict__ tp) {
   __shared__ float2 fr[kTile], fc[kTile];
   __shared__ float4 red[2][kTile][17];  // [rows | cols][state][thread] (A hi, A lo, C hi, C lo); 17: no bank clash
   const int tid = threadIdx.x, ti = tid >> 4, tj = tid & 15;
   for (int t = blockIdx.x; t < nt; t += gridDim.x) {
-    const int2 IJ = tiles[t];
-    const bool diag = IJ.x == IJ.y;
-    const int r0 = IJ.x * kTile, c0 = IJ.y * kTile;
-    if (tid < kTile) fr[tid] = r0 + tid < ns ? fg[r0 + tid] : make_float2(0.f, 0.f);
-    else if (tid < 2 * kTile) fc[tid - kTile] = c0 + tid - kTile < ns ? fg[c0 + tid - kTile] : make_float2(0.f, 0.f);
+    const TileD D = tiles[t];
+    const bool diag = D.I == D.J;
+    if (tid < kTile) fr[tid] = fg[D.I * kTile + tid];
+    else if (tid < 2 * kTile) fc[tid - kTile] = fg[D.J * kTile + tid - kTile];
     __syncthreads();
     float2 fcol[4];
 #pragma unroll
@@ -2247,9 +2243,7 @@ __global__ void __launch_bounds__(256, 3) k_stream_sym(const int2 *__restrict__ 
         A = ff_add(A, make_float2(v.x, v.y));
         C = ff_add(C, make_float2(v.z, v.w));
       }
-      const int st = (side == 0 ? r0 : c0) + x;
-      const int blk = side == 0 ? IJ.y : IJ.x;
-      tp[(long long)st * nb + blk] = make_float4(A.x, A.y, C.x, C.y);
+      tp[side == 0 ? D.rb + x * D.rs : D.cb + x * D.cs] = make_float4(A.x, A.y, C.x, C.y);
     }
     __syncthreads();
   }
@@ -2270,13 +2264,12 @@ constexpr int kSymThreads = 256;
 constexpr unsigned kTileBytes = kTile * kTile * sizeof(float4);
 constexpr unsigned kSymStageBytes = kTileBytes + 2 * kTile * sizeof(float2);
 constexpr size_t kSymColBytes = (size_t)(kSymThreads / 32) * 2 * kTile * sizeof(float2);  // one column table
-constexpr size_t kSymBulkSmem = (size_t)kSymStages * kSymStageBytes + 64 + 2 * kSymColBytes;
+constexpr size_t kSymBulkSmem = (size_t)kSymStages * kSymStageBytes + 128 + 2 * kSymColBytes;
 
 // the column partials of a finished off-diagonal tile: one (column, A | C) value per lane pair
-// (lanes l and l ^ 16 take warps 0-3 and 4-7), renormalised, into tp (slot: the tile's row block,
-// slotI; the batched sweep numbers a state's partner blocks within its instance)
-__device__ __forceinline__ void sym_columns_out(const float2 *__restrict__ colred, int2 IJ, int slotI, int nb, int lane,
-                                                int wid, float4 *__restrict__ tp) {
+// (lanes l and l ^ 16 take warps 0-3 and 4-7), renormalised, into the tile's column slots of tp
+__device__ __forceinline__ void sym_columns_out(const float2 *__restrict__ colred, int cb, int cs, int lane, int wid,
+                                                float4 *__restrict__ tp) {
   constexpr int NW = kSymThreads / 32, WG = NW / 2;
   const int g = lane >> 4;
   const int q = (lane & 15) + 16 * wid;  // 0 .. 127
@@ -2285,52 +2278,45 @@ __device__ __forceinline__ void sym_columns_out(const float2 *__restrict__ colre
 #pragma unroll
   for (int w = 1; w < WG; ++w) acc = ff_add(acc, colred[((g * WG + w) * 2 + comp) * kTile + col]);
   acc = ff_add(acc, make_float2(__shfl_xor_sync(0xFFFFFFFFu, acc.x, 16), __shfl_xor_sync(0xFFFFFFFFu, acc.y, 16)));
-  if (g == 0) ((float2 *)tp)[2 * ((long long)(IJ.y * kTile + col) * nb + slotI) + comp] = acc;
+  if (g == 0) ((float2 *)tp)[2 * (cb + col * cs) + comp] = acc;
 }
 
-__global__ void __launch_bounds__(kSymThreads, 1) k_stream_sym_bulk(const int2 *__restrict__ tiles, int nt,
+__global__ void __launch_bounds__(kSymThreads, 1) k_stream_sym_bulk(const TileD *__restrict__ tiles, int nt,
                                                                      const float4 *__restrict__ tc,
-                                                                     const float2 *__restrict__ fg, int ns, int nb,
+                                                                     const float2 *__restrict__ fg,
                                                                      float4 *__restrict__ tp, int *__restrict__ err) {
   constexpr int R = 4, NV = 2 * R;
   extern __shared__ __align__(128) unsigned char ssm[];
   unsigned long long *bars = (unsigned long long *)(ssm + kSymStages * kSymStageBytes);
-  int2 *stile = (int2 *)(bars + kSymStages);  // the tile held by each stage
-  float2 *colred0 = (float2 *)(ssm + kSymStages * kSymStageBytes + 64);  // 2 x [8 warps][A | C][64 columns]
+  TileD *stile = (TileD *)(bars + 4);  // the tile held by each stage
+  float2 *colred0 = (float2 *)(ssm + kSymStages * kSymStageBytes + 128);  // 2 x [8 warps][A | C][64 columns]
+  static_assert(kSymStages <= 3, "barriers and tile descriptors share 128 bytes");
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, tj = tid & 15, ti = tid >> 4;
   const int G = (int)gridDim.x;
   const int nloc = (int)blockIdx.x < nt ? (nt - 1 - (int)blockIdx.x) / G + 1 : 0;
-  // the f slices of every stage start as zeros (a copy of a last, partial block leaves the rest)
-  for (int i = tid; i < kSymStages * 2 * kTile; i += kSymThreads) {
-    float2 *fz = (float2 *)(ssm + (i / (2 * kTile)) * kSymStageBytes + kTileBytes);
-    fz[i % (2 * kTile)] = make_float2(0.f, 0.f);
-  }
   if (tid == 0) {
     for (int k = 0; k < kSymStages; ++k) mbar_init(bars + k, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  fence_proxy_async();  // the zeroed f slices before any bulk write to them
   __syncthreads();
   int issued = 0;
-  auto issue = [&](int k, int2 IJ) {
+  auto issue = [&](int k, const TileD &D) {
     const int s = k % kSymStages;
     const int t = (int)blockIdx.x + k * G;
-    stile[s] = IJ;
+    stile[s] = D;
     unsigned char *buf = ssm + (size_t)s * kSymStageBytes;
-    const int nr = min(kTile, ns - IJ.x * kTile), nc = min(kTile, ns - IJ.y * kTile);
-    const unsigned br = (unsigned)(nr * sizeof(float2) + 15) / 16 * 16, bc = (unsigned)(nc * sizeof(float2) + 15) / 16 * 16;
-    mbar_expect_tx(bars + s, kTileBytes + br + bc);
+    mbar_expect_tx(bars + s, kSymStageBytes);
     const unsigned char *src = (const unsigned char *)(tc + (size_t)t * kTile * kTile);
 #pragma unroll
     for (int q = 0; q < 4; ++q) bulk_g2s(buf + q * (kTileBytes / 4), src + q * (kTileBytes / 4), kTileBytes / 4, bars + s);
-    bulk_g2s(buf + kTileBytes, fg + (size_t)IJ.x * kTile, br, bars + s);
-    bulk_g2s(buf + kTileBytes + kTile * sizeof(float2), fg + (size_t)IJ.y * kTile, bc, bars + s);
+    bulk_g2s(buf + kTileBytes, fg + (size_t)D.I * kTile, kTile * sizeof(float2), bars + s);
+    bulk_g2s(buf + kTileBytes + kTile * sizeof(float2), fg + (size_t)D.J * kTile, kTile * sizeof(float2), bars + s);
   };
   if (tid == 0)
-    for (; issued < kSymStages && issued < nloc; ++issued) issue(issued, tiles[(int)blockIdx.x + issued * G]);
-  int2 nextIJ = make_int2(0, 0);  // thread 0: descriptor of the next tile to issue, loaded a tile ahead
-  if (tid == 0 && issued < nloc) nextIJ = tiles[(int)blockIdx.x + issued * G];
-  int2 prevIJ = make_int2(0, 0);  // the previous tile (its columns are combined in this iteration)
+    for (; issued < kSymStages && issued < nloc; ++issued) issue(issued, load_tile(tiles, (int)blockIdx.x + issued * G));
+  TileD next{};  // thread 0: descriptor of the next tile to issue, loaded a tile ahead
+  if (tid == 0 && issued < nloc) next = load_tile(tiles, (int)blockIdx.x + issued * G);
+  int pcb = -1, pcs = 0;  // column slots of the previous tile (combined in this iteration), -1: none
   bool ok = true;
   for (int k = 0; k <= nloc; ++k) {
     // thread 0 waits on the mbarrier of tile k (acquire); the CTA barrier publishes the stage
@@ -2342,17 +2328,17 @@ __global__ void __launch_bounds__(kSymThreads, 1) k_stream_sym_bulk(const int2 *
     }
     if (tid == 0 && k >= 1 && issued < nloc) {
       fence_proxy_async();  // order the generic reads of tile k-1's stage before its refill
-      issue(issued, nextIJ);
+      issue(issued, next);
       ++issued;
-      if (issued < nloc) nextIJ = tiles[(int)blockIdx.x + issued * G];
+      if (issued < nloc) next = load_tile(tiles, (int)blockIdx.x + issued * G);
     }
-    if (k >= 1 && prevIJ.x != prevIJ.y)
-      sym_columns_out(colred0 + ((k - 1) & 1) * (kSymColBytes / sizeof(float2)), prevIJ, prevIJ.x, nb, lane, wid, tp);
+    if (k >= 1 && pcb >= 0) sym_columns_out(colred0 + ((k - 1) & 1) * (kSymColBytes / sizeof(float2)), pcb, pcs, lane, wid, tp);
     if (!have) break;
     const int s = k % kSymStages;
-    const int2 IJ = stile[s];
-    prevIJ = IJ;
-    const bool diag = IJ.x == IJ.y;
+    const TileD D = stile[s];
+    const bool diag = D.I == D.J;
+    pcb = diag ? -1 : D.cb;
+    pcs = D.cs;
     const float4 *__restrict__ T = (const float4 *)(ssm + (size_t)s * kSymStageBytes);
     const float2 *__restrict__ fr = (const float2 *)(ssm + (size_t)s * kSymStageBytes + kTileBytes);
     const float2 *__restrict__ fc = fr + kTile;
@@ -2399,8 +2385,7 @@ __global__ void __launch_bounds__(kSymThreads, 1) k_stream_sym_bulk(const int2 *
       ff_reduce_scatter<NV, 8>(v, lane);
       const int idx = ((tj >> 3) & 1) * 4 + ((tj >> 2) & 1) * 2 + ((tj >> 1) & 1);
       if ((tj & 1) == 0) {  // lanes tj and tj ^ 1 hold the same total
-        const int row = IJ.x * kTile + ti * R + (idx >> 1);
-        ((float2 *)tp)[2 * ((long long)row * nb + IJ.y) + (idx & 1)] = v[0];
+        ((float2 *)tp)[2 * (D.rb + (ti * R + (idx >> 1)) * D.rs) + (idx & 1)] = v[0];
       }
     }
     if (!diag) {
@@ -2444,76 +2429,64 @@ constexpr unsigned kHalfTileBytes = kTileBytes / 2;
 constexpr unsigned kHalfStageBytes = kHalfTileBytes + (kTile / 2 + kTile) * sizeof(float2);
 template <int NST>
 constexpr size_t half_smem() {
-  return (size_t)NST * kHalfStageBytes + 64 + kSymColBytes;
+  return (size_t)NST * kHalfStageBytes + 192 + kSymColBytes;
 }
 
 // NST stages per CTA, CPS resident CTAs per SM (3 x 2 or 2 x 3 fit in the SM's shared memory)
-// lblk (batched sweep, else null): the block index of each block within its instance, which
-// numbers the partial slots; blocks are global otherwise.  rev: take the tile list from its end
-// (tile nt - 1 - t in place of t), so that a sweep following one in list order starts on the
-// tiles the L2 still holds; the partials do not depend on the order.
+// rev: take the tile list from its end (tile nt - 1 - t in place of t), so that a sweep following
+// one in list order starts on the tiles the L2 still holds; the partials do not depend on the order.
 template <int NST, int CPS>
-__global__ void __launch_bounds__(kSymThreads, CPS) k_stream_sym_half(const int2 *__restrict__ tiles, int nt,
+__global__ void __launch_bounds__(kSymThreads, CPS) k_stream_sym_half(const TileD *__restrict__ tiles, int nt,
                                                                        const float4 *__restrict__ tc,
-                                                                       const float2 *__restrict__ fg, int ns, int nb,
+                                                                       const float2 *__restrict__ fg,
                                                                        float4 *__restrict__ tp, int *__restrict__ err,
-                                                                       const int *__restrict__ lblk = nullptr,
                                                                        int rev = 0) {
   constexpr int kHalfStages = NST;
   static_assert(NST >= 2 && NST <= 4, "the ring needs 2..4 stages");
   constexpr int R = 2, NV = 2 * R, HR = kTile / 2;
   extern __shared__ __align__(128) unsigned char ssm[];
   unsigned long long *bars = (unsigned long long *)(ssm + kHalfStages * kHalfStageBytes);
-  int2 *stile = (int2 *)(bars + kHalfStages);  // the tile of each stage's unit
-  float2 *colred = (float2 *)(ssm + kHalfStages * kHalfStageBytes + 64);  // [8 warps][A | C][64 columns]
+  TileD *stile = (TileD *)(bars + 4);  // the tile of each stage's unit
+  float2 *colred = (float2 *)(ssm + kHalfStages * kHalfStageBytes + 192);  // [8 warps][A | C][64 columns]
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, tj = tid & 15, ti = tid >> 4;
   const int G = (int)gridDim.x;
   const int nloc = (int)blockIdx.x < nt ? (nt - 1 - (int)blockIdx.x) / G + 1 : 0;
   const int nunit = 2 * nloc;
-  for (int i = tid; i < kHalfStages * (HR + kTile); i += kSymThreads) {
-    float2 *fz = (float2 *)(ssm + (i / (HR + kTile)) * kHalfStageBytes + kHalfTileBytes);
-    fz[i % (HR + kTile)] = make_float2(0.f, 0.f);
-  }
   if (tid == 0) {
     for (int k = 0; k < kHalfStages; ++k) mbar_init(bars + k, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  fence_proxy_async();
   __syncthreads();
-  // thread 0: units are issued in order; issIJ is the tile being issued, aheadIJ the next one
+  // thread 0: units are issued in order; iss is the tile being issued, ahead the next one
   int issued = 0;
   auto tix = [&](int k) {  // the CTA's k-th tile
     const int t = (int)blockIdx.x + k * G;
     return rev ? nt - 1 - t : t;
   };
-  int2 issIJ = make_int2(0, 0), aheadIJ = make_int2(0, 0);
+  TileD iss{}, ahead{};
   if (tid == 0 && nloc > 0) {
-    issIJ = tiles[tix(0)];
-    if (nloc > 1) aheadIJ = tiles[tix(1)];
+    iss = load_tile(tiles, tix(0));
+    if (nloc > 1) ahead = load_tile(tiles, tix(1));
   }
   auto issue = [&](int v) {  // unit v = 2 k + h: half h of the CTA's tile k
     const int k = v >> 1, h = v & 1, s = v % kHalfStages;
     if (h == 0 && k > 0) {
-      issIJ = aheadIJ;
-      if (k + 1 < nloc) aheadIJ = tiles[tix(k + 1)];
+      iss = ahead;
+      if (k + 1 < nloc) ahead = load_tile(tiles, tix(k + 1));
     }
     const int t = tix(k);
-    stile[s] = issIJ;
+    stile[s] = iss;
     unsigned char *buf = ssm + (size_t)s * kHalfStageBytes;
-    const int nr = min(HR, ns - (issIJ.x * kTile + h * HR)), nc = min(kTile, ns - issIJ.y * kTile);
-    const unsigned br = nr > 0 ? (unsigned)(nr * sizeof(float2) + 15) / 16 * 16 : 0u;
-    const unsigned bc = (unsigned)(nc * sizeof(float2) + 15) / 16 * 16;
-    mbar_expect_tx(bars + s, kHalfTileBytes + br + bc);
+    mbar_expect_tx(bars + s, kHalfStageBytes);
     const unsigned char *src = (const unsigned char *)(tc + (size_t)t * kTile * kTile) + (size_t)h * kHalfTileBytes;
 #pragma unroll
     for (int q = 0; q < 2; ++q) bulk_g2s(buf + q * (kHalfTileBytes / 2), src + q * (kHalfTileBytes / 2), kHalfTileBytes / 2, bars + s);
-    if (br) bulk_g2s(buf + kHalfTileBytes, fg + (size_t)issIJ.x * kTile + h * HR, br, bars + s);
-    bulk_g2s(buf + kHalfTileBytes + HR * sizeof(float2), fg + (size_t)issIJ.y * kTile, bc, bars + s);
+    bulk_g2s(buf + kHalfTileBytes, fg + (size_t)iss.I * kTile + h * HR, HR * sizeof(float2), bars + s);
+    bulk_g2s(buf + kHalfTileBytes + HR * sizeof(float2), fg + (size_t)iss.J * kTile, kTile * sizeof(float2), bars + s);
   };
   if (tid == 0)
     for (; issued < kHalfStages && issued < nunit; ++issued) issue(issued);
-  int2 prevIJ = make_int2(0, 0);  // the tile of the previous unit
-  int prevI = 0;                  // its row block's slot index
+  int pcb = -1, pcs = 0;  // column slots of the previous unit's tile (-1: diagonal, or none)
   bool ok = true;
   float cA[4][2], cC[4][2];  // column sums of the current tile, carried across its halves
   for (int u = 0; u <= nunit; ++u) {
@@ -2529,14 +2502,13 @@ __global__ void __launch_bounds__(kSymThreads, CPS) k_stream_sym_half(const int2
       ++issued;
     }
     // the previous tile's column table (written after its second half) is complete
-    if ((u & 1) == 0 && u >= 2 && prevIJ.x != prevIJ.y) sym_columns_out(colred, prevIJ, prevI, nb, lane, wid, tp);
+    if ((u & 1) == 0 && u >= 2 && pcb >= 0) sym_columns_out(colred, pcb, pcs, lane, wid, tp);
     if (!have) break;
     const int s = u % kHalfStages, h = u & 1;
-    const int2 IJ = stile[s];
-    const int Il = lblk ? lblk[IJ.x] : IJ.x, Jl = lblk ? lblk[IJ.y] : IJ.y;  // slot blocks
-    prevIJ = IJ;
-    prevI = Il;
-    const bool diag = IJ.x == IJ.y;
+    const TileD D = stile[s];
+    const bool diag = D.I == D.J;
+    pcb = diag ? -1 : D.cb;
+    pcs = D.cs;
     const float4 *__restrict__ T = (const float4 *)(ssm + (size_t)s * kHalfStageBytes);
     const float2 *__restrict__ fr = (const float2 *)(ssm + (size_t)s * kHalfStageBytes + kHalfTileBytes);
     const float2 *__restrict__ fc = fr + HR;
@@ -2582,8 +2554,7 @@ __global__ void __launch_bounds__(kSymThreads, CPS) k_stream_sym_half(const int2
       ff_reduce_scatter<NV, 8>(v, lane);
       const int idx = tj >> 2;
       if ((tj & 3) == 0) {
-        const int row = IJ.x * kTile + h * HR + ti * R + (idx >> 1);
-        ((float2 *)tp)[2 * ((long long)row * nb + Jl) + (idx & 1)] = v[0];
+        ((float2 *)tp)[2 * (D.rb + (h * HR + ti * R + (idx >> 1)) * D.rs) + (idx & 1)] = v[0];
       }
     }
     if (!diag && h == 1) {
@@ -2636,12 +2607,9 @@ struct ItemSrc {
   __device__ __forceinline__ void get(int r, double &A, double &B) const { row_partials(item_ptr, part, r, A, B); }
 };
 struct TileSrc {
-  const float4 *tp;  // [nsp][nb]: state-major, one partial (A hi, A lo, C hi, C lo) per block of partner states
-  int nb, nsp;
-  // batched tiles: the padded row of every state and the block table (the number of partner
-  // blocks of a state is its system's, binfo[block].w); null for one system
-  const int *pmap = nullptr;
-  const int4 *binfo = nullptr;
+  const float4 *tp;  // one partial (A hi, A lo, C hi, C lo) per state and block of partner states
+  const int2 *prow;  // per state: its first slot in tp and its number of slots
+  const int *pmap;   // per state: its row in the padded energy order (the float-float stage input's)
 };
 
 // Collision epilogue fused with the RK4 stage arithmetic.
@@ -2666,7 +2634,7 @@ __device__ __forceinline__ FinIn fin_load(int r, const double *__restrict__ R, c
 }
 
 // out[r] = I (STAGE < 0), or the RK4 stage arithmetic with k_{STAGE+1} = I
-// ry: the state's row of yff when that is a padded state space (batched tiles), else r
+// ry: the state's row of yff when that is in the tiles' padded energy order, else r
 template <int STAGE, bool GSTATE>
 __device__ __forceinline__ void fin_stage(int r, double I, const FinIn &in, double *__restrict__ out,
                                           double *__restrict__ f, double *__restrict__ acc, double *__restrict__ y,
@@ -2739,25 +2707,27 @@ __global__ void __launch_bounds__(256) k_fin_tiles(TileSrc src, int ns, double c
   // warp 0 loads its state's epilogue inputs first, so that their latency overlaps the partials'
   const int r0 = base + lane;
   FinIn in{0.0, 0.0, 0.0, 0.0};
+  int ry = 0;
   if (wid == 0 && lane < SPC && r0 < ns) {
     if (RATE) in.R = R[r0];
     else in = fin_load<false, STAGE>(r0, R, ysrc, f, acc);
+    if (STAGE >= 0) ry = src.pmap[r0];
   }
-  // partials are stored for every padded state (r < nsp); the first three of every lane for
-  // the warp's states are loaded together (up to 96 partner blocks), the rest after
-  const int nb = src.nb;
+  // the first three partials of every lane for the warp's states are loaded together (up to 96
+  // partner blocks), the rest after
   float4 w[SPW][3];
-  int nbq[SPW];  // partner blocks of each state
+  int2 pr[SPW];
 #pragma unroll
   for (int q = 0; q < SPW; ++q) {
     const int r = base + SPW * wid + q;
-    const int pr = src.pmap && r < src.nsp ? src.pmap[r] : r;
-    nbq[q] = src.binfo && r < src.nsp ? src.binfo[pr / kTile].w : nb;
-    const float4 *__restrict__ row = src.tp + (long long)pr * nb;
+    pr[q] = r < ns ? src.prow[r] : make_int2(0, 0);
+  }
+#pragma unroll
+  for (int q = 0; q < SPW; ++q) {
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
       const int k = lane + 32 * m;
-      w[q][m] = r < src.nsp && k < nbq[q] ? row[k] : make_float4(0.f, 0.f, 0.f, 0.f);
+      w[q][m] = k < pr[q].y ? src.tp[pr[q].x + k] : make_float4(0.f, 0.f, 0.f, 0.f);
     }
   }
   float2 v[NV];
@@ -2770,14 +2740,10 @@ __global__ void __launch_bounds__(256) k_fin_tiles(TileSrc src, int ns, double c
       v[2 * q] = ff_add(v[2 * q], make_float2(w[q][m].x, w[q][m].y));
       v[2 * q + 1] = ff_add(v[2 * q + 1], make_float2(w[q][m].z, w[q][m].w));
     }
-    const int r = base + SPW * wid + q;
-    if (r < src.nsp) {
-      const float4 *__restrict__ row = src.tp + (long long)(src.pmap ? src.pmap[r] : r) * nb;
-      for (int k = lane + 96; k < nbq[q]; k += 32) {
-        const float4 x = row[k];
-        v[2 * q] = ff_add(v[2 * q], make_float2(x.x, x.y));
-        v[2 * q + 1] = ff_add(v[2 * q + 1], make_float2(x.z, x.w));
-      }
+    for (int k = lane + 96; k < pr[q].y; k += 32) {
+      const float4 x = src.tp[pr[q].x + k];
+      v[2 * q] = ff_add(v[2 * q], make_float2(x.x, x.y));
+      v[2 * q + 1] = ff_add(v[2 * q + 1], make_float2(x.z, x.w));
     }
   }
   ff_reduce_scatter<NV, 16>(v, lane);
@@ -2794,7 +2760,7 @@ __global__ void __launch_bounds__(256) k_fin_tiles(TileSrc src, int ns, double c
   if (RATE)
     out[r0] = c * (in.R - B);
   else
-    fin_apply<false, STAGE, false>(r0, A, B, c, in, out, f, acc, y, yff, dt, src.pmap ? src.pmap[r0] : r0);
+    fin_apply<false, STAGE, false>(r0, A, B, c, in, out, f, acc, y, yff, dt, ry);
 }
 
 template <bool LIT, typename SRC = ItemSrc>

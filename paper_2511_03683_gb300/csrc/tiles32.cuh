@@ -31,7 +31,7 @@ constexpr size_t kC32ColFloats = (size_t)(kC32Threads / 32) * kTile;  // [8 warp
 // dynamic shared memory of a launch shape with NST stages (and the double-buffered column table)
 template <int NST>
 constexpr size_t c32_smem() {
-  return (size_t)NST * kC32StageBytes + 128 + 2 * kC32ColFloats * sizeof(float);
+  return (size_t)NST * kC32StageBytes + 320 + 2 * kC32ColFloats * sizeof(float);
 }
 
 // (a, b) ~ (P_in, P_out) in FP32 with the ratio kept (see above); zero stays zero.
@@ -57,57 +57,29 @@ __device__ __forceinline__ float2 c32_round_pair(double pin, double pout) {
   return make_float2(ba, bb);
 }
 
-// tc[t][i][j] = rounded (P_in, P_out) of pair (64 I + i, 64 J + j) from the branch-merged
-// float-float coefficients of complete rows (entry (s, p) of row s is at srp[s] + p); zero
-// outside the nstate states.
-__global__ void k_tiles_fill_c32(const int2 *__restrict__ tiles, int nt, const float2 *__restrict__ coefA,
-                                 const float2 *__restrict__ coefB, const long long *__restrict__ srp, int ns,
-                                 float2 *__restrict__ tc) {
-  const long long n = (long long)nt * kTile * kTile;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-    const int t = (int)(e / (kTile * kTile)), k = (int)(e % (kTile * kTile));
-    const int2 IJ = tiles[t];
-    const int s = IJ.x * kTile + k / kTile, p = IJ.y * kTile + k % kTile;
-    float2 v = make_float2(0.f, 0.f);
-    if (s < ns && p < ns) {
-      const long long c = srp[s] + p;
-      const float2 a = coefA[c], b = coefB[c];
-      const double pin = ff_to_double(a.x, a.y), pout = pin + ff_to_double(b.x, b.y);
-      v = c32_round_pair(pin, pout);
-    }
-    tc[e] = v;
-  }
-}
-
-// The symmetric tiles from branch-merged pair rows that need not be complete (the batch's
-// systems, or one system whose rows miss some partners): one warp per row s, every stored pair
-// (s, p) whose block pair (I, J) lies in the upper triangle (I <= J) written to its tile entry;
-// the tiles were zeroed before, pairs without channels stay zero, and zero padding entries are
-// skipped.  Several systems share one padded block space through pmap (each state's padded row)
-// and binfo[g] of block g = (first block of its system, the system's first tile, its states, its
-// blocks); with both null there is one system of ns states in nbs blocks.  Tiles are numbered
-// row-major over each system's upper block triangle.  C32: the pairs rounded to FP32 with their
-// ratio kept, else float-float (float4 per entry).
+// The symmetric tiles from the branch-merged pair rows (complete or not): one warp per row s,
+// every stored pair (s, p) whose block pair (I, J) lies in the upper triangle written to its tile
+// entry; the tiles were zeroed before, pairs without channels stay zero.  pmap: each state's row in
+// the padded energy order (of one system, or of a batch's systems one after the other); tbase[I] =
+// (the index of tile (I, I), the last block column stored for block row I): tiles of a block row are
+// numbered consecutively, and pairs beyond the last column have zero coefficients (energy_reach).
+// C32: the pairs rounded to FP32 with their ratio kept, else float-float (float4 per entry).
 template <bool C32, typename IDX>
 __global__ void k_tiles_scatter(const long long *__restrict__ srp, int ns, const IDX *__restrict__ pidx,
                                 const float2 *__restrict__ coefA, const float2 *__restrict__ coefB,
-                                const int *__restrict__ pmap, const int4 *__restrict__ binfo, int nbs,
-                                void *__restrict__ tc) {
+                                const int *__restrict__ pmap, const int2 *__restrict__ tbase, void *__restrict__ tc) {
   const int lane = threadIdx.x & 31;
   const int w0 = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
   const int nw = (int)(((long long)gridDim.x * blockDim.x) >> 5);
   for (int r = w0; r < ns; r += nw) {
-    const int pr = pmap ? pmap[r] : r;
-    const int4 bi = binfo ? binfo[pr / kTile] : make_int4(0, 0, ns, nbs);
-    const int I = pr / kTile - bi.x;
+    const int pr = pmap[r], I = pr / kTile;
+    const int2 tb = tbase[I];
     for (long long e = srp[r] + lane; e < srp[r + 1]; e += 32) {
       const float2 a = coefA[e], b = coefB[e];
       if (a.x == 0.f && a.y == 0.f && b.x == 0.f && b.y == 0.f) continue;
-      const int pp = pmap ? pmap[pidx[e]] : (int)pidx[e];
-      const int J = pp / kTile - bi.x;
-      if (J < I) continue;
-      const long long t = (long long)bi.y + (long long)I * (2 * bi.w - I + 1) / 2 + (J - I);
-      const long long k = t * kTile * kTile + (pr % kTile) * kTile + pp % kTile;
+      const int pp = pmap[pidx[e]], J = pp / kTile;
+      if (J < I || J > tb.y) continue;
+      const long long k = (long long)(tb.x + (J - I)) * kTile * kTile + (pr % kTile) * kTile + pp % kTile;
       const double pin = ff_to_double(a.x, a.y), pout = pin + ff_to_double(b.x, b.y);
       if (C32) {
         ((float2 *)tc)[k] = c32_round_pair(pin, pout);
@@ -158,15 +130,14 @@ __device__ __forceinline__ void f32_reduce_scatter(float (&v)[NV], int lane) {
 }
 
 // the column sums of a finished off-diagonal tile: threads 0..63 add the 8 warps' values of
-// one column each and write them to the column state's partial for the tile's row block (slot
-// slotI)
-__device__ __forceinline__ void c32_columns_out(const float *__restrict__ colred, int2 IJ, int slotI, int nb, int tid,
+// one column each and write them to the tile's column slots
+__device__ __forceinline__ void c32_columns_out(const float *__restrict__ colred, int cb, int cs, int tid,
                                                 float *__restrict__ tp) {
   if (tid >= kTile) return;
   float acc = colred[tid];
 #pragma unroll
   for (int w = 1; w < kC32Threads / 32; ++w) acc = __fadd_rn(acc, colred[w * kTile + tid]);
-  tp[(long long)(IJ.y * kTile + tid) * nb + slotI] = acc;
+  tp[cb + tid * cs] = acc;
 }
 
 // One persistent 256-thread CTA (CPS per SM) streams its share of the tiles through NST
@@ -177,15 +148,13 @@ __device__ __forceinline__ void c32_columns_out(const float *__restrict__ colred
 // 1/tau_s summands P_out + f_p d (row s) and P_in - f_s d (column p, the reverse channel), each
 // with its f_l term.  The per-warp column table is double buffered and combined in the next
 // iteration, so a tile costs one CTA barrier.
-// lblk (batched sweep, else null): the block index of each block within its instance, which
-// numbers the partial slots.  rev: take the tile list from its end (tile nt - 1 - t in place of
-// t), so that a sweep following one in list order starts on the tiles the L2 still holds.
+// rev: take the tile list from its end (tile nt - 1 - t in place of t), so that a sweep following
+// one in list order starts on the tiles the L2 still holds.
 template <int MODE, int NST, int CPS>
-__global__ void __launch_bounds__(kC32Threads, CPS) k_stream_c32(const int2 *__restrict__ tiles, int nt,
+__global__ void __launch_bounds__(kC32Threads, CPS) k_stream_c32(const TileD *__restrict__ tiles, int nt,
                                                                   const float2 *__restrict__ tc,
-                                                                  const float2 *__restrict__ fg, int ns, int nb,
+                                                                  const float2 *__restrict__ fg,
                                                                   float *__restrict__ tp, int *__restrict__ err,
-                                                                  const int *__restrict__ lblk = nullptr,
                                                                   int rev = 0) {
   // the stage of tile k - 1 is refilled (with tile k - 1 + NST) only after the wait for tile k, so
   // one stage would wait for a copy not yet issued
@@ -193,46 +162,38 @@ __global__ void __launch_bounds__(kC32Threads, CPS) k_stream_c32(const int2 *__r
   constexpr int R = 4;
   extern __shared__ __align__(128) unsigned char ssm[];
   unsigned long long *bars = (unsigned long long *)(ssm + NST * kC32StageBytes);
-  int2 *stile = (int2 *)(bars + NST);
-  float *colred0 = (float *)(ssm + NST * kC32StageBytes + 128);
+  TileD *stile = (TileD *)(bars + 8);
+  float *colred0 = (float *)(ssm + NST * kC32StageBytes + 320);
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, tj = tid & 15, ti = tid >> 4;
   const int G = (int)gridDim.x;
   const int nloc = (int)blockIdx.x < nt ? (nt - 1 - (int)blockIdx.x) / G + 1 : 0;
-  for (int i = tid; i < NST * 2 * kTile; i += kC32Threads) {
-    float2 *fz = (float2 *)(ssm + (i / (2 * kTile)) * kC32StageBytes + kC32TileBytes);
-    fz[i % (2 * kTile)] = make_float2(0.f, 0.f);
-  }
   if (tid == 0) {
     for (int k = 0; k < NST; ++k) mbar_init(bars + k, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  fence_proxy_async();
   __syncthreads();
   int issued = 0;
   auto tix = [&](int k) {  // the CTA's k-th tile
     const int t = (int)blockIdx.x + k * G;
     return rev ? nt - 1 - t : t;
   };
-  auto issue = [&](int k, int2 IJ) {
+  auto issue = [&](int k, const TileD &D) {
     const int s = k % NST;
     const int t = tix(k);
-    stile[s] = IJ;
+    stile[s] = D;
     unsigned char *buf = ssm + (size_t)s * kC32StageBytes;
-    const int nr = min(kTile, ns - IJ.x * kTile), nc = min(kTile, ns - IJ.y * kTile);
-    const unsigned br = (unsigned)(nr * sizeof(float2) + 15) / 16 * 16, bc = (unsigned)(nc * sizeof(float2) + 15) / 16 * 16;
-    mbar_expect_tx(bars + s, kC32TileBytes + br + bc);
+    mbar_expect_tx(bars + s, kC32StageBytes);
     const unsigned char *src = (const unsigned char *)(tc + (size_t)t * kTile * kTile);
 #pragma unroll
     for (int q = 0; q < 2; ++q) bulk_g2s(buf + q * (kC32TileBytes / 2), src + q * (kC32TileBytes / 2), kC32TileBytes / 2, bars + s);
-    bulk_g2s(buf + kC32TileBytes, fg + (size_t)IJ.x * kTile, br, bars + s);
-    bulk_g2s(buf + kC32TileBytes + kTile * sizeof(float2), fg + (size_t)IJ.y * kTile, bc, bars + s);
+    bulk_g2s(buf + kC32TileBytes, fg + (size_t)D.I * kTile, kTile * sizeof(float2), bars + s);
+    bulk_g2s(buf + kC32TileBytes + kTile * sizeof(float2), fg + (size_t)D.J * kTile, kTile * sizeof(float2), bars + s);
   };
   if (tid == 0)
-    for (; issued < NST && issued < nloc; ++issued) issue(issued, tiles[tix(issued)]);
-  int2 nextIJ = make_int2(0, 0);
-  if (tid == 0 && issued < nloc) nextIJ = tiles[tix(issued)];
-  int2 prevIJ = make_int2(0, 0);
-  int prevI = 0;
+    for (; issued < NST && issued < nloc; ++issued) issue(issued, load_tile(tiles, tix(issued)));
+  TileD next{};
+  if (tid == 0 && issued < nloc) next = load_tile(tiles, tix(issued));
+  int pcb = -1, pcs = 0;  // column slots of the previous tile (-1: diagonal, or none)
   bool ok = true;
   for (int k = 0; k <= nloc; ++k) {
     const bool have = k < nloc;
@@ -242,19 +203,17 @@ __global__ void __launch_bounds__(kC32Threads, CPS) k_stream_c32(const int2 *__r
     }
     if (tid == 0 && k >= 1 && issued < nloc) {
       fence_proxy_async();  // the generic reads of tile k-1's stage before its refill
-      issue(issued, nextIJ);
+      issue(issued, next);
       ++issued;
-      if (issued < nloc) nextIJ = tiles[tix(issued)];
+      if (issued < nloc) next = load_tile(tiles, tix(issued));
     }
-    if (k >= 1 && prevIJ.x != prevIJ.y)
-      c32_columns_out(colred0 + ((k - 1) & 1) * kC32ColFloats, prevIJ, prevI, nb, tid, tp);
+    if (k >= 1 && pcb >= 0) c32_columns_out(colred0 + ((k - 1) & 1) * kC32ColFloats, pcb, pcs, tid, tp);
     if (!have) break;
     const int s = k % NST;
-    const int2 IJ = stile[s];
-    const int Il = lblk ? lblk[IJ.x] : IJ.x, Jl = lblk ? lblk[IJ.y] : IJ.y;  // slot blocks
-    prevIJ = IJ;
-    prevI = Il;
-    const bool diag = IJ.x == IJ.y;
+    const TileD D = stile[s];
+    const bool diag = D.I == D.J;
+    pcb = diag ? -1 : D.cb;
+    pcs = D.cs;
     const float2 *__restrict__ T = (const float2 *)(ssm + (size_t)s * kC32StageBytes);
     const float2 *__restrict__ fr = (const float2 *)(ssm + (size_t)s * kC32StageBytes + kC32TileBytes);
     const float2 *__restrict__ fc = fr + kTile;
@@ -287,7 +246,7 @@ __global__ void __launch_bounds__(kC32Threads, CPS) k_stream_c32(const int2 *__r
     }
     // rows: the 16 lanes of a half-warp share them; lanes 4i .. 4i + 3 end with the total of row i
     f32_reduce_scatter<R, 8>(rv, lane);
-    if ((tj & 3) == 0) tp[(long long)(IJ.x * kTile + ti * R + (tj >> 2)) * nb + Jl] = rv[0];
+    if ((tj & 3) == 0) tp[D.rb + (ti * R + (tj >> 2)) * D.rs] = rv[0];
     if (!diag) {
       // columns: lanes tj and tj + 16 share them (one level), then the 8 warps (next iteration)
       float *colred = colred0 + (k & 1) * kC32ColFloats;
@@ -321,68 +280,58 @@ constexpr unsigned kC32HalfBytes = kC32TileBytes / 2;
 constexpr unsigned kC32HalfStageBytes = kC32HalfBytes + (kTile / 2 + kTile) * sizeof(float2);
 template <int NST>
 constexpr size_t c32_half_smem() {
-  return (size_t)NST * kC32HalfStageBytes + 128 + kC32ColFloats * sizeof(float);
+  return (size_t)NST * kC32HalfStageBytes + 320 + kC32ColFloats * sizeof(float);
 }
 
 template <int MODE, int NST, int CPS>
-__global__ void __launch_bounds__(kC32Threads, CPS) k_stream_c32_half(const int2 *__restrict__ tiles, int nt,
+__global__ void __launch_bounds__(kC32Threads, CPS) k_stream_c32_half(const TileD *__restrict__ tiles, int nt,
                                                                        const float2 *__restrict__ tc,
-                                                                       const float2 *__restrict__ fg, int ns, int nb,
+                                                                       const float2 *__restrict__ fg,
                                                                        float *__restrict__ tp, int *__restrict__ err,
-                                                                       const int *__restrict__ lblk = nullptr,
                                                                        int rev = 0) {
   static_assert(NST >= 2 && NST <= 8, "the ring needs 2..8 stages");
   constexpr int R = 2, HR = kTile / 2;
   extern __shared__ __align__(128) unsigned char ssm[];
   unsigned long long *bars = (unsigned long long *)(ssm + NST * kC32HalfStageBytes);
-  int2 *stile = (int2 *)(bars + NST);
-  float *colred = (float *)(ssm + NST * kC32HalfStageBytes + 128);  // [8 warps][64 columns]
+  TileD *stile = (TileD *)(bars + 8);
+  float *colred = (float *)(ssm + NST * kC32HalfStageBytes + 320);  // [8 warps][64 columns]
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, tj = tid & 15, ti = tid >> 4;
   const int G = (int)gridDim.x;
   const int nloc = (int)blockIdx.x < nt ? (nt - 1 - (int)blockIdx.x) / G + 1 : 0;
   const int nunit = 2 * nloc;
-  for (int i = tid; i < NST * (HR + kTile); i += kC32Threads) {
-    float2 *fz = (float2 *)(ssm + (i / (HR + kTile)) * kC32HalfStageBytes + kC32HalfBytes);
-    fz[i % (HR + kTile)] = make_float2(0.f, 0.f);
-  }
   if (tid == 0) {
     for (int k = 0; k < NST; ++k) mbar_init(bars + k, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  fence_proxy_async();
   __syncthreads();
   int issued = 0;
   auto tix = [&](int k) {  // the CTA's k-th tile
     const int t = (int)blockIdx.x + k * G;
     return rev ? nt - 1 - t : t;
   };
-  int2 issIJ = make_int2(0, 0), aheadIJ = make_int2(0, 0);
+  TileD iss{}, ahead{};
   if (tid == 0 && nloc > 0) {
-    issIJ = tiles[tix(0)];
-    if (nloc > 1) aheadIJ = tiles[tix(1)];
+    iss = load_tile(tiles, tix(0));
+    if (nloc > 1) ahead = load_tile(tiles, tix(1));
   }
   auto issue = [&](int v) {  // unit v = 2 k + h: half h of the CTA's tile k
     const int k = v >> 1, h = v & 1, s = v % NST;
     if (h == 0 && k > 0) {
-      issIJ = aheadIJ;
-      if (k + 1 < nloc) aheadIJ = tiles[tix(k + 1)];
+      iss = ahead;
+      if (k + 1 < nloc) ahead = load_tile(tiles, tix(k + 1));
     }
     const int t = tix(k);
-    stile[s] = issIJ;
+    stile[s] = iss;
     unsigned char *buf = ssm + (size_t)s * kC32HalfStageBytes;
-    const int nr = min(HR, ns - (issIJ.x * kTile + h * HR)), nc = min(kTile, ns - issIJ.y * kTile);
-    const unsigned br = nr > 0 ? (unsigned)(nr * sizeof(float2) + 15) / 16 * 16 : 0u;
-    const unsigned bc = (unsigned)(nc * sizeof(float2) + 15) / 16 * 16;
-    mbar_expect_tx(bars + s, kC32HalfBytes + br + bc);
+    mbar_expect_tx(bars + s, kC32HalfStageBytes);
     const unsigned char *src = (const unsigned char *)(tc + (size_t)t * kTile * kTile) + (size_t)h * kC32HalfBytes;
     bulk_g2s(buf, src, kC32HalfBytes, bars + s);
-    if (br) bulk_g2s(buf + kC32HalfBytes, fg + (size_t)issIJ.x * kTile + h * HR, br, bars + s);
-    bulk_g2s(buf + kC32HalfBytes + HR * sizeof(float2), fg + (size_t)issIJ.y * kTile, bc, bars + s);
+    bulk_g2s(buf + kC32HalfBytes, fg + (size_t)iss.I * kTile + h * HR, HR * sizeof(float2), bars + s);
+    bulk_g2s(buf + kC32HalfBytes + HR * sizeof(float2), fg + (size_t)iss.J * kTile, kTile * sizeof(float2), bars + s);
   };
   if (tid == 0)
     for (; issued < NST && issued < nunit; ++issued) issue(issued);
-  int2 prevIJ = make_int2(0, 0);
-  int prevI = 0;
+  int pcb = -1, pcs = 0;  // column slots of the previous unit's tile (-1: diagonal, or none)
   bool ok = true;
   float cv[4];  // column sums of the current tile, carried across its halves
   for (int u = 0; u <= nunit; ++u) {
@@ -396,14 +345,13 @@ __global__ void __launch_bounds__(kC32Threads, CPS) k_stream_c32_half(const int2
       issue(issued);
       ++issued;
     }
-    if ((u & 1) == 0 && u >= 2 && prevIJ.x != prevIJ.y) c32_columns_out(colred, prevIJ, prevI, nb, tid, tp);
+    if ((u & 1) == 0 && u >= 2 && pcb >= 0) c32_columns_out(colred, pcb, pcs, tid, tp);
     if (!have) break;
     const int s = u % NST, h = u & 1;
-    const int2 IJ = stile[s];
-    const int Il = lblk ? lblk[IJ.x] : IJ.x, Jl = lblk ? lblk[IJ.y] : IJ.y;  // slot blocks
-    prevIJ = IJ;
-    prevI = Il;
-    const bool diag = IJ.x == IJ.y;
+    const TileD D = stile[s];
+    const bool diag = D.I == D.J;
+    pcb = diag ? -1 : D.cb;
+    pcs = D.cs;
     const float2 *__restrict__ T = (const float2 *)(ssm + (size_t)s * kC32HalfStageBytes);
     const float2 *__restrict__ fr = (const float2 *)(ssm + (size_t)s * kC32HalfStageBytes + kC32HalfBytes);
     const float2 *__restrict__ fc = fr + HR;
@@ -439,7 +387,7 @@ __global__ void __launch_bounds__(kC32Threads, CPS) k_stream_c32_half(const int2
     }
     // rows: the 16 lanes of a half-warp share them; lanes 8i .. 8i + 7 end with the total of row i
     f32_reduce_scatter<R, 8>(rv, lane);
-    if ((tj & 7) == 0) tp[(long long)(IJ.x * kTile + h * HR + ti * R + (tj >> 3)) * nb + Jl] = rv[0];
+    if ((tj & 7) == 0) tp[D.rb + (h * HR + ti * R + (tj >> 3)) * D.rs] = rv[0];
     if (!diag && h == 1) {
       // columns of the whole tile: lanes tj and tj + 16 share them (one level), then the warps
       // (after the next unit's barrier)
@@ -526,34 +474,33 @@ __global__ void k_pairs_c32(const float2 *__restrict__ A, const float2 *__restri
 // partials of SPC / 8 states (lanes over the blocks in float-float, then one 32-lane float-float
 // reduce-scatter of the SPC / 8 values), and warp 0 applies the prefactor and the RK4 stage
 // arithmetic in FP64, one lane per state.
-// pmap, binfo (batched tiles, else null): each state's padded row and the block table, whose
-// .w gives the partner blocks of a state's system; nsp is then the number of states
+// prow, pmap: as TileSrc
 template <int STAGE, bool RATE = false, int SPC = 32>
-__global__ void __launch_bounds__(256) k_fin_c32(const float *__restrict__ tp, int nb, int nsp, int ns, double c,
+__global__ void __launch_bounds__(256) k_fin_c32(const float *__restrict__ tp, const int2 *__restrict__ prow,
+                                                 const int *__restrict__ pmap, int ns, double c,
                                                  const double *__restrict__ ysrc, double *__restrict__ out,
                                                  double *__restrict__ f, double *__restrict__ acc,
-                                                 double *__restrict__ y, float2 *__restrict__ yff, double dt,
-                                                 const int *__restrict__ pmap = nullptr,
-                                                 const int4 *__restrict__ binfo = nullptr) {
+                                                 double *__restrict__ y, float2 *__restrict__ yff, double dt) {
   constexpr int SPW = SPC / 8, LPV = 32 / SPW;  // states per warp, lanes per state after the reduce-scatter
   __shared__ float2 tot[SPC];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int base = blockIdx.x * SPC;
   const int r0 = base + lane;
   FinIn in{0.0, 0.0, 0.0, 0.0};
+  int ry = 0;
   if (!RATE && wid == 0 && lane < SPC && r0 < ns) {
     if (STAGE >= 0) in.f = f[r0];
     if (STAGE >= 1) in.acc = acc[r0];
+    if (STAGE >= 0) ry = pmap[r0];
   }
   float2 v[SPW];
 #pragma unroll
   for (int q = 0; q < SPW; ++q) {
     const int r = base + SPW * wid + q;
     v[q] = make_float2(0.f, 0.f);
-    if (r < nsp) {
-      const int pr = pmap ? pmap[r] : r, nbr = binfo ? binfo[pr / kTile].w : nb;
-      const float *__restrict__ row = tp + (long long)pr * nb;
-      for (int k = lane; k < nbr; k += 32) v[q] = ff_add(v[q], make_float2(row[k], 0.f));
+    if (r < ns) {
+      const int2 pr = prow[r];
+      for (int k = lane; k < pr.y; k += 32) v[q] = ff_add(v[q], make_float2(tp[pr.x + k], 0.f));
     }
   }
   ff_reduce_scatter<SPW, 16>(v, lane);
@@ -566,7 +513,7 @@ __global__ void __launch_bounds__(256) k_fin_c32(const float *__restrict__ tp, i
     out[r0] = I;
     return;
   }
-  fin_stage<STAGE, false>(r0, I, in, out, f, acc, y, yff, dt, pmap ? pmap[r0] : r0);
+  fin_stage<STAGE, false>(r0, I, in, out, f, acc, y, yff, dt, ry);
 }
 
 }  // namespace dev
