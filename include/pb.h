@@ -179,7 +179,9 @@ typedef struct pb_dev_opts {
                                 4-channel groups per lane, 3 through L1 with one channel per lane;
                                 one channel per lane with lazily renormalised float-float sums: 4 one
                                 1024-thread CTA per SM with F in shared memory (5 if F does not fit) and
-                                the next trip in registers, 5 the same through L1, 6 = 3 with lazy sums;
+                                the next trip in registers, or, on a device with float-float symmetric
+                                tiles (dense_rows), the weights in the same energy-ordered tiles; 5 the
+                                same through L1, 6 = 3 with lazy sums;
                                 7 row blocks on complete branch-merged float-float rows: a warp takes
                                 four rows and one segment of their partners, each partner's F (shared
                                 memory) read once for the four rows, the weights through a per-warp
@@ -315,8 +317,8 @@ int pb_rtbte_rk4_host(pb_dev *dev, const double *f_host_in, double *f_host_out, 
  * PB_ENOCONV if maxit was reached first (F3 then holds the last iterate).  Each pass is
  * replayed from a CUDA graph, and the next pass is queued before the host reads the previous
  * pass's residual (one extra pass runs after the converged one; it changes neither F3 nor the
- * result); the residual numbers go through 48 bytes of page-locked host memory that the
- * handle allocates on its first solve and frees in pb_dev_destroy.
+ * result); the residual's block maxima go through a few KB (32 bytes per 32 states) of
+ * page-locked host memory that the handle allocates on its first solve and frees in pb_dev_destroy.
  * Needs a pb_dev created with opts.transport != 0. */
 int pb_iter_transport(pb_dev *dev, const double *f0, const double *vel3, double tol, int32_t maxit, double *F3,
                       int32_t *iters, double *resid, void *stream);

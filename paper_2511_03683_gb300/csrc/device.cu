@@ -52,7 +52,7 @@ struct Layout {
   size_t rp, item_ptr, items, col, coefA, coefB, g2, wt, eps, kc, R, omega, tab, part, acc, y, yff, fstage, Fa, Fb,
       Fff, tau, invtau, red, scal, obs, g2lo, gstate, tab32, col16, rp_real, vjpG, g2tab, vecs, hcol, hg2, hA, hB, sc,
       entries, hitems, titems, t_item_ptr, err, citems, citem_ptr, cpart, ccoefA, ccoefB, sidx16, sidx32, pcstart,
-      pcnt, srp, gitems, tiles, tcoef, tpart, pmap, prow, tbase, g2d, gditems, gdptr, gacc, gaccg, trptr, trpart, total;
+      pcnt, srp, gitems, tiles, tcoef, tpart, pmap, prow, tbase, ord, trlist, trsegr, trtpart, trf0, g2d, gditems, gdptr, gacc, gaccg, trptr, trpart, total;
 };
 
 struct Plan {
@@ -239,6 +239,8 @@ struct TilePlan {
   std::vector<int2> prow;         // [states] first partial slot, slots
   std::vector<int2> tbase;        // [blocks] index of tile (I, I), last block column of block row I
   std::vector<dev::TileD> tiles;  // block rows in order, columns ascending
+  std::vector<int2> span;         // [blocks] first block in reach, blocks in reach (both sides)
+  std::vector<int32_t> ord;       // [nsp] state of each padded row, -1 in the padding
 };
 
 // complete: every row holds every state (the reach alone decides); else the stored channels within
@@ -297,25 +299,62 @@ void tile_plan_add(const pb_channels *ch, bool complete, double reach, TilePlan 
       D.rs = hi[I] - lo[I] + 1;
       D.cb = (int)(first[J] + (I - lo[J]));
       D.cs = hi[J] - lo[J] + 1;
+      D.wu = (int)(first[I] / dev::kTile) + J - lo[I];
+      D.wl = (int)(first[J] / dev::kTile) + I - lo[J];
       T.tiles.push_back(D);
     }
+    T.span.push_back(make_int2(T.nb + lo[I], hi[I] - lo[I] + 1));
   }
   for (int64_t r = 0; r < ns; ++r) {
     const int K = pos[r] / dev::kTile, n = hi[K] - lo[K] + 1;
     T.pmap.push_back((int32_t)((int64_t)T.nb * dev::kTile + pos[r]));
     T.prow.push_back(make_int2((int)(first[K] + (int64_t)(pos[r] % dev::kTile) * n), n));
   }
+  for (int64_t i = 0; i < (int64_t)nb * dev::kTile; ++i) T.ord.push_back(i < ns ? ord[i] : -1);
   T.nb += nb;
   T.nt_full += (int64_t)nb * (nb + 1) / 2;
   T.nb_max = std::max(T.nb_max, nb);
   T.nsp = (int64_t)T.nb * dev::kTile;
 }
 
+// The transport weight tiles of a tile plan (kernels.cuh): the list of them, block-row-major, cut into
+// one contiguous range per CTA, and the segments (a CTA's tiles of one block row, at most
+// kTrSegTiles) with each block row's range of them.
+struct TrTilePlan {
+  std::vector<dev::TrTile> list;
+  std::vector<int2> segr;
+  int nseg = 0, grid = 0;
+};
+int64_t tr_tiles_of(const TilePlan &T) { return T.npart / dev::kTile; }
+int64_t tr_segs_cap(const TilePlan &T, int sm) {
+  return tr_tiles_of(T) / dev::kTrSegTiles + 2 * (int64_t)T.nb + (int64_t)sm * dev::kTrCtas + 1;
+}
+TrTilePlan tr_tile_plan(const TilePlan &T, int sm) {
+  TrTilePlan P;
+  const int64_t nw = tr_tiles_of(T);
+  P.grid = (int)std::max<int64_t>(1, std::min<int64_t>(nw, (int64_t)sm * dev::kTrCtas));
+  P.segr.assign((size_t)T.nb, make_int2(0, 0));
+  int64_t t = 0, cta = 0;
+  int run = 0;  // tiles of the open segment
+  for (int I = 0; I < T.nb; ++I) {
+    P.segr[I].x = P.nseg;
+    for (int q = 0; q < T.span[I].y; ++q, ++t) {
+      while (t >= (cta + 1) * nw / P.grid) ++cta;
+      const bool last = q + 1 == T.span[I].y || t + 1 == (cta + 1) * nw / P.grid || run + 1 == dev::kTrSegTiles;
+      P.list.push_back(dev::TrTile{T.span[I].x + q, P.nseg, last ? 1 : 0, 0});
+      run = last ? 0 : run + 1;
+      if (last) ++P.nseg;
+    }
+    P.segr[I].y = P.nseg;
+  }
+  return P;
+}
+
 // tp: the symmetric tiles (null: none); tile_entry: their bytes per pair (16 float-float, 8 for the
 // FP32 tiles of C32)
 Layout make_layout(const pb_channels *ch, const Plan &P, const Plan *S, int variant, bool transport,
                    int nfin_blocks, const TilePlan *tp = nullptr, const GDense &gd = GDense(), bool gacc = false,
-                   size_t tile_entry = sizeof(float4), int tr_nseg = 0) {
+                   size_t tile_entry = sizeof(float4), int tr_nseg = 0, int sm = 152) {
   Layout L{};
   size_t o = 0;
   auto take = [&](size_t bytes) {
@@ -352,7 +391,14 @@ Layout make_layout(const pb_channels *ch, const Plan &P, const Plan *S, int vari
   L.pmap = take(tp ? sizeof(int32_t) * ns : 0);
   L.prow = take(tp ? sizeof(int2) * ns : 0);
   L.tbase = take(tp ? sizeof(int2) * tp->nb : 0);
-  L.wt = take(transport ? sizeof(float2) * nsw : 0);
+  // float-float tiles: the transport weights in tiles, F and its partials in their order
+  const bool trt = transport && tp && tile_entry == sizeof(float4);
+  L.wt = take(transport ? sizeof(float2) * (trt ? std::max(nsw, (size_t)tr_tiles_of(*tp) * dev::kTile * dev::kTile) : nsw) : 0);
+  L.trlist = take(trt ? sizeof(dev::TrTile) * (size_t)tr_tiles_of(*tp) : 0);
+  L.trsegr = take(trt ? sizeof(int2) * tp->nb : 0);
+  L.trtpart = take(trt ? sizeof(float2) * 3 * dev::kTile * (size_t)tr_segs_cap(*tp, sm) : 0);
+  L.trf0 = take(trt ? sizeof(float4) * (size_t)tp->nsp : 0);
+  L.ord = take(tp ? sizeof(int32_t) * (size_t)tp->nsp : 0);
   L.eps = take(sizeof(double) * ns);
   L.kc = take(sizeof(short4) * ns);
   L.R = take(sizeof(double) * ns);
@@ -364,10 +410,10 @@ Layout make_layout(const pb_channels *ch, const Plan &P, const Plan *S, int vari
   L.fstage = take(sizeof(double) * ns);
   L.Fa = take(transport ? sizeof(double) * 3 * ns : 0);
   L.Fb = take(transport ? sizeof(double) * 3 * ns : 0);
-  L.Fff = take(transport ? sizeof(float2) * 3 * ns : 0);
+  L.Fff = take(transport ? sizeof(float2) * 3 * (trt ? std::max<size_t>((size_t)tp->nsp, ns) : ns) : 0);
   L.tau = take(sizeof(double) * ns);
   L.invtau = take(sizeof(double) * ns);
-  L.red = take(sizeof(double2) * (size_t)nfin_blocks);
+  L.red = take(sizeof(double2) * (size_t)std::max(nfin_blocks, tp ? 2 * tp->nb : 0));
   L.scal = take(sizeof(double) * 8);
   L.obs = take(sizeof(double) * 8);
   L.err = take(sizeof(int) * 4);
@@ -580,6 +626,16 @@ struct pb_dev {
   float4 *tpart = nullptr;
   int32_t *pmap = nullptr;  // as TilePlan
   int2 *prow = nullptr, *tbase = nullptr;
+  int32_t *ord = nullptr;
+  // transport over the tiles (transport_gather 0 and 4 on float-float tiles): wt then holds the weight tiles
+  // of the last pb_transport_setup (wt_tiles) and Fff the iterate in their order
+  bool tr_tiles = false, wt_tiles = false;
+  int tr_grid = 0, tr_nw = 0, nblk = 0;
+  dev::TrTile *trlist = nullptr;
+  int2 *trsegr = nullptr;
+  float2 *trtpart = nullptr;
+  float4 *trf0 = nullptr;
+  int nred() const { return wt_tiles ? 2 * nblk : nfin_blocks; }  // maxima that a transport epilogue leaves in red
   dev::TileSrc tile_src() const { return dev::TileSrc{tpart, prow, pmap}; }
   // PB_VARIANT_C32: the FF device whose tiles hold FP32 (P_in, P_out) (tiles32.cuh); its
   // partials in tpart are one FP32 value per (state, block)
@@ -590,9 +646,9 @@ struct pb_dev {
   // the next tile sweep takes the tile list from its end (the RK4 stages alternate, so that each
   // sweep starts on the tiles the previous one left in L2)
   int rev = 0;
-  // pb_iter_transport: page-locked host copies of the residual numbers of two successive
-  // passes (allocated on the first solve), so that the next pass runs while one is checked
-  double *hres = nullptr;
+  // pb_iter_transport: page-locked host copies of the epilogue's maxima of two successive passes
+  // (allocated on the first solve), so that the next pass runs while one is checked
+  double2 *hres = nullptr;
   cudaEvent_t hres_ev[2] = {nullptr, nullptr};
   float2 *tc32 = nullptr;
   int64_t *rp_real = nullptr;  // unpadded CSR row offsets [ns+1]
@@ -926,7 +982,7 @@ extern "C" int pb_dev_arena_bytes(const pb_channels *ch, const pb_dev_opts *opts
                                   "closure-checked list whose rows are complete or miss few partners (or dense_rows 3)");
     const TrRows tr = tr_rows_for(P.ns, sm, o.transport != 0, merged, complete, o.variant, o);
     *bytes = make_layout(ch, P, merged ? &S : nullptr, o.variant, o.transport != 0, nfin, sym ? &T : nullptr,
-                         gdense_for(ch, o, sm), o.adjoint != 0, c32 ? sizeof(float2) : sizeof(float4), tr.nseg)
+                         gdense_for(ch, o, sm), o.adjoint != 0, c32 ? sizeof(float2) : sizeof(float4), tr.nseg, sm)
                  .total;
   } catch (const std::bad_alloc &) {
     return set_error(PB_ENOMEM, "pb_dev_arena_bytes: out of host memory");
@@ -1021,7 +1077,7 @@ extern "C" int pb_dev_create(const pb_channels *ch, const pb_dev_opts *opts, voi
   d->tr_nseg = trr.nseg;
   d->tr_seglen = trr.seglen;
   d->L = make_layout(ch, P, merged ? &S : nullptr, o.variant, d->transport, d->nfin_blocks, sym ? &T : nullptr, gd,
-                     o.adjoint != 0, c32 ? sizeof(float2) : sizeof(float4), trr.nseg);
+                     o.adjoint != 0, c32 ? sizeof(float2) : sizeof(float4), trr.nseg, sm);
   if (arena_bytes < d->L.total) {
     const size_t need = d->L.total;
     delete d;
@@ -1106,6 +1162,16 @@ extern "C" int pb_dev_create(const pb_channels *ch, const pb_dev_opts *opts, voi
       d->pmap = (int32_t *)(A + L.pmap);
       d->prow = (int2 *)(A + L.prow);
       d->tbase = (int2 *)(A + L.tbase);
+      d->ord = (int32_t *)(A + L.ord);
+      d->nblk = T.nb;
+      if (d->transport && !c32 && (o.transport_gather == 0 || o.transport_gather == 4)) {
+        d->tr_tiles = true;
+        d->tr_nw = (int)tr_tiles_of(T);
+        d->trlist = (dev::TrTile *)(A + L.trlist);
+        d->trsegr = (int2 *)(A + L.trsegr);
+        d->trtpart = (float2 *)(A + L.trtpart);
+        d->trf0 = (float4 *)(A + L.trf0);
+      }
     }
   } else {
     d->citems = d->items;
@@ -1334,6 +1400,24 @@ extern "C" int pb_dev_create(const pb_channels *ch, const pb_dev_opts *opts, voi
           UP(d->pmap, T.pmap.data(), sizeof(int32_t) * T.pmap.size());
           UP(d->prow, T.prow.data(), sizeof(int2) * T.prow.size());
           UP(d->tbase, T.tbase.data(), sizeof(int2) * T.tbase.size());
+          UP(d->ord, T.ord.data(), sizeof(int32_t) * T.ord.size());
+          if (d->tr_tiles) {
+            const TrTilePlan W = tr_tile_plan(T, sm);
+            if (W.nseg > tr_segs_cap(T, sm)) {
+              status = set_error(PB_EINVAL, "pb_dev_create: transport segment plan mismatch");
+              break;
+            }
+            d->tr_grid = W.grid;
+            UP(d->trlist, W.list.data(), sizeof(dev::TrTile) * W.list.size());
+            UP(d->trsegr, W.segr.data(), sizeof(int2) * W.segr.size());
+            // the padding of f0 and F multiplies zero coefficients: it must hold zeros
+            cudaError_t e2 = cudaMemsetAsync(d->trf0, 0, sizeof(float4) * (size_t)d->nsp, st);
+            if (e2 == cudaSuccess) e2 = cudaMemsetAsync(d->Fff, 0, sizeof(float2) * 3 * (size_t)d->nsp, st);
+            if (e2 != cudaSuccess) {
+              status = cuda_fail(e2, "clear the transport padding");
+              break;
+            }
+          }
         }
         cudaError_t e_ = cudaStreamSynchronize(st);  // pageable sources above go out of scope
         if (e_ != cudaSuccess) {
@@ -1409,6 +1493,10 @@ extern "C" int pb_dev_create(const pb_channels *ch, const pb_dev_opts *opts, voi
   if (d->smem_F > 48 * 1024) {
     cudaFuncSetAttribute(dev::k_stream_tr<true, uint32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)d->smem_F);
     cudaFuncSetAttribute(dev::k_stream_tr<true, uint16_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)d->smem_F);
+  }
+  if (d->tr_tiles) {
+    if (dev::kTrTileSmem > (size_t)smem_optin) d->tr_tiles = false;
+    else cudaFuncSetAttribute(dev::k_stream_tr_tiles, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dev::kTrTileSmem);
   }
   if (d->smem_Frows > 48 * 1024)
     cudaFuncSetAttribute(dev::k_stream_tr_rows<dev::kTrRows>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1804,8 +1892,29 @@ int ensure_rk_graph(pb_dev *d, double *f, double dt) {
   return PB_OK;
 }
 
+int rates_seq(pb_dev *d, const double *f, double *inv_tau, cudaStream_t st);
+
 int ensure_weights(pb_dev *d, const double *f0, cudaStream_t st) {
   if (!d->transport) return set_error(PB_EINVAL, "transport buffers were not reserved (pb_dev_opts.transport = 0)");
+  const bool tiles = d->tr_tiles && d->sym;
+  if (tiles != d->wt_tiles) {
+    d->drop_call_graphs();  // the captured passes read the other form of the weights
+    d->wt_tiles = tiles;
+  }
+  if (tiles) {
+    // 1/tau at f0 is the scattering rate there; then the weight tiles
+    int rc = rates_seq(d, f0, d->invtau, st);
+    if (rc) return rc;
+    const int g = (int)((d->ns + 255) / 256);
+    dev::k_recip<<<g, 256, 0, st>>>(d->invtau, (int)d->ns, d->tau);
+    PB_LAUNCHED("k_recip");
+    dev::k_f0_map<<<g, 256, 0, st>>>(f0, (int)d->ns, d->pmap, d->trf0);
+    PB_LAUNCHED("k_f0_map");
+    dev::k_weight_tiles<<<(int)std::min<int64_t>(d->tnt, (int64_t)d->sm_count * 6), 256, 0, st>>>(
+        d->tiles, d->tnt, d->tcoef, d->trf0, d->wt);
+    PB_LAUNCHED("k_weight_tiles");
+    return PB_OK;
+  }
   const int grid = d->stream_grid(8);
   if (d->variant == PB_VARIANT_FF || d->variant == PB_VARIANT_F64) {
     // from the coefficient arrays (per state pair when branch-merged)
@@ -1859,9 +1968,23 @@ void launch_tr_lane(pb_dev *d, const IDX *col, const float2 *Fin, cudaStream_t s
   }
 }
 
-// res3: where the residual numbers go (d->scal when null)
+// res3: where the residual numbers go (d->scal when null).  With `maxima` (d->nred() of them) the
+// epilogue's per-CTA maxima go there and nothing reduces them.
 int transport_pass(pb_dev *d, const float2 *Fin_ff, const double *vel3, const double *Fold, double *Fnew,
-                   float2 *Fnew_ff, cudaStream_t st, double *res3 = nullptr) {
+                   float2 *Fnew_ff, cudaStream_t st, double *res3 = nullptr, double2 *maxima = nullptr) {
+  double2 *red = maxima ? maxima : d->red;
+  if (d->wt_tiles) {
+    dev::k_stream_tr_tiles<<<d->tr_grid, 256, dev::kTrTileSmem, st>>>(d->trlist, d->tr_nw, d->wt, Fin_ff, d->trtpart,
+                                                                      d->err);
+    PB_LAUNCHED("k_stream_tr_tiles");
+    dev::k_fin_tr_tiles<<<2 * d->nblk, 3 * dev::kFinTrStates, 0, st>>>(d->trsegr, d->trtpart, d->ord, d->c, d->tau,
+                                                                       vel3, Fold, Fnew, Fnew_ff, red);
+    PB_LAUNCHED("k_fin_tr_tiles");
+    if (maxima) return PB_OK;
+    dev::k_red_final<<<1, 256, 0, st>>>(d->red, d->nred(), res3 ? res3 : d->scal);
+    PB_LAUNCHED("k_red_final");
+    return PB_OK;
+  }
   const int n = (int)d->nitems;
   const float4 *W4 = (const float4 *)d->wt;
   const int64_t need = (d->nitems * 32 + dev::kBlock - 1) / dev::kBlock;
@@ -1885,9 +2008,10 @@ int transport_pass(pb_dev *d, const float2 *Fin_ff, const double *vel3, const do
   }
   PB_LAUNCHED("k_stream_tr");
   dev::k_fin_tr<<<fin_grid(d), kFinBlock, 0, st>>>(rows ? d->trptr : d->item_ptr, rows ? d->trpart : d->part,
-                                                    (int)d->ns, d->tau, vel3, Fold, Fnew, Fnew_ff, d->red);
+                                                    (int)d->ns, d->tau, vel3, Fold, Fnew, Fnew_ff, red);
   PB_LAUNCHED("k_fin_tr");
-  dev::k_red_final<<<1, 256, 0, st>>>(d->red, d->nfin_blocks, res3 ? res3 : d->scal);
+  if (maxima) return PB_OK;
+  dev::k_red_final<<<1, 256, 0, st>>>(d->red, d->nred(), res3 ? res3 : d->scal);
   PB_LAUNCHED("k_red_final");
   return PB_OK;
 }
@@ -1955,8 +2079,13 @@ bool pinned_host(const void *p) {
 // one transport pass: conversion of F3in, sweep, epilogue, residual (into res3, or the handle's
 // scalars when null)
 int transport_seq(pb_dev *d, const double *vel3, const double *F3in, double *F3out, double *res3, cudaStream_t st) {
-  int rc;
-  if ((rc = to_ff(d, F3in, 3 * d->ns, d->Fff, st))) return rc;
+  if (d->wt_tiles) {
+    dev::k_trF_map<<<(int)std::max<int64_t>(1, std::min<int64_t>((3 * d->ns + 255) / 256, 1024)), 256, 0, st>>>(
+        F3in, (int)d->ns, d->pmap, d->Fff);
+    PB_LAUNCHED("k_trF_map");
+  } else if (const int rc = to_ff(d, F3in, 3 * d->ns, d->Fff, st)) {
+    return rc;
+  }
   return transport_pass(d, d->Fff, vel3, F3in, F3out, d->Fff, st, res3);
 }
 }  // namespace
@@ -2005,10 +2134,6 @@ extern "C" int pb_dev_time_sweep(pb_dev *d, const double *f, int32_t nlaunch, in
   if (e != cudaSuccess) return cuda_fail(e, "pb_dev_time_sweep");
   *avg_ms = ms / (float)nlaunch;
   return PB_OK;
-}
-
-namespace {
-int rates_seq(pb_dev *d, const double *f, double *inv_tau, cudaStream_t st);
 }
 
 extern "C" int pb_scatter_rates(pb_dev *d, const double *f, double *inv_tau, void *stream) {
@@ -2162,22 +2287,26 @@ extern "C" int pb_iter_transport(pb_dev *d, const double *f0, const double *vel3
   int rc;
   if ((rc = ensure_weights(d, f0, st))) return rc;
   const int g3 = (int)((3 * d->ns + 255) / 256);
-  dev::k_tr_init<<<g3, 256, 0, st>>>(d->tau, vel3, (int)d->ns, d->Fa, d->Fff);
+  dev::k_tr_init<<<g3, 256, 0, st>>>(d->tau, vel3, (int)d->ns, d->wt_tiles ? d->pmap : nullptr, d->Fa, d->Fff);
   PB_LAUNCHED("k_tr_init");
   if (!d->hres) {
-    PB_CUDA(cudaMallocHost((void **)&d->hres, 6 * sizeof(double)));
+    PB_CUDA(cudaMallocHost((void **)&d->hres, 2 * sizeof(double2) * (size_t)std::max({1, d->nfin_blocks, 2 * d->nblk})));
     for (cudaEvent_t &e : d->hres_ev) PB_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
   }
   double *Fbuf[2] = {d->Fa, d->Fb};  // pass i reads Fbuf[i % 2] and writes Fbuf[(i + 1) % 2]
-  // pass i: replayed from one of two graphs (Fa -> Fb, Fb -> Fa), its residual numbers copied
-  // to hres[3 (i % 2)] and an event recorded after them
+  // pass i: replayed from one of two graphs (Fa -> Fb, Fb -> Fa) whose epilogue writes its maxima
+  // straight into the page-locked host memory, and an event recorded after it: the host reduces the
+  // few dozen numbers, so that a pass is two launches and no copy
+  const int nred = d->nred();
+  double2 *hres[2] = {d->hres, d->hres + std::max(d->nfin_blocks, 2 * d->nblk)};
   auto enqueue = [&](int32_t i) -> int {
     const double *Fc = Fbuf[i & 1];
     double *Fn = Fbuf[(i + 1) & 1];
     const int r = replay(d, kCallSolvePass, vel3, Fc, Fn, nullptr, st,
-                         [&](cudaStream_t s) -> int { return transport_pass(d, d->Fff, vel3, Fc, Fn, d->Fff, s); });
+                         [&](cudaStream_t s) -> int {
+                           return transport_pass(d, d->Fff, vel3, Fc, Fn, d->Fff, s, nullptr, hres[i & 1]);
+                         });
     if (r) return r;
-    PB_CUDA(cudaMemcpyAsync(d->hres + 3 * (i & 1), d->scal, 3 * sizeof(double), cudaMemcpyDeviceToHost, st));
     PB_CUDA(cudaEventRecord(d->hres_ev[i & 1], st));
     return PB_OK;
   };
@@ -2189,7 +2318,12 @@ extern "C" int pb_iter_transport(pb_dev *d, const double *f0, const double *vel3
   while (it < maxit) {
     if (it + 1 < maxit && (rc = enqueue(it + 1))) return rc;
     PB_CUDA(cudaEventSynchronize(d->hres_ev[it & 1]));
-    res = d->hres[3 * (it & 1)];
+    double dm = 0.0, fm = 0.0;
+    for (int k = 0; k < nred; ++k) {
+      dm = std::fmax(dm, hres[it & 1][k].x);
+      fm = std::fmax(fm, hres[it & 1][k].y);
+    }
+    res = fm > 0.0 ? dm / fm : 0.0;
     ++it;
     if (!std::isfinite(res)) break;
     if (res <= tol) break;

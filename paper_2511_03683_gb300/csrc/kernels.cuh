@@ -2177,12 +2177,13 @@ constexpr int kTile = 64;
 
 // One stored tile: its block row I and block column J, and where its partials go: state i of
 // block I has its slot at rb + i * rs, state j of block J at cb + j * cs.
+// wu, wl: the indices of its two transport weight tiles, (I, J) and (J, I).
 struct alignas(16) TileD {
-  int I, J, rb, rs, cb, cs, pad0, pad1;
+  int I, J, rb, rs, cb, cs, wu, wl;
 };
 __device__ __forceinline__ TileD load_tile(const TileD *__restrict__ tiles, int t) {
   const int4 a = reinterpret_cast<const int4 *>(tiles + t)[0], b = reinterpret_cast<const int4 *>(tiles + t)[1];
-  return TileD{a.x, a.y, a.z, a.w, b.x, b.y, 0, 0};
+  return TileD{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
 }
 
 // One tile per CTA trip (grid-stride over tiles); thread (ti, tj) takes rows 4ti..4ti+3 and
@@ -2585,6 +2586,179 @@ __global__ void __launch_bounds__(kSymThreads, CPS) k_stream_sym_half(const Tile
   }
 }
 
+// ------------------------------------------------------------ transport over tiles
+//
+// The transport weights W(s,p) = c (f0_p P_in(s,p) + (1 - f0_p) P_out(s,p)) on the energy-ordered
+// tiles.  W is not symmetric, so each tile (I, J) of the coefficients gives two weight tiles,
+// (I, J) and (J, I): 64 x 64 float-float weights without the prefactor c, row-major, the tiles of
+// a block row consecutive (the band of blocks in reach, 8.0M weights at 40^3 instead of the 22.6M
+// of the whole rows).  The positive two-product form loses nothing to cancellation, unlike
+// P_in + (1 - f0_p) D where D is close to -P_in.
+
+// (f, 1 - f) as float-float pairs in the padded energy order (the padding keeps its zeros)
+__global__ void k_f0_map(const double *__restrict__ f, int n, const int *__restrict__ pmap, float4 *__restrict__ out) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const double v = f[i];
+    const float2 a = ff_split(v), b = ff_split(1.0 - v);
+    out[pmap[i]] = make_float4(a.x, a.y, b.x, b.y);
+  }
+}
+
+// One CTA per coefficient tile (grid-stride): the weights of its rows go out directly, those of its
+// columns (the reverse direction: P_in and P_out swap) through a transposed copy in shared memory,
+// so both weight tiles are written in whole rows.  Float-float arithmetic: FP64 made the row form of
+// this pass cost 609 us at 40^3.
+__global__ void __launch_bounds__(256) k_weight_tiles(const TileD *__restrict__ tiles, int nt,
+                                                      const float4 *__restrict__ tc, const float4 *__restrict__ f0,
+                                                      float2 *__restrict__ W) {
+  __shared__ float2 tr[kTile][kTile + 1];
+  const int tid = threadIdx.x, col = tid & (kTile - 1), r0 = tid >> 6;
+  for (int t = blockIdx.x; t < nt; t += gridDim.x) {
+    const TileD D = tiles[t];
+    const bool diag = D.I == D.J;
+    const float4 *__restrict__ T = tc + (size_t)t * kTile * kTile;
+    float2 *__restrict__ Wu = W + (size_t)D.wu * kTile * kTile, *__restrict__ Wl = W + (size_t)D.wl * kTile * kTile;
+    const float4 fp = f0[D.J * kTile + col];
+#pragma unroll 4
+    for (int r = r0; r < kTile; r += 4) {
+      const float4 e = T[r * kTile + col];
+      const float2 pin = make_float2(e.x, e.y), pout = make_float2(e.z, e.w);
+      Wu[r * kTile + col] = ff_add(ff_mul(make_float2(fp.x, fp.y), pin), ff_mul(make_float2(fp.z, fp.w), pout));
+      if (!diag) {
+        const float4 fs = f0[D.I * kTile + r];
+        tr[col][r] = ff_add(ff_mul(make_float2(fs.x, fs.y), pout), ff_mul(make_float2(fs.z, fs.w), pin));
+      }
+    }
+    if (diag) continue;
+    __syncthreads();
+#pragma unroll 4
+    for (int r = r0; r < kTile; r += 4) Wl[r * kTile + col] = tr[r][col];
+    __syncthreads();
+  }
+}
+
+// F (natural state order, [n][3]) as float-float in the tiles' order: [block][direction][64]
+__device__ __forceinline__ size_t trF_at(int pos, int a) { return (size_t)(pos / kTile) * 3 * kTile + a * kTile + pos % kTile; }
+__global__ void k_trF_map(const double *__restrict__ F, int n, const int *__restrict__ pmap, float2 *__restrict__ out) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < 3 * n; i += gridDim.x * blockDim.x)
+    out[trF_at(pmap[i / 3], i % 3)] = ff_split(F[i]);
+}
+
+// The sweep: CTA b takes the contiguous range [b nw / G, (b + 1) nw / G) of the weight tiles
+// (block-row-major), staged through a two-deep ring of bulk copies (32 KB of weights and the 1.5 KB
+// of F of the column block per stage; three CTAs per SM).  Thread (ti, tj) takes rows 4 ti .. + 3 and
+// columns 2 tj, 2 tj + 1, 32 + 2 tj, 33 + 2 tj, three directions: 12 float-float sums that stay in
+// registers over all tiles of one block row (a segment; desc.w marks its last tile), lazily
+// renormalised (at most 4 terms per tile, 64 at most per segment, see kTrSegTiles), then
+// reduce-scattered over the 16 lanes of a row into part[segment][direction][row].  Bound by
+// instruction issue: per weight 3 multiply-adds of 12 operations and 0.5 shared-memory loads.
+// At 40^3 it replaces a row stream of every pair (48.8 us per pass).
+struct alignas(16) TrTile {
+  int J, seg, last, pad;
+};
+constexpr int kTrSegTiles = 16;  // tiles of one segment at most (64 terms per sum)
+constexpr unsigned kTrTileBytes = kTile * kTile * sizeof(float2);
+constexpr unsigned kTrStageBytes = kTrTileBytes + 3 * kTile * sizeof(float2);
+constexpr int kTrStages = 2, kTrCtas = 3;
+constexpr size_t kTrTileSmem = (size_t)kTrStages * kTrStageBytes + 64;
+
+__global__ void __launch_bounds__(256, kTrCtas) k_stream_tr_tiles(const TrTile *__restrict__ list, int nw,
+                                                                  const float2 *__restrict__ W,
+                                                                  const float2 *__restrict__ F,
+                                                                  float2 *__restrict__ part, int *__restrict__ err) {
+  extern __shared__ __align__(128) unsigned char trs[];
+  unsigned long long *bars = (unsigned long long *)(trs + kTrStages * kTrStageBytes);
+  TrTile *sdesc = (TrTile *)(bars + kTrStages);
+  const int tid = threadIdx.x, lane = tid & 31, tj = tid & 15, ti = tid >> 4;
+  const int t0 = (int)((long long)blockIdx.x * nw / gridDim.x), t1 = (int)((long long)(blockIdx.x + 1) * nw / gridDim.x);
+  const int nloc = t1 - t0;
+  if (tid == 0) {
+    for (int k = 0; k < kTrStages; ++k) mbar_init(bars + k, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  int issued = 0;
+  auto issue = [&](int k, const TrTile &D) {
+    const int s = k % kTrStages;
+    sdesc[s] = D;
+    unsigned char *buf = trs + (size_t)s * kTrStageBytes;
+    mbar_expect_tx(bars + s, kTrStageBytes);
+    const unsigned char *src = (const unsigned char *)(W + (size_t)(t0 + k) * kTile * kTile);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) bulk_g2s(buf + q * (kTrTileBytes / 2), src + q * (kTrTileBytes / 2), kTrTileBytes / 2, bars + s);
+    bulk_g2s(buf + kTrTileBytes, F + (size_t)D.J * 3 * kTile, 3 * kTile * sizeof(float2), bars + s);
+  };
+  auto desc = [&](int k) {
+    const int4 v = reinterpret_cast<const int4 *>(list)[t0 + k];
+    return TrTile{v.x, v.y, v.z, v.w};
+  };
+  if (tid == 0)
+    for (; issued < kTrStages && issued < nloc; ++issued) issue(issued, desc(issued));
+  TrTile next{};
+  if (tid == 0 && issued < nloc) next = desc(issued);
+  float acc[4][3][2];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) acc[i][c][0] = acc[i][c][1] = 0.f;
+  bool ok = true;
+  for (int k = 0; k < nloc; ++k) {
+    // thread 0 waits for tile k; the CTA barrier publishes it and frees the stage of tile k - 1
+    if (!__syncthreads_and(tid == 0 ? mbar_wait(bars + k % kTrStages, (unsigned)((k / kTrStages) & 1)) : true)) {
+      ok = false;
+      break;
+    }
+    if (tid == 0 && k >= 1 && issued < nloc) {
+      fence_proxy_async();  // the generic reads of tile k-1's stage before its refill
+      issue(issued, next);
+      ++issued;
+      if (issued < nloc) next = desc(issued);
+    }
+    const int s = k % kTrStages;
+    const TrTile D = sdesc[s];
+    const float4 *__restrict__ Wt = (const float4 *)(trs + (size_t)s * kTrStageBytes);
+    const float4 *__restrict__ Ft = (const float4 *)(trs + (size_t)s * kTrStageBytes + kTrTileBytes);
+    float4 fa[3], fb[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      fa[c] = Ft[c * (kTile / 2) + tj];
+      fb[c] = Ft[c * (kTile / 2) + 16 + tj];
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float4 w0 = Wt[(4 * ti + i) * (kTile / 2) + tj], w1 = Wt[(4 * ti + i) * (kTile / 2) + 16 + tj];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        ff_mac_lazy(acc[i][c][0], acc[i][c][1], make_float2(fa[c].x, fa[c].y), w0.x, w0.y);
+        ff_mac_lazy(acc[i][c][0], acc[i][c][1], make_float2(fa[c].z, fa[c].w), w0.z, w0.w);
+        ff_mac_lazy(acc[i][c][0], acc[i][c][1], make_float2(fb[c].x, fb[c].y), w1.x, w1.y);
+        ff_mac_lazy(acc[i][c][0], acc[i][c][1], make_float2(fb[c].z, fb[c].w), w1.z, w1.w);
+      }
+    }
+    if (D.last) {
+      float2 v[16];  // 12 sums (row i, direction c) and 4 zeros: lane tj ends with value tj
+#pragma unroll
+      for (int m = 0; m < 16; ++m)
+        v[m] = m < 12 ? make_float2(acc[m / 3][m % 3][0], acc[m / 3][m % 3][1]) : make_float2(0.f, 0.f);
+      ff_reduce_scatter<16, 8>(v, lane);
+      if (tj < 12) part[(size_t)D.seg * 3 * kTile + (tj % 3) * kTile + 4 * ti + tj / 3] = v[0];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) acc[i][c][0] = acc[i][c][1] = 0.f;
+    }
+  }
+  if (!ok) {
+    *err = 3;
+    if (tid == 0) {  // drain: wait (bounded) for every copy this CTA issued
+      for (int k = 0; k < kTrStages; ++k) {
+        const int uses = issued / kTrStages + (k < issued % kTrStages ? 1 : 0);
+        if (uses > 0) mbar_wait(bars + k, (unsigned)((uses - 1) & 1));
+      }
+    }
+  }
+}
+
 // ------------------------------------------------------------ finalisers
 
 // Row totals of the (A, B) partials (coefficient variants) or of the literal sums.
@@ -2836,6 +3010,55 @@ __global__ void __launch_bounds__(256) k_fin_tr(const int *__restrict__ item_ptr
   if (threadIdx.x == 0) red[blockIdx.x] = m;
 }
 
+// The same over the segments of the tile sweep (segr: each block's segments [x, y)): a CTA takes half
+// a block, 32 states in energy order (ord: their state numbers, -1 in the padding), with one warp per
+// direction, so that the FP64 arithmetic (1/64 of the FP32 rate) spreads over about as many SMs as
+// there are.  The weights lack the prefactor c, applied here.  red[2 block + half]: max |dF|, max |F|.
+constexpr int kFinTrStates = kTile / 2;
+__global__ void __launch_bounds__(3 * kFinTrStates) k_fin_tr_tiles(const int2 *__restrict__ segr,
+                                                                   const float2 *__restrict__ part,
+                                                                   const int *__restrict__ ord, double c,
+                                                                   const double *__restrict__ tau,
+                                                                   const double *__restrict__ vel3,
+                                                                   const double *__restrict__ Fold,
+                                                                   double *__restrict__ Fnew, float2 *__restrict__ Fff,
+                                                                   double2 *__restrict__ red) {
+  __shared__ double2 wm[3];
+  const int lane = threadIdx.x & 31, a = threadIdx.x >> 5, blk = blockIdx.x >> 1;
+  const int j = (blockIdx.x & 1) * kFinTrStates + lane, pos = blk * kTile + j;
+  const int2 sr = segr[blk];
+  const int r = ord[pos];
+  double t = 0.0, v = 0.0, fo = 0.0;
+  if (r >= 0) {
+    t = tau[r];
+    v = vel3[3 * r + a];
+    fo = Fold[3 * r + a];
+  }
+  float2 S = make_float2(0.f, 0.f);
+  const float2 *__restrict__ p = part + a * kTile + j;
+#pragma unroll 4
+  for (int q = sr.x; q < sr.y; ++q) S = ff_add(S, p[(size_t)q * 3 * kTile]);
+  double dm = 0.0, fm = 0.0;
+  if (r >= 0) {
+    const double Fn = t * (v + c * ff_to_double(S.x, S.y));
+    dm = fmax(0.0, fabs(Fn - fo));
+    fm = fmax(0.0, fabs(Fn));
+    Fnew[3 * r + a] = Fn;
+    Fff[trF_at(pos, a)] = ff_split(Fn);
+  }
+  // the maxima of non-negative numbers are those of their bit patterns (integer instructions)
+  unsigned long long du = (unsigned long long)__double_as_longlong(dm), fu = (unsigned long long)__double_as_longlong(fm);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    du = max(du, __shfl_xor_sync(0xFFFFFFFFu, du, o));
+    fu = max(fu, __shfl_xor_sync(0xFFFFFFFFu, fu, o));
+  }
+  if (lane == 0) wm[a] = make_double2(__longlong_as_double((long long)du), __longlong_as_double((long long)fu));
+  __syncthreads();
+  if (threadIdx.x == 0)
+    red[blockIdx.x] = make_double2(fmax(wm[0].x, fmax(wm[1].x, wm[2].x)), fmax(wm[0].y, fmax(wm[1].y, wm[2].y)));
+}
+
 __global__ void k_red_final(const double2 *__restrict__ red, int n, double *__restrict__ out) {
   double d = 0.0, m = 0.0;
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
@@ -2850,14 +3073,14 @@ __global__ void k_red_final(const double2 *__restrict__ red, int n, double *__re
   }
 }
 
-// F^0 = tau v and its float-float copy
+// F^0 = tau v and its float-float copy (pmap: in the tiles' order, else null)
 __global__ void k_tr_init(const double *__restrict__ tau, const double *__restrict__ vel3, int ns,
-                          double *__restrict__ F, float2 *__restrict__ Fff) {
+                          const int *__restrict__ pmap, double *__restrict__ F, float2 *__restrict__ Fff) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= 3 * ns) return;
   const double v = tau[i / 3] * vel3[i];
   F[i] = v;
-  Fff[i] = ff_split(v);
+  Fff[pmap ? trF_at(pmap[i / 3], i % 3) : (size_t)i] = ff_split(v);
 }
 
 // Deterministic single-block sums: out[0] = sum f, out[1] = sum eps f, out[2] = sum I.

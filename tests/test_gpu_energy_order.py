@@ -51,3 +51,46 @@ def test_energy_ordered_tiles_hold_every_nonzero_pair(pb, name, variant):  # noq
     if variant == "ff":
         dev.set_g2(T(ch.export()["g2"]))
         assert np.abs(dev.collision(T(f)).cpu().numpy() - I).max() <= MUTUAL * ab.max()
+
+
+@pytest.mark.parametrize("name", list(CASES))
+def test_transport_over_tiles(pb, name):  # noqa: F811
+    """The automatic transport shape on the tiles: one map against the oracle and the row sweep, the
+    residual numbers, the weights that stay in use after set_g2 until the next setup, and the row
+    form after it."""
+    m = CASES[name][0]()
+    o = oracle.Oracle(m)
+    ch = pb.Channels.from_model(m)
+    dev, rows = pb.Device(ch, transport=True), pb.Device(ch, transport=True, dense_rows=2)
+    rng = np.random.default_rng(43)
+    f0, v = o.window_values(m.f_fermi(m.emin() - 0.2)), o.window_values(m.vel)
+    F = rng.normal(size=(o.nstate, 3))
+    ref, _ = o.transport_map(f0, v, F)
+    got = dev.transport_map(T(f0), T(v), T(F)).cpu().numpy()
+    assert nrel(got, ref) <= TOL
+    assert nrel(rows.transport_map(T(f0), T(v), T(F)).cpu().numpy(), got) <= TOL
+    res = T(np.zeros(3))
+    dev.transport_iterate(T(v), T(F), resid=res)
+    d, top = np.abs(got - F).max(), np.abs(got).max()
+    assert np.abs(res.cpu().numpy() - np.array([d / top, d, top])).max() <= 1e-14 * max(d, top)
+    dev.set_g2(T(2.0 * ch.export()["g2"]))
+    assert np.array_equal(dev.transport_iterate(T(v), T(F)).cpu().numpy(), got)
+    dev.transport_setup(T(f0))
+    twice = dev.transport_iterate(T(v), T(F)).cpu().numpy()  # tau halves, tau W stays
+    assert np.abs(twice - (got - 0.5 * v / o.rates(f0)[:, None])).max() <= TOL * np.abs(got).max()
+    dev.check()
+
+
+def test_transport_segments_of_many_tiles(pb):  # noqa: F811
+    """A CTA's run of one block row longer than the 16 tiles that one lazily renormalised sum may
+    take (92 blocks of states at one energy): sampled rows against the oracle."""
+    m = synth.make_flat_einstein(18)
+    o = oracle.Oracle(m)
+    dev = pb.Device(pb.Channels.from_model(m), transport=True)
+    rng = np.random.default_rng(47)
+    f0, v, F = rng.uniform(0, 1, o.nstate), rng.normal(size=(o.nstate, 3)), rng.normal(size=(o.nstate, 3))
+    rows = np.concatenate([np.arange(3), rng.integers(0, o.nstate, 20), [o.nstate - 1]]).astype(np.int32)
+    ref, _ = o.transport_map(f0, v, F, rows=rows)
+    got = dev.transport_map(T(f0), T(v), T(F)).cpu().numpy()
+    assert np.abs(got[rows] - ref).max() <= TOL * np.abs(got).max()
+    dev.check()
