@@ -23,7 +23,7 @@
 //
 // Symmetric tiles (precision 1 and 2, every instance's channel list verified closed under
 // reversal): each instance takes a run of 64-state blocks of one padded state space, its states in
-// energy order, and the tiles of its upper block triangle within reach of a phonon are stored as
+// energy order (precision 2: in state order, all tiles of the triangle), and the tiles of its upper block triangle within reach of a phonon are stored as
 // 64 x 64 tiles (zero where a state pair has no channel), as in the single-system sweeps, so each
 // unordered state pair is streamed once for both of its directions and the pairs whose coefficients
 // are zero by their distance in energy are not streamed at all.  One launch of the single-system
@@ -451,7 +451,7 @@ BatchTiles batch_tiles_for(const pb_channels *const *chs, int32_t n, int prec, i
     so += ch->nstate;
     double gmax = 0.0;
     for (const double g : ch->g2) gmax = std::max(gmax, g);
-    tile_plan_add(ch, complete, energy_reach(ch, gmax), T);
+    tile_plan_add(ch, prec == 1, complete, energy_reach(ch, gmax), T);
   }
   const int64_t nt = (int64_t)T.tiles.size();
   if (nt == 0 || nt >= INT32_MAX / 2 || T.npart >= INT32_MAX) return T;

@@ -228,7 +228,7 @@ double energy_reach(const pb_channels *ch, double scale) {
 }
 
 // The symmetric tiles of one system or of a batch's systems one after the other: each system's
-// states in energy order, padded to whole blocks of kTile, and the tiles of its upper block
+// states in energy order (C32: in state order), padded to whole blocks of kTile, and the tiles of its upper block
 // triangle within reach of each other (kernels.cuh).
 struct TilePlan {
   int nb = 0;                     // blocks
@@ -245,17 +245,21 @@ struct TilePlan {
 
 // complete: every row holds every state (the reach alone decides); else the stored channels within
 // reach do.  In energy order the columns that meet block row I are I .. hi(I), hi made monotone, so
-// that the rows that meet block column J are a contiguous range too.
-void tile_plan_add(const pb_channels *ch, bool complete, double reach, TilePlan &T) {
+// that the rows that meet block column J are a contiguous range too.  energy false: the whole
+// triangle in state order, for the FP32 tiles (C32): their block sums are FP32, so another order of
+// the states changes df/dt by 1e-9 and more, the size of the sums' own rounding.
+void tile_plan_add(const pb_channels *ch, bool energy, bool complete, double reach, TilePlan &T) {
   const int64_t ns = ch->nstate;
   const double *eps = ch->eps.data();
   std::vector<int32_t> ord((size_t)ns), pos((size_t)ns);
   std::iota(ord.begin(), ord.end(), 0);
-  std::stable_sort(ord.begin(), ord.end(), [&](int32_t a, int32_t b) { return eps[a] < eps[b]; });
+  if (energy) std::stable_sort(ord.begin(), ord.end(), [&](int32_t a, int32_t b) { return eps[a] < eps[b]; });
   for (int64_t i = 0; i < ns; ++i) pos[ord[i]] = (int32_t)i;
   const int nb = (int)((ns + dev::kTile - 1) / dev::kTile);
   std::vector<int32_t> top((size_t)ns);  // last position in reach of each position
-  if (complete) {
+  if (!energy) {
+    std::fill(top.begin(), top.end(), (int32_t)std::max<int64_t>(ns - 1, 0));
+  } else if (complete) {
     for (int64_t i = 0, j = 0; i < ns; ++i) {
       j = std::max(j, i);
       while (j + 1 < ns && eps[ord[j + 1]] - eps[ord[i]] <= reach) ++j;
@@ -813,10 +817,11 @@ bool tiles_pay(int64_t nt, int64_t ns, int64_t nsw) {
 // serves (p, s) with P_in and P_out swapped); dense_rows 3, or automatic (0) on complete rows or
 // when the tiles stream fewer bytes than the rows (pays)
 // T: the tile plan, filled in when they may be taken.
-bool sym_for(const pb_channels *ch, const pb_dev_opts &o, bool merged, bool complete, int64_t nsw, TilePlan &T) {
+bool sym_for(const pb_channels *ch, const pb_dev_opts &o, bool c32, bool merged, bool complete, int64_t nsw,
+             TilePlan &T) {
   if (!(merged && ch->closed && o.variant == PB_VARIANT_FF && o.stream_mode != 2)) return false;
   if (o.dense_rows != 3 && o.dense_rows != 0) return false;
-  tile_plan_add(ch, complete, energy_reach(ch, 1.0), T);
+  tile_plan_add(ch, !c32, complete, energy_reach(ch, 1.0), T);
   if (T.tiles.size() >= (size_t)INT32_MAX / 2 || T.npart >= INT32_MAX) return false;
   return o.dense_rows == 3 || complete || tiles_pay((int64_t)T.tiles.size(), ch->nstate, nsw);
 }
@@ -976,7 +981,7 @@ extern "C" int pb_dev_arena_bytes(const pb_channels *ch, const pb_dev_opts *opts
     const bool merged = make_plans(ch, opts, o, sm, P, S, &complete);
     const int nfin = (int)((P.ns + kFinBlock - 1) / kFinBlock);
     TilePlan T;
-    const bool sym = sym_for(ch, o, merged, complete, S.nchp, T);
+    const bool sym = sym_for(ch, o, c32, merged, complete, S.nchp, T);
     if (c32 && !sym)
       return set_error(PB_EINVAL, "pb_dev: the FP32 coefficient tiles (C32) need the symmetric tiles: a "
                                   "closure-checked list whose rows are complete or miss few partners (or dense_rows 3)");
@@ -1018,7 +1023,7 @@ extern "C" int pb_dev_create(const pb_channels *ch, const pb_dev_opts *opts, voi
   bool merged = false, complete = false, sym = false;
   try {
     merged = make_plans(ch, opts, o, sm, P, S, &complete);
-    sym = sym_for(ch, o, merged, complete, S.nchp, T);
+    sym = sym_for(ch, o, c32, merged, complete, S.nchp, T);
   } catch (const std::bad_alloc &) {
     delete d;
     return set_error(PB_ENOMEM, "pb_dev_create: out of host memory");
