@@ -38,8 +38,10 @@ struct BInst {
   float k2;           // -log2(e) / (2 sigma^2)
   int soff;           // first global state of the instance
   int ns;             // states of the instance
-  long long doff;     // dense form: first (state, partner, branch) slot of the instance
-  int npp, nm;        // dense form: partner slots per state (ns rounded up to 32), branches
+  long long doff;     // dense form: the instance's first value in g2d
+  long long poff;     // its first slot in pidx
+  long long moff;     // its first entry in the slot map
+  int nm, pad;        // branches
 };
 
 template <int MODE>
@@ -99,35 +101,41 @@ __global__ void __launch_bounds__(512) k_stream_gbatch(const Item *__restrict__ 
 }
 
 // Dense pair-major form of the FP32 batch sweep (as k_stream_g_dense, per instance): every
-// instance keeps |g|^2 in one slot per (state, partner, branch), g2d[doff + (s * npp + p) * nm
-// + nu], zero where no channel exists, so no index is streamed.  An item is a run of partners
-// [I.start, I.start + I.len) of the global row I.row; partner records come through L1 (each CTA
-// takes a contiguous item range, mostly of one instance).  The per-pair arithmetic is
+// instance's pairs in reach have one slot each, their branches together at g2d[doff + slot * nm],
+// their partners (numbered within the instance) at pidx[poff + slot].  An item is a bundle of 32
+// chains of the global row I.row, its slots numbered within the instance (LanePlan); partner records
+// come through L1 (CTA b takes the items [cbeg[b], cbeg[b + 1]), ranges of about equal work, mostly
+// of one instance: rows differ tenfold in length over the instances).  The per-pair arithmetic is
 // k_stream_g_dense's (the bracket collected per pair).
 __global__ void __launch_bounds__(512, 2) k_stream_gbatch_dense(const Item *__restrict__ items,
-                                                             const int *__restrict__ item_inst, int nitems,
+                                                             const int *__restrict__ item_inst,
+                                                             const int *__restrict__ cbeg,
                                                              const BInst *__restrict__ inst,
                                                              const float *__restrict__ g2d,
+                                                             const uint32_t *__restrict__ pidx,
                                                              const uint4 *__restrict__ gstate,
                                                              Part4 *__restrict__ part) {
-  const int per = (nitems + gridDim.x - 1) / gridDim.x;
-  const int begin = blockIdx.x * per;
-  const int end = min(nitems, begin + per);
+  const int begin = cbeg[blockIdx.x], end = cbeg[blockIdx.x + 1];
   const int lane = threadIdx.x & 31;
   const int wib = threadIdx.x >> 5, nw = blockDim.x >> 5;
   for (int it = begin + wib; it < end; it += nw) {
     const Item I = items[it];
     const BInst B = inst[item_inst[it]];
     const uint4 ss = __ldg(gstate + I.row);
-    const int base = B.cpad - rec_lnm(ss);
+    const float2 *__restrict__ tab = B.tab + (B.cpad - rec_lnm(ss));
     const uint4 *__restrict__ gsi = gstate + B.soff;
     const int nm = B.nm;
-    const float *__restrict__ gr = g2d + B.doff + (long long)(I.row - B.soff) * B.npp * nm;
+    const float *__restrict__ gq = g2d + B.doff + (I.start + lane) * nm;  // the pair's nm branches
+    const uint32_t *__restrict__ pr = pidx + B.poff + I.start + lane;
     const float fs = __uint_as_float(ss.z), fsl = rec_f_lo(ss), es = __uint_as_float(ss.x), esl = rec_eps_lo(ss);
     float sum = 0.f, comp = 0.f;
-    for (int j = lane; j < I.len; j += 32) {
-      const int p = (int)I.start + j;
-      if (p >= B.ns) break;
+    uint32_t pn = pr[0];  // the next pair's partner, loaded a step ahead
+#pragma unroll 1
+    for (int left = I.len; left > 0; --left) {
+      const bool gap = pn >> 31;
+      const int p = (int)min(pn & 0x7FFFFFFFu, (uint32_t)(B.ns - 1));  // past the chain's end: zero |g|^2
+      pr += 32;
+      if (left > 1) pn = pr[0];
       const uint4 sp = __ldg(gsi + p);
       const float dh = __fsub_rn(es, __uint_as_float(sp.x));
       const float dl = __fsub_rn(esl, rec_eps_lo(sp));
@@ -136,8 +144,7 @@ __global__ void __launch_bounds__(512, 2) k_stream_gbatch_dense(const Item *__re
       const float delta = fmaf(fsl, fp, fpl * fs);
       const float alpha = (fs - fp) + (fsl - fpl);
       const float betap = (A + fsl) - delta, gammap = (Bq + fpl) - delta;
-      const float2 *__restrict__ tr = B.tab + (base + rec_lnm(sp));
-      const float *__restrict__ gq = gr + (long long)p * nm;
+      const float2 *__restrict__ tr = tab + rec_lnm(sp);
       auto term = [&](float gv, float2 t) {
         const float a = (dh + t.x) + dl;  // x + w
         const float e = (dh - t.x) + dl;  // x - w
@@ -148,7 +155,7 @@ __global__ void __launch_bounds__(512, 2) k_stream_gbatch_dense(const Item *__re
       };
       float acc = 0.f;
       if (nm <= kDenseBranches) {
-        // the pair's loads first; even nm: slot offsets are even (npp is a multiple of 32)
+        // the pair's loads first; even nm: slot offsets are even (doff too: slots come in bundles of 32)
         float gv[kDenseBranches];
         float2 tv[kDenseBranches];
         if ((nm & 1) == 0) {
@@ -174,31 +181,56 @@ __global__ void __launch_bounds__(512, 2) k_stream_gbatch_dense(const Item *__re
         for (int nu = 0; nu < nm; ++nu) acc += term(__ldcs(gq + nu), __ldg(tr + nu));
       }
       kahan_add(sum, comp, acc);
+      if (gap) kahan_add(sum, comp, 0.f);
+      gq += 32 * nm;
     }
     const double v = warp_sum_ff(make_float2(sum, -comp));
     if (lane == 0) part[it] = make_part4(v, 0.0, 0.0, 0.0);
   }
 }
 
-// g2d slots of every stored channel of the batch (the array is cleared before)
-__global__ void __launch_bounds__(kBlock) k_dense_g2_batch(const Item *__restrict__ items,
+// smap[moff + local row * ns + p] = the slot of every pair of the items (the map holds ~0 elsewhere)
+__global__ void __launch_bounds__(kBlock) k_slot_map_batch(const Item *__restrict__ items,
                                                            const int *__restrict__ item_inst, int nitems,
                                                            const BInst *__restrict__ inst,
-                                                           const uint32_t *__restrict__ col,
-                                                           const float *__restrict__ g2, float *__restrict__ g2d) {
+                                                           const uint32_t *__restrict__ pidx,
+                                                           uint32_t *__restrict__ smap) {
   const int lane = threadIdx.x & 31;
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int nwarps = (gridDim.x * blockDim.x) >> 5;
   for (int it = warp; it < nitems; it += nwarps) {
     const Item I = items[it];
     const BInst B = inst[item_inst[it]];
-    float *__restrict__ gr = g2d + B.doff + (long long)(I.row - B.soff) * B.npp * B.nm;
+    for (int j = 0; j < I.len; ++j) {
+      const long long slot = I.start + 32 * j + lane;
+      const uint32_t p = pidx[B.poff + slot] & 0x7FFFFFFFu;
+      if (p < (uint32_t)B.ns) smap[B.moff + (long long)(I.row - B.soff) * B.ns + p] = (uint32_t)slot;
+    }
+  }
+}
+
+// g2d values of every stored channel of the batch that has a slot (the array is cleared before)
+__global__ void __launch_bounds__(kBlock) k_dense_g2_batch(const Item *__restrict__ items,
+                                                           const int *__restrict__ item_inst, int nitems,
+                                                           const BInst *__restrict__ inst,
+                                                           const uint32_t *__restrict__ col,
+                                                           const float *__restrict__ g2,
+                                                           const uint32_t *__restrict__ smap,
+                                                           float *__restrict__ g2d) {
+  const int lane = threadIdx.x & 31;
+  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int nwarps = (gridDim.x * blockDim.x) >> 5;
+  for (int it = warp; it < nitems; it += nwarps) {
+    const Item I = items[it];
+    const BInst B = inst[item_inst[it]];
+    const uint32_t *__restrict__ sr = smap + B.moff + (long long)(I.row - B.soff) * B.ns;
     for (int j = lane; j < I.len; j += 32) {
       const long long c = I.start + j;
       const float v = g2[c];
       if (v == 0.f) continue;  // row padding (and channels with |g|^2 = 0, whose slot stays 0)
       const unsigned cw = col[c];
-      gr[(long long)(cw & 0xFFFFFFu) * B.nm + (cw >> 24)] = v;
+      const uint32_t slot = sr[cw & 0xFFFFFFu];
+      if (slot != ~0u) g2d[B.doff + (long long)slot * B.nm + (cw >> 24)] = v;
     }
   }
 }
@@ -250,10 +282,15 @@ struct pb_batch {
   std::vector<int64_t> lenp;       // padded length of every global row
   std::vector<int32_t> row_inst;   // instance of every global row
   std::vector<int64_t> nch;        // [n] stored channels per instance
-  // dense pair-major FP32 form (precision 0): |g|^2 in (state, partner, branch) slots
+  // dense pair-major FP32 form (precision 0): |g|^2 of the pairs in reach in slots; the instances'
+  // energies and reaches are kept for the plans of other item sizes (the channel lists may be gone)
   bool dense = false;
   float *g2d = nullptr;
-  std::vector<int32_t> npp;        // [n] partner slots per state of each instance
+  uint32_t *pidx0 = nullptr, *smap = nullptr;
+  int32_t *cbeg = nullptr;         // item ranges of the CTAs, one table per CTAs-per-SM choice
+  int64_t slot_cap = 0, value_cap = 0, map_size = 0;
+  std::vector<double> heps, reach;           // [ns], [n]
+  std::vector<pb::dev::BInst> hinst;         // [n]
   char *arena = nullptr;
   size_t bytes = 0;
   Item *items = nullptr;
@@ -297,16 +334,14 @@ struct BatchPlan {
   std::vector<int32_t> item_inst, item_ptr;
 };
 
-// dense: rows of npp partner slots, items of item_ch partners, Item.start = first partner
-void batch_plan(const pb_batch *b, int item_ch, BatchPlan &P, bool dense = false) {
+void batch_plan(const pb_batch *b, int item_ch, BatchPlan &P) {
   P.items.clear();
   P.item_inst.clear();
   P.item_ptr.assign(b->ns + 1, 0);
   int64_t off = 0;
   for (int64_t r = 0; r < b->ns; ++r) {
     P.item_ptr[r] = (int32_t)P.items.size();
-    const int64_t lenp = dense ? b->npp[b->row_inst[r]] : b->lenp[r];
-    if (dense) off = 0;
+    const int64_t lenp = b->lenp[r];
     if (lenp > 0) {
       const int64_t chunks = lenp / kRowPad;
       const int64_t np = std::max<int64_t>(1, (lenp + item_ch - 1) / item_ch);
@@ -338,36 +373,55 @@ int64_t batch_items_count(const std::vector<int64_t> &lenp, int item_ch) {
 
 // Dense pair-major FP32 batch (pb_batch_opts.layout 0 with precision 0): used when the stored
 // channels fill at least 85% of all instances' (state, partner, branch) slots; npp = nstate
-// rounded up to 32.  A dense work item takes item_ch / 4 partners (at least 32).
-int batch_npp(const pb_channels *ch) { return (int)((ch->nstate + 31) / 32 * 32); }
-int64_t batch_dense_slots(const pb_channels *const *chs, int32_t n) {
-  int64_t s = 0;
-  for (int i = 0; i < n; ++i) s += chs[i]->nstate * (int64_t)batch_npp(chs[i]) * chs[i]->nmodes;
-  return s;
-}
+// rounded up to 32.  A piece of a row (LanePlan) takes item_ch / 4 partners (at least 32).
+int64_t batch_npp(int64_t ns) { return (ns + 31) / 32 * 32; }
 bool batch_dense_for(const pb_channels *const *chs, int32_t n, const pb_batch_opts &o) {
   if (o.precision != 0 || o.layout != 0) return false;
-  int64_t nch = 0;
-  for (int i = 0; i < n; ++i) nch += chs[i]->nch;
-  return (double)nch >= 0.85 * (double)batch_dense_slots(chs, n);
+  int64_t nch = 0, slots = 0;
+  for (int i = 0; i < n; ++i) {
+    nch += chs[i]->nch;
+    slots += chs[i]->nstate * batch_npp(chs[i]->nstate) * chs[i]->nmodes;
+  }
+  return (double)nch >= 0.85 * (double)slots;
 }
 int batch_dense_part(int item_ch) { return std::max(32, item_ch / 4 / 8 * 8); }
-std::vector<int64_t> batch_dense_lenp(const pb_channels *const *chs, int32_t n) {
-  std::vector<int64_t> lenp;
-  for (int i = 0; i < n; ++i)
-    for (int64_t r = 0; r < chs[i]->nstate; ++r) lenp.push_back(batch_npp(chs[i]));
-  return lenp;
+// What the arena reserves, for any item size up to 4096 (the autotuner's largest) or the batch's own:
+// a row's bundles hold its pairs in reach and, since each is as long as its longest chain, at most 32
+// times the longest chain more; they are no more than its pieces.
+struct BatchDenseCaps {
+  int64_t items = 0, slots = 0, values = 0, map = 0;
+};
+BatchDenseCaps batch_dense_caps(const pb_channels *const *chs, int32_t n, int item_ch) {
+  BatchDenseCaps C;
+  for (int i = 0; i < n; ++i) {
+    const int64_t ns = chs[i]->nstate, npp = batch_npp(ns);
+    const int64_t longest = std::min<int64_t>(npp, (batch_dense_part(std::max(4096, item_ch)) + 31) / 32 * 32);
+    std::vector<double> e(chs[i]->eps.begin(), chs[i]->eps.begin() + ns);
+    std::sort(e.begin(), e.end());
+    const double reach = energy_reach_f32(chs[i]);
+    int64_t slots = ns * longest;
+    for (int64_t r = 0, a = 0, b = 0; r < ns; ++r) {
+      while (e[r] - e[a] > reach) ++a;
+      while (b < ns && e[b] - e[r] <= reach) ++b;
+      slots += b - a;
+    }
+    C.items += ns * std::max<int64_t>(1, (npp + batch_dense_part(1024) - 1) / batch_dense_part(1024));
+    C.slots += slots;
+    C.values += slots * chs[i]->nmodes;
+    C.map += ns * ns;
+  }
+  return C;
 }
 
 constexpr int kBatchMinItem = 1024;  // smallest item size the arena is planned for
 
 struct BatchLayout {
   size_t items, item_inst, item_ptr, col, g2, gstate, tabs, inst, cs, part, acc, y, omega_tmp, tab_tmp, eps_tmp,
-      kc_tmp, g2d, total;
+      kc_tmp, g2d, pidx, smap, cbeg, total;
 };
 
 BatchLayout batch_layout(const pb_channels *const *chs, int n, int64_t ns, int64_t nchp, int64_t nitems_cap,
-                         int64_t dense_slots = 0) {
+                         const BatchDenseCaps &dc, int sm) {
   BatchLayout L{};
   size_t o = 0;
   auto take = [&](size_t bytes) {
@@ -399,7 +453,10 @@ BatchLayout batch_layout(const pb_channels *const *chs, int n, int64_t ns, int64
   L.tab_tmp = take(sizeof(double2) * maxq);
   L.eps_tmp = take(sizeof(double) * maxs);
   L.kc_tmp = take(sizeof(short4) * maxs);
-  L.g2d = take(sizeof(float) * (size_t)dense_slots);
+  L.g2d = take(sizeof(float) * (size_t)dc.values);
+  L.pidx = take(sizeof(uint32_t) * (size_t)dc.slots);
+  L.smap = take(sizeof(uint32_t) * (size_t)dc.map);
+  L.cbeg = take(dc.slots ? sizeof(int32_t) * 4 * ((size_t)sm * 4 + 1) : 0);
   L.total = o;
   return L;
 }
@@ -559,10 +616,12 @@ std::vector<int64_t> batch_lenp(const pb_channels *const *chs, int32_t n) {
   return lenp;
 }
 
-int batch_upload_plan(pb_batch *b, int item_ch, cudaStream_t st, bool csr = false) {
-  BatchPlan P;
-  const bool dense = b->dense && !csr;
-  batch_plan(b, dense ? batch_dense_part(item_ch) : item_ch, P, dense);
+int batch_dense_grid(const pb_batch *b, int ctas) {
+  const int64_t need = (b->nitems * 32 + 511) / 512;
+  return (int)std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)b->sm_count * ctas));
+}
+
+int batch_upload_items(pb_batch *b, const BatchPlan &P, int item_ch, cudaStream_t st) {
   if ((int64_t)P.items.size() > b->nitems_cap)
     return set_error(PB_EINVAL, "pb_batch: item size %d needs more items than the arena holds", item_ch);
   PB_CUDA(cudaMemcpyAsync(b->items, P.items.data(), sizeof(Item) * P.items.size(), cudaMemcpyHostToDevice, st));
@@ -578,7 +637,83 @@ int batch_upload_plan(pb_batch *b, int item_ch, cudaStream_t st, bool csr = fals
   return PB_OK;
 }
 
-// the tile sweep of every instance in one launch (the single-system kernels, with the slot map)
+// The dense form's plan for an item size: the instances' lane plans, the slot map, the |g|^2 values
+// scattered into the slots from the channel list, and the CTAs' item ranges.
+int batch_upload_dense(pb_batch *b, int item_ch, cudaStream_t st) {
+  BatchPlan D, C;
+  std::vector<uint32_t> pidx;
+  int64_t values = 0, map = 0;
+  for (int i = 0; i < b->n; ++i) {
+    const int64_t s0 = b->soff[i], ns = b->soff[i + 1] - s0;
+    LanePlan<uint32_t> P;
+    lane_plan(b->heps.data() + s0, ns, batch_npp(ns), batch_dense_part(item_ch), b->reach[i], true, P);
+    auto &B = b->hinst[i];
+    B.doff = values;
+    B.poff = (long long)pidx.size();
+    B.moff = map;
+    values += P.slots * B.nm;
+    map += ns * ns;
+    pidx.insert(pidx.end(), P.pidx.begin(), P.pidx.end());
+    for (int64_t r = 0; r < ns; ++r) D.item_ptr.push_back((int32_t)D.items.size() + P.item_ptr[r]);
+    for (Item it : P.items) {
+      it.row += (int)s0;
+      D.items.push_back(it);
+      D.item_inst.push_back(i);
+    }
+  }
+  D.item_ptr.push_back((int32_t)D.items.size());
+  if ((int64_t)pidx.size() > b->slot_cap || values > b->value_cap)
+    return set_error(PB_EINVAL, "pb_batch: item size %d needs more slots than the arena holds", item_ch);
+  int rc;
+  PB_CUDA(cudaMemcpyAsync(b->inst, b->hinst.data(), sizeof(pb::dev::BInst) * b->hinst.size(), cudaMemcpyHostToDevice, st));
+  PB_CUDA(cudaMemcpyAsync(b->pidx0, pidx.data(), sizeof(uint32_t) * pidx.size(), cudaMemcpyHostToDevice, st));
+  PB_CUDA(cudaMemsetAsync(b->smap, 0xFF, sizeof(uint32_t) * (size_t)b->map_size, st));
+  PB_CUDA(cudaMemsetAsync(b->g2d, 0, sizeof(float) * (size_t)values, st));
+  auto grid = [&] {
+    const int64_t need = (b->nitems * 32 + dev::kBlock - 1) / dev::kBlock;
+    return (int)std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)b->sm_count * 8));
+  };
+  if ((rc = batch_upload_items(b, D, item_ch, st))) return rc;
+  dev::k_slot_map_batch<<<grid(), dev::kBlock, 0, st>>>(b->items, b->item_inst, (int)b->nitems, b->inst, b->pidx0, b->smap);
+  PB_LAUNCHED("k_slot_map_batch");
+  batch_plan(b, 2048, C);  // the channel list's own items, for the scatter
+  if ((rc = batch_upload_items(b, C, 2048, st))) return rc;
+  dev::k_dense_g2_batch<<<grid(), dev::kBlock, 0, st>>>(b->items, b->item_inst, (int)b->nitems, b->inst, b->col, b->g2,
+                                                        b->smap, b->g2d);
+  PB_LAUNCHED("k_dense_g2_batch");
+  PB_CUDA(cudaStreamSynchronize(st));
+  if ((rc = batch_upload_items(b, D, item_ch, st))) return rc;
+  // per CTAs-per-SM choice, item ranges of about equal work (steps times branches)
+  std::vector<int64_t> cost((size_t)b->nitems + 1, 0);
+  for (int64_t i = 0; i < b->nitems; ++i)
+    cost[i + 1] = cost[i] + (int64_t)D.items[i].len * (2 + b->hinst[D.item_inst[i]].nm) + 4;
+  const int stride = b->sm_count * 4 + 1;
+  std::vector<int32_t> cb((size_t)4 * stride, (int32_t)b->nitems);
+  for (int c = 1; c <= 4; ++c) {
+    const int g = batch_dense_grid(b, c);
+    for (int k = 0; k <= g; ++k)
+      cb[(size_t)(c - 1) * stride + k] =
+          (int32_t)(std::lower_bound(cost.begin(), cost.end(), cost[b->nitems] * k / g) - cost.begin());
+  }
+  PB_CUDA(cudaMemcpyAsync(b->cbeg, cb.data(), sizeof(int32_t) * cb.size(), cudaMemcpyHostToDevice, st));
+  PB_CUDA(cudaStreamSynchronize(st));
+  return PB_OK;
+}
+
+int batch_upload_plan(pb_batch *b, int item_ch, cudaStream_t st) {
+  if (b->dense) {
+    try {
+      return batch_upload_dense(b, item_ch, st);
+    } catch (const std::bad_alloc &) {
+      return set_error(PB_ENOMEM, "pb_batch: out of host memory");
+    }
+  }
+  BatchPlan P;
+  batch_plan(b, item_ch, P);
+  return batch_upload_items(b, P, item_ch, st);
+}
+
+// the tile sweep of every instance in one launch (the single-system kernels)
 int batch_sweep_tiles(pb_batch *b, cudaStream_t st) {
   const int nt = b->tnt;
   if (b->prec == 2) {
@@ -626,11 +761,11 @@ int batch_sweep(pb_batch *b, cudaStream_t st) {
     PB_LAUNCHED("k_stream_ff (batch)");
     return PB_OK;
   }
-  const int64_t need = (b->nitems * 32 + 511) / 512;
-  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)b->sm_count * b->ctas));
+  const int grid = batch_dense_grid(b, b->ctas);  // of 512 threads
   if (b->dense) {
-    pb::dev::k_stream_gbatch_dense<<<grid, 512, 0, st>>>(b->items, b->item_inst, (int)b->nitems, b->inst, b->g2d,
-                                                          b->gstate, b->part);
+    pb::dev::k_stream_gbatch_dense<<<grid, 512, 0, st>>>(b->items, b->item_inst,
+                                                          b->cbeg + (size_t)(b->ctas - 1) * (b->sm_count * 4 + 1),
+                                                          b->inst, b->g2d, b->pidx0, b->gstate, b->part);
     PB_LAUNCHED("k_stream_gbatch_dense");
     return PB_OK;
   }
@@ -926,9 +1061,12 @@ extern "C" int pb_batch_arena_bytes(const pb_channels *const *chs, int32_t n, co
       pb_batch_opts o{};
       if (opts) o = *opts;
       const bool dense = batch_dense_for(chs, n, o);
-      const int64_t cap = std::max(batch_items_count(batch_lenp(chs, n), kBatchMinItem),
-                                   dense ? batch_items_count(batch_dense_lenp(chs, n), batch_dense_part(kBatchMinItem)) : 0);
-      *bytes = batch_layout(chs, n, ns, nchp, cap, dense ? batch_dense_slots(chs, n) : 0).total;
+      const BatchDenseCaps dc = dense ? batch_dense_caps(chs, n, o.item_channels) : BatchDenseCaps{};
+      const int64_t cap = std::max(batch_items_count(batch_lenp(chs, n), kBatchMinItem), dc.items);
+      int sm = 152, devid = 0;
+      if (cudaGetDevice(&devid) == cudaSuccess) cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, devid);
+      else cudaGetLastError();
+      *bytes = batch_layout(chs, n, ns, nchp, cap, dc, sm).total;
     }
   } catch (const std::bad_alloc &) {
     return set_error(PB_ENOMEM, "pb_batch_arena_bytes: out of host memory");
@@ -973,10 +1111,11 @@ extern "C" int pb_batch_create(const pb_channels *const *chs, int32_t n, const p
     b->lenp = b->prec >= 1 ? batch_pair_lenp(chs, n) : batch_lenp(chs, n);
     b->nitems_cap = batch_items_count(b->lenp, kBatchMinItem);
     b->dense = batch_dense_for(chs, n, o);
-    if (b->dense)
-      b->nitems_cap = std::max(b->nitems_cap,
-                               batch_items_count(batch_dense_lenp(chs, n), batch_dense_part(kBatchMinItem)));
-    for (int i = 0; i < n; ++i) b->npp.push_back(batch_npp(chs[i]));
+    const BatchDenseCaps dc = b->dense ? batch_dense_caps(chs, n, o.item_channels) : BatchDenseCaps{};
+    b->nitems_cap = std::max(b->nitems_cap, dc.items);
+    b->slot_cap = dc.slots;
+    b->value_cap = dc.values;
+    b->map_size = dc.map;
     b->soff.assign(n + 1, 0);
     for (int i = 0; i < n; ++i) {
       b->soff[i + 1] = b->soff[i] + chs[i]->nstate;
@@ -1047,7 +1186,7 @@ extern "C" int pb_batch_create(const pb_channels *const *chs, int32_t n, const p
       *out = b;
       return PB_OK;
     }
-    const BatchLayout L = batch_layout(chs, n, ns, nchp, b->nitems_cap, b->dense ? batch_dense_slots(chs, n) : 0);
+    const BatchLayout L = batch_layout(chs, n, ns, nchp, b->nitems_cap, dc, sm);
     if (bytes < L.total) {
       delete b;
       return set_error(PB_ENOMEM, "pb_batch_create: arena of %zu bytes is smaller than the %zu needed", bytes, L.total);
@@ -1067,7 +1206,16 @@ extern "C" int pb_batch_create(const pb_channels *const *chs, int32_t n, const p
     b->part = (Part4 *)(A + L.part);
     b->acc = (double *)(A + L.acc);
     b->y = (double *)(A + L.y);
-    if (b->dense) b->g2d = (float *)(A + L.g2d);
+    if (b->dense) {
+      b->g2d = (float *)(A + L.g2d);
+      b->pidx0 = (uint32_t *)(A + L.pidx);
+      b->smap = (uint32_t *)(A + L.smap);
+      b->cbeg = (int32_t *)(A + L.cbeg);
+      for (int i = 0; i < n; ++i) {
+        b->heps.insert(b->heps.end(), chs[i]->eps.begin(), chs[i]->eps.begin() + chs[i]->nstate);
+        b->reach.push_back(energy_reach_f32(chs[i]));
+      }
+    }
     double *om = (double *)(A + L.omega_tmp);
     double2 *tt = (double2 *)(A + L.tab_tmp);
     double *ep = (double *)(A + L.eps_tmp);
@@ -1102,9 +1250,7 @@ extern "C" int pb_batch_create(const pb_channels *const *chs, int32_t n, const p
       hin[i].k2 = (float)(-1.4426950408889634 / (2.0 * ch->sigma * ch->sigma));
       hin[i].soff = (int)b->soff[i];
       hin[i].ns = (int)ch->nstate;
-      hin[i].npp = batch_npp(ch);
       hin[i].nm = ch->nmodes;
-      hin[i].doff = i == 0 ? 0 : hin[i - 1].doff + (long long)chs[i - 1]->nstate * hin[i - 1].npp * hin[i - 1].nm;
       for (int64_t s = 0; s < ch->nstate; ++s) hcs[b->soff[i] + s] = c * norm;
       // the instance's rows in parallel from their first padded channel (hg2 is zero-filled)
       std::vector<int64_t> rs((size_t)ch->nstate + 1, coff);
@@ -1155,21 +1301,7 @@ extern "C" int pb_batch_create(const pb_channels *const *chs, int32_t n, const p
       if (e == cudaSuccess) e = cudaStreamSynchronize(st);
       if (e != cudaSuccess) status = cuda_fail(e, "pb_batch_create: upload");
     }
-    if (status == PB_OK && b->dense) {
-      // the dense slots from the channel list (through the channel plan), then the dense plan
-      cudaError_t e = cudaMemsetAsync(b->g2d, 0, sizeof(float) * (size_t)batch_dense_slots(chs, n), st);
-      if (e != cudaSuccess) status = cuda_fail(e, "pb_batch_create: clear dense slots");
-      if (status == PB_OK) status = batch_upload_plan(b, 2048, st, true);
-      if (status == PB_OK) {
-        const int64_t need = (b->nitems * 32 + dev::kBlock - 1) / dev::kBlock;
-        const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)b->sm_count * 8));
-        dev::k_dense_g2_batch<<<grid, dev::kBlock, 0, st>>>(b->items, b->item_inst, (int)b->nitems, b->inst, b->col,
-                                                            b->g2, b->g2d);
-        e = cudaGetLastError();
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) status = cuda_fail(e, "k_dense_g2_batch");
-      }
-    }
+    b->hinst = hin;
     if (status == PB_OK) {
       b->ctas = o.ctas_per_sm ? o.ctas_per_sm : 2;
       status = batch_upload_plan(b, o.item_channels ? o.item_channels : 2048, st);

@@ -52,7 +52,7 @@ struct Layout {
   size_t rp, item_ptr, items, col, coefA, coefB, g2, wt, eps, kc, R, omega, tab, part, acc, y, yff, fstage, Fa, Fb,
       Fff, tau, invtau, red, scal, obs, g2lo, gstate, tab32, col16, rp_real, vjpG, g2tab, vecs, hcol, hg2, hA, hB, sc,
       entries, hitems, titems, t_item_ptr, err, citems, citem_ptr, cpart, ccoefA, ccoefB, sidx16, sidx32, pcstart,
-      pcnt, srp, gitems, tiles, tcoef, tpart, pmap, prow, tbase, ord, trlist, trsegr, trtpart, trf0, g2d, gditems, gdptr, gacc, gaccg, trptr, trpart, total;
+      pcnt, srp, gitems, gdidx, gdmap, gdorder, gdwbeg, tiles, tcoef, tpart, pmap, prow, tbase, ord, trlist, trsegr, trtpart, trf0, g2d, gditems, gdptr, gacc, gaccg, trptr, trpart, total;
 };
 
 struct Plan {
@@ -166,33 +166,134 @@ size_t coef_bytes(int variant) {
 // over channels and the channel-only regions are empty).
 void plan_items(const std::vector<int64_t> &rp, int item_ch, std::vector<Item> &items, std::vector<int32_t> &ptr);
 
+// The energy distance beyond which both Gaussians of a channel are flushed to zero in FP32:
+// ex2.approx.ftz returns 0 below 2^-126, so at (x +- w)^2 / (2 sigma^2) > 126 ln 2; 127 and 0.1%
+// cover the FP32 rounding of x +- w and of the exponent.
+double energy_reach_f32(const pb_channels *ch) {
+  double wmax = 0.0;
+  for (const double w : ch->omega) wmax = std::max(wmax, w);
+  const double e = (wmax + std::sqrt(2.0 * 127.0 * std::log(2.0)) * ch->sigma) * 1.001;
+  return std::isfinite(e) ? e : INFINITY;
+}
+
+// The dense mixed-precision sweep's pairs (kernels.cuh): row r's partners 0 .. ns - 1 are cut into
+// pieces of at most `item` slots of npp (multiples of 8) and dealt to the 32 lanes of each; a lane's
+// partners within reach are a chain.  The row's chains, longest first, form bundles of 32, one work
+// item each: start = its first slot, len = steps, lane l's k-th pair at start + 32 k + l: its partner,
+// with the top bit of IDX set when partners out of reach follow it in the lane's order; all lower bits
+// set past the chain's end.
+template <typename IDX>
+struct LanePlan {
+  std::vector<Item> items;        // row = the list's state
+  std::vector<int32_t> item_ptr;  // [ns + 1]
+  std::vector<IDX> pidx;          // [slots] partner
+  int64_t slots = 0;
+};
+template <typename IDX>
+void lane_plan(const double *eps, int64_t ns, int64_t npp, int64_t item, double reach, bool fill, LanePlan<IDX> &P) {
+  const int64_t chunks = npp / kRowPad, np = std::max<int64_t>(1, (npp + item - 1) / item);
+  std::vector<int64_t> p0((size_t)np + 1, 0);  // first partner of every piece
+  for (int64_t k = 0; k < np; ++k) p0[k + 1] = p0[k] + kRowPad * (chunks / np + (k < chunks % np ? 1 : 0));
+  std::vector<std::vector<int32_t>> steps((size_t)ns);  // of every row's bundles
+  // the chain of every partner in reach, the chains' ranks by length (stable), the bundles
+  auto row = [&](int64_t r, std::vector<int32_t> &cnt, std::vector<int32_t> &rank) {
+    cnt.assign((size_t)np * 32, 0);
+    for (int64_t k = 0; k < np; ++k)
+      for (int64_t p = p0[k]; p < std::min(p0[k + 1], ns); ++p)
+        if (std::fabs(eps[r] - eps[p]) <= reach) ++cnt[(size_t)(k * 32 + (p - p0[k]) % 32)];
+    rank.resize(cnt.size());
+    std::iota(rank.begin(), rank.end(), 0);
+    std::stable_sort(rank.begin(), rank.end(), [&](int32_t a, int32_t b) { return cnt[a] > cnt[b]; });
+  };
+#pragma omp parallel
+  {
+    std::vector<int32_t> cnt, rank;
+#pragma omp for schedule(dynamic, 16)
+    for (int64_t r = 0; r < ns; ++r) {
+      row(r, cnt, rank);
+      for (size_t q = 0; q < rank.size() && cnt[rank[q]] > 0; q += 32) steps[r].push_back(cnt[rank[q]]);
+    }
+  }
+  P.item_ptr.assign((size_t)ns + 1, 0);
+  for (int64_t r = 0; r < ns; ++r) {
+    P.item_ptr[r] = (int32_t)P.items.size();
+    for (const int32_t n : steps[r]) {
+      Item it;
+      it.start = P.slots;
+      it.len = n;
+      it.row = (int)r;
+      P.items.push_back(it);
+      P.slots += 32 * (int64_t)n;
+    }
+  }
+  P.item_ptr[ns] = (int32_t)P.items.size();
+  if (!fill) return;
+  constexpr IDX kGap = (IDX)((IDX)1 << (8 * sizeof(IDX) - 1));
+  P.pidx.assign((size_t)P.slots, (IDX)(kGap - 1));
+#pragma omp parallel
+  {
+    std::vector<int32_t> cnt, rank, at, prev;
+#pragma omp for schedule(dynamic, 16)
+    for (int64_t r = 0; r < ns; ++r) {
+      row(r, cnt, rank);
+      at.assign(cnt.size(), -1);  // bundle and lane of every chain: 32 bundle + lane
+      for (size_t q = 0; q < rank.size() && cnt[rank[q]] > 0; ++q) at[rank[q]] = (int32_t)q;
+      std::fill(cnt.begin(), cnt.end(), 0);
+      prev.assign(cnt.size(), 0);
+      for (int64_t k = 0; k < np; ++k)
+        for (int64_t p = p0[k]; p < std::min(p0[k + 1], ns); ++p)
+          if (std::fabs(eps[r] - eps[p]) <= reach) {
+            const size_t c = (size_t)(k * 32 + (p - p0[k]) % 32);
+            const Item &it = P.items[(size_t)P.item_ptr[r] + at[c] / 32];
+            const size_t slot = (size_t)it.start + 32 * (size_t)cnt[c] + at[c] % 32;
+            P.pidx[slot] = (IDX)p;
+            if (cnt[c]++ > 0 && p - prev[c] > 32) P.pidx[slot - 32] |= kGap;
+            prev[c] = (int32_t)p;
+          }
+    }
+  }
+}
+
 // Dense pair-major form of the mixed-precision sweep (pb_dev_opts.channel_per_lane 5, or 0 when
-// the channel list fills at least 85% of the (row, branch, partner) slots): |g|^2 in one slot
-// per (row, branch, partner), rows of npp partner slots (nstate rounded up to 32), items of
-// `item` partners, about two per resident warp.
+// the channel list fills at least 85% of the (row, branch, partner) slots): the pairs in reach in
+// one slot each (LanePlan), their branches together; a piece of a row is about half a resident
+// warp's share of all pairs.
 struct GDense {
   bool on = false;
-  int npp = 0, nm = 0, item = 0;
-  int64_t nitems = 0;
+  int nm = 0;
   size_t bytes = 0;
+  int grid = 0;  // CTAs of the sweep (kDenseThreads threads, one per SM)
+  LanePlan<uint16_t> plan;
+  std::vector<int32_t> order, wbeg;  // items by length; each warp's range of them
 };
-GDense gdense_for(const pb_channels *ch, const pb_dev_opts &o, int sm) {
+GDense gdense_for(const pb_channels *ch, const pb_dev_opts &o, int sm, bool fill) {
   GDense g;
   const bool mixed = o.variant == PB_VARIANT_G32 || o.variant == PB_VARIANT_G16 || o.variant == PB_VARIANT_H16;
   if (!mixed || (o.channel_per_lane != 0 && o.channel_per_lane != 5)) return g;
   const int64_t ns = ch->nstate, nm = ch->nmodes;
-  if (ns == 0 || nm == 0) return g;
+  if (ns == 0 || nm == 0 || ns >= dev::kGapBit) return g;  // (more states than shared memory holds are refused later)
   const int64_t npp = (ns + 31) / 32 * 32;
   const double slots = (double)ns * (double)nm * (double)npp;
   if (o.channel_per_lane == 0 && (double)ch->row_ptr[ns] < 0.85 * slots) return g;
   g.on = true;
-  g.npp = (int)npp;
   g.nm = (int)nm;
   const int64_t warps = (int64_t)sm * 32;
-  const int64_t item = (ns * npp / (2 * warps) + 31) / 32 * 32;
-  g.item = (int)std::max<int64_t>(256, std::min<int64_t>(item, npp));
-  g.nitems = ns * std::max<int64_t>(1, (npp + g.item - 1) / g.item);
-  g.bytes = (size_t)(o.variant == PB_VARIANT_G32 ? 4 : 2) * (size_t)slots;
+  int64_t item = (ns * npp / (2 * warps) + 31) / 32 * 32;
+  item = std::max<int64_t>(256, std::min<int64_t>(item, npp));
+  lane_plan(ch->eps.data(), ns, npp, item, energy_reach_f32(ch), fill, g.plan);
+  g.bytes = (size_t)(o.variant == PB_VARIANT_G32 ? 4 : 2) * (size_t)nm * (size_t)g.plan.slots;
+  const auto &it = g.plan.items;
+  const int64_t n = (int64_t)it.size();
+  g.grid = (int)std::max<int64_t>(1, std::min<int64_t>((n * 32 + dev::kDenseThreads - 1) / dev::kDenseThreads, sm));
+  if (!fill) return g;
+  g.order.resize((size_t)n);
+  std::iota(g.order.begin(), g.order.end(), 0);
+  std::stable_sort(g.order.begin(), g.order.end(), [&](int32_t a, int32_t b) { return it[a].len > it[b].len; });
+  std::vector<int64_t> cost((size_t)n + 1, 0);  // in FP32-form branch evaluations, with a step's and an item's own work
+  for (int64_t q = 0; q < n; ++q) cost[q + 1] = cost[q] + (int64_t)it[g.order[q]].len * (2 + nm) + 4;
+  const int64_t nw = (int64_t)g.grid * (dev::kDenseThreads / 32);
+  for (int64_t w = 0; w <= nw; ++w)
+    g.wbeg.push_back((int32_t)(std::lower_bound(cost.begin(), cost.end(), (cost[n] * w + nw - 1) / nw) - cost.begin()));
   return g;
 }
 
@@ -439,11 +540,15 @@ Layout make_layout(const pb_channels *ch, const Plan &P, const Plan *S, int vari
   L.hitems = take(sizeof(Item) * nhi);
   L.titems = take(sizeof(Item) * ((variant == PB_VARIANT_PAPER) ? z.nentp / kRowPad + (int64_t)ns : 0));
   L.t_item_ptr = take(sizeof(int32_t) * (ns + 1));
-  L.part = take(sizeof(Part4) * std::max<int64_t>(std::max<int64_t>(W.nitems, gd.nitems),
+  L.part = take(sizeof(Part4) * std::max<int64_t>(std::max<int64_t>(W.nitems, (int64_t)gd.plan.items.size()),
                                                   (variant == PB_VARIANT_PAPER) ? z.nentp / kRowPad + (int64_t)ns : 0));
   L.g2d = take(gd.on ? gd.bytes : 0);
-  L.gditems = take(gd.on ? sizeof(Item) * (size_t)gd.nitems : 0);
+  L.gditems = take(gd.on ? sizeof(Item) * (size_t)(int64_t)gd.plan.items.size() : 0);
   L.gdptr = take(gd.on ? sizeof(int32_t) * (ns + 1) : 0);
+  L.gdidx = take(gd.on ? sizeof(uint16_t) * (size_t)gd.plan.slots : 0);
+  L.gdmap = take(gd.on ? sizeof(uint32_t) * ns * ns : 0);
+  L.gdorder = take(gd.on ? sizeof(int32_t) * gd.plan.items.size() : 0);
+  L.gdwbeg = take(gd.on ? sizeof(int32_t) * ((size_t)gd.grid * (dev::kDenseThreads / 32) + 1) : 0);
   L.rp_real = take(sizeof(int64_t) * (ns + 1));
   L.vjpG = take(sizeof(float2) * 3 * ns);
   L.g2tab = take(sizeof(float4) * 2 * 4 * ns);
@@ -588,8 +693,11 @@ struct pb_dev {
   void *g2lo = nullptr;     // |g|^2 in FP32 or BF16 (mixed-precision variants)
   // dense pair-major mixed-precision sweep (GDense)
   bool gdense = false;
-  int gd_npp = 0, gd_nitems = 0;
-  size_t gd_bytes = 0;
+  int gd_nitems = 0, gd_grid = 0;
+  int32_t *gd_order = nullptr, *gd_wbeg = nullptr;
+  uint16_t *gd_idx = nullptr;  // the partner of every slot
+  uint32_t *gd_map = nullptr;  // the slot of every pair [ns][ns]
+  size_t gd_bytes = 0, gd_slots = 0;
   void *g2d = nullptr;
   Item *gd_items = nullptr;
   int32_t *gd_item_ptr = nullptr;
@@ -987,7 +1095,7 @@ extern "C" int pb_dev_arena_bytes(const pb_channels *ch, const pb_dev_opts *opts
                                   "closure-checked list whose rows are complete or miss few partners (or dense_rows 3)");
     const TrRows tr = tr_rows_for(P.ns, sm, o.transport != 0, merged, complete, o.variant, o);
     *bytes = make_layout(ch, P, merged ? &S : nullptr, o.variant, o.transport != 0, nfin, sym ? &T : nullptr,
-                         gdense_for(ch, o, sm), o.adjoint != 0, c32 ? sizeof(float2) : sizeof(float4), tr.nseg, sm)
+                         gdense_for(ch, o, sm, false), o.adjoint != 0, c32 ? sizeof(float2) : sizeof(float4), tr.nseg, sm)
                  .total;
   } catch (const std::bad_alloc &) {
     return set_error(PB_ENOMEM, "pb_dev_arena_bytes: out of host memory");
@@ -1073,11 +1181,17 @@ extern "C" int pb_dev_create(const pb_channels *ch, const pb_dev_opts *opts, voi
   d->half_cps = (opts && opts->ctas_per_sm == 2) ? 2 : 3;
   d->tnt = (int)T.tiles.size();
   d->nsp = T.nsp;
-  const GDense gd = gdense_for(ch, o, sm);
+  GDense gd;
+  try {
+    gd = gdense_for(ch, o, sm, true);
+  } catch (const std::bad_alloc &) {
+    delete d;
+    return set_error(PB_ENOMEM, "pb_dev_create: out of host memory");
+  }
   d->gdense = gd.on;
-  d->gd_npp = gd.npp;
-  d->gd_nitems = (int)gd.nitems;
+  d->gd_nitems = (int)(int64_t)gd.plan.items.size();
   d->gd_bytes = gd.bytes;
+  d->gd_slots = (size_t)gd.plan.slots;
   const TrRows trr = tr_rows_for(d->ns, sm, d->transport, merged, complete, o.variant, o);
   d->tr_nseg = trr.nseg;
   d->tr_seglen = trr.seglen;
@@ -1124,6 +1238,11 @@ extern "C" int pb_dev_create(const pb_channels *ch, const pb_dev_opts *opts, voi
     d->g2d = A + L.g2d;
     d->gd_items = (Item *)(A + L.gditems);
     d->gd_item_ptr = (int32_t *)(A + L.gdptr);
+    d->gd_idx = (uint16_t *)(A + L.gdidx);
+    d->gd_order = (int32_t *)(A + L.gdorder);
+    d->gd_wbeg = (int32_t *)(A + L.gdwbeg);
+    d->gd_grid = gd.grid;
+    d->gd_map = (uint32_t *)(A + L.gdmap);
   }
   d->gstate = (uint4 *)(A + L.gstate);
   d->tab32 = (float2 *)(A + L.tab32);
@@ -1329,13 +1448,22 @@ extern "C" int pb_dev_create(const pb_channels *ch, const pb_dev_opts *opts, voi
         }
       }
       if (d->gdense) {
-        std::vector<int64_t> rpd((size_t)d->ns + 1);
-        for (int64_t r = 0; r <= d->ns; ++r) rpd[r] = r * gd.npp;
-        std::vector<Item> gi;
-        std::vector<int32_t> gp;
-        plan_items(rpd, gd.item, gi, gp);
-        UP(d->gd_items, gi.data(), sizeof(Item) * gi.size());
-        UP(d->gd_item_ptr, gp.data(), sizeof(int32_t) * gp.size());
+        UP(d->gd_items, gd.plan.items.data(), sizeof(Item) * gd.plan.items.size());
+        UP(d->gd_item_ptr, gd.plan.item_ptr.data(), sizeof(int32_t) * gd.plan.item_ptr.size());
+        UP(d->gd_order, gd.order.data(), sizeof(int32_t) * gd.order.size());
+        UP(d->gd_wbeg, gd.wbeg.data(), sizeof(int32_t) * gd.wbeg.size());
+        UP(d->gd_idx, gd.plan.pidx.data(), sizeof(uint16_t) * gd.plan.pidx.size());
+        cudaError_t e_ = cudaMemsetAsync(d->gd_map, 0xFF, sizeof(uint32_t) * (size_t)d->ns * (size_t)d->ns, st);
+        if (e_ == cudaSuccess) {
+          const int64_t need = ((int64_t)d->gd_nitems * 32 + dev::kBlock - 1) / dev::kBlock;
+          dev::k_slot_map<<<(int)std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)sm * 8)), dev::kBlock, 0, st>>>(
+              d->gd_items, d->gd_nitems, d->gd_idx, (int)d->ns, d->gd_map);
+          e_ = cudaGetLastError();
+        }
+        if (e_ != cudaSuccess) {
+          status = cuda_fail(e_, "k_slot_map");
+          break;
+        }
       }
       if (d->tr_nseg) {  // the row-block transport sweep's partials: row r owns r * nseg .. (r + 1) * nseg
         std::vector<int32_t> tp((size_t)d->ns + 1);
@@ -1617,8 +1745,8 @@ extern "C" int pb_dev_get_info(const pb_dev *d, pb_dev_info *info) {
     case PB_VARIANT_G32:
     case PB_VARIANT_G16:
     case PB_VARIANT_H16:
-      // dense pair-major: the (state, partner, branch) slots, zeros included; else |g|^2 + word
-      info->bytes_per_channel = d->gdense ? (d->nch ? (double)d->gd_bytes / (double)d->nch : 0.0)
+      // dense pair-major: the slots of the pairs in reach (each with its partner); else |g|^2 + word
+      info->bytes_per_channel = d->gdense ? (d->nch ? (double)(d->gd_bytes + d->gd_slots * sizeof(uint16_t)) / (double)d->nch : 0.0)
                                           : (d->variant == PB_VARIANT_G32 ? 4.0 : 2.0) + sizeof(uint32_t);
       break;
     case PB_VARIANT_PAPER:  // step 2: P_in, D, index, sc_col write; step 3: entry + sc_col gather
@@ -1730,12 +1858,10 @@ int launch_stream_t(pb_dev *d, int mode, const double *fd, const float2 *fff, co
       using T = std::remove_pointer_t<decltype(tag)>;
       const T *gl = (const T *)d->g2lo;
       if (d->gdense) {
-        const int gdg = (int)std::max<int64_t>(
-            1, std::min<int64_t>(((int64_t)d->gd_nitems * 32 + dev::kDenseThreads - 1) / dev::kDenseThreads, d->sm_count));
-        const int nd = d->gd_nitems, npp = d->gd_npp, nm = d->nmodes;
+        const int nm = d->nmodes;
         const T *gd = (const T *)d->g2d;
-        if (coll) dev::k_stream_g_dense<dev::MODE_COLL, T><<<gdg, dev::kDenseThreads, d->smem_f, st>>>(d->gd_items, nd, g, gd, npp, nm, d->gstate, ns, part);
-        else      dev::k_stream_g_dense<dev::MODE_RATE, T><<<gdg, dev::kDenseThreads, d->smem_f, st>>>(d->gd_items, nd, g, gd, npp, nm, d->gstate, ns, part);
+        if (coll) dev::k_stream_g_dense<dev::MODE_COLL, T><<<d->gd_grid, dev::kDenseThreads, d->smem_f, st>>>(d->gd_items, d->gd_order, d->gd_wbeg, g, gd, d->gd_idx, nm, d->gstate, ns, part);
+        else      dev::k_stream_g_dense<dev::MODE_RATE, T><<<d->gd_grid, dev::kDenseThreads, d->smem_f, st>>>(d->gd_items, d->gd_order, d->gd_wbeg, g, gd, d->gd_idx, nm, d->gstate, ns, part);
       } else if (d->g_lane) {
         launch_g_lane<T>(d->g_shape, coll, gg, d->sm_count, d->smem_f, st, d->items, n, g, gl, d->gstate, ns, part);
       } else {
@@ -2416,7 +2542,7 @@ int coef_setup(pb_dev *d, cudaStream_t st) {
       with_g2t(d->variant, [&](auto tag) {
         using T = std::remove_pointer_t<decltype(tag)>;
         dev::k_dense_g2<T><<<d->chan_grid(8), dev::kBlock, 0, st>>>(d->items, (int)d->nitems, rp, rr, d->col, d->g2,
-                                                                    d->nmodes, d->gd_npp, (T *)d->g2d, d->g2s);
+                                                                    d->gd_map, (int)d->ns, d->nmodes, (T *)d->g2d, d->g2s);
       });
       PB_LAUNCHED("k_dense_g2");
     }
@@ -2443,12 +2569,10 @@ int vjp_launch_mixed(pb_dev *d, const double *f, const double *lam, double wl, c
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((d->nitems * 32 + 511) / 512, (int64_t)d->sm_count * ctas));
   if (d->gdense) {
     // the dense pair-major sweep with the rate summands weighted by lam_s - lam_p
-    const int gdg = (int)std::max<int64_t>(
-        1, std::min<int64_t>(((int64_t)d->gd_nitems * 32 + dev::kDenseThreads - 1) / dev::kDenseThreads, d->sm_count));
     with_g2t(d->variant, [&](auto tag) {
       using T = std::remove_pointer_t<decltype(tag)>;
-      dev::k_stream_g_dense<dev::MODE_VJP, T><<<gdg, dev::kDenseThreads, smem, st>>>(
-          d->gd_items, d->gd_nitems, g, (const T *)d->g2d, d->gd_npp, d->nmodes, d->gstate, ns, d->part, lam32);
+      dev::k_stream_g_dense<dev::MODE_VJP, T><<<d->gd_grid, dev::kDenseThreads, smem, st>>>(
+          d->gd_items, d->gd_order, d->gd_wbeg, g, (const T *)d->g2d, d->gd_idx, d->nmodes, d->gstate, ns, d->part, lam32);
     });
     PB_LAUNCHED("k_stream_g_dense (vjp)");
   } else {

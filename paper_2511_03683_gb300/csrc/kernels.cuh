@@ -1337,26 +1337,37 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 3 : 1) k_stream_g_lane(const I
   }
 }
 
-// Dense pair-major form of the mixed-precision sweep.  |g|^2 is stored in one slot per
-// (row s, partner p, branch nu): g2d[(s * npp + p) * nm + nu], zero where the channel does not
-// exist, so no index is streamed; a pair's branches are contiguous (a few vector loads at fixed
-// offsets) and a warp's 32 partners one contiguous run.  A lane takes one partner at a time:
-// the partner record, the energy difference and the occupation products once per pair, then
-// the nm branches with their (hbar w, N) from the table row of q = k_p - k_s.  g_term's bracket
+// Dense pair-major form of the mixed-precision sweep.  Every state pair within reach of a phonon
+// has one slot, g2d[slot * nm + nu] for its branches (zero where the channel does not exist;
+// contiguous, a few vector loads at fixed offsets) and pidx[slot] = its partner; beyond that reach
+// both Gaussians are flushed to zero in FP32 and the pair adds exactly nothing (a third of the pairs
+// of the windowed grids is left).  A lane takes one pair at a time: the partner record, the energy
+// difference and the occupation products once per pair, then the nm branches with their (hbar w, N) from the table row of q = k_p - k_s.  g_term's bracket
 // with its first-order low-part corrections is bilinear in (G_a, G_e); collected per pair it is
 //   u = G_a (N alpha - gamma') + G_e (N alpha + beta'),   alpha = (f_s - f_p) + (f_s,lo - f_p,lo),
 //   delta = f_s,lo f_p + f_p,lo f_s,  beta' = A + f_s,lo - delta,  gamma' = B + f_p,lo - delta
 // (A = f_s (1 - f_p), B = (1 - f_s) f_p as g_term forms them), and the rate summand is
 // G_a (N + f_p) + G_e (N + 1 - f_p) with f_p = hi + lo: a few operations per branch besides the
-// Gaussians.  A lane's nm terms are summed and added to its compensated sum once per pair.  An
-// item is a run of partners of one row (I.start = s * npp + first partner); its partial goes to
-// part[item].x.  MODE_VJP: the FP32 adjoint's sum, the rate summands of each pair weighted by
+// Gaussians.  A lane's nm terms are summed and added to its compensated sum once per pair.
+// An item is a bundle of 32 chains of one row: chain = the pairs in reach that lane l takes when
+// the row's partners are dealt to the lanes in state order (partners p0 + l, p0 + l + 32, ... of one
+// piece of the row), the row's chains sorted by length (LanePlan on the host).  So the compensated
+// sums add the same terms in the same order as over all partners, where the pairs out of reach add
+// zeros (kGapBit of pidx: some follow this pair; the first zero may still move the compensation into
+// the sum, the others change nothing), while a bundle's lanes are busy for all of its I.len steps (lane l's slots are I.start + l
+// + 32 k).  Its partial goes to part[item].x.  Warp w takes the items order[wbeg[w]] ..
+// order[wbeg[w + 1] - 1], longest first and about equal steps for every warp (a small system has
+// little more than one bundle per resident warp, three to eight steps long).  MODE_VJP: the FP32 adjoint's sum, the rate summands of each pair weighted by
 // lam_s - lam_p (lam in FP32 after the records in shared memory; see k_stream_g_vjp).
 constexpr int kDenseBranches = 6;  // branches whose loads a lane issues together (more: one at a time)
+constexpr int kGapBit = 0x8000;
 constexpr int kDenseThreads = 1024;  // one CTA per SM (768 threads without spills measured slower)
 template <int MODE, typename G2T>
-__global__ void __launch_bounds__(kDenseThreads, 1) k_stream_g_dense(const Item *__restrict__ items, int nitems, GGeom g,
-                                                            const G2T *__restrict__ g2d, int npp, int nm,
+__global__ void __launch_bounds__(kDenseThreads, 1) k_stream_g_dense(const Item *__restrict__ items,
+                                                            const int *__restrict__ order,
+                                                            const int *__restrict__ wbeg, GGeom g,
+                                                            const G2T *__restrict__ g2d,
+                                                            const uint16_t *__restrict__ pidx, int nm,
                                                             const uint4 *__restrict__ gstate, int ns,
                                                             Part4 *__restrict__ part,
                                                             const float *__restrict__ lam32 = nullptr) {
@@ -1369,20 +1380,23 @@ __global__ void __launch_bounds__(kDenseThreads, 1) k_stream_g_dense(const Item 
   __syncthreads();
   const int lane = threadIdx.x & 31;
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int nwarps = (gridDim.x * blockDim.x) >> 5;
-  for (int it = warp; it < nitems; it += nwarps) {
+  const int qe = wbeg[warp + 1];
+  for (int q = wbeg[warp]; q < qe; ++q) {
+    const int it = order[q];
     const Item I = items[it];
     const int s = I.row;
     const uint4 ss = gsd[s];
     const int base = g.cpad - rec_lnm(ss);
-    const int p0 = (int)(I.start - (long long)s * npp);
-    const G2T *__restrict__ gr = g2d + (size_t)s * npp * nm;
+    const G2T *__restrict__ gr = g2d + (size_t)(I.start + lane) * nm;
+    const uint16_t *__restrict__ pr = pidx + I.start + lane;
     const float fs = __uint_as_float(ss.z), fsl = rec_f_lo(ss), es = __uint_as_float(ss.x), esl = rec_eps_lo(ss);
     const float ls = MODE == MODE_VJP ? lsm[s] : 0.f;
     float sum = 0.f, comp = 0.f;
-    for (int j = lane; j < I.len; j += 32) {
-      const int p = p0 + j;
-      if (p >= ns) break;  // the row's padding slots (zero |g|^2, no record)
+    int pn = pr[0];  // the next pair's partner, loaded a step ahead
+    for (int j = 0; j < I.len; ++j) {
+      const bool gap = pn & kGapBit;
+      const int p = min(pn & (kGapBit - 1), ns - 1);  // past the end of the lane's chain: zero |g|^2
+      if (j + 1 < I.len) pn = pr[32 * (j + 1)];
       const uint4 sp = gsd[p];
       const float dh = __fsub_rn(es, __uint_as_float(sp.x));
       const float dl = __fsub_rn(esl, rec_eps_lo(sp));
@@ -1415,7 +1429,7 @@ __global__ void __launch_bounds__(kDenseThreads, 1) k_stream_g_dense(const Item 
         return gv * u;
       };
       float acc = 0.f;
-      const G2T *__restrict__ gq = gr + (size_t)p * nm;  // the pair's nm slots
+      const G2T *__restrict__ gq = gr + (size_t)(32 * j) * nm;  // the pair's nm branches
       if (nm <= kDenseBranches) {
         // all of the pair's loads first (|g|^2 from HBM, (hbar w, N) from L1/L2), then the terms
         float gv[kDenseBranches];
@@ -1449,6 +1463,7 @@ __global__ void __launch_bounds__(kDenseThreads, 1) k_stream_g_dense(const Item 
         for (int nu = 0; nu < nm; ++nu) acc += term(g2_at(gq, nu), __ldg(tr + nu));
       }
       kahan_add(sum, comp, MODE == MODE_VJP ? (ls - lsm[p]) * acc : acc);
+      if (gap) kahan_add(sum, comp, 0.f);
     }
     // float-float tree of (sum, -comp), then one conversion
     const double v = warp_sum_ff(make_float2(sum, -comp));
@@ -1456,15 +1471,32 @@ __global__ void __launch_bounds__(kDenseThreads, 1) k_stream_g_dense(const Item 
   }
 }
 
-// g2d[(r * npp + p) * nm + nu] = s2 |g|^2 of the stored channel (r, p, nu) in the storage type
-// (round to nearest; s2 a power of two); the array is cleared before, so missing channels keep
-// zero slots
+// smap[row * ns + p] = the slot of every pair (row, p) of the items (the map holds ~0 elsewhere)
+__global__ void k_slot_map(const Item *__restrict__ items, int nitems, const uint16_t *__restrict__ pidx, int ns,
+                           uint32_t *__restrict__ smap) {
+  const int lane = threadIdx.x & 31;
+  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int nwarps = (gridDim.x * blockDim.x) >> 5;
+  for (int it = warp; it < nitems; it += nwarps) {
+    const Item I = items[it];
+    for (int j = 0; j < I.len; ++j) {
+      const long long slot = I.start + 32 * j + lane;
+      const int p = pidx[slot] & (kGapBit - 1);
+      if (p < ns) smap[(size_t)I.row * ns + p] = (uint32_t)slot;
+    }
+  }
+}
+
+// g2d[smap(r, p) * nm + nu] = s2 |g|^2 of the stored channel (r, p, nu) in the storage type (round to
+// nearest; s2 a power of two); the array is cleared before, so missing channels keep zeros, and
+// channels out of reach have no slot
 template <typename G2T>
 __global__ void __launch_bounds__(kBlock) k_dense_g2(const Item *__restrict__ items, int nitems,
                                                      const long long *__restrict__ rp_pad,
                                                      const long long *__restrict__ rp_real,
                                                      const uint32_t *__restrict__ col, const double *__restrict__ g2,
-                                                     int nm, int npp, G2T *__restrict__ g2d, double s2) {
+                                                     const uint32_t *__restrict__ smap, int ns, int nm,
+                                                     G2T *__restrict__ g2d, double s2) {
   const int lane = threadIdx.x & 31;
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -1477,8 +1509,8 @@ __global__ void __launch_bounds__(kBlock) k_dense_g2(const Item *__restrict__ it
       if (off + j >= real_len) break;
       const long long c = I.start + j;
       const unsigned cw = col[c];
-      const size_t slot = ((size_t)r * npp + (cw & 0xFFFFFFu)) * (size_t)nm + (cw >> 24);
-      g2_store(g2d, slot, s2 * g2[c]);
+      const uint32_t slot = smap[(size_t)r * ns + (cw & 0xFFFFFFu)];
+      if (slot != ~0u) g2_store(g2d, (size_t)slot * nm + (cw >> 24), s2 * g2[c]);
     }
   }
 }

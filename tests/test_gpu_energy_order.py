@@ -94,3 +94,35 @@ def test_transport_segments_of_many_tiles(pb):  # noqa: F811
     got = dev.transport_map(T(f0), T(v), T(F)).cpu().numpy()
     assert np.abs(got[rows] - ref).max() <= TOL * np.abs(got).max()
     dev.check()
+
+
+@pytest.mark.parametrize("name", list(CASES))
+def test_dense_mixed_sweep_skips_pairs_out_of_reach(pb, name):  # noqa: F811
+    """The dense FP32 |g|^2 sweep over the pairs in reach, alone and in the batch, and its adjoint
+    against the channel-list form of the same device type, which sweeps every channel: both evaluate
+    the same FP32 Gaussians (whose own error against FP64 is about 2^-24 of the exponent: beyond
+    1e-6 where a narrow delta function leaves only far tails), so they agree to FP32 rounding of the
+    terms."""
+    m = CASES[name][0]()
+    o = oracle.Oracle(m)
+    ch = pb.Channels.from_model(m)
+    dev, lanes = pb.Device(ch, variant="g32", channel_per_lane=5), pb.Device(ch, variant="g32", channel_per_lane=4)
+    b = pb.Batch([ch, ch])
+    rng = np.random.default_rng(53)
+    f, lam = rng.uniform(0, 1, o.nstate), rng.normal(size=o.nstate)
+    ab = o.collision(f, with_abs=True)[1]
+    ref = lanes.collision(T(f)).cpu().numpy()
+    assert np.abs(dev.collision(T(f)).cpu().numpy() - ref).max() <= 1e-6 * ab.max()
+    both = b.collision(T(np.concatenate([f, f]))).cpu().numpy()
+    assert np.array_equal(both[:o.nstate], both[o.nstate:])
+    assert np.abs(both[:o.nstate] - ref).max() <= 1e-6 * ab.max()
+    assert nrel(dev.rates(T(f)).cpu().numpy(), lanes.rates(T(f)).cpu().numpy()) <= 1e-6
+    f0 = o.window_values(m.f_hot())
+    ft, fb, want = T(f0), T(np.concatenate([f0, f0])), T(f0)
+    dev.rk4(ft, 1.0, 2)
+    b.rk4(fb, 1.0, 2)
+    lanes.rk4(want, 1.0, 2)
+    want = want.cpu().numpy()
+    assert nrel(ft.cpu().numpy(), want) <= 1e-6 and nrel(fb.cpu().numpy()[o.nstate:], want) <= 1e-6
+    g = [d.collision_vjp(T(f), T(lam), grad_g2=T(np.zeros(ch.nchannels))).cpu().numpy() for d in (dev, lanes)]
+    assert np.abs(g[0] - g[1]).max() <= 1e-6 * np.abs(o.rates(f)).max() * np.abs(lam).max()
