@@ -716,29 +716,32 @@ int batch_upload_plan(pb_batch *b, int item_ch, cudaStream_t st) {
 // the tile sweep of every instance in one launch (the single-system kernels)
 int batch_sweep_tiles(pb_batch *b, cudaStream_t st) {
   const int nt = b->tnt;
-  if (b->prec == 2) {
-    with_c32_shape(b->tshape, [&](auto nst, auto cps, auto half) {
-      const int gs = (int)std::max<int64_t>(1, std::min<int64_t>(nt, (int64_t)b->sm_count * cps()));
-      const float2 *tc = (const float2 *)b->tc;
-      float *tp = (float *)b->tp;
-      if constexpr (decltype(half)::value)
-        dev::k_stream_c32_half<dev::MODE_COLL, nst(), cps()><<<gs, dev::kC32Threads, dev::c32_half_smem<nst()>(), st>>>(
-            b->tl, nt, tc, b->yff, tp, b->err, b->rev);
-      else
-        dev::k_stream_c32<dev::MODE_COLL, nst(), cps()><<<gs, dev::kC32Threads, dev::c32_smem<nst()>(), st>>>(
-            b->tl, nt, tc, b->yff, tp, b->err, b->rev);
-    });
-    PB_LAUNCHED("k_stream_c32 (batch tiles)");
-    return PB_OK;
-  }
-  const float4 *tc = (const float4 *)b->tc;
-  float4 *tp = (float4 *)b->tp;
-  const int gs = (int)std::max<int64_t>(1, std::min<int64_t>(nt, (int64_t)b->sm_count * b->tshape));
-  if (b->tshape == 3)
-    dev::k_stream_sym_half<2, 3><<<gs, dev::kSymThreads, dev::half_smem<2>(), st>>>(b->tl, nt, tc, b->yff, tp, b->err, b->rev);
-  else
-    dev::k_stream_sym_half<3, 2><<<gs, dev::kSymThreads, dev::half_smem<3>(), st>>>(b->tl, nt, tc, b->yff, tp, b->err, b->rev);
-  PB_LAUNCHED("k_stream_sym_half (batch tiles)");
+  with_bool(chain_pdl(nt, b->sm_count), [&](auto pdl) {
+    if (b->prec == 2) {
+      with_c32_shape(b->tshape, [&](auto nst, auto cps, auto half) {
+        const int gs = (int)std::max<int64_t>(1, std::min<int64_t>(nt, (int64_t)b->sm_count * cps()));
+        const float2 *tc = (const float2 *)b->tc;
+        float *tp = (float *)b->tp;
+        if constexpr (decltype(half)::value)
+          launch_pdl(pdl(), dev::k_stream_c32_half<dev::MODE_COLL, nst(), cps(), pdl()>, gs, dev::kC32Threads,
+                     dev::c32_half_smem<nst()>(), st, b->tl, nt, tc, b->yff, tp, b->err, b->rev);
+        else
+          launch_pdl(pdl(), dev::k_stream_c32<dev::MODE_COLL, nst(), cps(), pdl()>, gs, dev::kC32Threads,
+                     dev::c32_smem<nst()>(), st, b->tl, nt, tc, b->yff, tp, b->err, b->rev);
+      });
+      return;
+    }
+    const float4 *tc = (const float4 *)b->tc;
+    float4 *tp = (float4 *)b->tp;
+    const int gs = (int)std::max<int64_t>(1, std::min<int64_t>(nt, (int64_t)b->sm_count * b->tshape));
+    if (b->tshape == 3)
+      launch_pdl(pdl(), dev::k_stream_sym_half<2, 3, pdl()>, gs, dev::kSymThreads, dev::half_smem<2>(), st, b->tl, nt, tc,
+                 b->yff, tp, b->err, b->rev);
+    else
+      launch_pdl(pdl(), dev::k_stream_sym_half<3, 2, pdl()>, gs, dev::kSymThreads, dev::half_smem<3>(), st, b->tl, nt, tc,
+                 b->yff, tp, b->err, b->rev);
+  });
+  PB_LAUNCHED("tile sweep (batch)");
   return PB_OK;
 }
 
@@ -782,16 +785,16 @@ int batch_fin(pb_batch *b, double *out, double *f, double dt, cudaStream_t st, c
     // the instances' prefactors are folded into the tiles: c = 1; states index f, y and the
     // outputs, their padded rows the partials and the next stage's float-float input
     const int ns = (int)b->ns;
-    if (b->prec == 2) {
-      dev::k_fin_c32<STAGE><<<(ns + 31) / 32, 256, 0, st>>>((const float *)b->tp, b->prow, b->pmap, ns, 1.0, src,
-                                                            out, f, b->acc, b->y, b->yff, dt);
-      PB_LAUNCHED("k_fin_c32 (batch tiles)");
-    } else {
-      const dev::TileSrc ts{(const float4 *)b->tp, b->prow, b->pmap};
-      dev::k_fin_tiles<STAGE><<<(ns + 31) / 32, 256, 0, st>>>(ts, ns, 1.0, b->Rg, src, out, f, b->acc, b->y, b->yff,
-                                                              dt);
-      PB_LAUNCHED("k_fin_tiles (batch tiles)");
-    }
+    with_bool(chain_pdl(b->tnt, b->sm_count), [&](auto pdl) {
+      if (b->prec == 2)
+        launch_pdl(pdl(), dev::k_fin_c32<STAGE, false, 32, pdl()>, (ns + 31) / 32, 256, 0, st, (const float *)b->tp,
+                   b->prow, b->pmap, ns, 1.0, src, out, f, b->acc, b->y, b->yff, dt);
+      else
+        launch_pdl(pdl(), dev::k_fin_tiles<STAGE, false, 32, pdl()>, (ns + 31) / 32, 256, 0, st,
+                   dev::TileSrc{(const float4 *)b->tp, b->prow, b->pmap}, ns, 1.0, b->Rg, src, out, f, b->acc, b->y,
+                   b->yff, dt);
+    });
+    PB_LAUNCHED("tile epilogue (batch)");
     return PB_OK;
   }
   if (b->prec == 2) {
@@ -1014,19 +1017,10 @@ int batch_setup_tiles(pb_batch *b, const TilePlan &T, cudaStream_t st) {
   PB_LAUNCHED("k_tiles_scatter (batch)");
   PB_CUDA(cudaStreamSynchronize(st));  // the host tables are released on return
   // dynamic shared memory of every launch shape the autotuner may pick
-  const cudaFuncAttribute A = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  if (b->prec == 2) {
-    for (int shape : {2, 3, 4, 7, 8})
-      with_c32_shape(shape, [&](auto nst, auto cps, auto half) {
-        if constexpr (decltype(half)::value)
-          cudaFuncSetAttribute(dev::k_stream_c32_half<dev::MODE_COLL, nst(), cps()>, A, (int)dev::c32_half_smem<nst()>());
-        else
-          cudaFuncSetAttribute(dev::k_stream_c32<dev::MODE_COLL, nst(), cps()>, A, (int)dev::c32_smem<nst()>());
-      });
-  } else {
-    cudaFuncSetAttribute(dev::k_stream_sym_half<2, 3>, A, (int)dev::half_smem<2>());
-    cudaFuncSetAttribute(dev::k_stream_sym_half<3, 2>, A, (int)dev::half_smem<3>());
-  }
+  if (b->prec == 2)
+    for (int shape : {2, 3, 4, 7, 8}) set_c32_smem(shape);
+  else
+    set_half_smem();
   PB_CUDA(cudaGetLastError());
   return PB_OK;
 }

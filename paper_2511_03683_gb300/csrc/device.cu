@@ -46,6 +46,13 @@ void with_c32_shape(int shape, F &&fn) {
   }
 }
 
+// fn(std::true_type or std::false_type)
+template <typename F>
+void with_bool(bool b, F &&fn) {
+  if (b) fn(std::true_type());
+  else fn(std::false_type());
+}
+
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 struct Layout {
@@ -597,6 +604,30 @@ int cuda_fail(cudaError_t e, const char *what) {
     if (e_ != cudaSuccess) return cuda_fail(e_, #call);         \
   } while (0)
 
+// Which tile sweeps and epilogues form such chains: those of at most one tile per SM, where a stage
+// is little more than the two launches (four-band window, us per RK4 step of 20: 16^3 22.8 against
+// 27.2 as ordinary launches, 28^3 25.7 against 28.5; at 32^3 with the cutoffs, 195 tiles, 18.5 against
+// 16.9, and at 40^3 76 against 68: sweep CTAs that come in while the epilogue runs slow it down).
+bool chain_pdl(int64_t tiles, int sm_count) { return tiles <= sm_count; }
+
+// kernel<<<grid, block, smem, st>>>(args...), with pdl as a programmatic dependent of the kernel
+// before it in the stream (kernels.cuh, pdl_trigger); only for kernels that wait for it themselves.
+// Errors are left to cudaGetLastError, as with the launch syntax.
+template <typename... P, typename... A>
+void launch_pdl(bool pdl, void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = pdl ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 #define PB_LAUNCHED(what)                                       \
   do {                                                          \
     cudaError_t e_ = cudaGetLastError();                        \
@@ -748,6 +779,7 @@ struct pb_dev {
   float2 *trtpart = nullptr;
   float4 *trf0 = nullptr;
   int nred() const { return wt_tiles ? 2 * nblk : nfin_blocks; }  // maxima that a transport epilogue leaves in red
+  bool chain() const { return chain_pdl(tnt, sm_count); }
   dev::TileSrc tile_src() const { return dev::TileSrc{tpart, prow, pmap}; }
   // PB_VARIANT_C32: the FF device whose tiles hold FP32 (P_in, P_out) (tiles32.cuh); its
   // partials in tpart are one FP32 value per (state, block)
@@ -793,6 +825,12 @@ struct pb_dev {
   cudaStream_t cap = nullptr;
   cudaGraphExec_t rk_exec = nullptr;
   cudaGraphExec_t rk_exec_in = nullptr;  // the same step preceded by the stage-input conversion of f
+  // kRkRun steps in one graph, captured once rk_exec has been replayed kRkRunAfter times: a graph
+  // launch costs about as much as one of the small kernels in it, but capturing eight steps costs
+  // half a millisecond, which a few dozen steps on one f do not earn back
+  cudaGraphExec_t rk_exec_run = nullptr;
+  static constexpr int kRkRun = 8, kRkRunAfter = 64;
+  int64_t rk_replays = 0;
   // graphs of the short launch sequences of pb_collision, pb_scatter_rates and
   // pb_transport_iterate, one per call kind and argument set, the last kGraphs kept
   static constexpr int kGraphs = 12;
@@ -1057,6 +1095,33 @@ int paper_setup(pb_dev *d, const pb_channels *ch, int item_ch, cudaStream_t st) 
   return PB_OK;
 }
 
+// dynamic shared memory of the tile sweeps
+void set_half_smem() {
+  for (const bool b : {false, true})
+    with_bool(b, [](auto pdl) {
+      const cudaFuncAttribute A = cudaFuncAttributeMaxDynamicSharedMemorySize;
+      cudaFuncSetAttribute(dev::k_stream_sym_half<3, 2, pdl()>, A, (int)dev::half_smem<3>());
+      cudaFuncSetAttribute(dev::k_stream_sym_half<2, 3, pdl()>, A, (int)dev::half_smem<2>());
+    });
+}
+void set_c32_smem(int shape) {
+  for (const bool b : {false, true})
+    with_bool(b, [&](auto pdl) {
+      with_c32_shape(shape, [&](auto nst, auto cps, auto half) {
+        const cudaFuncAttribute A = cudaFuncAttributeMaxDynamicSharedMemorySize;
+        if constexpr (decltype(half)::value) {
+          const int sm32 = (int)dev::c32_half_smem<nst()>();
+          cudaFuncSetAttribute(dev::k_stream_c32_half<dev::MODE_COLL, nst(), cps(), pdl()>, A, sm32);
+          cudaFuncSetAttribute(dev::k_stream_c32_half<dev::MODE_RATE, nst(), cps(), pdl()>, A, sm32);
+        } else {
+          const int sm32 = (int)dev::c32_smem<nst()>();
+          cudaFuncSetAttribute(dev::k_stream_c32<dev::MODE_COLL, nst(), cps(), pdl()>, A, sm32);
+          cudaFuncSetAttribute(dev::k_stream_c32<dev::MODE_RATE, nst(), cps(), pdl()>, A, sm32);
+        }
+      });
+    });
+}
+
 template <typename IDX>
 void set_stream_smem(int bytes) {
   cudaFuncSetAttribute(dev::k_stream_ff<dev::MODE_COLL, true, IDX>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
@@ -1105,6 +1170,7 @@ extern "C" int pb_dev_arena_bytes(const pb_channels *ch, const pb_dev_opts *opts
 
 namespace {
 int coef_setup(pb_dev *d, cudaStream_t st);
+void drop_rk_graphs(pb_dev *d);
 }
 
 extern "C" int pb_dev_create(const pb_channels *ch, const pb_dev_opts *opts, void *arena, size_t arena_bytes,
@@ -1599,25 +1665,10 @@ extern "C" int pb_dev_create(const pb_channels *ch, const pb_dev_opts *opts, voi
       d->sym_half = false;
     } else {
       cudaFuncSetAttribute(dev::k_stream_sym_bulk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dev::kSymBulkSmem);
-      cudaFuncSetAttribute(dev::k_stream_sym_half<3, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)dev::half_smem<3>());
-      cudaFuncSetAttribute(dev::k_stream_sym_half<2, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)dev::half_smem<2>());
+      set_half_smem();
     }
   }
-  if (d->c32)
-    with_c32_shape(d->c32_shape, [&](auto nst, auto cps, auto half) {
-      const cudaFuncAttribute A = cudaFuncAttributeMaxDynamicSharedMemorySize;
-      if constexpr (decltype(half)::value) {
-        const int sm32 = (int)dev::c32_half_smem<nst()>();
-        cudaFuncSetAttribute(dev::k_stream_c32_half<dev::MODE_COLL, nst(), cps()>, A, sm32);
-        cudaFuncSetAttribute(dev::k_stream_c32_half<dev::MODE_RATE, nst(), cps()>, A, sm32);
-      } else {
-        const int sm32 = (int)dev::c32_smem<nst()>();
-        cudaFuncSetAttribute(dev::k_stream_c32<dev::MODE_COLL, nst(), cps()>, A, sm32);
-        cudaFuncSetAttribute(dev::k_stream_c32<dev::MODE_RATE, nst(), cps()>, A, sm32);
-      }
-    });
+  if (d->c32) set_c32_smem(d->c32_shape);
   if (d->smem_f > 48 * 1024) {
     set_stream_smem<uint32_t>((int)d->smem_f);
     set_stream_smem<uint16_t>((int)d->smem_f);
@@ -1708,8 +1759,7 @@ extern "C" int pb_dev_selftest_wait(pb_dev *d, int32_t wait_us, void *stream) {
 
 extern "C" void pb_dev_destroy(pb_dev *d) {
   if (!d) return;
-  if (d->rk_exec) cudaGraphExecDestroy(d->rk_exec);
-  if (d->rk_exec_in) cudaGraphExecDestroy(d->rk_exec_in);
+  drop_rk_graphs(d);
   d->drop_call_graphs();
   if (d->cap) cudaStreamDestroy(d->cap);
   if (d->hres) cudaFreeHost(d->hres);
@@ -1779,35 +1829,31 @@ int launch_stream_t(pb_dev *d, int mode, const double *fd, const float2 *fff, co
     float *tp = (float *)d->tpart;
     with_c32_shape(d->c32_shape, [&](auto nst, auto cps, auto half) {
       const int gs = (int)std::max<int64_t>(1, std::min<int64_t>(d->tnt, (int64_t)d->sm_count * cps()));
-      if constexpr (decltype(half)::value) {
-        const size_t sm32 = dev::c32_half_smem<nst()>();
-        if (coll)
-          dev::k_stream_c32_half<dev::MODE_COLL, nst(), cps()><<<gs, dev::kC32Threads, sm32, st>>>(
-              d->tiles, d->tnt, d->tc32, fff, tp, d->err, d->rev);
-        else
-          dev::k_stream_c32_half<dev::MODE_RATE, nst(), cps()><<<gs, dev::kC32Threads, sm32, st>>>(
-              d->tiles, d->tnt, d->tc32, fff, tp, d->err, d->rev);
-      } else {
-        const size_t sm32 = dev::c32_smem<nst()>();
-        if (coll)
-          dev::k_stream_c32<dev::MODE_COLL, nst(), cps()><<<gs, dev::kC32Threads, sm32, st>>>(
-              d->tiles, d->tnt, d->tc32, fff, tp, d->err, d->rev);
-        else
-          dev::k_stream_c32<dev::MODE_RATE, nst(), cps()><<<gs, dev::kC32Threads, sm32, st>>>(
-              d->tiles, d->tnt, d->tc32, fff, tp, d->err, d->rev);
-      }
+      with_bool(d->chain(), [&](auto pdl) {
+        with_bool(coll, [&](auto cm) {
+          constexpr int M = cm() ? dev::MODE_COLL : dev::MODE_RATE;
+          if constexpr (decltype(half)::value)
+            launch_pdl(pdl(), dev::k_stream_c32_half<M, nst(), cps(), pdl()>, gs, dev::kC32Threads,
+                       dev::c32_half_smem<nst()>(), st, d->tiles, d->tnt, d->tc32, fff, tp, d->err, d->rev);
+          else
+            launch_pdl(pdl(), dev::k_stream_c32<M, nst(), cps(), pdl()>, gs, dev::kC32Threads, dev::c32_smem<nst()>(),
+                       st, d->tiles, d->tnt, d->tc32, fff, tp, d->err, d->rev);
+        });
+      });
     });
   } else if (d->variant == PB_VARIANT_FF && d->sym && !d->c32 && part == d->part) {
     // symmetric tiles; the rate mode needs the same (A, B) partials
     if (d->sym_half && fff == d->yff) {
       const int cps = d->half_cps;
       const int gs = (int)std::max<int64_t>(1, std::min<int64_t>(d->tnt, (int64_t)d->sm_count * cps));
-      if (cps == 3)
-        dev::k_stream_sym_half<2, 3><<<gs, dev::kSymThreads, dev::half_smem<2>(), st>>>(
-            d->tiles, d->tnt, d->tcoef, fff, d->tpart, d->err, d->rev);
-      else
-        dev::k_stream_sym_half<3, 2><<<gs, dev::kSymThreads, dev::half_smem<3>(), st>>>(
-            d->tiles, d->tnt, d->tcoef, fff, d->tpart, d->err, d->rev);
+      with_bool(d->chain(), [&](auto pdl) {
+        if (cps == 3)
+          launch_pdl(pdl(), dev::k_stream_sym_half<2, 3, pdl()>, gs, dev::kSymThreads, dev::half_smem<2>(), st, d->tiles,
+                     d->tnt, d->tcoef, fff, d->tpart, d->err, d->rev);
+        else
+          launch_pdl(pdl(), dev::k_stream_sym_half<3, 2, pdl()>, gs, dev::kSymThreads, dev::half_smem<3>(), st, d->tiles,
+                     d->tnt, d->tcoef, fff, d->tpart, d->err, d->rev);
+      });
     } else if (d->sym_nt && fff == d->yff) {  // the bulk copies read f from this padded arena buffer
       const int gs = (int)std::max<int64_t>(1, std::min<int64_t>(d->tnt, (int64_t)d->sm_count));
       dev::k_stream_sym_bulk<<<gs, dev::kSymThreads, dev::kSymBulkSmem, st>>>(d->tiles, d->tnt, d->tcoef, fff,
@@ -1894,6 +1940,22 @@ int fin_grid(const pb_dev *d) { return d->nfin_blocks; }
 // per CTA a 40^3 step had 149 CTAs for 152 SMs, and the C32 RK4 step ran 14% slower)
 bool fin_small(const pb_dev *d) { return (d->ns + 31) / 32 < 4 * (int64_t)d->sm_count; }
 
+template <int STAGE, bool RATE>
+void launch_fin_tiles(pb_dev *d, const double *ysrc, double *out, double *f, double *y, double dt, cudaStream_t st) {
+  with_bool(d->chain(), [&](auto pdl) {
+    with_bool(fin_small(d), [&](auto small) {
+      constexpr int SPC = small() ? 8 : 32;
+      const int grid = (int)((d->ns + SPC - 1) / SPC);
+      if (d->c32)
+        launch_pdl(pdl(), dev::k_fin_c32<STAGE, RATE, SPC, pdl()>, grid, 256, 0, st, (const float *)d->tpart, d->prow,
+                   d->pmap, (int)d->ns, d->c, ysrc, out, f, d->acc, y, d->yff, dt);
+      else
+        launch_pdl(pdl(), dev::k_fin_tiles<STAGE, RATE, SPC, pdl()>, grid, 256, 0, st, d->tile_src(), (int)d->ns, d->c,
+                   d->R, ysrc, out, f, d->acc, y, d->yff, dt);
+    });
+  });
+}
+
 // ydst: where a stage writes the next stage's input (default d->y)
 template <int STAGE>
 void launch_fin(pb_dev *d, const double *ysrc, double *out, double *f, double dt, cudaStream_t st,
@@ -1908,20 +1970,8 @@ void launch_fin(pb_dev *d, const double *ysrc, double *out, double *f, double dt
     dev::k_fin_coll<true, STAGE><<<fin_grid(d), kFinBlock, 0, st>>>(
         dev::ItemSrc{d->variant == PB_VARIANT_PAPER ? d->t_item_ptr : d->item_ptr, d->part}, (int)d->ns, d->c, d->R, ysrc,
                                                                     out, f, d->acc, y, d->yff, dt);
-  else if (d->sym && d->c32)
-    if (fin_small(d))
-      dev::k_fin_c32<STAGE, false, 8><<<(int)((d->ns + 7) / 8), 256, 0, st>>>(
-          (const float *)d->tpart, d->prow, d->pmap, (int)d->ns, d->c, ysrc, out, f, d->acc, y, d->yff, dt);
-    else
-      dev::k_fin_c32<STAGE><<<(int)((d->ns + 31) / 32), 256, 0, st>>>(
-          (const float *)d->tpart, d->prow, d->pmap, (int)d->ns, d->c, ysrc, out, f, d->acc, y, d->yff, dt);
   else if (d->sym)
-    if (fin_small(d))
-      dev::k_fin_tiles<STAGE, false, 8><<<(int)((d->ns + 7) / 8), 256, 0, st>>>(
-          d->tile_src(), (int)d->ns, d->c, d->R, ysrc, out, f, d->acc, y, d->yff, dt);
-    else
-      dev::k_fin_tiles<STAGE><<<(int)((d->ns + 31) / 32), 256, 0, st>>>(
-          d->tile_src(), (int)d->ns, d->c, d->R, ysrc, out, f, d->acc, y, d->yff, dt);
+    launch_fin_tiles<STAGE, false>(d, ysrc, out, f, y, dt, st);
   else
     dev::k_fin_coll<false, STAGE><<<fin_grid(d), kFinBlock, 0, st>>>(dev::ItemSrc{d->item_ptr, d->part}, (int)d->ns, d->c, d->R, ysrc,
                                                                      out, f, d->acc, y, d->yff, dt);
@@ -1983,9 +2033,33 @@ int rk4_launches(pb_dev *d, double *f, double dt, cudaStream_t st) {
 }
 
 void drop_rk_graphs(pb_dev *d) {
-  if (d->rk_exec) cudaGraphExecDestroy(d->rk_exec);
-  if (d->rk_exec_in) cudaGraphExecDestroy(d->rk_exec_in);
-  d->rk_exec = d->rk_exec_in = nullptr;
+  for (cudaGraphExec_t *e : {&d->rk_exec, &d->rk_exec_in, &d->rk_exec_run}) {
+    if (*e) cudaGraphExecDestroy(*e);
+    *e = nullptr;
+  }
+  d->rk_replays = 0;
+}
+
+// a graph of `steps` RK4 steps on f, with the conversion of f into the stage input first or not
+int capture_rk_graph(pb_dev *d, double *f, double dt, int steps, bool with_input, cudaGraphExec_t &exec) {
+  if (!d->cap) PB_CUDA(cudaStreamCreateWithFlags(&d->cap, cudaStreamNonBlocking));
+  PB_CUDA(cudaStreamBeginCapture(d->cap, cudaStreamCaptureModeThreadLocal));
+  int rc = with_input ? stage_input(d, f, d->cap) : PB_OK;
+  for (int i = 0; i < steps && rc == PB_OK; ++i) rc = rk4_launches(d, f, dt, d->cap);
+  cudaGraph_t graph = nullptr;
+  cudaError_t e = cudaStreamEndCapture(d->cap, &graph);
+  if (rc) {
+    if (graph) cudaGraphDestroy(graph);
+    return rc;
+  }
+  if (e != cudaSuccess) return cuda_fail(e, "cudaStreamEndCapture");
+  e = cudaGraphInstantiate(&exec, graph, 0);
+  cudaGraphDestroy(graph);
+  if (e != cudaSuccess) {
+    exec = nullptr;
+    return cuda_fail(e, "cudaGraphInstantiate");
+  }
+  return PB_OK;
 }
 
 // two graphs of one RK4 step on f: rk_exec (its stage input already in yff, as the last stage
@@ -1993,30 +2067,11 @@ void drop_rk_graphs(pb_dev *d) {
 int ensure_rk_graph(pb_dev *d, double *f, double dt) {
   if (d->rk_exec && d->rk_exec_in && d->rk_f == f && d->rk_dt == dt) return PB_OK;
   drop_rk_graphs(d);
-  if (!d->cap) PB_CUDA(cudaStreamCreateWithFlags(&d->cap, cudaStreamNonBlocking));
-  for (int with_input = 0; with_input < 2; ++with_input) {
-    PB_CUDA(cudaStreamBeginCapture(d->cap, cudaStreamCaptureModeThreadLocal));
-    int rc = with_input ? stage_input(d, f, d->cap) : PB_OK;
-    if (rc == PB_OK) rc = rk4_launches(d, f, dt, d->cap);
-    cudaGraph_t graph = nullptr;
-    cudaError_t e = cudaStreamEndCapture(d->cap, &graph);
-    if (rc) {
-      if (graph) cudaGraphDestroy(graph);
-      drop_rk_graphs(d);
-      return rc;
-    }
-    if (e != cudaSuccess) {
-      drop_rk_graphs(d);
-      return cuda_fail(e, "cudaStreamEndCapture");
-    }
-    cudaGraphExec_t &exec = with_input ? d->rk_exec_in : d->rk_exec;
-    e = cudaGraphInstantiate(&exec, graph, 0);
-    cudaGraphDestroy(graph);
-    if (e != cudaSuccess) {
-      exec = nullptr;
-      drop_rk_graphs(d);
-      return cuda_fail(e, "cudaGraphInstantiate");
-    }
+  int rc = capture_rk_graph(d, f, dt, 1, false, d->rk_exec);
+  if (rc == PB_OK) rc = capture_rk_graph(d, f, dt, 1, true, d->rk_exec_in);
+  if (rc) {
+    drop_rk_graphs(d);
+    return rc;
   }
   d->rk_f = f;
   d->rk_dt = dt;
@@ -2284,22 +2339,8 @@ int rates_seq(pb_dev *d, const double *f, double *inv_tau, cudaStream_t st) {
   if (d->variant == PB_VARIANT_LITERAL || d->mixed())
     dev::k_fin_rate<true><<<fin_grid(d), kFinBlock, 0, st>>>(dev::ItemSrc{d->fwd_item_ptr(), d->part}, (int)d->ns,
                                                              d->mixed() ? d->gscale() : d->c, d->R, inv_tau);
-  else if (d->sym && d->c32 && fin_small(d))
-    dev::k_fin_c32<-1, true, 8><<<(int)((d->ns + 7) / 8), 256, 0, st>>>((const float *)d->tpart, d->prow, d->pmap,
-                                                                       (int)d->ns, d->c, nullptr, inv_tau, nullptr,
-                                                                       nullptr, nullptr, nullptr, 0.0);
-  else if (d->sym && d->c32)
-    dev::k_fin_c32<-1, true><<<(int)((d->ns + 31) / 32), 256, 0, st>>>((const float *)d->tpart, d->prow, d->pmap,
-                                                                       (int)d->ns, d->c, nullptr, inv_tau, nullptr,
-                                                                       nullptr, nullptr, nullptr, 0.0);
-  else if (d->sym && fin_small(d))
-    dev::k_fin_tiles<-1, true, 8><<<(int)((d->ns + 7) / 8), 256, 0, st>>>(
-        d->tile_src(), (int)d->ns, d->c, d->R, nullptr, inv_tau, nullptr, nullptr, nullptr,
-        nullptr, 0.0);
   else if (d->sym)
-    dev::k_fin_tiles<-1, true><<<(int)((d->ns + 31) / 32), 256, 0, st>>>(
-        d->tile_src(), (int)d->ns, d->c, d->R, nullptr, inv_tau, nullptr, nullptr, nullptr,
-        nullptr, 0.0);
+    launch_fin_tiles<-1, true>(d, nullptr, inv_tau, nullptr, nullptr, 0.0, st);
   else
     dev::k_fin_rate<false><<<fin_grid(d), kFinBlock, 0, st>>>(dev::ItemSrc{d->item_ptr, d->part}, (int)d->ns, d->c, d->R, inv_tau);
   PB_LAUNCHED("k_fin_rate");
@@ -2316,7 +2357,13 @@ extern "C" int pb_rtbte_rk4_step(pb_dev *d, double *f, double dt, int32_t nsteps
   int rc = ensure_rk_graph(d, f, dt);
   if (rc) return rc;
   PB_CUDA(cudaGraphLaunch(d->rk_exec_in, st));  // the first step converts f itself
-  for (int32_t i = 1; i < nsteps; ++i) PB_CUDA(cudaGraphLaunch(d->rk_exec, st));
+  int32_t left = nsteps - 1;
+  if (left >= pb_dev::kRkRun && (d->rk_exec_run || d->rk_replays >= pb_dev::kRkRunAfter)) {
+    if (!d->rk_exec_run && (rc = capture_rk_graph(d, f, dt, pb_dev::kRkRun, false, d->rk_exec_run))) return rc;
+    for (; left >= pb_dev::kRkRun; left -= pb_dev::kRkRun) PB_CUDA(cudaGraphLaunch(d->rk_exec_run, st));
+  }
+  d->rk_replays += left;
+  for (; left > 0; --left) PB_CUDA(cudaGraphLaunch(d->rk_exec, st));
   return PB_OK;
 }
 

@@ -176,6 +176,16 @@ __global__ void k_table(const double *__restrict__ omega, long long n, double kT
   }
 }
 
+// Programmatic dependent launch (griddepcontrol, PTX ISA).  The kernels of the sweep chains are
+// launched so that a kernel may start while the one before it runs: launch_dependents, at a CTA's last
+// unit of work, lets the next kernel in once all CTAs are there, and before the first access to
+// anything that an earlier kernel of the chain writes (or still reads) each kernel waits for the
+// completion of the one before it, which has waited for its own predecessor.  Only constants of the
+// handle (tables, coefficients) are read before the wait.  Kernels have both forms (template PDL):
+// the instructions cost a large sweep more than the early start gains (chain_pdl on the host).
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __global__ void k_to_ff(const double *__restrict__ x, long long n, float2 *__restrict__ out) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     out[i] = ff_split(x[i]);
@@ -184,6 +194,7 @@ __global__ void k_to_ff(const double *__restrict__ x, long long n, float2 *__res
 // the same into the tiles' padded energy order: out[pmap[i]] (the padding keeps its zeros)
 __global__ void k_to_ff_map(const double *__restrict__ x, int n, const int *__restrict__ pmap,
                             float2 *__restrict__ out) {
+  pdl_trigger();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) out[pmap[i]] = ff_split(x[i]);
 }
 
@@ -2468,7 +2479,7 @@ constexpr size_t half_smem() {
 // NST stages per CTA, CPS resident CTAs per SM (3 x 2 or 2 x 3 fit in the SM's shared memory)
 // rev: take the tile list from its end (tile nt - 1 - t in place of t), so that a sweep following
 // one in list order starts on the tiles the L2 still holds; the partials do not depend on the order.
-template <int NST, int CPS>
+template <int NST, int CPS, bool PDL>
 __global__ void __launch_bounds__(kSymThreads, CPS) k_stream_sym_half(const TileD *__restrict__ tiles, int nt,
                                                                        const float4 *__restrict__ tc,
                                                                        const float2 *__restrict__ fg,
@@ -2501,7 +2512,13 @@ __global__ void __launch_bounds__(kSymThreads, CPS) k_stream_sym_half(const Tile
     iss = load_tile(tiles, tix(0));
     if (nloc > 1) ahead = load_tile(tiles, tix(1));
   }
-  auto issue = [&](int v) {  // unit v = 2 k + h: half h of the CTA's tile k
+  auto issue_f = [&](int v, const TileD &D) {  // the f slices of unit v
+    const int h = v & 1, s = v % kHalfStages;
+    unsigned char *buf = ssm + (size_t)s * kHalfStageBytes + kHalfTileBytes;
+    bulk_g2s(buf, fg + (size_t)D.I * kTile + h * HR, HR * sizeof(float2), bars + s);
+    bulk_g2s(buf + HR * sizeof(float2), fg + (size_t)D.J * kTile, kTile * sizeof(float2), bars + s);
+  };
+  auto issue = [&](int v) {  // unit v = 2 k + h: half h of the CTA's tile k (coefficients)
     const int k = v >> 1, h = v & 1, s = v % kHalfStages;
     if (h == 0 && k > 0) {
       iss = ahead;
@@ -2514,11 +2531,17 @@ __global__ void __launch_bounds__(kSymThreads, CPS) k_stream_sym_half(const Tile
     const unsigned char *src = (const unsigned char *)(tc + (size_t)t * kTile * kTile) + (size_t)h * kHalfTileBytes;
 #pragma unroll
     for (int q = 0; q < 2; ++q) bulk_g2s(buf + q * (kHalfTileBytes / 2), src + q * (kHalfTileBytes / 2), kHalfTileBytes / 2, bars + s);
-    bulk_g2s(buf + kHalfTileBytes, fg + (size_t)iss.I * kTile + h * HR, HR * sizeof(float2), bars + s);
-    bulk_g2s(buf + kHalfTileBytes + HR * sizeof(float2), fg + (size_t)iss.J * kTile, kTile * sizeof(float2), bars + s);
   };
-  if (tid == 0)
-    for (; issued < kHalfStages && issued < nunit; ++issued) issue(issued);
+  if (tid == 0) {
+    for (; issued < kHalfStages && issued < nunit; ++issued) {
+      issue(issued);
+      if (!PDL) issue_f(issued, iss);
+    }
+    if (PDL) {
+      pdl_wait();  // f comes from the kernel before this one, which may still read the partials
+      for (int v = 0; v < issued; ++v) issue_f(v, stile[v]);
+    }
+  }
   int pcb = -1, pcs = 0;  // column slots of the previous unit's tile (-1: diagonal, or none)
   bool ok = true;
   float cA[4][2], cC[4][2];  // column sums of the current tile, carried across its halves
@@ -2532,11 +2555,13 @@ __global__ void __launch_bounds__(kSymThreads, CPS) k_stream_sym_half(const Tile
     if (tid == 0 && u >= 1 && issued < nunit) {
       fence_proxy_async();  // the generic reads of unit u-1's stage before its refill
       issue(issued);
+      issue_f(issued, iss);
       ++issued;
     }
     // the previous tile's column table (written after its second half) is complete
     if ((u & 1) == 0 && u >= 2 && pcb >= 0) sym_columns_out(colred, pcb, pcs, lane, wid, tp);
     if (!have) break;
+    if (PDL && u + 1 == nunit) pdl_trigger();
     const int s = u % kHalfStages, h = u & 1;
     const TileD D = stile[s];
     const bool diag = D.I == D.J;
@@ -2901,7 +2926,7 @@ __global__ void k_fin_coll(SRC src, int ns, double c, const double *__restrict__
 // cost the same with one active lane as with 32 on this part, so a lane-0-per-state epilogue
 // spent most of its time there).  RATE: 1/tau.
 // SPC states per CTA (8 or 32; few states take 8, for more CTAs in flight)
-template <int STAGE, bool RATE = false, int SPC = 32>
+template <int STAGE, bool RATE, int SPC, bool PDL>
 __global__ void __launch_bounds__(256) k_fin_tiles(TileSrc src, int ns, double c, const double *__restrict__ R,
                                                    const double *__restrict__ ysrc, double *__restrict__ out,
                                                    double *__restrict__ f, double *__restrict__ acc,
@@ -2910,6 +2935,18 @@ __global__ void __launch_bounds__(256) k_fin_tiles(TileSrc src, int ns, double c
   __shared__ float4 tot[SPC];  // (A hi, A lo, C hi, C lo) per state
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int base = blockIdx.x * SPC;
+  int2 pr[SPW];
+  auto load_rows = [&] {
+#pragma unroll
+    for (int q = 0; q < SPW; ++q) {
+      const int r = base + SPW * wid + q;
+      pr[q] = r < ns ? src.prow[r] : make_int2(0, 0);
+    }
+  };
+  if (PDL) {
+    load_rows();
+    pdl_wait();
+  }
   // warp 0 loads its state's epilogue inputs first, so that their latency overlaps the partials'
   const int r0 = base + lane;
   FinIn in{0.0, 0.0, 0.0, 0.0};
@@ -2922,12 +2959,7 @@ __global__ void __launch_bounds__(256) k_fin_tiles(TileSrc src, int ns, double c
   // the first three partials of every lane for the warp's states are loaded together (up to 96
   // partner blocks), the rest after
   float4 w[SPW][3];
-  int2 pr[SPW];
-#pragma unroll
-  for (int q = 0; q < SPW; ++q) {
-    const int r = base + SPW * wid + q;
-    pr[q] = r < ns ? src.prow[r] : make_int2(0, 0);
-  }
+  if (!PDL) load_rows();
 #pragma unroll
   for (int q = 0; q < SPW; ++q) {
 #pragma unroll
@@ -2952,6 +2984,7 @@ __global__ void __launch_bounds__(256) k_fin_tiles(TileSrc src, int ns, double c
       v[2 * q + 1] = ff_add(v[2 * q + 1], make_float2(x.z, x.w));
     }
   }
+  if (PDL) pdl_trigger();
   ff_reduce_scatter<NV, 16>(v, lane);
   if ((lane & (LPV - 1)) == 0) {
     const int idx = lane / LPV;  // the top lane bits: (state q, A | C)

@@ -155,7 +155,7 @@ __device__ __forceinline__ void c32_columns_out(const float *__restrict__ colred
 // iteration, so a tile costs one CTA barrier.
 // rev: take the tile list from its end (tile nt - 1 - t in place of t), so that a sweep following
 // one in list order starts on the tiles the L2 still holds.
-template <int MODE, int NST, int CPS>
+template <int MODE, int NST, int CPS, bool PDL>
 __global__ void __launch_bounds__(kC32Threads, CPS) k_stream_c32(const TileD *__restrict__ tiles, int nt,
                                                                   const float2 *__restrict__ tc,
                                                                   const float2 *__restrict__ fg,
@@ -182,7 +182,13 @@ __global__ void __launch_bounds__(kC32Threads, CPS) k_stream_c32(const TileD *__
     const int t = (int)blockIdx.x + k * G;
     return rev ? nt - 1 - t : t;
   };
-  auto issue = [&](int k, const TileD &D) {
+  auto issue_f = [&](int k, const TileD &D) {  // the f slices of the CTA's tile k
+    const int s = k % NST;
+    unsigned char *buf = ssm + (size_t)s * kC32StageBytes + kC32TileBytes;
+    bulk_g2s(buf, fg + (size_t)D.I * kTile, kTile * sizeof(float2), bars + s);
+    bulk_g2s(buf + kTile * sizeof(float2), fg + (size_t)D.J * kTile, kTile * sizeof(float2), bars + s);
+  };
+  auto issue = [&](int k, const TileD &D) {  // its coefficients
     const int s = k % NST;
     const int t = tix(k);
     stile[s] = D;
@@ -191,11 +197,18 @@ __global__ void __launch_bounds__(kC32Threads, CPS) k_stream_c32(const TileD *__
     const unsigned char *src = (const unsigned char *)(tc + (size_t)t * kTile * kTile);
 #pragma unroll
     for (int q = 0; q < 2; ++q) bulk_g2s(buf + q * (kC32TileBytes / 2), src + q * (kC32TileBytes / 2), kC32TileBytes / 2, bars + s);
-    bulk_g2s(buf + kC32TileBytes, fg + (size_t)D.I * kTile, kTile * sizeof(float2), bars + s);
-    bulk_g2s(buf + kC32TileBytes + kTile * sizeof(float2), fg + (size_t)D.J * kTile, kTile * sizeof(float2), bars + s);
   };
-  if (tid == 0)
-    for (; issued < NST && issued < nloc; ++issued) issue(issued, load_tile(tiles, tix(issued)));
+  if (tid == 0) {
+    for (; issued < NST && issued < nloc; ++issued) {
+      const TileD D = load_tile(tiles, tix(issued));
+      issue(issued, D);
+      if (!PDL) issue_f(issued, D);
+    }
+    if (PDL) {
+      pdl_wait();  // f comes from the kernel before this one, which may still read the partials
+      for (int k = 0; k < issued; ++k) issue_f(k, stile[k]);
+    }
+  }
   TileD next{};
   if (tid == 0 && issued < nloc) next = load_tile(tiles, tix(issued));
   int pcb = -1, pcs = 0;  // column slots of the previous tile (-1: diagonal, or none)
@@ -209,11 +222,13 @@ __global__ void __launch_bounds__(kC32Threads, CPS) k_stream_c32(const TileD *__
     if (tid == 0 && k >= 1 && issued < nloc) {
       fence_proxy_async();  // the generic reads of tile k-1's stage before its refill
       issue(issued, next);
+      issue_f(issued, next);
       ++issued;
       if (issued < nloc) next = load_tile(tiles, tix(issued));
     }
     if (k >= 1 && pcb >= 0) c32_columns_out(colred0 + ((k - 1) & 1) * kC32ColFloats, pcb, pcs, tid, tp);
     if (!have) break;
+    if (PDL && k + 1 == nloc) pdl_trigger();
     const int s = k % NST;
     const TileD D = stile[s];
     const bool diag = D.I == D.J;
@@ -288,7 +303,7 @@ constexpr size_t c32_half_smem() {
   return (size_t)NST * kC32HalfStageBytes + 320 + kC32ColFloats * sizeof(float);
 }
 
-template <int MODE, int NST, int CPS>
+template <int MODE, int NST, int CPS, bool PDL>
 __global__ void __launch_bounds__(kC32Threads, CPS) k_stream_c32_half(const TileD *__restrict__ tiles, int nt,
                                                                        const float2 *__restrict__ tc,
                                                                        const float2 *__restrict__ fg,
@@ -319,7 +334,13 @@ __global__ void __launch_bounds__(kC32Threads, CPS) k_stream_c32_half(const Tile
     iss = load_tile(tiles, tix(0));
     if (nloc > 1) ahead = load_tile(tiles, tix(1));
   }
-  auto issue = [&](int v) {  // unit v = 2 k + h: half h of the CTA's tile k
+  auto issue_f = [&](int v, const TileD &D) {  // the f slices of unit v
+    const int h = v & 1, s = v % NST;
+    unsigned char *buf = ssm + (size_t)s * kC32HalfStageBytes + kC32HalfBytes;
+    bulk_g2s(buf, fg + (size_t)D.I * kTile + h * HR, HR * sizeof(float2), bars + s);
+    bulk_g2s(buf + HR * sizeof(float2), fg + (size_t)D.J * kTile, kTile * sizeof(float2), bars + s);
+  };
+  auto issue = [&](int v) {  // (coefficients) unit v = 2 k + h: half h of the CTA's tile k
     const int k = v >> 1, h = v & 1, s = v % NST;
     if (h == 0 && k > 0) {
       iss = ahead;
@@ -331,11 +352,17 @@ __global__ void __launch_bounds__(kC32Threads, CPS) k_stream_c32_half(const Tile
     mbar_expect_tx(bars + s, kC32HalfStageBytes);
     const unsigned char *src = (const unsigned char *)(tc + (size_t)t * kTile * kTile) + (size_t)h * kC32HalfBytes;
     bulk_g2s(buf, src, kC32HalfBytes, bars + s);
-    bulk_g2s(buf + kC32HalfBytes, fg + (size_t)iss.I * kTile + h * HR, HR * sizeof(float2), bars + s);
-    bulk_g2s(buf + kC32HalfBytes + HR * sizeof(float2), fg + (size_t)iss.J * kTile, kTile * sizeof(float2), bars + s);
   };
-  if (tid == 0)
-    for (; issued < NST && issued < nunit; ++issued) issue(issued);
+  if (tid == 0) {
+    for (; issued < NST && issued < nunit; ++issued) {
+      issue(issued);
+      if (!PDL) issue_f(issued, iss);
+    }
+    if (PDL) {
+      pdl_wait();  // f comes from the kernel before this one, which may still read the partials
+      for (int v = 0; v < issued; ++v) issue_f(v, stile[v]);
+    }
+  }
   int pcb = -1, pcs = 0;  // column slots of the previous unit's tile (-1: diagonal, or none)
   bool ok = true;
   float cv[4];  // column sums of the current tile, carried across its halves
@@ -348,10 +375,12 @@ __global__ void __launch_bounds__(kC32Threads, CPS) k_stream_c32_half(const Tile
     if (tid == 0 && u >= 1 && issued < nunit) {
       fence_proxy_async();  // the generic reads of unit u-1's stage before its refill
       issue(issued);
+      issue_f(issued, iss);
       ++issued;
     }
     if ((u & 1) == 0 && u >= 2 && pcb >= 0) c32_columns_out(colred, pcb, pcs, tid, tp);
     if (!have) break;
+    if (PDL && u + 1 == nunit) pdl_trigger();
     const int s = u % NST, h = u & 1;
     const TileD D = stile[s];
     const bool diag = D.I == D.J;
@@ -480,7 +509,7 @@ __global__ void k_pairs_c32(const float2 *__restrict__ A, const float2 *__restri
 // reduce-scatter of the SPC / 8 values), and warp 0 applies the prefactor and the RK4 stage
 // arithmetic in FP64, one lane per state.
 // prow, pmap: as TileSrc
-template <int STAGE, bool RATE = false, int SPC = 32>
+template <int STAGE, bool RATE, int SPC, bool PDL>
 __global__ void __launch_bounds__(256) k_fin_c32(const float *__restrict__ tp, const int2 *__restrict__ prow,
                                                  const int *__restrict__ pmap, int ns, double c,
                                                  const double *__restrict__ ysrc, double *__restrict__ out,
@@ -493,21 +522,31 @@ __global__ void __launch_bounds__(256) k_fin_c32(const float *__restrict__ tp, c
   const int r0 = base + lane;
   FinIn in{0.0, 0.0, 0.0, 0.0};
   int ry = 0;
+  int2 pr[SPW];
+  auto load_rows = [&] {
+#pragma unroll
+    for (int q = 0; q < SPW; ++q) {
+      const int r = base + SPW * wid + q;
+      pr[q] = r < ns ? prow[r] : make_int2(0, 0);
+    }
+  };
+  if (PDL) {
+    load_rows();
+    pdl_wait();
+  }
   if (!RATE && wid == 0 && lane < SPC && r0 < ns) {
     if (STAGE >= 0) in.f = f[r0];
     if (STAGE >= 1) in.acc = acc[r0];
     if (STAGE >= 0) ry = pmap[r0];
   }
   float2 v[SPW];
+  if (!PDL) load_rows();
 #pragma unroll
   for (int q = 0; q < SPW; ++q) {
-    const int r = base + SPW * wid + q;
     v[q] = make_float2(0.f, 0.f);
-    if (r < ns) {
-      const int2 pr = prow[r];
-      for (int k = lane; k < pr.y; k += 32) v[q] = ff_add(v[q], make_float2(tp[pr.x + k], 0.f));
-    }
+    for (int k = lane; k < pr[q].y; k += 32) v[q] = ff_add(v[q], make_float2(tp[pr[q].x + k], 0.f));
   }
+  if (PDL) pdl_trigger();
   ff_reduce_scatter<SPW, 16>(v, lane);
   if ((lane & (LPV - 1)) == 0) tot[SPW * wid + lane / LPV] = v[0];
   __syncthreads();
