@@ -562,7 +562,7 @@ BatchLayoutFF batch_layout_ff(const pb_channels *const *chs, int n, int64_t ns, 
   L.pC = take(c32 && !T.on ? sizeof(float2) * nent : 0);
   L.pidx = take(sizeof(uint32_t) * nent);
   L.Rg = take(sizeof(double) * ns);
-  L.yff = take(sizeof(float2) * (T.on ? T.nsp : ns));  // tiles: the padded state space
+  L.yff = take(T.on ? sizeof(float4) * T.nsp : sizeof(float2) * ns);  // tiles: the padded state space
   L.part = take(sizeof(Part4) * nitems_cap);
   L.acc = take(sizeof(double) * ns);
   L.y = take(sizeof(double) * ns);
@@ -731,15 +731,15 @@ int batch_sweep_tiles(pb_batch *b, cudaStream_t st) {
       });
       return;
     }
-    const float4 *tc = (const float4 *)b->tc;
-    float4 *tp = (float4 *)b->tp;
+    const float4 *tc = (const float4 *)b->tc, *fg = (const float4 *)b->yff;
+    float2 *tp = (float2 *)b->tp;
     const int gs = (int)std::max<int64_t>(1, std::min<int64_t>(nt, (int64_t)b->sm_count * b->tshape));
     if (b->tshape == 3)
-      launch_pdl(pdl(), dev::k_stream_sym_half<2, 3, pdl()>, gs, dev::kSymThreads, dev::half_smem<2>(), st, b->tl, nt, tc,
-                 b->yff, tp, b->err, b->rev);
+      launch_pdl(pdl(), dev::k_stream_sym_half<dev::MODE_COLL, 2, 3, pdl()>, gs, dev::kSymThreads, dev::half_smem<2>(),
+                 st, b->tl, nt, tc, fg, tp, b->err, b->rev);
     else
-      launch_pdl(pdl(), dev::k_stream_sym_half<3, 2, pdl()>, gs, dev::kSymThreads, dev::half_smem<3>(), st, b->tl, nt, tc,
-                 b->yff, tp, b->err, b->rev);
+      launch_pdl(pdl(), dev::k_stream_sym_half<dev::MODE_COLL, 3, 2, pdl()>, gs, dev::kSymThreads, dev::half_smem<3>(),
+                 st, b->tl, nt, tc, fg, tp, b->err, b->rev);
   });
   PB_LAUNCHED("tile sweep (batch)");
   return PB_OK;
@@ -787,12 +787,11 @@ int batch_fin(pb_batch *b, double *out, double *f, double dt, cudaStream_t st, c
     const int ns = (int)b->ns;
     with_bool(chain_pdl(b->tnt, b->sm_count), [&](auto pdl) {
       if (b->prec == 2)
-        launch_pdl(pdl(), dev::k_fin_c32<STAGE, false, 32, pdl()>, (ns + 31) / 32, 256, 0, st, (const float *)b->tp,
-                   b->prow, b->pmap, ns, 1.0, src, out, f, b->acc, b->y, b->yff, dt);
+        launch_pdl(pdl(), dev::k_fin_net<float, STAGE, false, 32, pdl()>, (ns + 31) / 32, 256, 0, st, (const float *)b->tp,
+                   b->prow, b->pmap, ns, 1.0, nullptr, out, f, b->acc, b->y, b->yff, dt);
       else
-        launch_pdl(pdl(), dev::k_fin_tiles<STAGE, false, 32, pdl()>, (ns + 31) / 32, 256, 0, st,
-                   dev::TileSrc{(const float4 *)b->tp, b->prow, b->pmap}, ns, 1.0, b->Rg, src, out, f, b->acc, b->y,
-                   b->yff, dt);
+        launch_pdl(pdl(), dev::k_fin_net<float2, STAGE, false, 32, pdl()>, (ns + 31) / 32, 256, 0, st,
+                   (const float2 *)b->tp, b->prow, b->pmap, ns, 1.0, nullptr, out, f, b->acc, b->y, b->yff, dt);
     });
     PB_LAUNCHED("tile epilogue (batch)");
     return PB_OK;
@@ -820,9 +819,10 @@ int batch_fin(pb_batch *b, double *out, double *f, double dt, cudaStream_t st, c
 
 int batch_stage_input(pb_batch *b, const double *f, cudaStream_t st) {
   if (b->tiles) {
-    dev::k_to_ff_map<<<(int)std::max<int64_t>(1, std::min<int64_t>((b->ns + 255) / 256, 1024)), 256, 0, st>>>(
-        f, (int)b->ns, b->pmap, b->yff);
-    PB_LAUNCHED("k_to_ff_map (batch tiles)");
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((b->ns + 255) / 256, 1024));
+    if (b->prec == 1) dev::k_f0_map<<<grid, 256, 0, st>>>(f, (int)b->ns, b->pmap, (float4 *)b->yff);
+    else dev::k_to_ff_map<<<grid, 256, 0, st>>>(f, (int)b->ns, b->pmap, b->yff);
+    PB_LAUNCHED("stage input (batch tiles)");
     return PB_OK;
   }
   if (b->prec >= 1) {
@@ -1157,7 +1157,7 @@ extern "C" int pb_batch_create(const pb_channels *const *chs, int32_t n, const p
       {
         // the error word; the padding of the stage input stays zero
         cudaError_t e = cudaMemsetAsync(b->err, 0, sizeof(int), st);
-        if (e == cudaSuccess && T.on) e = cudaMemsetAsync(b->yff, 0, sizeof(float2) * (size_t)T.nsp, st);
+        if (e == cudaSuccess && T.on) e = cudaMemsetAsync(b->yff, 0, sizeof(float4) * (size_t)T.nsp, st);
         if (e != cudaSuccess) status = cuda_fail(e, "pb_batch_create: clear");
       }
       if (status == PB_OK) status = batch_setup_ff(b, chs, n, LF, st);

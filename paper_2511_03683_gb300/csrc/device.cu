@@ -518,7 +518,7 @@ Layout make_layout(const pb_channels *ch, const Plan &P, const Plan *S, int vari
   L.tab = take(sizeof(double2) * (size_t)ch->nq * ch->nmodes);
   L.acc = take(sizeof(double) * ns);
   L.y = take(sizeof(double) * ns);
-  L.yff = take(sizeof(float2) * (tp ? std::max<size_t>((size_t)tp->nsp, ns) : ns));
+  L.yff = take(tp ? sizeof(float4) * (size_t)tp->nsp + sizeof(float2) * ns : sizeof(float2) * ns);
   L.fstage = take(sizeof(double) * ns);
   L.Fa = take(transport ? sizeof(double) * 3 * ns : 0);
   L.Fb = take(transport ? sizeof(double) * 3 * ns : 0);
@@ -604,11 +604,12 @@ int cuda_fail(cudaError_t e, const char *what) {
     if (e_ != cudaSuccess) return cuda_fail(e_, #call);         \
   } while (0)
 
-// Which tile sweeps and epilogues form such chains: those of at most one tile per SM, where a stage
-// is little more than the two launches (four-band window, us per RK4 step of 20: 16^3 22.8 against
-// 27.2 as ordinary launches, 28^3 25.7 against 28.5; at 32^3 with the cutoffs, 195 tiles, 18.5 against
-// 16.9, and at 40^3 76 against 68: sweep CTAs that come in while the epilogue runs slow it down).
-bool chain_pdl(int64_t tiles, int sm_count) { return tiles <= sm_count; }
+// Which tile sweeps and epilogues form such chains: those of at most three tiles per two SMs, where a
+// stage is little more than the two launches (four-band window, us per RK4 step: 16^3 22.4 against
+// 25.2 as ordinary launches, 24^3 22.7 against 25.4, 30^3 28.0 against 30.6; at 32^3, 296 tiles, 31.4
+// against 31.0, and at 40^3, 1017 tiles, 64.0 against 59.3: sweep CTAs that come in while the epilogue
+// runs slow it down).
+bool chain_pdl(int64_t tiles, int sm_count) { return 2 * tiles <= 3 * (int64_t)sm_count; }
 
 // kernel<<<grid, block, smem, st>>>(args...), with pdl as a programmatic dependent of the kernel
 // before it in the stream (kernels.cuh, pdl_trigger); only for kernels that wait for it themselves.
@@ -1100,8 +1101,10 @@ void set_half_smem() {
   for (const bool b : {false, true})
     with_bool(b, [](auto pdl) {
       const cudaFuncAttribute A = cudaFuncAttributeMaxDynamicSharedMemorySize;
-      cudaFuncSetAttribute(dev::k_stream_sym_half<3, 2, pdl()>, A, (int)dev::half_smem<3>());
-      cudaFuncSetAttribute(dev::k_stream_sym_half<2, 3, pdl()>, A, (int)dev::half_smem<2>());
+      cudaFuncSetAttribute(dev::k_stream_sym_half<dev::MODE_COLL, 3, 2, pdl()>, A, (int)dev::half_smem<3>());
+      cudaFuncSetAttribute(dev::k_stream_sym_half<dev::MODE_COLL, 2, 3, pdl()>, A, (int)dev::half_smem<2>());
+      cudaFuncSetAttribute(dev::k_stream_sym_half<dev::MODE_RATE, 3, 2, pdl()>, A, (int)dev::half_smem<3>());
+      cudaFuncSetAttribute(dev::k_stream_sym_half<dev::MODE_RATE, 2, 3, pdl()>, A, (int)dev::half_smem<2>());
     });
 }
 void set_c32_smem(int shape) {
@@ -1498,7 +1501,7 @@ extern "C" int pb_dev_create(const pb_channels *ch, const pb_dev_opts *opts, voi
         }
         // the tile sweeps read f in whole blocks: its padding must hold zeros (it multiplies zero
         // coefficients)
-        e_ = cudaMemsetAsync(d->yff, 0, sizeof(float2) * (size_t)std::max<int64_t>(d->sym ? d->nsp : 0, d->ns), st);
+        e_ = cudaMemsetAsync(d->yff, 0, d->sym ? sizeof(float4) * (size_t)d->nsp : sizeof(float2) * (size_t)d->ns, st);
         if (e_ != cudaSuccess) {
           status = cuda_fail(e_, "clear the stage input");
           break;
@@ -1842,17 +1845,22 @@ int launch_stream_t(pb_dev *d, int mode, const double *fd, const float2 *fff, co
       });
     });
   } else if (d->variant == PB_VARIANT_FF && d->sym && !d->c32 && part == d->part) {
-    // symmetric tiles; the rate mode needs the same (A, B) partials
+    // symmetric tiles (the rate mode of the forms other than half-tiles needs the same (A, B) partials)
     if (d->sym_half && fff == d->yff) {
       const int cps = d->half_cps;
       const int gs = (int)std::max<int64_t>(1, std::min<int64_t>(d->tnt, (int64_t)d->sm_count * cps));
       with_bool(d->chain(), [&](auto pdl) {
-        if (cps == 3)
-          launch_pdl(pdl(), dev::k_stream_sym_half<2, 3, pdl()>, gs, dev::kSymThreads, dev::half_smem<2>(), st, d->tiles,
-                     d->tnt, d->tcoef, fff, d->tpart, d->err, d->rev);
-        else
-          launch_pdl(pdl(), dev::k_stream_sym_half<3, 2, pdl()>, gs, dev::kSymThreads, dev::half_smem<3>(), st, d->tiles,
-                     d->tnt, d->tcoef, fff, d->tpart, d->err, d->rev);
+        with_bool(coll, [&](auto cm) {
+          constexpr int M = cm() ? dev::MODE_COLL : dev::MODE_RATE;
+          const float4 *fg = (const float4 *)fff;
+          float2 *tp = (float2 *)d->tpart;
+          if (cps == 3)
+            launch_pdl(pdl(), dev::k_stream_sym_half<M, 2, 3, pdl()>, gs, dev::kSymThreads, dev::half_smem<2>(), st,
+                       d->tiles, d->tnt, d->tcoef, fg, tp, d->err, d->rev);
+          else
+            launch_pdl(pdl(), dev::k_stream_sym_half<M, 3, 2, pdl()>, gs, dev::kSymThreads, dev::half_smem<3>(), st,
+                       d->tiles, d->tnt, d->tcoef, fg, tp, d->err, d->rev);
+        });
       });
     } else if (d->sym_nt && fff == d->yff) {  // the bulk copies read f from this padded arena buffer
       const int gs = (int)std::max<int64_t>(1, std::min<int64_t>(d->tnt, (int64_t)d->sm_count));
@@ -1947,11 +1955,14 @@ void launch_fin_tiles(pb_dev *d, const double *ysrc, double *out, double *f, dou
       constexpr int SPC = small() ? 8 : 32;
       const int grid = (int)((d->ns + SPC - 1) / SPC);
       if (d->c32)
-        launch_pdl(pdl(), dev::k_fin_c32<STAGE, RATE, SPC, pdl()>, grid, 256, 0, st, (const float *)d->tpart, d->prow,
-                   d->pmap, (int)d->ns, d->c, ysrc, out, f, d->acc, y, d->yff, dt);
+        launch_pdl(pdl(), dev::k_fin_net<float, STAGE, RATE, SPC, pdl()>, grid, 256, 0, st, (const float *)d->tpart,
+                   d->prow, d->pmap, (int)d->ns, d->c, nullptr, out, f, d->acc, y, d->yff, dt);
+      else if (d->sym_half)
+        launch_pdl(pdl(), dev::k_fin_net<float2, STAGE, RATE, SPC, pdl()>, grid, 256, 0, st, (const float2 *)d->tpart,
+                   d->prow, d->pmap, (int)d->ns, d->c, d->R, out, f, d->acc, y, d->yff, dt);
       else
-        launch_pdl(pdl(), dev::k_fin_tiles<STAGE, RATE, SPC, pdl()>, grid, 256, 0, st, d->tile_src(), (int)d->ns, d->c,
-                   d->R, ysrc, out, f, d->acc, y, d->yff, dt);
+        dev::k_fin_tiles<STAGE, RATE, SPC><<<grid, 256, 0, st>>>(d->tile_src(), (int)d->ns, d->c, d->R, ysrc, out, f,
+                                                                 d->acc, y, d->yff, dt);
     });
   });
 }
@@ -1987,10 +1998,11 @@ int to_ff(pb_dev *d, const double *x, int64_t n, float2 *out, cudaStream_t st) {
 // Stage-input conversion the streaming kernel of this variant reads (once per call: splitting
 // f inside every CTA of the sweep instead costs more, FP64 being slow on this part).
 int stage_input(pb_dev *d, const double *f, cudaStream_t st) {
-  if (d->variant == PB_VARIANT_FF && d->sym) {  // in the tiles' energy order
-    dev::k_to_ff_map<<<(int)std::max<int64_t>(1, std::min<int64_t>((d->ns + 255) / 256, 1024)), 256, 0, st>>>(
-        f, (int)d->ns, d->pmap, d->yff);
-    PB_LAUNCHED("k_to_ff_map");
+  if (d->variant == PB_VARIANT_FF && d->sym) {  // in the tiles' order
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((d->ns + 255) / 256, 1024));
+    if (d->sym_half) dev::k_f0_map<<<grid, 256, 0, st>>>(f, (int)d->ns, d->pmap, (float4 *)d->yff);
+    else dev::k_to_ff_map<<<grid, 256, 0, st>>>(f, (int)d->ns, d->pmap, d->yff);
+    PB_LAUNCHED("stage input");
     return PB_OK;
   }
   if (d->variant == PB_VARIANT_FF || d->variant == PB_VARIANT_PAPER) return to_ff(d, f, d->ns, d->yff, st);

@@ -2460,38 +2460,84 @@ __global__ void __launch_bounds__(kSymThreads, 1) k_stream_sym_bulk(const TileD 
   }
 }
 
-// The same float-float tile sweep in half-tiles: the unit of staging is 32 rows x 64 columns of a
-// tile (32 KB, contiguous in the tile's row-major layout), so a CTA of 256 threads holds three
-// units in shared memory and two CTAs fit on an SM (16 warps, each CTA with its own barrier).
-// A CTA takes both halves of each of its tiles in turn: rows are complete within a half (one
-// float-float (A, C) partial per row and partner block, as above); the column sums of a tile
-// stay in registers across its two halves and go to the per-warp table after the second, and
-// the table is combined after the next unit's barrier.  Columns are written only every other
-// unit, so one table suffices.  Thread (ti, tj) takes rows 2 ti, 2 ti + 1 of the half and
-// columns tj, tj + 16, tj + 32, tj + 48.
+// The default float-float tile sweep, in half-tiles and net terms.
+//
+// Net terms.  The pair (s, p) adds t = f_p (1 - f_s) P_in - f_s (1 - f_p) P_out to I_s / c and -t to
+// I_p / c (the reverse channel swaps P_in and P_out), so an entry needs one float-float value and
+// each state one sum, I_s = c sum_p t(s, p), in place of the four multiply-adds into the A and C sums
+// of both states that the forms above take.  With f and g = 1 - f staged as float-float (fg), t is the
+// difference of two products of two, 24 operations, and two lazy additions of 8: 40 operations
+// against 48, with half the sums to carry and to reduce, half the partials, and an epilogue of two
+// FP64 operations instead of seven per state.  The terms cancel before they are rounded together, and
+// neither R_s nor the closing difference A - f_s (R - B) is needed (error of df/dt at 35^3 7.8e-15 ->
+// 4.8e-15).  MODE_RATE: B = sum f D for both sides, 1/tau = c (R - B) (the positive summands
+// f_p P_in + g_p P_out instead of R, which is summed in FP64, would be six times less accurate).
+//
+// Half-tiles.  The unit of staging is 32 rows x 64 columns of a tile (32 KB, contiguous in the tile's
+// row-major layout); two stages and the column table take 73 KB, so three CTAs of 256 threads fit on
+// an SM.  A CTA takes both halves of each of its tiles in turn: thread (ti, tj) takes rows 2 ti,
+// 2 ti + 1 of the half and columns tj, tj + 16, tj + 32, tj + 48; row and column sums stay in
+// registers across the two halves.  After the second, the tile's row sums are reduce-scattered over
+// the 16 lanes of a row and the column sums go through one shuffle level and a per-warp table that is
+// combined after the next unit's barrier.  Bound by instruction issue at 40^3.
 constexpr unsigned kHalfTileBytes = kTileBytes / 2;
-constexpr unsigned kHalfStageBytes = kHalfTileBytes + (kTile / 2 + kTile) * sizeof(float2);
+constexpr unsigned kHalfStageBytes = kHalfTileBytes + (kTile / 2 + kTile) * sizeof(float4);
+constexpr size_t kNetColBytes = (size_t)(kSymThreads / 32) * kTile * sizeof(float2);  // the column table
 template <int NST>
 constexpr size_t half_smem() {
-  return (size_t)NST * kHalfStageBytes + 192 + kSymColBytes;
+  return (size_t)NST * kHalfStageBytes + 192 + kNetColBytes;
+}
+
+// (h, l) += (ah, al) without renormalising: h takes the exact TwoSum, l the rest (as ff_mac_lazy)
+__device__ __forceinline__ void ff_add_lazy(float &h, float &l, float ah, float al) {
+  const float s = __fadd_rn(h, ah);
+  const float bb = __fsub_rn(s, h);
+  const float err = __fadd_rn(__fsub_rn(h, __fsub_rn(s, bb)), __fsub_rn(ah, bb));
+  l = __fadd_rn(l, __fadd_rn(err, al));
+  h = s;
+}
+
+// t above from the entry e = (P_in, P_out) and fs, fp = (f hi, f lo, g hi, g lo); not renormalised
+__device__ __forceinline__ float2 net_term(float4 e, float4 fs, float4 fp) {
+  float mh, ml, nh, nl, uh, ul, vh, vl;
+  ff_prod(mh, ml, make_float2(fp.x, fp.y), fs.z, fs.w);  // f_p g_s
+  ff_prod(nh, nl, make_float2(fs.x, fs.y), fp.z, fp.w);  // f_s g_p
+  ff_prod(uh, ul, make_float2(mh, ml), e.x, e.y);
+  ff_prod(vh, vl, make_float2(nh, nl), e.z, e.w);
+  const float s = __fsub_rn(uh, vh);
+  const float bb = __fsub_rn(s, uh);
+  const float err = __fsub_rn(__fsub_rn(uh, __fsub_rn(s, bb)), __fadd_rn(vh, bb));
+  return make_float2(s, __fadd_rn(err, __fsub_rn(ul, vl)));
+}
+
+// the column sums of a finished off-diagonal tile: four lanes per column (l, l ^ 8, l ^ 16, l ^ 24) add
+// two warps' values each, renormalised, into the tile's column slots of tp
+__device__ __forceinline__ void net_columns_out(const float2 *__restrict__ colred, int cb, int cs, int lane, int wid,
+                                                float2 *__restrict__ tp) {
+  const int g = lane >> 3, col = (lane & 7) + 8 * wid;
+  float2 acc = ff_add(colred[2 * g * kTile + col], colred[(2 * g + 1) * kTile + col]);
+#pragma unroll
+  for (int o = 8; o <= 16; o <<= 1)
+    acc = ff_add(acc, make_float2(__shfl_xor_sync(0xFFFFFFFFu, acc.x, o), __shfl_xor_sync(0xFFFFFFFFu, acc.y, o)));
+  if (g == 0) tp[cb + col * cs] = acc;
 }
 
 // NST stages per CTA, CPS resident CTAs per SM (3 x 2 or 2 x 3 fit in the SM's shared memory)
 // rev: take the tile list from its end (tile nt - 1 - t in place of t), so that a sweep following
 // one in list order starts on the tiles the L2 still holds; the partials do not depend on the order.
-template <int NST, int CPS, bool PDL>
+template <int MODE, int NST, int CPS, bool PDL>
 __global__ void __launch_bounds__(kSymThreads, CPS) k_stream_sym_half(const TileD *__restrict__ tiles, int nt,
                                                                        const float4 *__restrict__ tc,
-                                                                       const float2 *__restrict__ fg,
-                                                                       float4 *__restrict__ tp, int *__restrict__ err,
+                                                                       const float4 *__restrict__ fg,
+                                                                       float2 *__restrict__ tp, int *__restrict__ err,
                                                                        int rev = 0) {
   constexpr int kHalfStages = NST;
   static_assert(NST >= 2 && NST <= 4, "the ring needs 2..4 stages");
-  constexpr int R = 2, NV = 2 * R, HR = kTile / 2;
+  constexpr int HR = kTile / 2;
   extern __shared__ __align__(128) unsigned char ssm[];
   unsigned long long *bars = (unsigned long long *)(ssm + kHalfStages * kHalfStageBytes);
   TileD *stile = (TileD *)(bars + 4);  // the tile of each stage's unit
-  float2 *colred = (float2 *)(ssm + kHalfStages * kHalfStageBytes + 192);  // [8 warps][A | C][64 columns]
+  float2 *colred = (float2 *)(ssm + kHalfStages * kHalfStageBytes + 192);  // [8 warps][64 columns]
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, tj = tid & 15, ti = tid >> 4;
   const int G = (int)gridDim.x;
   const int nloc = (int)blockIdx.x < nt ? (nt - 1 - (int)blockIdx.x) / G + 1 : 0;
@@ -2515,8 +2561,8 @@ __global__ void __launch_bounds__(kSymThreads, CPS) k_stream_sym_half(const Tile
   auto issue_f = [&](int v, const TileD &D) {  // the f slices of unit v
     const int h = v & 1, s = v % kHalfStages;
     unsigned char *buf = ssm + (size_t)s * kHalfStageBytes + kHalfTileBytes;
-    bulk_g2s(buf, fg + (size_t)D.I * kTile + h * HR, HR * sizeof(float2), bars + s);
-    bulk_g2s(buf + HR * sizeof(float2), fg + (size_t)D.J * kTile, kTile * sizeof(float2), bars + s);
+    bulk_g2s(buf, fg + (size_t)D.I * kTile + h * HR, HR * sizeof(float4), bars + s);
+    bulk_g2s(buf + HR * sizeof(float4), fg + (size_t)D.J * kTile, kTile * sizeof(float4), bars + s);
   };
   auto issue = [&](int v) {  // unit v = 2 k + h: half h of the CTA's tile k (coefficients)
     const int k = v >> 1, h = v & 1, s = v % kHalfStages;
@@ -2544,7 +2590,7 @@ __global__ void __launch_bounds__(kSymThreads, CPS) k_stream_sym_half(const Tile
   }
   int pcb = -1, pcs = 0;  // column slots of the previous unit's tile (-1: diagonal, or none)
   bool ok = true;
-  float cA[4][2], cC[4][2];  // column sums of the current tile, carried across its halves
+  float c[4][2], r0[2][2];  // column sums of the current tile; row sums of its first half
   for (int u = 0; u <= nunit; ++u) {
     const bool have = u < nunit;
     if (!__syncthreads_and(tid == 0 && have ? mbar_wait(bars + u % kHalfStages, (unsigned)((u / kHalfStages) & 1))
@@ -2559,7 +2605,7 @@ __global__ void __launch_bounds__(kSymThreads, CPS) k_stream_sym_half(const Tile
       ++issued;
     }
     // the previous tile's column table (written after its second half) is complete
-    if ((u & 1) == 0 && u >= 2 && pcb >= 0) sym_columns_out(colred, pcb, pcs, lane, wid, tp);
+    if ((u & 1) == 0 && u >= 2 && pcb >= 0) net_columns_out(colred, pcb, pcs, lane, wid, tp);
     if (!have) break;
     if (PDL && u + 1 == nunit) pdl_trigger();
     const int s = u % kHalfStages, h = u & 1;
@@ -2568,67 +2614,71 @@ __global__ void __launch_bounds__(kSymThreads, CPS) k_stream_sym_half(const Tile
     pcb = diag ? -1 : D.cb;
     pcs = D.cs;
     const float4 *__restrict__ T = (const float4 *)(ssm + (size_t)s * kHalfStageBytes);
-    const float2 *__restrict__ fr = (const float2 *)(ssm + (size_t)s * kHalfStageBytes + kHalfTileBytes);
-    const float2 *__restrict__ fc = fr + HR;
-    float2 fcol[4];
+    const float4 *__restrict__ fr = (const float4 *)(ssm + (size_t)s * kHalfStageBytes + kHalfTileBytes);
+    const float4 *__restrict__ fc = fr + HR;
+    float4 fcol[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) fcol[j] = fc[tj + 16 * j];
-    float rA[R][2], rC[R][2];
+    if (h == 0) {
 #pragma unroll
-    for (int i = 0; i < R; ++i) {
-      const int row = ti * R + i;
-      const float2 fs = fr[row];
-      float4 e[4];
+      for (int j = 0; j < 4; ++j) c[j][0] = c[j][1] = 0.f;
+    }
+    float r[2][2];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) e[j] = T[row * kTile + tj + 16 * j];
+    for (int i = 0; i < 2; ++i) {
+      const int row = ti * 2 + i;
+      const float4 fs = fr[row];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        if (j == 0) {
-          ff_prod(rA[i][0], rA[i][1], fcol[j], e[j].x, e[j].y);
-          ff_prod(rC[i][0], rC[i][1], fcol[j], e[j].z, e[j].w);
-        } else {
-          ff_mac_lazy(rA[i][0], rA[i][1], fcol[j], e[j].x, e[j].y);
-          ff_mac_lazy(rC[i][0], rC[i][1], fcol[j], e[j].z, e[j].w);
-        }
-        if (!diag) {
-          if (h == 0 && i == 0) {
-            ff_prod(cA[j][0], cA[j][1], fs, e[j].z, e[j].w);
-            ff_prod(cC[j][0], cC[j][1], fs, e[j].x, e[j].y);
+        const float4 e = T[row * kTile + tj + 16 * j];
+        if (MODE == MODE_COLL) {
+          const float2 t = net_term(e, fs, fcol[j]);
+          if (j == 0) {
+            r[i][0] = t.x;
+            r[i][1] = t.y;
           } else {
-            ff_mac_lazy(cA[j][0], cA[j][1], fs, e[j].z, e[j].w);
-            ff_mac_lazy(cC[j][0], cC[j][1], fs, e[j].x, e[j].y);
+            ff_add_lazy(r[i][0], r[i][1], t.x, t.y);
+          }
+          if (!diag) ff_add_lazy(c[j][0], c[j][1], -t.x, -t.y);
+        } else {
+          if (j == 0) ff_prod(r[i][0], r[i][1], make_float2(fcol[j].x, fcol[j].y), e.z, e.w);
+          else ff_mac_lazy(r[i][0], r[i][1], make_float2(fcol[j].x, fcol[j].y), e.z, e.w);
+          ff_mac_lazy(r[i][0], r[i][1], make_float2(fcol[j].x, fcol[j].y), -e.x, -e.y);
+          if (!diag) {
+            ff_mac_lazy(c[j][0], c[j][1], make_float2(fs.x, fs.y), e.x, e.y);
+            ff_mac_lazy(c[j][0], c[j][1], make_float2(fs.x, fs.y), -e.z, -e.w);
           }
         }
       }
     }
-    // rows: the 16 lanes of a half-warp share them; lanes 4m .. 4m + 3 end with value m = (row, A | C)
-    {
-      float2 v[NV];
+    if (h == 0) {
 #pragma unroll
-      for (int i = 0; i < R; ++i) {
-        v[2 * i] = make_float2(rA[i][0], rA[i][1]);
-        v[2 * i + 1] = make_float2(rC[i][0], rC[i][1]);
+      for (int i = 0; i < 2; ++i) {
+        r0[i][0] = r[i][0];
+        r0[i][1] = r[i][1];
       }
-      ff_reduce_scatter<NV, 8>(v, lane);
-      const int idx = tj >> 2;
-      if ((tj & 3) == 0) {
-        ((float2 *)tp)[2 * (D.rb + (h * HR + ti * R + (idx >> 1)) * D.rs) + (idx & 1)] = v[0];
-      }
+      continue;
     }
-    if (!diag && h == 1) {
+    // rows: the 16 lanes of a half-warp share them; lanes 4m .. 4m + 3 end with row m's total
+    // (rows 2 ti, 2 ti + 1 of the first half, then of the second)
+    {
+      float2 v[4] = {make_float2(r0[0][0], r0[0][1]), make_float2(r0[1][0], r0[1][1]), make_float2(r[0][0], r[0][1]),
+                     make_float2(r[1][0], r[1][1])};
+      ff_reduce_scatter<4, 8>(v, lane);
+      const int m = tj >> 2;
+      if ((tj & 3) == 0) tp[D.rb + ((m >> 1) * HR + ti * 2 + (m & 1)) * D.rs] = v[0];
+    }
+    if (!diag) {
       // columns of the whole tile: lanes tj and tj + 16 share them (one level), then the warps
       // (after the next unit's barrier)
       const bool up = lane & 16;
 #pragma unroll
-      for (int m = 0; m < 4; ++m) {
-        const int jk = m >> 1, jo = jk + 2;  // kept / sent column slot
-        const float2 a = (m & 1) ? make_float2(cC[jk][0], cC[jk][1]) : make_float2(cA[jk][0], cA[jk][1]);
-        const float2 c = (m & 1) ? make_float2(cC[jo][0], cC[jo][1]) : make_float2(cA[jo][0], cA[jo][1]);
-        const float2 send = up ? a : c, keep = up ? c : a;
-        const float2 w = ff_add(keep, make_float2(__shfl_xor_sync(0xFFFFFFFFu, send.x, 16),
-                                                  __shfl_xor_sync(0xFFFFFFFFu, send.y, 16)));
-        const int col = tj + 16 * ((up ? 2 : 0) + jk);
-        colred[(wid * 2 + (m & 1)) * kTile + col] = w;
+      for (int jk = 0; jk < 2; ++jk) {
+        const int jo = jk + 2;  // kept / sent column slot
+        const float2 a = make_float2(c[jk][0], c[jk][1]), b = make_float2(c[jo][0], c[jo][1]);
+        const float2 send = up ? a : b, keep = up ? b : a;
+        colred[wid * kTile + tj + 16 * ((up ? 2 : 0) + jk)] =
+            ff_add(keep, make_float2(__shfl_xor_sync(0xFFFFFFFFu, send.x, 16), __shfl_xor_sync(0xFFFFFFFFu, send.y, 16)));
       }
     }
   }
@@ -2654,6 +2704,7 @@ __global__ void __launch_bounds__(kSymThreads, CPS) k_stream_sym_half(const Tile
 
 // (f, 1 - f) as float-float pairs in the padded energy order (the padding keeps its zeros)
 __global__ void k_f0_map(const double *__restrict__ f, int n, const int *__restrict__ pmap, float4 *__restrict__ out) {
+  pdl_trigger();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const double v = f[i];
     const float2 a = ff_split(v), b = ff_split(1.0 - v);
@@ -2866,7 +2917,19 @@ __device__ __forceinline__ FinIn fin_load(int r, const double *__restrict__ R, c
 
 // out[r] = I (STAGE < 0), or the RK4 stage arithmetic with k_{STAGE+1} = I
 // ry: the state's row of yff when that is in the tiles' padded energy order, else r
-template <int STAGE, bool GSTATE>
+enum { OUT_FF = 0, OUT_REC = 1, OUT_FG = 2 };  // the sweep's input: float2 f, uint4 records, float4 (f, 1 - f)
+
+// (f, 1 - f) as float-float pairs; 1 - f by float-float arithmetic (FP32 only)
+__device__ __forceinline__ float4 fg_of(double f) {
+  const float2 a = ff_split(f);
+  const float s = __fsub_rn(1.f, a.x);
+  const float bb = __fsub_rn(s, 1.f);
+  const float e = __fsub_rn(__fsub_rn(__fsub_rn(1.f, __fsub_rn(s, bb)), __fadd_rn(a.x, bb)), a.y);
+  const float h = __fadd_rn(s, e);
+  return make_float4(a.x, a.y, h, __fsub_rn(e, __fsub_rn(h, s)));
+}
+
+template <int STAGE, int OUT>
 __device__ __forceinline__ void fin_stage(int r, double I, const FinIn &in, double *__restrict__ out,
                                           double *__restrict__ f, double *__restrict__ acc, double *__restrict__ y,
                                           float2 *__restrict__ yff, double dt, int ry = -1) {
@@ -2890,17 +2953,19 @@ __device__ __forceinline__ void fin_stage(int r, double I, const FinIn &in, doub
     f[r] = yn;
   }
   y[r] = yn;
-  if (GSTATE)
-    rec_set_f(reinterpret_cast<uint4 *>(yff) + r, yn);  // yff points at the uint4 record array
+  if (OUT == OUT_REC)
+    rec_set_f(reinterpret_cast<uint4 *>(yff) + r, yn);
+  else if (OUT == OUT_FG)
+    reinterpret_cast<float4 *>(yff)[ry] = fg_of(yn);
   else
     yff[ry < 0 ? r : ry] = ff_split(yn);
 }
 
-template <bool LIT, int STAGE, bool GSTATE>
+template <bool LIT, int STAGE, int OUT>
 __device__ __forceinline__ void fin_apply(int r, double A, double B, double c, const FinIn &in,
                                           double *__restrict__ out, double *__restrict__ f, double *__restrict__ acc,
                                           double *__restrict__ y, float2 *__restrict__ yff, double dt, int ry = -1) {
-  fin_stage<STAGE, GSTATE>(r, LIT ? -c * A : c * (A - in.y * (in.R - B)), in, out, f, acc, y, yff, dt, ry);
+  fin_stage<STAGE, OUT>(r, LIT ? -c * A : c * (A - in.y * (in.R - B)), in, out, f, acc, y, yff, dt, ry);
 }
 
 template <bool LIT, int STAGE, bool GSTATE = false, typename SRC = ItemSrc>
@@ -2912,7 +2977,7 @@ __global__ void k_fin_coll(SRC src, int ns, double c, const double *__restrict__
   const FinIn in = fin_load<LIT, STAGE>(r, R, ysrc, f, acc);
   double A, B;
   src.get(r, A, B);
-  fin_apply<LIT, STAGE, GSTATE>(r, A, B, c, in, out, f, acc, y, yff, dt);
+  fin_apply<LIT, STAGE, GSTATE ? OUT_REC : OUT_FF>(r, A, B, c, in, out, f, acc, y, yff, dt);
 }
 
 // The same epilogue over symmetric-tile partials, one warp per state: lanes add the block
@@ -2926,7 +2991,7 @@ __global__ void k_fin_coll(SRC src, int ns, double c, const double *__restrict__
 // cost the same with one active lane as with 32 on this part, so a lane-0-per-state epilogue
 // spent most of its time there).  RATE: 1/tau.
 // SPC states per CTA (8 or 32; few states take 8, for more CTAs in flight)
-template <int STAGE, bool RATE, int SPC, bool PDL>
+template <int STAGE, bool RATE, int SPC>
 __global__ void __launch_bounds__(256) k_fin_tiles(TileSrc src, int ns, double c, const double *__restrict__ R,
                                                    const double *__restrict__ ysrc, double *__restrict__ out,
                                                    double *__restrict__ f, double *__restrict__ acc,
@@ -2935,18 +3000,6 @@ __global__ void __launch_bounds__(256) k_fin_tiles(TileSrc src, int ns, double c
   __shared__ float4 tot[SPC];  // (A hi, A lo, C hi, C lo) per state
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int base = blockIdx.x * SPC;
-  int2 pr[SPW];
-  auto load_rows = [&] {
-#pragma unroll
-    for (int q = 0; q < SPW; ++q) {
-      const int r = base + SPW * wid + q;
-      pr[q] = r < ns ? src.prow[r] : make_int2(0, 0);
-    }
-  };
-  if (PDL) {
-    load_rows();
-    pdl_wait();
-  }
   // warp 0 loads its state's epilogue inputs first, so that their latency overlaps the partials'
   const int r0 = base + lane;
   FinIn in{0.0, 0.0, 0.0, 0.0};
@@ -2959,7 +3012,12 @@ __global__ void __launch_bounds__(256) k_fin_tiles(TileSrc src, int ns, double c
   // the first three partials of every lane for the warp's states are loaded together (up to 96
   // partner blocks), the rest after
   float4 w[SPW][3];
-  if (!PDL) load_rows();
+  int2 pr[SPW];
+#pragma unroll
+  for (int q = 0; q < SPW; ++q) {
+    const int r = base + SPW * wid + q;
+    pr[q] = r < ns ? src.prow[r] : make_int2(0, 0);
+  }
 #pragma unroll
   for (int q = 0; q < SPW; ++q) {
 #pragma unroll
@@ -2984,7 +3042,6 @@ __global__ void __launch_bounds__(256) k_fin_tiles(TileSrc src, int ns, double c
       v[2 * q + 1] = ff_add(v[2 * q + 1], make_float2(x.z, x.w));
     }
   }
-  if (PDL) pdl_trigger();
   ff_reduce_scatter<NV, 16>(v, lane);
   if ((lane & (LPV - 1)) == 0) {
     const int idx = lane / LPV;  // the top lane bits: (state q, A | C)
@@ -2999,7 +3056,7 @@ __global__ void __launch_bounds__(256) k_fin_tiles(TileSrc src, int ns, double c
   if (RATE)
     out[r0] = c * (in.R - B);
   else
-    fin_apply<false, STAGE, false>(r0, A, B, c, in, out, f, acc, y, yff, dt, ry);
+    fin_apply<false, STAGE, OUT_FF>(r0, A, B, c, in, out, f, acc, y, yff, dt, ry);
 }
 
 template <bool LIT, typename SRC = ItemSrc>

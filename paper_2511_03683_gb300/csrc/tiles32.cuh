@@ -504,15 +504,19 @@ __global__ void k_pairs_c32(const float2 *__restrict__ A, const float2 *__restri
   }
 }
 
-// Epilogue of the C32 sweep: a 256-thread CTA takes SPC states; each warp adds the block
+// Epilogue of the net-term sweeps (PT = float: C32; float2: the float-float half-tile sweep, whose
+// next input is (f, 1 - f)): a 256-thread CTA takes SPC states; each warp adds the block
 // partials of SPC / 8 states (lanes over the blocks in float-float, then one 32-lane float-float
 // reduce-scatter of the SPC / 8 values), and warp 0 applies the prefactor and the RK4 stage
 // arithmetic in FP64, one lane per state.
-// prow, pmap: as TileSrc
-template <int STAGE, bool RATE, int SPC, bool PDL>
-__global__ void __launch_bounds__(256) k_fin_c32(const float *__restrict__ tp, const int2 *__restrict__ prow,
+// prow, pmap: as TileSrc.  RATE: 1/tau = c (R - sum) for the float-float sweep (partials of B), c sum
+// for C32 (partials of the summands themselves).
+__device__ __forceinline__ float2 as_ff(float v) { return make_float2(v, 0.f); }
+__device__ __forceinline__ float2 as_ff(float2 v) { return v; }
+template <typename PT, int STAGE, bool RATE, int SPC, bool PDL>
+__global__ void __launch_bounds__(256) k_fin_net(const PT *__restrict__ tp, const int2 *__restrict__ prow,
                                                  const int *__restrict__ pmap, int ns, double c,
-                                                 const double *__restrict__ ysrc, double *__restrict__ out,
+                                                 const double *__restrict__ R, double *__restrict__ out,
                                                  double *__restrict__ f, double *__restrict__ acc,
                                                  double *__restrict__ y, float2 *__restrict__ yff, double dt) {
   constexpr int SPW = SPC / 8, LPV = 32 / SPW;  // states per warp, lanes per state after the reduce-scatter
@@ -534,6 +538,8 @@ __global__ void __launch_bounds__(256) k_fin_c32(const float *__restrict__ tp, c
     load_rows();
     pdl_wait();
   }
+  double Rr = 0.0;
+  if (RATE && R && wid == 0 && lane < SPC && r0 < ns) Rr = R[r0];
   if (!RATE && wid == 0 && lane < SPC && r0 < ns) {
     if (STAGE >= 0) in.f = f[r0];
     if (STAGE >= 1) in.acc = acc[r0];
@@ -544,7 +550,7 @@ __global__ void __launch_bounds__(256) k_fin_c32(const float *__restrict__ tp, c
 #pragma unroll
   for (int q = 0; q < SPW; ++q) {
     v[q] = make_float2(0.f, 0.f);
-    for (int k = lane; k < pr[q].y; k += 32) v[q] = ff_add(v[q], make_float2(tp[pr[q].x + k], 0.f));
+    for (int k = lane; k < pr[q].y; k += 32) v[q] = ff_add(v[q], as_ff(tp[pr[q].x + k]));
   }
   if (PDL) pdl_trigger();
   ff_reduce_scatter<SPW, 16>(v, lane);
@@ -552,12 +558,12 @@ __global__ void __launch_bounds__(256) k_fin_c32(const float *__restrict__ tp, c
   __syncthreads();
   if (wid != 0 || lane >= SPC || r0 >= ns) return;
   const float2 Tt = tot[lane];
-  const double I = c * ff_to_double(Tt.x, Tt.y);
   if (RATE) {
-    out[r0] = I;
+    out[r0] = c * (R ? Rr - ff_to_double(Tt.x, Tt.y) : ff_to_double(Tt.x, Tt.y));
     return;
   }
-  fin_stage<STAGE, false>(r0, I, in, out, f, acc, y, yff, dt, ry);
+  const double I = c * ff_to_double(Tt.x, Tt.y);
+  fin_stage<STAGE, sizeof(PT) == sizeof(float) ? OUT_FF : OUT_FG>(r0, I, in, out, f, acc, y, yff, dt, ry);
 }
 
 }  // namespace dev
