@@ -492,7 +492,7 @@ struct BatchTiles : TilePlan {
 };
 // nent: the padded pair entries of all rows; lenp: those of every row (batch_pair_lenp)
 BatchTiles batch_tiles_for(const pb_channels *const *chs, int32_t n, int prec, int layout,
-                           const std::vector<int64_t> &lenp) {
+                           const std::vector<int64_t> &lenp, int sm) {
   BatchTiles T;
   if (prec < 1 || layout == 1) return T;
   int64_t nent = 0, so = 0;
@@ -515,6 +515,7 @@ BatchTiles batch_tiles_for(const pb_channels *const *chs, int32_t n, int prec, i
   const double tile_bytes = (double)nt * dev::kTile * dev::kTile * (prec == 2 ? 8.0 : 16.0);
   const double row_bytes = (double)nent * (prec == 2 ? 12.0 : 20.0);
   T.on = layout == 2 || tile_bytes <= 0.7 * row_bytes;
+  if (T.on && prec == 1 && chain_pdl(nt, sm)) tile_plan_halve(T);
   return T;
 }
 
@@ -716,8 +717,12 @@ int batch_upload_plan(pb_batch *b, int item_ch, cudaStream_t st) {
 // the tile sweep of every instance in one launch (the single-system kernels)
 int batch_sweep_tiles(pb_batch *b, cudaStream_t st) {
   const int nt = b->tnt;
-  with_bool(chain_pdl(nt, b->sm_count), [&](auto pdl) {
-    if (b->prec == 2) {
+  const bool chain = chain_pdl(nt, b->sm_count);
+  if (b->prec == 1)
+    launch_half_tiles<dev::MODE_COLL>(chain, b->tshape, b->sm_count, b->tl, nt, (const float4 *)b->tc, b->yff, b->tp,
+                                      b->err, b->rev, st);
+  else
+    with_bool(chain, [&](auto pdl) {
       with_c32_shape(b->tshape, [&](auto nst, auto cps, auto half) {
         const int gs = (int)std::max<int64_t>(1, std::min<int64_t>(nt, (int64_t)b->sm_count * cps()));
         const float2 *tc = (const float2 *)b->tc;
@@ -729,18 +734,7 @@ int batch_sweep_tiles(pb_batch *b, cudaStream_t st) {
           launch_pdl(pdl(), dev::k_stream_c32<dev::MODE_COLL, nst(), cps(), pdl()>, gs, dev::kC32Threads,
                      dev::c32_smem<nst()>(), st, b->tl, nt, tc, b->yff, tp, b->err, b->rev);
       });
-      return;
-    }
-    const float4 *tc = (const float4 *)b->tc, *fg = (const float4 *)b->yff;
-    float2 *tp = (float2 *)b->tp;
-    const int gs = (int)std::max<int64_t>(1, std::min<int64_t>(nt, (int64_t)b->sm_count * b->tshape));
-    if (b->tshape == 3)
-      launch_pdl(pdl(), dev::k_stream_sym_half<dev::MODE_COLL, 2, 3, pdl()>, gs, dev::kSymThreads, dev::half_smem<2>(),
-                 st, b->tl, nt, tc, fg, tp, b->err, b->rev);
-    else
-      launch_pdl(pdl(), dev::k_stream_sym_half<dev::MODE_COLL, 3, 2, pdl()>, gs, dev::kSymThreads, dev::half_smem<3>(),
-                 st, b->tl, nt, tc, fg, tp, b->err, b->rev);
-  });
+    });
   PB_LAUNCHED("tile sweep (batch)");
   return PB_OK;
 }
@@ -1044,12 +1038,15 @@ extern "C" int pb_batch_arena_bytes(const pb_channels *const *chs, int32_t n, co
       if (!chs[i]->closed)
         return set_error(PB_EINVAL, "pb_batch: layout 2 (symmetric tiles) needs channel lists built with the "
                                     "closure check (list %d was not)", i);
+  int sm = 152, devid = 0;
+  if (cudaGetDevice(&devid) == cudaSuccess) cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, devid);
+  else cudaGetLastError();
   try {
     if (prec >= 1) {
       const std::vector<int64_t> lenp = batch_pair_lenp(chs, n);
       int64_t nent = 0;
       for (int64_t l : lenp) nent += l;
-      const BatchTiles T = batch_tiles_for(chs, n, prec, opts ? opts->layout : 0, lenp);
+      const BatchTiles T = batch_tiles_for(chs, n, prec, opts ? opts->layout : 0, lenp, sm);
       *bytes = batch_layout_ff(chs, n, ns, nent, batch_items_count(lenp, kBatchMinItem), prec == 2, T, lenp).total;
     } else {
       pb_batch_opts o{};
@@ -1057,9 +1054,6 @@ extern "C" int pb_batch_arena_bytes(const pb_channels *const *chs, int32_t n, co
       const bool dense = batch_dense_for(chs, n, o);
       const BatchDenseCaps dc = dense ? batch_dense_caps(chs, n, o.item_channels) : BatchDenseCaps{};
       const int64_t cap = std::max(batch_items_count(batch_lenp(chs, n), kBatchMinItem), dc.items);
-      int sm = 152, devid = 0;
-      if (cudaGetDevice(&devid) == cudaSuccess) cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, devid);
-      else cudaGetLastError();
       *bytes = batch_layout(chs, n, ns, nchp, cap, dc, sm).total;
     }
   } catch (const std::bad_alloc &) {
@@ -1119,7 +1113,7 @@ extern "C" int pb_batch_create(const pb_channels *const *chs, int32_t n, const p
     if (b->prec >= 1) {
       int64_t nent = 0;
       for (int64_t l : b->lenp) nent += l;
-      const BatchTiles T = batch_tiles_for(chs, n, b->prec, o.layout, b->lenp);
+      const BatchTiles T = batch_tiles_for(chs, n, b->prec, o.layout, b->lenp, sm);
       const BatchLayoutFF LF = batch_layout_ff(chs, n, ns, nent, b->nitems_cap, b->prec == 2, T, b->lenp);
       if (bytes < LF.total) {
         delete b;

@@ -429,6 +429,31 @@ void tile_plan_add(const pb_channels *ch, bool energy, bool complete, double rea
   T.nsp = (int64_t)T.nb * dev::kTile;
 }
 
+// A second column slot for every off-diagonal tile of the plan, for the sweep whose CTAs take half a tile
+// (k_stream_sym_unit): a state of block K then has two slots per tile of block column K, its row slots
+// after them.
+void tile_plan_halve(TilePlan &T) {
+  std::vector<int64_t> first((size_t)T.nb);
+  std::vector<int> slots((size_t)T.nb);
+  auto ncol = [&](int K) { return K - T.span[K].x; };  // tiles above the diagonal in block column K
+  T.npart = 0;
+  for (int K = 0; K < T.nb; ++K) {
+    slots[K] = T.span[K].y + ncol(K);
+    first[K] = T.npart;
+    T.npart += (int64_t)slots[K] * dev::kTile;
+  }
+  for (size_t r = 0; r < T.pmap.size(); ++r) {
+    const int K = T.pmap[r] / dev::kTile;
+    T.prow[r] = make_int2((int)(first[K] + (int64_t)(T.pmap[r] % dev::kTile) * slots[K]), slots[K]);
+  }
+  for (dev::TileD &D : T.tiles) {
+    D.rb = (int)(first[D.I] + 2 * ncol(D.I) + (D.J - D.I));
+    D.rs = slots[D.I];
+    D.cb = (int)(first[D.J] + 2 * (D.I - T.span[D.J].x));
+    D.cs = slots[D.J];
+  }
+}
+
 // The transport weight tiles of a tile plan (kernels.cuh): the list of them, block-row-major, cut into
 // one contiguous range per CTA, and the segments (a CTA's tiles of one block row, at most
 // kTrSegTiles) with each block row's range of them.
@@ -437,7 +462,11 @@ struct TrTilePlan {
   std::vector<int2> segr;
   int nseg = 0, grid = 0;
 };
-int64_t tr_tiles_of(const TilePlan &T) { return T.npart / dev::kTile; }
+int64_t tr_tiles_of(const TilePlan &T) {
+  int64_t n = 0;
+  for (const int2 s : T.span) n += s.y;
+  return n;
+}
 int64_t tr_segs_cap(const TilePlan &T, int sm) {
   return tr_tiles_of(T) / dev::kTrSegTiles + 2 * (int64_t)T.nb + (int64_t)sm * dev::kTrCtas + 1;
 }
@@ -964,13 +993,15 @@ bool tiles_pay(int64_t nt, int64_t ns, int64_t nsw) {
 // serves (p, s) with P_in and P_out swapped); dense_rows 3, or automatic (0) on complete rows or
 // when the tiles stream fewer bytes than the rows (pays)
 // T: the tile plan, filled in when they may be taken.
-bool sym_for(const pb_channels *ch, const pb_dev_opts &o, bool c32, bool merged, bool complete, int64_t nsw,
+bool sym_for(const pb_channels *ch, const pb_dev_opts &o, bool c32, bool merged, bool complete, int64_t nsw, int sm,
              TilePlan &T) {
   if (!(merged && ch->closed && o.variant == PB_VARIANT_FF && o.stream_mode != 2)) return false;
   if (o.dense_rows != 3 && o.dense_rows != 0) return false;
   tile_plan_add(ch, !c32, complete, energy_reach(ch, 1.0), T);
   if (T.tiles.size() >= (size_t)INT32_MAX / 2 || T.npart >= INT32_MAX) return false;
-  return o.dense_rows == 3 || complete || tiles_pay((int64_t)T.tiles.size(), ch->nstate, nsw);
+  if (!(o.dense_rows == 3 || complete || tiles_pay((int64_t)T.tiles.size(), ch->nstate, nsw))) return false;
+  if (!c32 && o.tile_sweep == 3 && chain_pdl((int64_t)T.tiles.size(), sm)) tile_plan_halve(T);
+  return true;
 }
 
 // work-item size of the branch-merged sweep: the caller's, the bulk ring's, or the default
@@ -1098,14 +1129,24 @@ int paper_setup(pb_dev *d, const pb_channels *ch, int item_ch, cudaStream_t st) 
 
 // dynamic shared memory of the tile sweeps
 void set_half_smem() {
-  for (const bool b : {false, true})
-    with_bool(b, [](auto pdl) {
-      const cudaFuncAttribute A = cudaFuncAttributeMaxDynamicSharedMemorySize;
-      cudaFuncSetAttribute(dev::k_stream_sym_half<dev::MODE_COLL, 3, 2, pdl()>, A, (int)dev::half_smem<3>());
-      cudaFuncSetAttribute(dev::k_stream_sym_half<dev::MODE_COLL, 2, 3, pdl()>, A, (int)dev::half_smem<2>());
-      cudaFuncSetAttribute(dev::k_stream_sym_half<dev::MODE_RATE, 3, 2, pdl()>, A, (int)dev::half_smem<3>());
-      cudaFuncSetAttribute(dev::k_stream_sym_half<dev::MODE_RATE, 2, 3, pdl()>, A, (int)dev::half_smem<2>());
-    });
+  const cudaFuncAttribute A = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  cudaFuncSetAttribute(dev::k_stream_sym_half<dev::MODE_COLL, 3, 2>, A, (int)dev::half_smem<3>());
+  cudaFuncSetAttribute(dev::k_stream_sym_half<dev::MODE_COLL, 2, 3>, A, (int)dev::half_smem<2>());
+  cudaFuncSetAttribute(dev::k_stream_sym_half<dev::MODE_RATE, 3, 2>, A, (int)dev::half_smem<3>());
+  cudaFuncSetAttribute(dev::k_stream_sym_half<dev::MODE_RATE, 2, 3>, A, (int)dev::half_smem<2>());
+}
+// The half-tile sweep of nt tiles.  fg: the padded (f, 1 - f) records; tp: the float2 partials.
+template <int MODE>
+void launch_half_tiles(bool chain, int cps, int sm_count, const dev::TileD *tiles, int nt, const float4 *tc, const void *fg_,
+                       void *tp_, int *err, int rev, cudaStream_t st) {
+  const float4 *fg = (const float4 *)fg_;
+  float2 *tp = (float2 *)tp_;
+  const int gs = (int)std::max<int64_t>(1, std::min<int64_t>(nt, (int64_t)sm_count * cps));
+  if (chain) launch_pdl(true, dev::k_stream_sym_unit<MODE>, 2 * nt, dev::kSymThreads, 0, st, tiles, tc, fg, tp);
+  else if (cps == 3)
+    dev::k_stream_sym_half<MODE, 2, 3><<<gs, dev::kSymThreads, dev::half_smem<2>(), st>>>(tiles, nt, tc, fg, tp, err, rev);
+  else
+    dev::k_stream_sym_half<MODE, 3, 2><<<gs, dev::kSymThreads, dev::half_smem<3>(), st>>>(tiles, nt, tc, fg, tp, err, rev);
 }
 void set_c32_smem(int shape) {
   for (const bool b : {false, true})
@@ -1157,7 +1198,7 @@ extern "C" int pb_dev_arena_bytes(const pb_channels *ch, const pb_dev_opts *opts
     const bool merged = make_plans(ch, opts, o, sm, P, S, &complete);
     const int nfin = (int)((P.ns + kFinBlock - 1) / kFinBlock);
     TilePlan T;
-    const bool sym = sym_for(ch, o, c32, merged, complete, S.nchp, T);
+    const bool sym = sym_for(ch, o, c32, merged, complete, S.nchp, sm, T);
     if (c32 && !sym)
       return set_error(PB_EINVAL, "pb_dev: the FP32 coefficient tiles (C32) need the symmetric tiles: a "
                                   "closure-checked list whose rows are complete or miss few partners (or dense_rows 3)");
@@ -1200,7 +1241,7 @@ extern "C" int pb_dev_create(const pb_channels *ch, const pb_dev_opts *opts, voi
   bool merged = false, complete = false, sym = false;
   try {
     merged = make_plans(ch, opts, o, sm, P, S, &complete);
-    sym = sym_for(ch, o, c32, merged, complete, S.nchp, T);
+    sym = sym_for(ch, o, c32, merged, complete, S.nchp, sm, T);
   } catch (const std::bad_alloc &) {
     delete d;
     return set_error(PB_ENOMEM, "pb_dev_create: out of host memory");
@@ -1665,7 +1706,7 @@ extern "C" int pb_dev_create(const pb_channels *ch, const pb_dev_opts *opts, voi
   if (d->sym_nt) {
     if (dev::kSymBulkSmem > (size_t)smem_optin) {
       d->sym_nt = 0;  // the global-load tile sweep needs no opt-in shared memory
-      d->sym_half = false;
+      d->sym_half = d->sym_half && d->chain();  // (its small form needs none either)
     } else {
       cudaFuncSetAttribute(dev::k_stream_sym_bulk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dev::kSymBulkSmem);
       set_half_smem();
@@ -1847,20 +1888,9 @@ int launch_stream_t(pb_dev *d, int mode, const double *fd, const float2 *fff, co
   } else if (d->variant == PB_VARIANT_FF && d->sym && !d->c32 && part == d->part) {
     // symmetric tiles (the rate mode of the forms other than half-tiles needs the same (A, B) partials)
     if (d->sym_half && fff == d->yff) {
-      const int cps = d->half_cps;
-      const int gs = (int)std::max<int64_t>(1, std::min<int64_t>(d->tnt, (int64_t)d->sm_count * cps));
-      with_bool(d->chain(), [&](auto pdl) {
-        with_bool(coll, [&](auto cm) {
-          constexpr int M = cm() ? dev::MODE_COLL : dev::MODE_RATE;
-          const float4 *fg = (const float4 *)fff;
-          float2 *tp = (float2 *)d->tpart;
-          if (cps == 3)
-            launch_pdl(pdl(), dev::k_stream_sym_half<M, 2, 3, pdl()>, gs, dev::kSymThreads, dev::half_smem<2>(), st,
-                       d->tiles, d->tnt, d->tcoef, fg, tp, d->err, d->rev);
-          else
-            launch_pdl(pdl(), dev::k_stream_sym_half<M, 3, 2, pdl()>, gs, dev::kSymThreads, dev::half_smem<3>(), st,
-                       d->tiles, d->tnt, d->tcoef, fg, tp, d->err, d->rev);
-        });
+      with_bool(coll, [&](auto cm) {
+        launch_half_tiles<cm() ? dev::MODE_COLL : dev::MODE_RATE>(d->chain(), d->half_cps, d->sm_count, d->tiles, d->tnt,
+                                                                 d->tcoef, fff, d->tpart, d->err, d->rev, st);
       });
     } else if (d->sym_nt && fff == d->yff) {  // the bulk copies read f from this padded arena buffer
       const int gs = (int)std::max<int64_t>(1, std::min<int64_t>(d->tnt, (int64_t)d->sm_count));

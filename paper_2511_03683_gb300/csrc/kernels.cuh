@@ -2510,7 +2510,45 @@ __device__ __forceinline__ float2 net_term(float4 e, float4 fs, float4 fp) {
   return make_float2(s, __fadd_rn(err, __fsub_rn(ul, vl)));
 }
 
-// the column sums of a finished off-diagonal tile: four lanes per column (l, l ^ 8, l ^ 16, l ^ 24) add
+// one entry into the row sum r (first: its first term) and, off the diagonal, the column sum c
+template <int MODE>
+__device__ __forceinline__ void net_entry(float4 e, float4 fs, float4 fp, bool diag, bool first, float (&r)[2],
+                                          float (&c)[2]) {
+  if (MODE == MODE_COLL) {
+    const float2 t = net_term(e, fs, fp);
+    if (first) {
+      r[0] = t.x;
+      r[1] = t.y;
+    } else {
+      ff_add_lazy(r[0], r[1], t.x, t.y);
+    }
+    if (!diag) ff_add_lazy(c[0], c[1], -t.x, -t.y);
+  } else {
+    if (first) ff_prod(r[0], r[1], make_float2(fp.x, fp.y), e.z, e.w);
+    else ff_mac_lazy(r[0], r[1], make_float2(fp.x, fp.y), e.z, e.w);
+    ff_mac_lazy(r[0], r[1], make_float2(fp.x, fp.y), -e.x, -e.y);
+    if (!diag) {
+      ff_mac_lazy(c[0], c[1], make_float2(fs.x, fs.y), e.x, e.y);
+      ff_mac_lazy(c[0], c[1], make_float2(fs.x, fs.y), -e.z, -e.w);
+    }
+  }
+}
+
+// the column sums of an off-diagonal tile into the per-warp table: lanes tj and tj + 16 share a column,
+// and each keeps two of the four
+__device__ __forceinline__ void net_columns_in(const float (&c)[4][2], float2 *colred, int lane, int wid) {
+  const bool up = lane & 16;
+#pragma unroll
+  for (int jk = 0; jk < 2; ++jk) {
+    const int jo = jk + 2;  // kept / sent column slot
+    const float2 a = make_float2(c[jk][0], c[jk][1]), b = make_float2(c[jo][0], c[jo][1]);
+    const float2 send = up ? a : b, keep = up ? b : a;
+    colred[wid * kTile + (lane & 15) + 16 * ((up ? 2 : 0) + jk)] =
+        ff_add(keep, make_float2(__shfl_xor_sync(0xFFFFFFFFu, send.x, 16), __shfl_xor_sync(0xFFFFFFFFu, send.y, 16)));
+  }
+}
+
+// the sums in the table: four lanes per column (l, l ^ 8, l ^ 16, l ^ 24) add
 // two warps' values each, renormalised, into the tile's column slots of tp
 __device__ __forceinline__ void net_columns_out(const float2 *__restrict__ colred, int cb, int cs, int lane, int wid,
                                                 float2 *__restrict__ tp) {
@@ -2525,7 +2563,7 @@ __device__ __forceinline__ void net_columns_out(const float2 *__restrict__ colre
 // NST stages per CTA, CPS resident CTAs per SM (3 x 2 or 2 x 3 fit in the SM's shared memory)
 // rev: take the tile list from its end (tile nt - 1 - t in place of t), so that a sweep following
 // one in list order starts on the tiles the L2 still holds; the partials do not depend on the order.
-template <int MODE, int NST, int CPS, bool PDL>
+template <int MODE, int NST, int CPS>
 __global__ void __launch_bounds__(kSymThreads, CPS) k_stream_sym_half(const TileD *__restrict__ tiles, int nt,
                                                                        const float4 *__restrict__ tc,
                                                                        const float4 *__restrict__ fg,
@@ -2578,16 +2616,11 @@ __global__ void __launch_bounds__(kSymThreads, CPS) k_stream_sym_half(const Tile
 #pragma unroll
     for (int q = 0; q < 2; ++q) bulk_g2s(buf + q * (kHalfTileBytes / 2), src + q * (kHalfTileBytes / 2), kHalfTileBytes / 2, bars + s);
   };
-  if (tid == 0) {
+  if (tid == 0)
     for (; issued < kHalfStages && issued < nunit; ++issued) {
       issue(issued);
-      if (!PDL) issue_f(issued, iss);
+      issue_f(issued, iss);
     }
-    if (PDL) {
-      pdl_wait();  // f comes from the kernel before this one, which may still read the partials
-      for (int v = 0; v < issued; ++v) issue_f(v, stile[v]);
-    }
-  }
   int pcb = -1, pcs = 0;  // column slots of the previous unit's tile (-1: diagonal, or none)
   bool ok = true;
   float c[4][2], r0[2][2];  // column sums of the current tile; row sums of its first half
@@ -2607,7 +2640,6 @@ __global__ void __launch_bounds__(kSymThreads, CPS) k_stream_sym_half(const Tile
     // the previous tile's column table (written after its second half) is complete
     if ((u & 1) == 0 && u >= 2 && pcb >= 0) net_columns_out(colred, pcb, pcs, lane, wid, tp);
     if (!have) break;
-    if (PDL && u + 1 == nunit) pdl_trigger();
     const int s = u % kHalfStages, h = u & 1;
     const TileD D = stile[s];
     const bool diag = D.I == D.J;
@@ -2629,27 +2661,7 @@ __global__ void __launch_bounds__(kSymThreads, CPS) k_stream_sym_half(const Tile
       const int row = ti * 2 + i;
       const float4 fs = fr[row];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const float4 e = T[row * kTile + tj + 16 * j];
-        if (MODE == MODE_COLL) {
-          const float2 t = net_term(e, fs, fcol[j]);
-          if (j == 0) {
-            r[i][0] = t.x;
-            r[i][1] = t.y;
-          } else {
-            ff_add_lazy(r[i][0], r[i][1], t.x, t.y);
-          }
-          if (!diag) ff_add_lazy(c[j][0], c[j][1], -t.x, -t.y);
-        } else {
-          if (j == 0) ff_prod(r[i][0], r[i][1], make_float2(fcol[j].x, fcol[j].y), e.z, e.w);
-          else ff_mac_lazy(r[i][0], r[i][1], make_float2(fcol[j].x, fcol[j].y), e.z, e.w);
-          ff_mac_lazy(r[i][0], r[i][1], make_float2(fcol[j].x, fcol[j].y), -e.x, -e.y);
-          if (!diag) {
-            ff_mac_lazy(c[j][0], c[j][1], make_float2(fs.x, fs.y), e.x, e.y);
-            ff_mac_lazy(c[j][0], c[j][1], make_float2(fs.x, fs.y), -e.z, -e.w);
-          }
-        }
-      }
+      for (int j = 0; j < 4; ++j) net_entry<MODE>(T[row * kTile + tj + 16 * j], fs, fcol[j], diag, j == 0, r[i], c[j]);
     }
     if (h == 0) {
 #pragma unroll
@@ -2669,17 +2681,8 @@ __global__ void __launch_bounds__(kSymThreads, CPS) k_stream_sym_half(const Tile
       if ((tj & 3) == 0) tp[D.rb + ((m >> 1) * HR + ti * 2 + (m & 1)) * D.rs] = v[0];
     }
     if (!diag) {
-      // columns of the whole tile: lanes tj and tj + 16 share them (one level), then the warps
-      // (after the next unit's barrier)
-      const bool up = lane & 16;
-#pragma unroll
-      for (int jk = 0; jk < 2; ++jk) {
-        const int jo = jk + 2;  // kept / sent column slot
-        const float2 a = make_float2(c[jk][0], c[jk][1]), b = make_float2(c[jo][0], c[jo][1]);
-        const float2 send = up ? a : b, keep = up ? b : a;
-        colred[wid * kTile + tj + 16 * ((up ? 2 : 0) + jk)] =
-            ff_add(keep, make_float2(__shfl_xor_sync(0xFFFFFFFFu, send.x, 16), __shfl_xor_sync(0xFFFFFFFFu, send.y, 16)));
-      }
+      // columns of the whole tile: one shuffle level, then the warps (after the next unit's barrier)
+      net_columns_in(c, colred, lane, wid);
     }
   }
   if (!ok) {
@@ -2691,6 +2694,51 @@ __global__ void __launch_bounds__(kSymThreads, CPS) k_stream_sym_half(const Tile
       }
     }
   }
+}
+
+// The same sums for a small tile list (chain_pdl): one CTA per half-tile, all of them resident at once, so
+// neither ring nor loop.  Each thread loads its eight entries straight into registers before it waits
+// for the kernel before (only f comes from that one), so the coefficients' latency passes under the
+// epilogue.  The two halves of a tile leave their column sums in two slots.
+template <int MODE>
+__global__ void __launch_bounds__(kSymThreads, 3) k_stream_sym_unit(const TileD *__restrict__ tiles,
+                                                                     const float4 *__restrict__ tc, const float4 *fg,
+                                                                     float2 *__restrict__ tp) {
+  constexpr int HR = kTile / 2;
+  __shared__ float2 colred[kSymThreads / 32 * kTile];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, tj = tid & 15, ti = tid >> 4;
+  const int h = blockIdx.x & 1;
+  const TileD D = load_tile(tiles, blockIdx.x >> 1);
+  const float4 *__restrict__ T = tc + (size_t)blockIdx.x * (HR * kTile);
+  float4 e[2][4];
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) e[i][j] = T[(ti * 2 + i) * kTile + tj + 16 * j];
+  pdl_wait();  // the kernel before this one writes f, and may still read the partials
+  pdl_trigger();
+  float4 fs[2], fcol[4];
+#pragma unroll
+  for (int i = 0; i < 2; ++i) fs[i] = __ldcg(fg + (size_t)D.I * kTile + h * HR + ti * 2 + i);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) fcol[j] = __ldcg(fg + (size_t)D.J * kTile + tj + 16 * j);
+  const bool diag = D.I == D.J;
+  float r[2][2], c[4][2];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) c[j][0] = c[j][1] = 0.f;
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) net_entry<MODE>(e[i][j], fs[i], fcol[j], diag, j == 0, r[i], c[j]);
+  {
+    float2 v[2] = {make_float2(r[0][0], r[0][1]), make_float2(r[1][0], r[1][1])};
+    ff_reduce_scatter<2, 8>(v, lane);
+    if ((tj & 7) == 0) tp[D.rb + (h * HR + ti * 2 + (tj >> 3)) * D.rs] = v[0];
+  }
+  if (diag) return;
+  net_columns_in(c, colred, lane, wid);
+  __syncthreads();
+  net_columns_out(colred, D.cb + h, D.cs, lane, wid, tp);
 }
 
 // ------------------------------------------------------------ transport over tiles

@@ -126,3 +126,31 @@ def test_dense_mixed_sweep_skips_pairs_out_of_reach(pb, name):  # noqa: F811
     assert nrel(ft.cpu().numpy(), want) <= 1e-6 and nrel(fb.cpu().numpy()[o.nstate:], want) <= 1e-6
     g = [d.collision_vjp(T(f), T(lam), grad_g2=T(np.zeros(ch.nchannels))).cpu().numpy() for d in (dev, lanes)]
     assert np.abs(g[0] - g[1]).max() <= 1e-6 * np.abs(o.rates(f)).max() * np.abs(lam).max()
+
+
+@pytest.mark.parametrize("ctas", [0, 2])
+@pytest.mark.parametrize("n", [3, 4, 10, 11])
+def test_half_tile_sweep_of_small_and_larger_lists(pb, n, ctas):  # noqa: F811
+    """Whole triangles around the lines of the half-tile sweep: 27 and 64 states (one diagonal tile,
+    ragged and full), 1000 states (136 tiles: a CTA per half-tile, chained; twice that in the batch, which
+    takes the ring) and 1331 (231 tiles, the ring), against the oracle; the batch also with itself."""
+    m = synth.make_flat_einstein(n)
+    o = oracle.Oracle(m)
+    ch = pb.Channels.from_model(m)
+    dev = pb.Device(ch, dense_rows=3, ctas_per_sm=ctas)
+    rng = np.random.default_rng(59)
+    f = rng.uniform(0, 1, o.nstate)
+    ref, ab = o.collision(f, with_abs=True)
+    check_I(dev.collision(T(f)).cpu().numpy(), ref, ab)
+    assert nrel(dev.rates(T(f)).cpu().numpy(), o.rates(f)) <= TOL
+    ft = T(f)
+    dev.rk4(ft, 1.0, 3)
+    assert nrel(ft.cpu().numpy(), o.rk4(f, 1.0, 3)) <= TOL
+    dev.check()
+    b = pb.Batch([ch, ch], precision="ff", layout=2)
+    both = b.collision(T(np.concatenate([f, f]))).cpu().numpy()
+    assert np.array_equal(both[:o.nstate], both[o.nstate:])
+    check_I(both[:o.nstate], ref, ab)
+    fb = T(np.concatenate([f, f]))
+    b.rk4(fb, 1.0, 3)
+    assert nrel(fb.cpu().numpy()[o.nstate:], o.rk4(f, 1.0, 3)) <= TOL
