@@ -586,7 +586,7 @@ Layout make_layout(const pb_channels *ch, const Plan &P, const Plan *S, int vari
   L.gdorder = take(gd.on ? sizeof(int32_t) * gd.plan.items.size() : 0);
   L.gdwbeg = take(gd.on ? sizeof(int32_t) * ((size_t)gd.grid * (dev::kDenseThreads / 32) + 1) : 0);
   L.rp_real = take(sizeof(int64_t) * (ns + 1));
-  L.vjpG = take(sizeof(float2) * 3 * ns);
+  L.vjpG = take(sizeof(float2) * 3 * (tp ? std::max<size_t>((size_t)tp->nsp, ns) : ns));
   L.g2tab = take(sizeof(float4) * 2 * 4 * ns);
   L.vecs = take(sizeof(double) * 9 * ns);
   L.trptr = take(tr_nseg ? sizeof(int32_t) * (ns + 1) : 0);
@@ -826,7 +826,7 @@ struct pb_dev {
   cudaEvent_t hres_ev[2] = {nullptr, nullptr};
   float2 *tc32 = nullptr;
   int64_t *rp_real = nullptr;  // unpadded CSR row offsets [ns+1]
-  float2 *vjpG = nullptr;      // adjoint gather table [ns][3]
+  float2 *vjpG = nullptr;      // adjoint gather table [ns][3]; tiles: [nsp] (f, 1 - f), then [nsp] cotangents
   int tr_nseg = 0, tr_seglen = 0;  // row-block transport sweep: segments per row, partners per segment
   int32_t *trptr = nullptr;        // its partial ranges per row (r * tr_nseg) for the finaliser
   Part4 *trpart = nullptr;         // its (row, segment) partials [ns][tr_nseg]
@@ -1142,6 +1142,7 @@ void launch_half_tiles(bool chain, int cps, int sm_count, const dev::TileD *tile
   const float4 *fg = (const float4 *)fg_;
   float2 *tp = (float2 *)tp_;
   const int gs = (int)std::max<int64_t>(1, std::min<int64_t>(nt, (int64_t)sm_count * cps));
+  if (nt < 1) return;
   if (chain) launch_pdl(true, dev::k_stream_sym_unit<MODE>, 2 * nt, dev::kSymThreads, 0, st, tiles, tc, fg, tp);
   else if (cps == 3)
     dev::k_stream_sym_half<MODE, 2, 3><<<gs, dev::kSymThreads, dev::half_smem<2>(), st>>>(tiles, nt, tc, fg, tp, err, rev);
@@ -1543,8 +1544,9 @@ extern "C" int pb_dev_create(const pb_channels *ch, const pb_dev_opts *opts, voi
         // the tile sweeps read f in whole blocks: its padding must hold zeros (it multiplies zero
         // coefficients)
         e_ = cudaMemsetAsync(d->yff, 0, d->sym ? sizeof(float4) * (size_t)d->nsp : sizeof(float2) * (size_t)d->ns, st);
+        if (e_ == cudaSuccess && d->sym) e_ = cudaMemsetAsync(d->vjpG, 0, sizeof(float2) * 3 * (size_t)d->nsp, st);
         if (e_ != cudaSuccess) {
-          status = cuda_fail(e_, "clear the stage input");
+          status = cuda_fail(e_, "clear the stage inputs");
           break;
         }
       }
@@ -2680,6 +2682,11 @@ int vjp_launch_mixed(pb_dev *d, const double *f, const double *lam, double wl, c
   return PB_OK;
 }
 
+// whether the FF adjoint runs over the symmetric tiles (any tile_sweep), and its inputs there
+bool vjp_tiles(const pb_dev *d) { return d->sym && !d->c32; }
+float4 *vjp_fg(pb_dev *d) { return (float4 *)d->vjpG; }
+float2 *vjp_lam(pb_dev *d) { return d->vjpG + 2 * (size_t)d->nsp; }
+
 // FF adjoint in three launches per call: vjp_prep_ff (the cotangent g = wl lam + wm mprev,
 // mprev may be null, and its gather table; slot >= 0 also writes that stage of the
 // |g|^2-gradient table), vjp_sweep_ff (k_stream_vjp) and vjp_fin_ff (mu = J(f)^T g, out = mu
@@ -2687,6 +2694,12 @@ int vjp_launch_mixed(pb_dev *d, const double *f, const double *lam, double wl, c
 int vjp_prep_ff(pb_dev *d, const double *f, const double *lam, double wl, const double *mprev, double wm,
                  double *gbuf, int slot, cudaStream_t st) {
   const int ns = (int)d->ns;
+  if (vjp_tiles(d)) {
+    dev::k_vjp_prep_map<<<(ns + 255) / 256, 256, 0, st>>>(f, lam, wl, ns, d->pmap, vjp_fg(d), vjp_lam(d), -d->c,
+                                                          slot >= 0 ? d->g2tab + 2 * (size_t)slot * ns : nullptr);
+    PB_LAUNCHED("k_vjp_prep_map");
+    return PB_OK;
+  }
   dev::k_vjp_prep<<<(ns + 255) / 256, 256, 0, st>>>(f, lam, wl, mprev, wm, ns, gbuf, d->vjpG, -d->c,
                                                     slot >= 0 ? d->g2tab + 2 * (size_t)slot * ns : nullptr);
   PB_LAUNCHED("k_vjp_prep");
@@ -2694,6 +2707,16 @@ int vjp_prep_ff(pb_dev *d, const double *f, const double *lam, double wl, const 
 }
 
 int vjp_sweep_ff(pb_dev *d, cudaStream_t st) {
+  if (vjp_tiles(d)) {
+    float2 *tp = (float2 *)d->tpart;
+    if (d->tnt < 1) return PB_OK;
+    if (d->sym_half && d->chain())
+      launch_pdl(true, dev::k_vjp_tiles<1>, 2 * d->tnt, dev::kSymThreads, 0, st, d->tiles, d->tcoef, vjp_fg(d), vjp_lam(d), tp);
+    else
+      dev::k_vjp_tiles<2><<<d->tnt, dev::kSymThreads, 0, st>>>(d->tiles, d->tcoef, vjp_fg(d), vjp_lam(d), tp);
+    PB_LAUNCHED("k_vjp_tiles");
+    return PB_OK;
+  }
   const int ns = (int)d->ns, n = (int)d->nitems;
   const int grid = d->stream_grid(d->smem_G ? std::max(1, std::min(d->ctas, (int)((228 * 1024) / (d->smem_G + 1024)))) : d->ctas);
   const float4 *A4 = (const float4 *)d->coefA, *B4 = (const float4 *)d->coefB;
@@ -2711,6 +2734,15 @@ int vjp_sweep_ff(pb_dev *d, cudaStream_t st) {
 int vjp_fin_ff(pb_dev *d, const double *gbuf, double *mu, const double *acc_in, double *acc_out,
                 const dev::VjpNext &nx, cudaStream_t st) {
   const int ns = (int)d->ns;
+  if (vjp_tiles(d)) {
+    with_bool(ns <= 2048, [&](auto small) {
+      constexpr int SPC = small() ? 8 : 32;
+      launch_pdl(d->chain(), dev::k_fin_vjp_net<SPC>, (ns + SPC - 1) / SPC, 256, 0, st, (const float2 *)d->tpart, d->prow,
+                 d->pmap, ns, d->c, mu, acc_in, acc_out, nx, vjp_fg(d), vjp_lam(d), -d->c);
+    });
+    PB_LAUNCHED("k_fin_vjp_net");
+    return PB_OK;
+  }
   if (ns <= 2048)  // few states: more, smaller CTAs
     dev::k_fin_vjp<8><<<(ns + 7) / 8, 256, 0, st>>>(d->item_ptr, d->part, ns, d->c, d->R, gbuf, mu, acc_in, acc_out, nx,
                                                    d->vjpG, -d->c);

@@ -3009,6 +3009,153 @@ __device__ __forceinline__ void fin_stage(int r, double I, const FinIn &in, doub
     yff[ry < 0 ? r : ry] = ff_split(yn);
 }
 
+// ------------------------------------------------------------ adjoint over the symmetric tiles
+//
+// The transposed sum of the adjoint section above is, with g = 1 - f,
+//   (J^T lam)_s = c sum_p (lam_p - lam_s) a(s, p),   a(s, p) = g_p P_out(s, p) + f_p P_in(s, p),
+// (a = P_in + D - f_p D, and R_s - B_s = sum_p a) and the reverse entry gives the partner's term
+// (lam_s - lam_p) (g_s P_in + f_s P_out): one tile entry serves both states, with one float-float sum
+// each, as in the forward sweep, and only the tiles within reach are read, where the row sweep reads 18
+// bytes of every directed pair, takes four sums per state and subtracts lam_s (R - B) at the end.
+// About 64 operations per entry.  Eight entries per thread per half-tile are loaded straight into
+// registers.  NH halves per CTA: 1 where the plan has two column slots per tile (small lists), else 2,
+// with the column sums carried in registers.  Latency bound at 24^3 (four-band window, 1028 states,
+// 69 tiles in reach of 153): a 20-step trajectory's gradient 3.22 -> 2.49 ms, of which the row sweep
+// took 16 us of each of 80 calls.
+template <int NH>
+__global__ void __launch_bounds__(kSymThreads, 2) k_vjp_tiles(const TileD *__restrict__ tiles,
+                                                               const float4 *__restrict__ tc, const float4 *fg,
+                                                               const float2 *lam, float2 *__restrict__ tp) {
+  constexpr int HR = kTile / 2;
+  __shared__ float2 colred[kSymThreads / 32 * kTile];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, tj = tid & 15, ti = tid >> 4;
+  const int u0 = (int)blockIdx.x * NH;  // first half-tile
+  const TileD D = load_tile(tiles, u0 >> 1);
+  const bool diag = D.I == D.J;
+  float4 fcol[4];
+  float2 lcol[4];
+  float c[4][2];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) c[j][0] = c[j][1] = 0.f;
+#pragma unroll
+  for (int k = 0; k < NH; ++k) {
+    const int h = NH == 1 ? u0 & 1 : k;
+    const float4 *__restrict__ T = tc + (size_t)(u0 + k) * (HR * kTile);
+    float4 e[2][4];
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) e[i][j] = T[(ti * 2 + i) * kTile + tj + 16 * j];
+    if (k == 0) {
+      pdl_wait();  // the kernel before this one writes fg and lam, and may still read the partials
+      pdl_trigger();
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        fcol[j] = __ldcg(fg + (size_t)D.J * kTile + tj + 16 * j);
+        lcol[j] = __ldcg(lam + (size_t)D.J * kTile + tj + 16 * j);
+      }
+    }
+    float2 v[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const size_t row = (size_t)D.I * kTile + h * HR + ti * 2 + i;
+      const float4 fs = __ldcg(fg + row);
+      const float2 ls = __ldcg(lam + row);
+      float rh = 0.f, rl = 0.f;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        // w = lam_p - lam_s: the exact difference of the high parts and the low parts
+        const float wh = __fsub_rn(lcol[j].x, ls.x);
+        const float bb = __fsub_rn(wh, lcol[j].x);
+        const float er = __fsub_rn(__fsub_rn(lcol[j].x, __fsub_rn(wh, bb)), __fadd_rn(ls.x, bb));
+        const float2 w = make_float2(wh, __fadd_rn(er, __fsub_rn(lcol[j].y, ls.y)));
+        float ah, al;
+        ff_prod(ah, al, make_float2(fcol[j].x, fcol[j].y), e[i][j].x, e[i][j].y);
+        ff_mac_lazy(ah, al, make_float2(fcol[j].z, fcol[j].w), e[i][j].z, e[i][j].w);
+        if (j == 0) ff_prod(rh, rl, w, ah, al);
+        else ff_mac_lazy(rh, rl, w, ah, al);
+        if (!diag) {
+          ff_prod(ah, al, make_float2(fs.z, fs.w), e[i][j].x, e[i][j].y);
+          ff_mac_lazy(ah, al, make_float2(fs.x, fs.y), e[i][j].z, e[i][j].w);
+          ff_mac_lazy(c[j][0], c[j][1], w, -ah, -al);
+        }
+      }
+      v[i] = make_float2(rh, rl);
+    }
+    ff_reduce_scatter<2, 8>(v, lane);
+    if ((tj & 7) == 0) tp[D.rb + (h * HR + ti * 2 + (tj >> 3)) * D.rs] = v[0];
+  }
+  if (diag) return;
+  net_columns_in(c, colred, lane, wid);
+  __syncthreads();
+  net_columns_out(colred, D.cb + (NH == 1 ? u0 & 1 : 0), D.cs, lane, wid, tp);
+}
+
+// A state's inputs of the sweep above, in the tiles' order, and the stage table of the gradient
+__device__ __forceinline__ void vjp_prep_tile_at(int i, int row, double fi, double li, float4 *__restrict__ fg,
+                                                 float2 *__restrict__ lamff, double scale, float4 *__restrict__ tab) {
+  fg[row] = fg_of(fi);
+  lamff[row] = ff_split(li);
+  if (tab) {
+    const double gi = 1.0 - fi, sl = scale * li;
+    const float2 a = ff_split(sl * fi), b = ff_split(sl * gi), fs = ff_split(fi), gs = ff_split(gi);
+    tab[2 * i] = make_float4(a.x, a.y, b.x, b.y);
+    tab[2 * i + 1] = make_float4(fs.x, fs.y, gs.x, gs.y);
+  }
+}
+
+__global__ void k_vjp_prep_map(const double *__restrict__ f, const double *__restrict__ lam, double wl, int n,
+                               const int *__restrict__ pmap, float4 *__restrict__ fg, float2 *__restrict__ lamff,
+                               double scale, float4 *__restrict__ tab) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) vjp_prep_tile_at(i, pmap[i], f[i], wl * lam[i], fg, lamff, scale, tab);
+}
+
+// mu = J^T g from the partials of k_vjp_tiles; out, acc_in, acc_out and nx as in k_fin_vjp
+template <int SPC>
+__global__ void __launch_bounds__(256) k_fin_vjp_net(const float2 *tp, const int2 *__restrict__ prow,
+                                                     const int *__restrict__ pmap, int ns, double c, double *out,
+                                                     const double *acc_in, double *acc_out, VjpNext nx, float4 *fg,
+                                                     float2 *lamff, double scale) {
+  constexpr int SPW = SPC / 8, LPV = 32 / SPW;  // states per warp, lanes per state after the reduce-scatter
+  __shared__ float2 tot[SPC];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int base = blockIdx.x * SPC;
+  const int r0 = base + lane;
+  const bool fin = wid == 0 && lane < SPC && r0 < ns;
+  int2 pr[SPW];
+#pragma unroll
+  for (int q = 0; q < SPW; ++q) {
+    const int r = base + SPW * wid + q;
+    pr[q] = r < ns ? prow[r] : make_int2(0, 0);
+  }
+  const int row = fin ? pmap[r0] : 0;
+  pdl_wait();
+  double ai = 0.0, fn = 0.0, ln = 0.0;
+  if (fin) {
+    if (acc_out) ai = acc_in[r0];
+    if (nx.f) {
+      fn = nx.f[r0];
+      ln = nx.lam[r0];
+    }
+  }
+  float2 v[SPW];
+#pragma unroll
+  for (int q = 0; q < SPW; ++q) {
+    v[q] = make_float2(0.f, 0.f);
+    for (int k = lane; k < pr[q].y; k += 32) v[q] = ff_add(v[q], tp[pr[q].x + k]);
+  }
+  pdl_trigger();
+  ff_reduce_scatter<SPW, 16>(v, lane);
+  if ((lane & (LPV - 1)) == 0) tot[SPW * wid + lane / LPV] = v[0];
+  __syncthreads();
+  if (!fin) return;
+  const double mu = c * ff_to_double(tot[lane].x, tot[lane].y);
+  if (out) out[r0] = mu;
+  if (acc_out) acc_out[r0] = ai + mu;
+  if (nx.f) vjp_prep_tile_at(r0, row, fn, nx.wl * ln + nx.wm * mu, fg, lamff, scale, nx.tab);
+}
+
 template <bool LIT, int STAGE, int OUT>
 __device__ __forceinline__ void fin_apply(int r, double A, double B, double c, const FinIn &in,
                                           double *__restrict__ out, double *__restrict__ f, double *__restrict__ acc,

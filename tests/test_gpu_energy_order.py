@@ -154,3 +154,31 @@ def test_half_tile_sweep_of_small_and_larger_lists(pb, n, ctas):  # noqa: F811
     fb = T(np.concatenate([f, f]))
     b.rk4(fb, 1.0, 3)
     assert nrel(fb.cpu().numpy()[o.nstate:], o.rk4(f, 1.0, 3)) <= TOL
+
+
+@pytest.mark.parametrize("opts", [{}, dict(tile_sweep=1)])
+@pytest.mark.parametrize("name", list(CASES) + ["ring"])
+def test_adjoint_over_tiles(pb, name, opts):  # noqa: F811
+    """The FF adjoint over the tiles (a CTA per half-tile; "ring", 231 tiles, and tile_sweep 1 a CTA per
+    tile) against the oracle and, for the |g|^2 gradient, the row form, which takes the same table."""
+    m = synth.make_flat_einstein(11) if name == "ring" else CASES[name][0]()
+    o = oracle.Oracle(m)
+    ch = pb.Channels.from_model(m)
+    dev, rows = pb.Device(ch, dense_rows=3, **opts), pb.Device(ch, dense_rows=2)
+    rng = np.random.default_rng(61)
+    f, lam = rng.uniform(0, 1, o.nstate), rng.normal(size=o.nstate)
+    gg = [T(np.zeros(ch.nchannels)) for _ in range(2)]
+    got, ref = [d.collision_vjp(T(f), T(lam), grad_g2=q).cpu().numpy() for d, q in zip((dev, rows), gg)]
+    assert nrel(got, o.collision_vjp(f, lam)) <= 1e-11
+    assert nrel(got, ref) <= 1e-11
+    assert np.array_equal(gg[0].cpu().numpy(), gg[1].cpu().numpy())
+    f0 = o.window_values(m.f_hot())
+    l1 = T(lam)
+    for _ in range(2):  # twice: the replayed sequence too
+        l1.copy_(T(lam))
+        dev.rk4_vjp(T(f0), l1, 1.0)
+        assert nrel(l1.cpu().numpy(), o.rk4_vjp(f0, 1.0, 1, lam)) <= 1e-11
+    # after set_g2 the rows replace the tiles
+    dev.set_g2(T(ch.export()["g2"]))
+    assert nrel(dev.collision_vjp(T(f), T(lam)).cpu().numpy(), got) <= 1e-11
+    dev.check()
