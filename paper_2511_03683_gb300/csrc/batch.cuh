@@ -780,12 +780,16 @@ int batch_fin(pb_batch *b, double *out, double *f, double dt, cudaStream_t st, c
     // outputs, their padded rows the partials and the next stage's float-float input
     const int ns = (int)b->ns;
     with_bool(chain_pdl(b->tnt, b->sm_count), [&](auto pdl) {
-      if (b->prec == 2)
-        launch_pdl(pdl(), dev::k_fin_net<float, STAGE, false, 32, pdl()>, (ns + 31) / 32, 256, 0, st, (const float *)b->tp,
-                   b->prow, b->pmap, ns, 1.0, nullptr, out, f, b->acc, b->y, b->yff, dt);
-      else
-        launch_pdl(pdl(), dev::k_fin_net<float2, STAGE, false, 32, pdl()>, (ns + 31) / 32, 256, 0, st,
-                   (const float2 *)b->tp, b->prow, b->pmap, ns, 1.0, nullptr, out, f, b->acc, b->y, b->yff, dt);
+      with_bool(fin_small(ns, b->sm_count), [&](auto small) {
+        constexpr int SPC = small() ? 8 : 32;
+        const int grid = (ns + SPC - 1) / SPC;
+        if (b->prec == 2)
+          launch_pdl(pdl(), dev::k_fin_net<float, STAGE, false, SPC, pdl()>, grid, 256, 0, st, (const float *)b->tp,
+                     b->prow, b->pmap, ns, 1.0, nullptr, out, f, b->acc, b->y, b->yff, dt);
+        else
+          launch_pdl(pdl(), dev::k_fin_net<float2, STAGE, false, SPC, pdl()>, grid, 256, 0, st, (const float2 *)b->tp,
+                     b->prow, b->pmap, ns, 1.0, nullptr, out, f, b->acc, b->y, b->yff, dt);
+      });
     });
     PB_LAUNCHED("tile epilogue (batch)");
     return PB_OK;

@@ -640,6 +640,11 @@ int cuda_fail(cudaError_t e, const char *what) {
 // runs slow it down).
 bool chain_pdl(int64_t tiles, int sm_count) { return 2 * tiles <= 3 * (int64_t)sm_count; }
 
+// The tile epilogues, single systems' and batches': 8 states per CTA unless 32 per CTA still give four
+// CTAs per SM (with 32 per CTA a 40^3 step had 149 CTAs for 152 SMs, and the C32 RK4 step ran 14%
+// slower; the sums do not depend on it).
+bool fin_small(int64_t ns, int sm_count) { return (ns + 31) / 32 < 4 * (int64_t)sm_count; }
+
 // kernel<<<grid, block, smem, st>>>(args...), with pdl as a programmatic dependent of the kernel
 // before it in the stream (kernels.cuh, pdl_trigger); only for kernels that wait for it themselves.
 // Errors are left to cudaGetLastError, as with the launch syntax.
@@ -1976,14 +1981,10 @@ int launch_stream(pb_dev *d, int mode, const double *fd, const float2 *fff, cuda
 
 int fin_grid(const pb_dev *d) { return d->nfin_blocks; }
 
-// the tile epilogues: 8 states per CTA unless 32 per CTA still give four CTAs per SM (with 32
-// per CTA a 40^3 step had 149 CTAs for 152 SMs, and the C32 RK4 step ran 14% slower)
-bool fin_small(const pb_dev *d) { return (d->ns + 31) / 32 < 4 * (int64_t)d->sm_count; }
-
 template <int STAGE, bool RATE>
 void launch_fin_tiles(pb_dev *d, const double *ysrc, double *out, double *f, double *y, double dt, cudaStream_t st) {
   with_bool(d->chain(), [&](auto pdl) {
-    with_bool(fin_small(d), [&](auto small) {
+    with_bool(fin_small(d->ns, d->sm_count), [&](auto small) {
       constexpr int SPC = small() ? 8 : 32;
       const int grid = (int)((d->ns + SPC - 1) / SPC);
       if (d->c32)
@@ -2735,7 +2736,7 @@ int vjp_fin_ff(pb_dev *d, const double *gbuf, double *mu, const double *acc_in, 
                 const dev::VjpNext &nx, cudaStream_t st) {
   const int ns = (int)d->ns;
   if (vjp_tiles(d)) {
-    with_bool(ns <= 2048, [&](auto small) {
+    with_bool(fin_small(ns, d->sm_count), [&](auto small) {
       constexpr int SPC = small() ? 8 : 32;
       launch_pdl(d->chain(), dev::k_fin_vjp_net<SPC>, (ns + SPC - 1) / SPC, 256, 0, st, (const float2 *)d->tpart, d->prow,
                  d->pmap, ns, d->c, mu, acc_in, acc_out, nx, vjp_fg(d), vjp_lam(d), -d->c);
