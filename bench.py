@@ -165,7 +165,8 @@ def function_source(text: str, name: str) -> str:
 HOT_FUNCTIONS = ("ff_split", "ff_to_double", "ff_mac", "ff_mac_lazy", "ff_add", "warp_sum", "partners4", "group_f",
                  "k_stream_ff", "k_stream_sym", "ff_prod", "ff_reduce_scatter",
                  "sym_columns_out", "mbar_init", "mbar_expect_tx", "mbar_try_wait", "mbar_wait", "bulk_g2s",
-                 "fence_proxy_async", "k_stream_sym_bulk", "half_smem", "k_stream_sym_half")
+                 "fence_proxy_async", "k_stream_sym_bulk", "half_smem", "load_tile", "ff_add_lazy", "net_term",
+                 "net_entry", "net_columns_in", "net_columns_out", "k_stream_sym_half", "k_stream_sym_unit")
 
 
 # the FP32 coefficient-tile sweep (tiles32.cuh) and the helpers of kernels.cuh it inlines
@@ -201,6 +202,19 @@ def ncu_traffic(workload: str, variant: str, bytes_per_launch: float):
         return float(e["dram_bytes_per_launch"])
     except (OSError, KeyError, ValueError):
         return None
+
+
+def l2_note(args, sweep_bytes: float, ns: int) -> str:
+    """What the timed steps find in the 129 MB L2."""
+    if args.workload != "window40":
+        return "inputs fit in L2 (latency/parity workload)"
+    if sweep_bytes > 129e6:
+        return f"inputs larger than L2 ({sweep_bytes / 1e9:.2f} GB streamed per sweep vs 0.13 GB L2)"
+    note = f"no flush between steps; {sweep_bytes / 1e9:.3f} GB streamed per collision sweep, which a step's sweeps share"
+    if args.variant == "ff" and args.transport_gather in (0, 4):  # both weights of a tile's pairs, 8 bytes each
+        weights = (2 * sweep_bytes / 65536 - (ns + 63) // 64) * 32768
+        note = f"a step's inputs ({(sweep_bytes + weights) / 1e9:.4f} GB of tiles and transport weights) larger than the 0.129 GB L2; " + note
+    return note
 
 
 def max_over_ranks(x: float, ws: int, device=None) -> float:
@@ -741,7 +755,7 @@ def run_ours(args):
         torch.cuda.synchronize()
         rates_ms = statistics.mean(a.elapsed_time(b) for a, b in evs[:10])
     # the sweep kernel alone: CUDA events on this stream around back-to-back launches of it
-    # (its 0.19 GB exceed the L2), and one launch at a time with L2 flushed before each
+    # (FF: the 67 MB of tiles stay in the L2), and one launch at a time with L2 flushed before each
     sweep_ms = dev.time_sweep(f, 50, stream=stream)
     sweep_ms_fl = sweep_ms_flushed(dev, f, 30, stream)
     # back-to-back launches alternating the tile order, as the RK4 stages run them (each sweep
@@ -814,9 +828,7 @@ def run_ours(args):
         cfg = workload_config(args.workload)
         cfg.update({"nstate": ns, "channels": nch, "variant": args.variant, "tile_sweep": args.tile_sweep,
                     "ctas_per_sm": args.ctas_per_sm, "transport_gather": args.transport_gather,
-                    "l2": "inputs larger than L2 "
-                    f"({dev.bytes_per_channel * nch / 1e9:.2f} GB streamed per sweep vs 0.13 GB L2)"
-                    if args.workload == "window40" else "inputs fit in L2 (latency/parity workload)",
+                    "l2": l2_note(args, bytes_launch, ns),
                     "parallelism": f"{ws} independent replica(s)"})
         emit({
             "metric": "e-ph channels/s", "value": value, "unit": "channels/s", "n_gpus": ws, "steps": args.steps,

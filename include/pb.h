@@ -209,10 +209,11 @@ typedef struct pb_dev_opts {
                                 rows' bytes; else 2); 1 (complete rows only) the collision, rate and
                                 transport sweeps take each entry's partner from its position and stream no
                                 index (16 instead of 18 bytes per entry); 3 as 1 where the rows are complete,
-                                and the collision and rate sweeps stream the upper block triangle of the pair
-                                matrix as 64 x 64 tiles of (P_in, P_out), zero where a pair has no channel,
-                                adding each tile to its rows and, through the reverse channels (P_in(p,s) =
-                                P_out(s,p)), to its columns: about 8 bytes per state pair (only for a list
+                                and the collision, rate, transport and adjoint sweeps stream the pair matrix as
+                                64 x 64 tiles of (P_in, P_out), zero where a pair has no channel: the states in
+                                energy order, of the upper block triangle only the tiles within reach of a
+                                phonon (C32: state order, the whole triangle), each added to its rows and, through
+                                the reverse channels (P_in(p,s) = P_out(s,p)), to its columns (only for a list
                                 built with check_closure, which guarantees those reverse channels; 1 or 2
                                 otherwise); 2 always stream the index */
   int32_t tile_sweep;        /* the symmetric tile sweep (dense_rows 3): 0 automatic (= 3); 1 each thread
@@ -222,7 +223,8 @@ typedef struct pb_dev_opts {
                                 its bounded waits reporting through pb_dev_check; 3 the same ring in
                                 half-tiles (32 x 64 entries, 32 KB), the column sums of a tile carried in
                                 registers across its two halves: two stages per CTA and three CTAs per SM
-                                (ctas_per_sm 2: three stages, two CTAs).  PB_VARIANT_C32: 0 or 2 its
+                                (ctas_per_sm 2: three stages, two CTAs), or one CTA per
+                                half-tile and no ring for at most 1.5 tiles per SM.  PB_VARIANT_C32: 0 or 2 its
                                 default launch shape (two stages, three CTAs per SM), 3..6 other shapes
                                 (3 x 2, 2 x 2, 4 x 1, 6 x 1 stages x CTAs), 7 and 8 half-tiles
                                 (3 x 4, 4 x 3) */
@@ -430,9 +432,9 @@ typedef struct pb_batch_opts {
                              precision 1 and 2: 0 automatic (symmetric tiles when every instance's list
                              was built with check_closure and the tiles stream at most 0.7 of the rows'
                              bytes: each instance's states in 64-state blocks of one padded state space,
-                             the upper block triangle of each instance stored as 64 x 64 tiles, one
-                             unordered state pair per entry for both directions, zero where a pair has
-                             no channel); 1 rows (one entry per directed state pair); 2 symmetric tiles
+                             the upper block triangle of each instance (precision 1: the tiles within reach)
+                             stored as 64 x 64 tiles, one unordered state pair per entry for both
+                             directions, zero where a pair has no channel); 1 rows (one entry per directed state pair); 2 symmetric tiles
                              whatever their bytes (PB_EINVAL for a list built without check_closure) */
 } pb_batch_opts;
 

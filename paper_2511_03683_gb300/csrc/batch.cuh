@@ -23,7 +23,8 @@
 //
 // Symmetric tiles (precision 1 and 2, every instance's channel list verified closed under
 // reversal): each instance takes a run of 64-state blocks of one padded state space, its states in
-// energy order (precision 2: in state order, all tiles of the triangle), and the tiles of its upper block triangle within reach of a phonon are stored as
+// energy order (precision 2: in state order, all tiles of the triangle), and the tiles of its upper
+// block triangle within reach of a phonon are stored as
 // 64 x 64 tiles (zero where a state pair has no channel), as in the single-system sweeps, so each
 // unordered state pair is streamed once for both of its directions and the pairs whose coefficients
 // are zero by their distance in energy are not streamed at all.  One launch of the single-system

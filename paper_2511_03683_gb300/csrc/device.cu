@@ -633,11 +633,11 @@ int cuda_fail(cudaError_t e, const char *what) {
     if (e_ != cudaSuccess) return cuda_fail(e_, #call);         \
   } while (0)
 
-// Which tile sweeps and epilogues form such chains: those of at most three tiles per two SMs, where a
-// stage is little more than the two launches (four-band window, us per RK4 step: 16^3 22.4 against
-// 25.2 as ordinary launches, 24^3 22.7 against 25.4, 30^3 28.0 against 30.6; at 32^3, 296 tiles, 31.4
-// against 31.0, and at 40^3, 1017 tiles, 64.0 against 59.3: sweep CTAs that come in while the epilogue
-// runs slow it down).
+// Which tile sweeps and epilogues form such chains: those of at most three tiles per two SMs (then all
+// half-tiles are resident at once, k_stream_sym_unit), where a stage is little more than the two
+// launches (four-band window, us per RK4 step: 16^3 17.0 against 25.2 with the ring and ordinary
+// launches, 24^3 18.5 against 25.4, 30^3 24.9 against 30.7; at 32^3, 296 tiles, 31.2 against 31.1, and at
+// 40^3, 1017 tiles, 61.9 against 59.7: sweep CTAs that come in while the epilogue runs slow it down).
 bool chain_pdl(int64_t tiles, int sm_count) { return 2 * tiles <= 3 * (int64_t)sm_count; }
 
 // The tile epilogues, single systems' and batches': 8 states per CTA unless 32 per CTA still give four
@@ -949,8 +949,8 @@ int resolve_opts(const pb_channels *ch, const pb_dev_opts *opts, int sm_count, p
   if (d.tile_sweep < 0 || d.tile_sweep > 8 || (d.tile_sweep > 3 && d.variant != PB_VARIANT_C32))
     return set_error(PB_EINVAL, "pb_dev: tile_sweep must be 0..3 (0..8 for the FP32 coefficient tiles)");
   if (d.adjoint < 0 || d.adjoint > 1) return set_error(PB_EINVAL, "pb_dev: adjoint must be 0 or 1");
-  // automatic: the half-tile ring (measured 38.8 us per 40^3 sweep against 42.6 us for whole tiles);
-  // for C32 its own default shape
+  // automatic: the half-tile ring (with A and C sums over the whole 40^3 triangle, 38.8 us per sweep
+  // against 42.6 us for whole tiles); for C32 its own default shape
   if (d.tile_sweep == 0) d.tile_sweep = d.variant == PB_VARIANT_C32 ? 2 : 3;
   if (d.variant == PB_VARIANT_C32 && (d.tile_sweep == 1 || d.stream_mode == 2 || d.merge_branches == 2 ||
                                       d.dense_rows == 1 || d.dense_rows == 2))
