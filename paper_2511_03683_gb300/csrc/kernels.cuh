@@ -183,6 +183,11 @@ __global__ void k_table(const double *__restrict__ omega, long long n, double kT
 // completion of the one before it, which has waited for its own predecessor.  Only constants of the
 // handle (tables, coefficients) are read before the wait.  Kernels have both forms (template PDL):
 // the instructions cost a large sweep more than the early start gains (chain_pdl on the host).
+// A buffer that an earlier kernel of the chain writes is not read-only for the lifetime of a kernel
+// that starts under it, so in these kernels it is not a `const ... __restrict__` parameter (the
+// compiler could take the non-coherent path for it, or move its loads above the wait) and is loaded
+// after the wait, the sweep's inputs and partials with __ldcg; __restrict__ const is left to the
+// handle's constants.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -3146,7 +3151,7 @@ __global__ void __launch_bounds__(256) k_fin_vjp_net(const float2 *tp, const int
 #pragma unroll
   for (int q = 0; q < SPW; ++q) {
     v[q] = make_float2(0.f, 0.f);
-    for (int k = lane; k < pr[q].y; k += 32) v[q] = ff_add(v[q], tp[pr[q].x + k]);
+    for (int k = lane; k < pr[q].y; k += 32) v[q] = ff_add(v[q], __ldcg(tp + pr[q].x + k));
   }
   pdl_trigger();
   ff_reduce_scatter<SPW, 16>(v, lane);

@@ -158,7 +158,7 @@ __device__ __forceinline__ void c32_columns_out(const float *__restrict__ colred
 template <int MODE, int NST, int CPS, bool PDL>
 __global__ void __launch_bounds__(kC32Threads, CPS) k_stream_c32(const TileD *__restrict__ tiles, int nt,
                                                                   const float2 *__restrict__ tc,
-                                                                  const float2 *__restrict__ fg,
+                                                                  const float2 *fg,
                                                                   float *__restrict__ tp, int *__restrict__ err,
                                                                   int rev = 0) {
   // the stage of tile k - 1 is refilled (with tile k - 1 + NST) only after the wait for tile k, so
@@ -306,7 +306,7 @@ constexpr size_t c32_half_smem() {
 template <int MODE, int NST, int CPS, bool PDL>
 __global__ void __launch_bounds__(kC32Threads, CPS) k_stream_c32_half(const TileD *__restrict__ tiles, int nt,
                                                                        const float2 *__restrict__ tc,
-                                                                       const float2 *__restrict__ fg,
+                                                                       const float2 *fg,
                                                                        float *__restrict__ tp, int *__restrict__ err,
                                                                        int rev = 0) {
   static_assert(NST >= 2 && NST <= 8, "the ring needs 2..8 stages");
@@ -514,11 +514,10 @@ __global__ void k_pairs_c32(const float2 *__restrict__ A, const float2 *__restri
 __device__ __forceinline__ float2 as_ff(float v) { return make_float2(v, 0.f); }
 __device__ __forceinline__ float2 as_ff(float2 v) { return v; }
 template <typename PT, int STAGE, bool RATE, int SPC, bool PDL>
-__global__ void __launch_bounds__(256) k_fin_net(const PT *__restrict__ tp, const int2 *__restrict__ prow,
+__global__ void __launch_bounds__(256) k_fin_net(const PT *tp, const int2 *__restrict__ prow,
                                                  const int *__restrict__ pmap, int ns, double c,
-                                                 const double *__restrict__ R, double *__restrict__ out,
-                                                 double *__restrict__ f, double *__restrict__ acc,
-                                                 double *__restrict__ y, float2 *__restrict__ yff, double dt) {
+                                                 const double *__restrict__ R, double *out, double *f, double *acc,
+                                                 double *y, float2 *yff, double dt) {
   constexpr int SPW = SPC / 8, LPV = 32 / SPW;  // states per warp, lanes per state after the reduce-scatter
   __shared__ float2 tot[SPC];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -550,7 +549,7 @@ __global__ void __launch_bounds__(256) k_fin_net(const PT *__restrict__ tp, cons
 #pragma unroll
   for (int q = 0; q < SPW; ++q) {
     v[q] = make_float2(0.f, 0.f);
-    for (int k = lane; k < pr[q].y; k += 32) v[q] = ff_add(v[q], as_ff(tp[pr[q].x + k]));
+    for (int k = lane; k < pr[q].y; k += 32) v[q] = ff_add(v[q], as_ff(__ldcg(tp + pr[q].x + k)));
   }
   if (PDL) pdl_trigger();
   ff_reduce_scatter<SPW, 16>(v, lane);
