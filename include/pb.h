@@ -316,7 +316,8 @@ int pb_rtbte_rk4_host(pb_dev *dev, const double *f_host_in, double *f_host_out, 
  * from F^0 = tau v until max|F^{i+1}-F^i| <= tol * max|F^{i+1}|.
  * f0: device double[nstate]; vel3, F3: device double[nstate][3].  On return (stream
  * synchronised) *iters holds the iterations done and *resid the last relative change;
- * PB_ENOCONV if maxit was reached first (F3 then holds the last iterate).  Each pass is
+ * PB_ENOCONV if maxit was reached first or an iterate holds a number that is not finite (F3 then
+ * holds the last iterate, and in the second case *resid is infinite).  Each pass is
  * replayed from a CUDA graph, and the next pass is queued before the host reads the previous
  * pass's residual (one extra pass runs after the converged one; it changes neither F3 nor the
  * result); the residual's block maxima go through a few KB (32 bytes per 32 states) of
@@ -333,7 +334,8 @@ int pb_transport_setup(pb_dev *dev, const double *f0, void *stream);
 /* One pass of the transport map with the weights of the last pb_transport_setup:
  * F3out = tau (v + W F3in), all device double[nstate][3], without any host
  * synchronisation.  If resid3 (device double[3]) is not NULL it receives
- * (max|F3out-F3in| / max|F3out|, max|F3out-F3in|, max|F3out|).  The pass's four launches are
+ * (max|F3out-F3in| / max|F3out|, max|F3out-F3in|, max|F3out|), not finite where a number of
+ * either iterate is not.  The pass's four launches are
  * replayed from a CUDA graph kept per set of pointers, as for pb_collision (an iteration that
  * alternates between two buffers replays two graphs). */
 int pb_transport_iterate(pb_dev *dev, const double *vel3, const double *F3in, double *F3out, double *resid3,

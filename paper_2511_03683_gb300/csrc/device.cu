@@ -2542,11 +2542,14 @@ extern "C" int pb_iter_transport(pb_dev *d, const double *f0, const double *vel3
     if (it + 1 < maxit && (rc = enqueue(it + 1))) return rc;
     PB_CUDA(cudaEventSynchronize(d->hres_ev[it & 1]));
     double dm = 0.0, fm = 0.0;
+    bool finite = true;  // (the maxima are NaN or infinite as soon as one number is: max_abs)
     for (int k = 0; k < nred; ++k) {
-      dm = std::fmax(dm, hres[it & 1][k].x);
-      fm = std::fmax(fm, hres[it & 1][k].y);
+      const double2 m = hres[it & 1][k];
+      finite = finite && std::isfinite(m.x) && std::isfinite(m.y);
+      dm = std::max(dm, m.x);
+      fm = std::max(fm, m.y);
     }
-    res = fm > 0.0 ? dm / fm : 0.0;
+    res = !finite ? INFINITY : fm > 0.0 ? dm / fm : 0.0;
     ++it;
     if (!std::isfinite(res)) break;
     if (res <= tol) break;

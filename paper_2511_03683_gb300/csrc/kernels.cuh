@@ -3272,16 +3272,25 @@ __global__ void k_fin_rate(SRC src, int ns, double c, const double *__restrict__
   out[r] = LIT ? c * A : c * (Rr - B);
 }
 
-// F_new = tau (v + sum W F); ff copy for the next pass; per-block max |dF| and max |F|.
-// max over the block of (a, b), both non-negative: warp shuffles, then one step through shared
+// Maxima of non-negative numbers are those of their bit patterns (integer instructions), and with
+// the sign cleared a NaN's pattern lies above infinity's: a NaN anywhere is the maximum, where fmax
+// would drop it and a solve whose iterate is NaN would look converged.
+__device__ __forceinline__ unsigned long long abs_bits(double v) {
+  return (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull;
+}
+__device__ __forceinline__ double max_abs(double a, double b) {
+  return __longlong_as_double((long long)max(abs_bits(a), abs_bits(b)));
+}
+
+// max |.| over the block of a and of b: warp shuffles, then one step through shared
 // memory (exact, so the order does not matter); the result is valid in thread 0
 __device__ __forceinline__ double2 block_max2(double a, double b) {
   __shared__ double2 wm[32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-    a = fmax(a, __shfl_xor_sync(0xFFFFFFFFu, a, o));
-    b = fmax(b, __shfl_xor_sync(0xFFFFFFFFu, b, o));
+    a = max_abs(a, __shfl_xor_sync(0xFFFFFFFFu, a, o));
+    b = max_abs(b, __shfl_xor_sync(0xFFFFFFFFu, b, o));
   }
   if (lane == 0) wm[wid] = make_double2(a, b);
   __syncthreads();
@@ -3290,12 +3299,14 @@ __device__ __forceinline__ double2 block_max2(double a, double b) {
     v = lane < (int)((blockDim.x + 31) >> 5) ? wm[lane] : make_double2(0.0, 0.0);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-      v.x = fmax(v.x, __shfl_xor_sync(0xFFFFFFFFu, v.x, o));
-      v.y = fmax(v.y, __shfl_xor_sync(0xFFFFFFFFu, v.y, o));
+      v.x = max_abs(v.x, __shfl_xor_sync(0xFFFFFFFFu, v.x, o));
+      v.y = max_abs(v.y, __shfl_xor_sync(0xFFFFFFFFu, v.y, o));
     }
   }
   return v;
 }
+
+// F_new = tau (v + sum W F); ff copy for the next pass; per-block max |dF| and max |F|.
 
 __global__ void __launch_bounds__(256) k_fin_tr(const int *__restrict__ item_ptr, const Part4 *__restrict__ part,
                                                 int ns, const double *__restrict__ tau,
@@ -3325,8 +3336,8 @@ __global__ void __launch_bounds__(256) k_fin_tr(const int *__restrict__ item_ptr
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       const double Fn = t * (vv[a] + S[a]);
-      if (Fold) dm = fmax(dm, fabs(Fn - fo[a]));
-      fm = fmax(fm, fabs(Fn));
+      if (Fold) dm = max_abs(dm, Fn - fo[a]);
+      fm = max_abs(fm, Fn);
       Fnew[3 * r + a] = Fn;
       Fff[3 * r + a] = ff_split(Fn);
     }
@@ -3366,13 +3377,12 @@ __global__ void __launch_bounds__(3 * kFinTrStates) k_fin_tr_tiles(const int2 *_
   double dm = 0.0, fm = 0.0;
   if (r >= 0) {
     const double Fn = t * (v + c * ff_to_double(S.x, S.y));
-    dm = fmax(0.0, fabs(Fn - fo));
-    fm = fmax(0.0, fabs(Fn));
+    dm = Fn - fo;
+    fm = Fn;
     Fnew[3 * r + a] = Fn;
     Fff[trF_at(pos, a)] = ff_split(Fn);
   }
-  // the maxima of non-negative numbers are those of their bit patterns (integer instructions)
-  unsigned long long du = (unsigned long long)__double_as_longlong(dm), fu = (unsigned long long)__double_as_longlong(fm);
+  unsigned long long du = abs_bits(dm), fu = abs_bits(fm);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     du = max(du, __shfl_xor_sync(0xFFFFFFFFu, du, o));
@@ -3381,18 +3391,18 @@ __global__ void __launch_bounds__(3 * kFinTrStates) k_fin_tr_tiles(const int2 *_
   if (lane == 0) wm[a] = make_double2(__longlong_as_double((long long)du), __longlong_as_double((long long)fu));
   __syncthreads();
   if (threadIdx.x == 0)
-    red[blockIdx.x] = make_double2(fmax(wm[0].x, fmax(wm[1].x, wm[2].x)), fmax(wm[0].y, fmax(wm[1].y, wm[2].y)));
+    red[blockIdx.x] = make_double2(max_abs(wm[0].x, max_abs(wm[1].x, wm[2].x)), max_abs(wm[0].y, max_abs(wm[1].y, wm[2].y)));
 }
 
 __global__ void k_red_final(const double2 *__restrict__ red, int n, double *__restrict__ out) {
   double d = 0.0, m = 0.0;
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    d = fmax(d, red[i].x);
-    m = fmax(m, red[i].y);
+    d = max_abs(d, red[i].x);
+    m = max_abs(m, red[i].y);
   }
   const double2 v = block_max2(d, m);
   if (threadIdx.x == 0) {
-    out[0] = v.y > 0.0 ? v.x / v.y : 0.0;
+    out[0] = v.y == 0.0 && isfinite(v.x) ? 0.0 : v.x / v.y;  // not finite: NaN or infinite
     out[1] = v.x;
     out[2] = v.y;
   }
