@@ -2133,17 +2133,18 @@ int ensure_weights(pb_dev *d, const double *f0, cudaStream_t st) {
     d->wt_tiles = tiles;
   }
   if (tiles) {
-    // 1/tau at f0 is the scattering rate there; then the weight tiles
+    // the scattering rate at f0, the weight tiles with their sums (in the rate sweep's partials, which
+    // are spent), and 1/tau from the one or the other
     int rc = rates_seq(d, f0, d->invtau, st);
     if (rc) return rc;
-    const int g = (int)((d->ns + 255) / 256);
-    dev::k_recip<<<g, 256, 0, st>>>(d->invtau, (int)d->ns, d->tau);
-    PB_LAUNCHED("k_recip");
-    dev::k_f0_map<<<g, 256, 0, st>>>(f0, (int)d->ns, d->pmap, d->trf0);
+    dev::k_f0_map<<<(int)((d->ns + 255) / 256), 256, 0, st>>>(f0, (int)d->ns, d->pmap, d->trf0);
     PB_LAUNCHED("k_f0_map");
-    dev::k_weight_tiles<<<(int)std::min<int64_t>(d->tnt, (int64_t)d->sm_count * 6), 256, 0, st>>>(
-        d->tiles, d->tnt, d->tcoef, d->trf0, d->wt);
+    dev::k_weight_tiles<<<(int)std::min<int64_t>(d->tnt, (int64_t)d->sm_count * 5), 256, 0, st>>>(
+        d->tiles, d->tnt, d->tcoef, d->trf0, d->sym_half && d->chain() ? 2 : 1, d->wt, (double *)d->tpart);
     PB_LAUNCHED("k_weight_tiles");
+    dev::k_tau_tiles<<<(int)((d->ns + 7) / 8), 256, 0, st>>>((const double *)d->tpart, d->prow, d->R, (int)d->ns, d->c,
+                                                             d->invtau, d->tau);
+    PB_LAUNCHED("k_tau_tiles");
     return PB_OK;
   }
   const int grid = d->stream_grid(8);

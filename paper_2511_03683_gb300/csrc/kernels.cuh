@@ -2768,37 +2768,132 @@ __global__ void k_f0_map(const double *__restrict__ f, int n, const int *__restr
   }
 }
 
+// A float-float sum with what its two words drop in a third: the weights' row sums below lose nothing to
+// the additions.
+struct FF3 {
+  float h, l, e;
+};
+__device__ __forceinline__ void two_sum(float a, float b, float &s, float &err) {
+  s = __fadd_rn(a, b);
+  const float bb = __fsub_rn(s, a);
+  err = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+}
+__device__ __forceinline__ void ff3_add(FF3 &t, float h, float l) {
+  float e1, e2, e3;
+  two_sum(t.h, h, t.h, e1);
+  two_sum(t.l, l, t.l, e2);
+  two_sum(t.l, e1, t.l, e3);
+  t.e = __fadd_rn(t.e, __fadd_rn(e2, e3));
+}
+__device__ __forceinline__ void ff3_add(FF3 &t, const FF3 &v) {
+  ff3_add(t, v.h, v.l);
+  t.e = __fadd_rn(t.e, v.e);
+}
+__device__ __forceinline__ FF3 ff3_shfl_xor(const FF3 &v, int mask) {
+  return FF3{__shfl_xor_sync(0xFFFFFFFFu, v.h, mask), __shfl_xor_sync(0xFFFFFFFFu, v.l, mask),
+             __shfl_xor_sync(0xFFFFFFFFu, v.e, mask)};
+}
+__device__ __forceinline__ double ff3_to_double(const FF3 &v) {
+  return (double)v.h + ((double)v.l + (double)v.e);
+}
+
 // One CTA per coefficient tile (grid-stride): the weights of its rows go out directly, those of its
 // columns (the reverse direction: P_in and P_out swap) through a transposed copy in shared memory,
 // so both weight tiles are written in whole rows.  Float-float arithmetic: FP64 made the row form of
-// this pass cost 609 us at 40^3.
+// this pass cost 609 us at 40^3.  The weights' sums over the tile's rows and columns go to the tile's
+// partial slots in FP64 (sums; ncs: column slots per tile, the second of two is zeroed): positive
+// terms, so 1/tau keeps its accuracy where R - B cancels (k_tau_tiles).  A warp's half-rows are added
+// in a reduce-scatter of four rows at a time, a thread's column in registers, and one thread per row
+// and column converts (a conversion costs as much as 64 FP32 operations).
 __global__ void __launch_bounds__(256) k_weight_tiles(const TileD *__restrict__ tiles, int nt,
                                                       const float4 *__restrict__ tc, const float4 *__restrict__ f0,
-                                                      float2 *__restrict__ W) {
+                                                      int ncs, float2 *__restrict__ W, double *__restrict__ sums) {
   __shared__ float2 tr[kTile][kTile + 1];
-  const int tid = threadIdx.x, col = tid & (kTile - 1), r0 = tid >> 6;
+  __shared__ FF3 su[2][kTile], sl[4][kTile];
+  const int tid = threadIdx.x, col = tid & (kTile - 1), r0 = tid >> 6, lane = tid & 31;
   for (int t = blockIdx.x; t < nt; t += gridDim.x) {
     const TileD D = tiles[t];
     const bool diag = D.I == D.J;
     const float4 *__restrict__ T = tc + (size_t)t * kTile * kTile;
     float2 *__restrict__ Wu = W + (size_t)D.wu * kTile * kTile, *__restrict__ Wl = W + (size_t)D.wl * kTile * kTile;
     const float4 fp = f0[D.J * kTile + col];
-#pragma unroll 4
-    for (int r = r0; r < kTile; r += 4) {
-      const float4 e = T[r * kTile + col];
-      const float2 pin = make_float2(e.x, e.y), pout = make_float2(e.z, e.w);
-      Wu[r * kTile + col] = ff_add(ff_mul(make_float2(fp.x, fp.y), pin), ff_mul(make_float2(fp.z, fp.w), pout));
-      if (!diag) {
-        const float4 fs = f0[D.I * kTile + r];
-        tr[col][r] = ff_add(ff_mul(make_float2(fs.x, fs.y), pout), ff_mul(make_float2(fs.z, fs.w), pin));
+    FF3 cs{0.f, 0.f, 0.f};
+#pragma unroll 1
+    for (int q = 0; q < kTile; q += 16) {  // rows q + r0 + 4 k
+      FF3 v[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int r = q + r0 + 4 * k;
+        const float4 e = T[r * kTile + col];
+        const float2 pin = make_float2(e.x, e.y), pout = make_float2(e.z, e.w);
+        const float2 w = ff_add(ff_mul(make_float2(fp.x, fp.y), pin), ff_mul(make_float2(fp.z, fp.w), pout));
+        Wu[r * kTile + col] = w;
+        v[k] = FF3{w.x, w.y, 0.f};
+        if (!diag) {
+          const float4 fs = f0[D.I * kTile + r];
+          const float2 u = ff_add(ff_mul(make_float2(fs.x, fs.y), pout), ff_mul(make_float2(fs.z, fs.w), pin));
+          tr[col][r] = u;
+          ff3_add(cs, u.x, u.y);
+        }
       }
+      // lanes 8 k .. 8 k + 7 end with row k
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const bool up = lane & 16;
+        const FF3 send = up ? v[k] : v[k + 2];
+        if (up) v[k] = v[k + 2];
+        ff3_add(v[k], ff3_shfl_xor(send, 16));
+      }
+      {
+        const bool up = lane & 8;
+        const FF3 send = up ? v[0] : v[1];
+        if (up) v[0] = v[1];
+        ff3_add(v[0], ff3_shfl_xor(send, 8));
+      }
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) ff3_add(v[0], ff3_shfl_xor(v[0], o));
+      if ((lane & 7) == 0) su[(tid >> 5) & 1][q + r0 + 4 * (lane >> 3)] = v[0];
     }
-    if (diag) continue;
+    sl[r0][col] = cs;
     __syncthreads();
+    if (tid < kTile) {
+      FF3 s = su[0][tid];
+      ff3_add(s, su[1][tid]);
+      sums[D.rb + tid * D.rs] = ff3_to_double(s);
+    } else if (tid < 2 * kTile && !diag) {
+      FF3 s = sl[0][col];
+#pragma unroll
+      for (int k = 1; k < 4; ++k) ff3_add(s, sl[k][col]);
+      sums[D.cb + col * D.cs] = ff3_to_double(s);
+      if (ncs == 2) sums[D.cb + col * D.cs + 1] = 0.0;
+    }
+    if (!diag) {
 #pragma unroll 4
-    for (int r = r0; r < kTile; r += 4) Wl[r * kTile + col] = tr[r][col];
+      for (int r = r0; r < kTile; r += 4) Wl[r * kTile + col] = tr[r][col];
+    }
     __syncthreads();
   }
+}
+
+// tau at f0, one warp per state, from the rate sweep's 1/tau = c (R - B) (in inv_tau) and the sums of the
+// weights.  R is summed in FP64 from the channels, so the difference is the better one (3e-16 to 7e-16 in
+// the worst state at 16^3, 300 K, against 1.4e-15 from the float-float weights) until it cancels: with
+// occupied partners at 100 K and sigma 0.4 meV it is off by 2e-13, the weights' sum by 1.5e-15.  The line
+// is R - B = R / 4, where both are at about 1.5e-15.
+__global__ void k_tau_tiles(const double *__restrict__ sums, const int2 *__restrict__ prow,
+                            const double *__restrict__ R, int ns, double c, double *__restrict__ inv_tau,
+                            double *__restrict__ tau) {
+  const int r = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+  if (r >= ns) return;
+  const int2 pr = prow[r];
+  double s = 0.0;
+  for (int k = lane; k < pr.y; k += 32) s += sums[pr.x + k];
+  s = warp_sum(s);
+  if (lane) return;
+  double v = inv_tau[r];
+  if (!(v >= 0.25 * (c * R[r]))) v = c * s;
+  inv_tau[r] = v;
+  tau[r] = v > 0.0 ? 1.0 / v : 0.0;
 }
 
 // F (natural state order, [n][3]) as float-float in the tiles' order: [block][direction][64]

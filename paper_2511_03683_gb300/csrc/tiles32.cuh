@@ -62,13 +62,17 @@ __device__ __forceinline__ float2 c32_round_pair(double pin, double pout) {
   return make_float2(ba, bb);
 }
 
-// The symmetric tiles from the branch-merged pair rows (complete or not): one warp per row s,
-// every stored pair (s, p) whose block pair (I, J) lies in the upper triangle written to its tile
-// entry; the tiles were zeroed before, pairs without channels stay zero.  pmap: each state's row in
-// the padded energy order (of one system, or of a batch's systems one after the other); tbase[I] =
-// (the index of tile (I, I), the last block column stored for block row I): tiles of a block row are
-// numbered consecutively, and pairs beyond the last column have zero coefficients (energy_reach).
-// C32: the pairs rounded to FP32 with their ratio kept, else float-float (float4 per entry).
+// The symmetric tiles from the branch-merged pair rows (complete or not): one warp per row s, every
+// stored pair (s, p) written to its tile entries; the tiles were zeroed before, pairs without channels
+// stay zero.  pmap: each state's row in the padded energy order (of one system, or of a batch's systems
+// one after the other); tbase[I] = (the index of tile (I, I), the last block column stored for block
+// row I): tiles of a block row are numbered consecutively, and pairs beyond the last column have zero
+// coefficients (energy_reach).
+// Float-float (float4 per entry): a pair's P_in(s, p) is P_in of entry (s, p) and, by the reverse
+// channels, P_out of entry (p, s), so each half of an entry is one row's stored P_in to 2^-49.  P_in + D
+// of one row would lose the smaller direction to cancellation (P_out / P_in = exp(-hbar w / kT): the
+// absorption rates were off by up to 5e-13 at 100 K, and the scattering rates of occupied states with them).
+// C32: the pairs P_in, P_in + D of the upper triangle rounded to FP32 with their ratio kept.
 template <bool C32, typename IDX>
 __global__ void k_tiles_scatter(const long long *__restrict__ srp, int ns, const IDX *__restrict__ pidx,
                                 const float2 *__restrict__ coefA, const float2 *__restrict__ coefB,
@@ -80,17 +84,25 @@ __global__ void k_tiles_scatter(const long long *__restrict__ srp, int ns, const
     const int pr = pmap[r], I = pr / kTile;
     const int2 tb = tbase[I];
     for (long long e = srp[r] + lane; e < srp[r + 1]; e += 32) {
-      const float2 a = coefA[e], b = coefB[e];
-      if (a.x == 0.f && a.y == 0.f && b.x == 0.f && b.y == 0.f) continue;
-      const int pp = pmap[pidx[e]], J = pp / kTile;
-      if (J < I || J > tb.y) continue;
-      const long long k = (long long)(tb.x + (J - I)) * kTile * kTile + (pr % kTile) * kTile + pp % kTile;
-      const double pin = ff_to_double(a.x, a.y), pout = pin + ff_to_double(b.x, b.y);
+      const float2 a = coefA[e];
       if (C32) {
+        const float2 b = coefB[e];
+        if (a.x == 0.f && a.y == 0.f && b.x == 0.f && b.y == 0.f) continue;
+        const int pp = pmap[pidx[e]], J = pp / kTile;
+        if (J < I || J > tb.y) continue;
+        const long long k = (long long)(tb.x + (J - I)) * kTile * kTile + (pr % kTile) * kTile + pp % kTile;
+        const double pin = ff_to_double(a.x, a.y), pout = pin + ff_to_double(b.x, b.y);
         ((float2 *)tc)[k] = c32_round_pair(pin, pout);
       } else {
-        const float2 x = ff_split(pin), y = ff_split(pout);
-        ((float4 *)tc)[k] = make_float4(x.x, x.y, y.x, y.y);
+        if (a.x == 0.f && a.y == 0.f) continue;
+        const int pp = pmap[pidx[e]], J = pp / kTile;
+        if (J >= I && J <= tb.y)
+          ((float2 *)tc)[2 * ((long long)(tb.x + (J - I)) * kTile * kTile + (pr % kTile) * kTile + pp % kTile)] = a;
+        if (J <= I) {
+          const int2 tj = tbase[J];
+          if (I <= tj.y)
+            ((float2 *)tc)[2 * ((long long)(tj.x + (I - J)) * kTile * kTile + (pp % kTile) * kTile + pr % kTile) + 1] = a;
+        }
       }
     }
   }
