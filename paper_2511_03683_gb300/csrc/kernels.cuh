@@ -62,6 +62,13 @@ __device__ __forceinline__ float2 ff_split(double v) {
 
 __device__ __forceinline__ double ff_to_double(float h, float l) { return (double)h + (double)l; }
 
+// s + err = a + b exactly
+__device__ __forceinline__ void two_sum(float a, float b, float &s, float &err) {
+  s = __fadd_rn(a, b);
+  const float bb = __fsub_rn(s, a);
+  err = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+}
+
 // (h, l) += x * (ah, al)
 __device__ __forceinline__ void ff_mac(float &h, float &l, float2 x, float ah, float al) {
   const float p = __fmul_rn(x.x, ah);
@@ -2758,13 +2765,40 @@ __global__ void __launch_bounds__(kSymThreads, 3) k_stream_sym_unit(const TileD 
 // of the whole rows).  The positive two-product form loses nothing to cancellation, unlike
 // P_in + (1 - f0_p) D where D is close to -P_in.
 
+// (f, 1 - f) as float-float pairs, both correctly rounded: in a nearly full state the 48 bits kept of f
+// leave few of 1 - f, so the last bits of the FP64 number go into it too.  The one definition of the
+// sweeps' input, at a call's start and between the stages: n steps in one call are n calls of one step.
+// f is cut into words of 24, 24 and 5 bits by integer instructions and everything after is FP32:
+// ff_split(f) and ff_split(1.0 - f) take nine instructions of the FP64 pipe (1/64 of the FP32 rate) one
+// after the other at the end of every stage (16^3, 20 steps: 335 us with them, 328 so).
+__device__ __forceinline__ float4 fg_of(double f) {
+  const unsigned hi = (unsigned)__double2hiint(f), lo = (unsigned)__double2loint(f);
+  const int E = (int)((hi >> 20) & 0x7FFu) - 1023;
+  if (E < -74 || E > 100) {  // zero, words below FP32's normal range, far too large, not finite
+    const float2 a = ff_split(f), b = ff_split(1.0 - f);
+    return make_float4(a.x, a.y, b.x, b.y);
+  }
+  const unsigned sign = hi & 0x80000000u;
+  const float h = __uint_as_float(sign | (unsigned)(E + 127) << 23 | (hi & 0xFFFFFu) << 3 | lo >> 29);
+  const float sc = __uint_as_float(sign | (unsigned)(E - 47 + 127) << 23);
+  const float m = __fmul_rn((float)((lo >> 5) & 0xFFFFFFu), sc), l = __fmul_rn((float)(lo & 31u), __fmul_rn(sc, 0x1p-5f));
+  // f = ax + ay + r exactly
+  const float ax = __fadd_rn(h, m), em = __fsub_rn(m, __fsub_rn(ax, h));
+  const float ay = __fadd_rn(em, l), r = __fsub_rn(l, __fsub_rn(ay, em));
+  // 1 - ax - ay - r = s2 + p + (q - r)
+  float s1, e1, s2, e2, p, q;
+  two_sum(1.f, -ax, s1, e1);
+  two_sum(s1, -ay, s2, e2);
+  two_sum(e1, e2, p, q);
+  const float gh = __fadd_rn(s2, p);
+  return make_float4(ax, ay, gh, __fadd_rn(__fsub_rn(p, __fsub_rn(gh, s2)), __fsub_rn(q, r)));
+}
+
 // (f, 1 - f) as float-float pairs in the padded energy order (the padding keeps its zeros)
 __global__ void k_f0_map(const double *__restrict__ f, int n, const int *__restrict__ pmap, float4 *__restrict__ out) {
   pdl_trigger();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const double v = f[i];
-    const float2 a = ff_split(v), b = ff_split(1.0 - v);
-    out[pmap[i]] = make_float4(a.x, a.y, b.x, b.y);
+    out[pmap[i]] = fg_of(f[i]);
   }
 }
 
@@ -2773,11 +2807,6 @@ __global__ void k_f0_map(const double *__restrict__ f, int n, const int *__restr
 struct FF3 {
   float h, l, e;
 };
-__device__ __forceinline__ void two_sum(float a, float b, float &s, float &err) {
-  s = __fadd_rn(a, b);
-  const float bb = __fsub_rn(s, a);
-  err = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-}
 __device__ __forceinline__ void ff3_add(FF3 &t, float h, float l) {
   float e1, e2, e3;
   two_sum(t.h, h, t.h, e1);
@@ -3069,16 +3098,6 @@ __device__ __forceinline__ FinIn fin_load(int r, const double *__restrict__ R, c
 // out[r] = I (STAGE < 0), or the RK4 stage arithmetic with k_{STAGE+1} = I
 // ry: the state's row of yff when that is in the tiles' padded energy order, else r
 enum { OUT_FF = 0, OUT_REC = 1, OUT_FG = 2 };  // the sweep's input: float2 f, uint4 records, float4 (f, 1 - f)
-
-// (f, 1 - f) as float-float pairs; 1 - f by float-float arithmetic (FP32 only)
-__device__ __forceinline__ float4 fg_of(double f) {
-  const float2 a = ff_split(f);
-  const float s = __fsub_rn(1.f, a.x);
-  const float bb = __fsub_rn(s, 1.f);
-  const float e = __fsub_rn(__fsub_rn(__fsub_rn(1.f, __fsub_rn(s, bb)), __fadd_rn(a.x, bb)), a.y);
-  const float h = __fadd_rn(s, e);
-  return make_float4(a.x, a.y, h, __fsub_rn(e, __fsub_rn(h, s)));
-}
 
 template <int STAGE, int OUT>
 __device__ __forceinline__ void fin_stage(int r, double I, const FinIn &in, double *__restrict__ out,
