@@ -298,7 +298,8 @@ int pb_scatter_rates(pb_dev *dev, const double *f, double *inv_tau, void *stream
  * step dt (fs), in place on the device vector f.  Steps are replayed from CUDA graphs captured
  * on first use per (f, dt) (the capture uses an internal stream): the call's first step from a
  * graph that also converts f into the sweeps' stage input, the others from one that takes it
- * from the step before. */
+ * from the step before.  The call that brings the steps on one (f, dt) to 64 captures a graph of
+ * eight steps before it launches anything (about 0.14 ms, once) and takes the rest in eights. */
 int pb_rtbte_rk4_step(pb_dev *dev, double *f, double dt, int32_t nsteps, void *stream);
 
 /* Same as pb_rtbte_rk4_step with HOST buffers: copies f_host_in (double[nstate]) to the

@@ -860,9 +860,10 @@ struct pb_dev {
   cudaStream_t cap = nullptr;
   cudaGraphExec_t rk_exec = nullptr;
   cudaGraphExec_t rk_exec_in = nullptr;  // the same step preceded by the stage-input conversion of f
-  // kRkRun steps in one graph, captured once rk_exec has been replayed kRkRunAfter times: a graph
-  // launch costs about as much as one of the small kernels in it, but capturing eight steps costs
-  // half a millisecond, which a few dozen steps on one f do not earn back
+  // kRkRun steps in one graph, captured by the call that brings the steps on one (f, dt) to kRkRunAfter: a
+  // graph launch costs about as much as one of the small kernels in it (16^3 18.8 -> 15.4 us per step,
+  // 24^3 18.9 -> 16.7, 40^3 60.0 -> 57.1), and capturing eight steps costs 0.14 ms, which a few dozen
+  // steps do not earn back
   cudaGraphExec_t rk_exec_run = nullptr;
   static constexpr int kRkRun = 8, kRkRunAfter = 64;
   int64_t rk_replays = 0;
@@ -2402,12 +2403,17 @@ extern "C" int pb_rtbte_rk4_step(pb_dev *d, double *f, double dt, int32_t nsteps
   cudaStream_t st = (cudaStream_t)stream;
   int rc = ensure_rk_graph(d, f, dt);
   if (rc) return rc;
-  PB_CUDA(cudaGraphLaunch(d->rk_exec_in, st));  // the first step converts f itself
   int32_t left = nsteps - 1;
-  if (left >= pb_dev::kRkRun && (d->rk_exec_run || d->rk_replays >= pb_dev::kRkRunAfter)) {
-    if (!d->rk_exec_run && (rc = capture_rk_graph(d, f, dt, pb_dev::kRkRun, false, d->rk_exec_run))) return rc;
-    for (; left >= pb_dev::kRkRun; left -= pb_dev::kRkRun) PB_CUDA(cudaGraphLaunch(d->rk_exec_run, st));
+  // the eight-step graph, if it is due, before anything is launched; the steps do not need it
+  if (!d->rk_exec_run && left >= pb_dev::kRkRun && d->rk_replays + left >= pb_dev::kRkRunAfter &&
+      capture_rk_graph(d, f, dt, pb_dev::kRkRun, false, d->rk_exec_run)) {
+    cudaGetLastError();
+    clear_error();
+    d->rk_replays = 0;  // (tried again later)
   }
+  PB_CUDA(cudaGraphLaunch(d->rk_exec_in, st));  // the first step converts f itself
+  if (d->rk_exec_run)
+    for (; left >= pb_dev::kRkRun; left -= pb_dev::kRkRun) PB_CUDA(cudaGraphLaunch(d->rk_exec_run, st));
   d->rk_replays += left;
   for (; left > 0; --left) PB_CUDA(cudaGraphLaunch(d->rk_exec, st));
   return PB_OK;

@@ -1,0 +1,104 @@
+"""The library's host code against a stand-in for the CUDA runtime (fake_cudart.cpp): its own objects,
+linked with functions that count launches and can be told to fail, in a process of their own."""
+import os
+import shutil
+import subprocess
+import sys
+import textwrap
+
+import pytest
+
+import paper_2511_03683_gb300 as pb
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    b = pb.builder()
+    objs = [os.path.join(b.OBJDIR, s + ".o") for s in b.CU_SOURCES + b.CPP_SOURCES]
+    newest = max(os.path.getmtime(s) for s in b._sources())
+    if not all(os.path.exists(o) and os.path.getmtime(o) >= newest for o in objs):
+        b.build(force=True)
+    inc = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"))),
+                       "include")
+    out = str(tmp_path_factory.mktemp("fake") / "libfake.so")
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-fPIC", "-shared", "-I" + inc, os.path.join(HERE, "fake_cudart.cpp"),
+                           *objs, "-Wl,-Bsymbolic", "-Wl,-z,defs", "-fopenmp", "-o", out])
+    return out
+
+
+PRELUDE = """
+import ctypes, sys
+import numpy as np
+sys.path.insert(0, {root!r})
+import synth
+import paper_2511_03683_gb300 as pb
+pb.LIB_PATH, pb._lib = {lib!r}, None
+L = pb.lib()
+L.fake_fail.argtypes = L.fake_fail_new.argtypes = [ctypes.c_long]
+L.fake_news.restype = L.fake_count.restype = ctypes.c_long
+
+def aligned(n):
+    a = np.zeros(n + 256, np.uint8)
+    o = -a.ctypes.data % 256
+    return a[o:o + n]
+
+def opts(**kw):
+    o = pb._DevOpts()
+    for k, v in kw.items():
+        setattr(o, k, v)
+    return o
+
+def device(ch, **kw):
+    o, n, h = opts(**kw), ctypes.c_size_t(0), ctypes.c_void_p()
+    rc = L.pb_dev_arena_bytes(ch._h, ctypes.byref(o), ctypes.byref(n))
+    if rc:
+        return rc, None, None
+    arena = aligned(n.value)
+    rc = L.pb_dev_create(ch._h, ctypes.byref(o), ctypes.c_void_p(arena.ctypes.data), n, None, ctypes.byref(h))
+    return rc, h, arena
+"""
+
+
+def child(fake, body):
+    src = PRELUDE.format(root=os.path.dirname(HERE), lib=fake) + textwrap.dedent(body)
+    r = subprocess.run([sys.executable, "-c", src], capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0, r.stdout + r.stderr
+
+
+@pytest.mark.parametrize("fail", [False, True])
+def test_rk4_eight_step_graph(fake, fail):
+    """Every call runs its n steps whatever graphs it replays (one launch for the input, eight per step):
+    one by one at first, eight at a time later and in a long call; and where the eight-step graph
+    cannot be made, one by one again, with no step done twice or left out and no error."""
+    child(fake, f"""
+    ch = pb.Channels.from_model(synth.make_window4(8))
+    rc, h, arena = device(ch)
+    assert rc == pb.PB_OK, L.pb_last_error().decode()
+    f = np.zeros(ch.nstate)
+
+    def steps(n):
+        a, g = L.fake_count(0), L.fake_count(1)
+        rc = L.pb_rtbte_rk4_step(h, ctypes.c_void_p(f.ctypes.data), 1.0, n, None)
+        assert rc == pb.PB_OK, L.pb_last_error().decode()
+        assert L.fake_count(0) - a == 1 + 8 * n, (n, L.fake_count(0) - a)
+        return L.fake_count(1) - g  # graph launches
+
+    assert steps(1) == 1 and steps(9) == 9
+    assert steps(41) == 41
+    if {fail}:
+        L.fake_fail(1)
+        assert steps(41) == 41  # the eight-step graph fails: one by one
+        assert steps(9) == 9
+    else:
+        assert steps(41) == 1 + 5  # 1 + 8 * 5
+        assert steps(12) == 1 + 1 + 3
+        g = np.zeros(ch.nstate)
+        f = g  # another vector: the graphs start over, and a long call takes the eight-step one by itself
+        assert steps(20) == 20
+        assert steps(4001) == 1 + 500
+        f = np.zeros(ch.nstate)
+        assert steps(4001) == 1 + 500
+    L.pb_dev_destroy(h)
+    """)
