@@ -507,9 +507,7 @@ BatchTiles batch_tiles_for(const pb_channels *const *chs, int32_t n, int prec, i
     const int64_t full = (ch->nstate + kRowPad - 1) / kRowPad * kRowPad;
     for (int64_t r = 0; r < ch->nstate; ++r) complete = complete && lenp[so + r] == full;
     so += ch->nstate;
-    double gmax = 0.0;
-    for (const double g : ch->g2) gmax = std::max(gmax, g);
-    tile_plan_add(ch, prec == 1, complete, energy_reach(ch, gmax), T);
+    tile_plan_add(ch, prec == 1, complete, energy_reach(ch, ch->g2_max), T);
   }
   const int64_t nt = (int64_t)T.tiles.size();
   if (nt == 0 || nt >= INT32_MAX / 2 || T.npart >= INT32_MAX) return T;

@@ -266,6 +266,10 @@ extern "C" int pb_build_channels(const pb_model *m, pb_g2_fn g2fn, void *user, c
       ch->g2.shrink_to_fit();
     }
     ch->nch = nch;
+    double top = 0.0;
+#pragma omp parallel for num_threads(nt) schedule(static) reduction(max : top)
+    for (int64_t c = 0; c < nch; ++c) top = std::max(top, ch->g2[c]);
+    ch->g2_max = top;
     int64_t mx = 0;
     for (int64_t r = 0; r < ns; ++r) mx = std::max(mx, ch->row_ptr[r + 1] - ch->row_ptr[r]);
     ch->max_row = mx;

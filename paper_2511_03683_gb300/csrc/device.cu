@@ -1276,8 +1276,7 @@ extern "C" int pb_dev_create(const pb_channels *ch, const pb_dev_opts *opts, voi
     // FP16 |g|^2: the largest value at creation maps into [2^9, 2^10), so every value down to
     // 2^-23 of it stays a normal FP16 number (11 significand bits; FP16's smallest normal is
     // 2^-14) and pb_dev_set_g2 may raise them up to 63-fold
-    double gmax = 0.0;
-    for (const double v : ch->g2) gmax = std::max(gmax, std::fabs(v));
+    const double gmax = ch->g2_max;
     if (gmax > 0.0 && std::isfinite(gmax)) d->g2s = std::ldexp(1.0, 10 - std::ilogb(gmax) - 1);
   }
   d->sm_count = sm;
