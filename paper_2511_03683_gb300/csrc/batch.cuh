@@ -511,9 +511,12 @@ BatchTiles batch_tiles_for(const pb_channels *const *chs, int32_t n, int prec, i
   }
   const int64_t nt = (int64_t)T.tiles.size();
   if (nt == 0 || nt >= INT32_MAX / 2 || T.npart >= INT32_MAX) return T;
-  const double tile_bytes = (double)nt * dev::kTile * dev::kTile * (prec == 2 ? 8.0 : 16.0);
   const double row_bytes = (double)nent * (prec == 2 ? 12.0 : 20.0);
-  T.on = layout == 2 || tile_bytes <= 0.7 * row_bytes;
+  auto pay = [&](int64_t tiles) {
+    return (double)tiles * dev::kTile * dev::kTile * (prec == 2 ? 8.0 : 16.0) <= 0.7 * row_bytes;
+  };
+  T.band = layout != 2 && !pay(T.nt_full);
+  T.on = !T.band || pay(nt);
   if (T.on && prec == 1 && chain_pdl(nt, sm)) tile_plan_halve(T);
   return T;
 }
@@ -586,8 +589,8 @@ BatchLayoutFF batch_layout_ff(const pb_channels *const *chs, int n, int64_t ns, 
   L.pmap = take(T.on ? sizeof(int32_t) * ns : 0);
   L.prow = take(T.on ? sizeof(int2) * ns : 0);
   L.tbase = take(T.on ? sizeof(int2) * T.nb : 0);
-  L.tc = take(T.on ? te * (size_t)T.nt_full * dev::kTile * dev::kTile : 0);
-  L.tp = take(T.on ? pe * (size_t)T.nsp * T.nb_max : 0);
+  L.tc = take(T.on ? te * (size_t)T.tiles_reserved() * dev::kTile * dev::kTile : 0);
+  L.tp = take(T.on ? T.part_bytes(pe) : 0);
   L.err = take(sizeof(int));
   L.total = o;
   return L;

@@ -341,8 +341,17 @@ double energy_reach(const pb_channels *ch, double scale) {
 struct TilePlan {
   int nb = 0;                     // blocks
   int64_t nsp = 0, npart = 0;     // padded states; partial slots
-  int64_t nt_full = 0;            // tiles of the whole triangles, and the blocks of the largest system:
-  int nb_max = 0;                 // what the arena reserves, whatever the reach
+  int64_t nt_full = 0;            // tiles of the whole triangles
+  int nb_max = 0;                 // blocks of the largest system
+  // What the arena reserves: the whole triangles, a size known from the numbers of states, or with `band`
+  // what is stored.  Band: the lists that take the tiles because of the reach (the whole triangle would not
+  // have paid): they would hold a region that grows with the square of the states for a fraction of it.
+  bool band = false, halved = false;
+  int64_t tiles_reserved() const { return band ? (int64_t)tiles.size() : nt_full; }
+  size_t part_bytes(size_t slot) const {  // slot: bytes of one partial of the sweeps that take whole tiles
+    if (band) return halved ? sizeof(float2) * (size_t)npart : slot * (size_t)npart;
+    return slot * (size_t)nsp * (size_t)nb_max;
+  }
   std::vector<int32_t> pmap;      // [states] row in the padded energy order
   std::vector<int2> prow;         // [states] first partial slot, slots
   std::vector<int2> tbase;        // [blocks] index of tile (I, I), last block column of block row I
@@ -435,6 +444,7 @@ void tile_plan_add(const pb_channels *ch, bool energy, bool complete, double rea
 void tile_plan_halve(TilePlan &T) {
   std::vector<int64_t> first((size_t)T.nb);
   std::vector<int> slots((size_t)T.nb);
+  T.halved = true;
   auto ncol = [&](int K) { return K - T.span[K].x; };  // tiles above the diagonal in block column K
   T.npart = 0;
   for (int K = 0; K < T.nb; ++K) {
@@ -527,8 +537,8 @@ Layout make_layout(const pb_channels *ch, const Plan &P, const Plan *S, int vari
   L.gacc = take(S && gacc && variant == PB_VARIANT_FF ? sizeof(float4) * nsw : 0);
   L.gaccg = take(gacc && (variant == PB_VARIANT_G32 || variant == PB_VARIANT_G16 || variant == PB_VARIANT_H16) ? 3 * sizeof(double) * (size_t)ns * (size_t)ns : 0);
   L.tiles = take(tp ? sizeof(dev::TileD) * tp->tiles.size() : 0);
-  L.tcoef = take(tp ? tile_entry * (size_t)tp->nt_full * dev::kTile * dev::kTile : 0);
-  L.tpart = take(tp ? sizeof(float4) * (size_t)tp->nb_max * (size_t)tp->nsp : 0);
+  L.tcoef = take(tp ? tile_entry * (size_t)tp->tiles_reserved() * dev::kTile * dev::kTile : 0);
+  L.tpart = take(tp ? tp->part_bytes(sizeof(float4)) : 0);
   L.pmap = take(tp ? sizeof(int32_t) * ns : 0);
   L.prow = take(tp ? sizeof(int2) * ns : 0);
   L.tbase = take(tp ? sizeof(int2) * tp->nb : 0);
@@ -1005,7 +1015,8 @@ bool sym_for(const pb_channels *ch, const pb_dev_opts &o, bool c32, bool merged,
   if (o.dense_rows != 3 && o.dense_rows != 0) return false;
   tile_plan_add(ch, !c32, complete, energy_reach(ch, 1.0), T);
   if (T.tiles.size() >= (size_t)INT32_MAX / 2 || T.npart >= INT32_MAX) return false;
-  if (!(o.dense_rows == 3 || complete || tiles_pay((int64_t)T.tiles.size(), ch->nstate, nsw))) return false;
+  T.band = !(o.dense_rows == 3 || complete || tiles_pay(T.nt_full, ch->nstate, nsw));
+  if (T.band && !tiles_pay((int64_t)T.tiles.size(), ch->nstate, nsw)) return false;
   if (!c32 && o.tile_sweep == 3 && chain_pdl((int64_t)T.tiles.size(), sm)) tile_plan_halve(T);
   return true;
 }

@@ -1,4 +1,4 @@
-"""Host side of the batched forms: what sizing a batch costs and reserves (no GPU)."""
+"""What sizing a device or a batch costs and reserves (host only, no GPU)."""
 import ctypes
 import time
 
@@ -24,3 +24,24 @@ def test_sizing_a_tiled_batch_does_not_walk_every_coupling():
     rows = min(arena(lists, 1, layout=1)[1] for _ in range(7))
     for prec in (1, 2):
         assert min(arena(lists, prec)[1] for _ in range(7)) <= 4 * rows
+
+
+def dev_arena(ch, **kw):
+    o, n = pb._DevOpts(), ctypes.c_size_t(0)
+    for k, v in kw.items():
+        setattr(o, k, v)
+    assert pb.lib().pb_dev_arena_bytes(ch._h, ctypes.byref(o), ctypes.byref(n)) == pb.PB_OK
+    return n.value
+
+
+def test_lists_that_take_the_tiles_for_their_reach_reserve_the_stored_tiles():
+    """A cutoff list whose whole upper triangle would not pay (28^3: 325 tiles, 21 MB) but whose
+    hundred tiles in reach do reserves those and not the triangle, alone and in a batch; forced tiles
+    reserve the triangle, a size that follows from the number of states."""
+    ch = pb.Channels.from_model(synth.make_window4(28), g2_min=1e-5, delta_nsigma=6.0)
+    nb = (ch.nstate + 63) // 64
+    triangle = 16 * 4096 * nb * (nb + 1) // 2
+    assert 0 < dev_arena(ch) - dev_arena(ch, dense_rows=2) < triangle // 2
+    assert dev_arena(ch, dense_rows=3) - dev_arena(ch, dense_rows=2) >= triangle
+    assert 0 < arena([ch, ch], 1)[0] - arena([ch, ch], 1, layout=1)[0] < triangle
+    assert arena([ch, ch], 1, layout=2)[0] - arena([ch, ch], 1, layout=1)[0] >= 2 * triangle
