@@ -386,9 +386,10 @@ bool batch_dense_for(const pb_channels *const *chs, int32_t n, const pb_batch_op
   return (double)nch >= 0.85 * (double)slots;
 }
 int batch_dense_part(int item_ch) { return std::max(32, item_ch / 4 / 8 * 8); }
-// What the arena reserves, for any item size up to 4096 (the autotuner's largest) or the batch's own:
-// a row's bundles hold its pairs in reach and, since each is as long as its longest chain, at most 32
-// times the longest chain more; they are no more than its pieces.
+// What the arena reserves, for the autotuner's item sizes and the batch's own: a row's bundles hold its
+// pairs in reach and, since each is as long as its longest chain, at most 32 times the longest chain
+// more; nor can they hold more than the pieces do with every lane as long as the piece's longest (the
+// chains sorted by length never need more steps than piece by piece).
 struct BatchDenseCaps {
   int64_t items = 0, slots = 0, values = 0, map = 0;
 };
@@ -396,15 +397,25 @@ BatchDenseCaps batch_dense_caps(const pb_channels *const *chs, int32_t n, int it
   BatchDenseCaps C;
   for (int i = 0; i < n; ++i) {
     const int64_t ns = chs[i]->nstate, npp = batch_npp(ns);
-    const int64_t longest = std::min<int64_t>(npp, (batch_dense_part(std::max(4096, item_ch)) + 31) / 32 * 32);
     std::vector<double> e(chs[i]->eps.begin(), chs[i]->eps.begin() + ns);
     std::sort(e.begin(), e.end());
     const double reach = energy_reach_f32(chs[i]);
-    int64_t slots = ns * longest;
+    std::vector<int64_t> near((size_t)ns);  // pairs in reach of every state, in energy order
     for (int64_t r = 0, a = 0, b = 0; r < ns; ++r) {
       while (e[r] - e[a] > reach) ++a;
       while (b < ns && e[b] - e[r] <= reach) ++b;
-      slots += b - a;
+      near[r] = b - a;
+    }
+    int64_t slots = 0;
+    for (const int item : {1024, 2048, 4096, item_ch}) {
+      if (item <= 0) continue;
+      int64_t longest = 0, pieces = 0, s = 0;  // 32 times the longest lane of any piece, of all pieces
+      for (const int64_t n : lane_pieces(npp, batch_dense_part(item))) {
+        longest = std::max(longest, (n + 31) / 32 * 32);
+        pieces += (n + 31) / 32 * 32;
+      }
+      for (const int64_t p : near) s += std::min(p + longest, pieces);
+      slots = std::max(slots, s);
     }
     C.items += ns * std::max<int64_t>(1, (npp + batch_dense_part(1024) - 1) / batch_dense_part(1024));
     C.slots += slots;

@@ -196,11 +196,19 @@ struct LanePlan {
   std::vector<IDX> pidx;          // [slots] partner
   int64_t slots = 0;
 };
+// the sizes of the pieces that a row of npp slots is cut into
+std::vector<int64_t> lane_pieces(int64_t npp, int64_t item) {
+  const int64_t chunks = npp / kRowPad, np = std::max<int64_t>(1, (npp + item - 1) / item);
+  std::vector<int64_t> n((size_t)np);
+  for (int64_t k = 0; k < np; ++k) n[k] = kRowPad * (chunks / np + (k < chunks % np ? 1 : 0));
+  return n;
+}
 template <typename IDX>
 void lane_plan(const double *eps, int64_t ns, int64_t npp, int64_t item, double reach, bool fill, LanePlan<IDX> &P) {
-  const int64_t chunks = npp / kRowPad, np = std::max<int64_t>(1, (npp + item - 1) / item);
+  const std::vector<int64_t> pieces = lane_pieces(npp, item);
+  const int64_t np = (int64_t)pieces.size();
   std::vector<int64_t> p0((size_t)np + 1, 0);  // first partner of every piece
-  for (int64_t k = 0; k < np; ++k) p0[k + 1] = p0[k] + kRowPad * (chunks / np + (k < chunks % np ? 1 : 0));
+  for (int64_t k = 0; k < np; ++k) p0[k + 1] = p0[k] + pieces[k];
   std::vector<std::vector<int32_t>> steps((size_t)ns);  // of every row's bundles
   // the chain of every partner in reach, the chains' ranks by length (stable), the bundles
   auto row = [&](int64_t r, std::vector<int32_t> &cnt, std::vector<int32_t> &rank) {

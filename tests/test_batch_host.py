@@ -45,3 +45,14 @@ def test_lists_that_take_the_tiles_for_their_reach_reserve_the_stored_tiles():
     assert dev_arena(ch, dense_rows=3) - dev_arena(ch, dense_rows=2) >= triangle
     assert 0 < arena([ch, ch], 1)[0] - arena([ch, ch], 1, layout=1)[0] < triangle
     assert arena([ch, ch], 1, layout=2)[0] - arena([ch, ch], 1, layout=1)[0] >= 2 * triangle
+
+
+def test_dense_batch_reserves_no_more_slots_than_pairs():
+    """The default FP32 batch: per (state, partner) slot 8 bytes of list and 4 of dense |g|^2 per branch,
+    4 of partner and 4 of slot map, each grid's padded phonon table and a few hundred bytes per state; its
+    chains never need more slots than there are partners (rounded up to 32 in each piece of a row)."""
+    ns = (16, 18, 20, 22)
+    lists = [pb.Channels.from_model(synth.make_window4(n)) for n in ns]
+    slots = sum(c.nstate * ((c.nstate + 31) // 32 * 32) for c in lists)
+    tables = sum((2 * n) ** 3 * 6 * 8 for n in ns)
+    assert arena(lists, 0)[0] <= slots * (12 * 6 + 8) + tables + 400 * sum(c.nstate for c in lists) + (1 << 20)

@@ -102,3 +102,26 @@ def test_rk4_eight_step_graph(fake, fail):
         assert steps(4001) == 1 + 500
     L.pb_dev_destroy(h)
     """)
+
+
+def test_dense_batch_plans_fit_the_arena(fake):
+    """pb_batch_arena_bytes bounds the slots of every item size that the autotuner tries and of the
+    batch's own, whatever the reach: narrow, ordinary, the whole spectrum, a single energy."""
+    child(fake, """
+    ms = [synth.make_window4(16, sigma=4e-4), synth.make_window4(17), synth.make_window4(22), synth.make_window4(12, sigma=0.3),
+          synth.make_flat_einstein(5), synth.make_tiny(6).with_(T=20.0)]
+    chs = [pb.Channels.from_model(m) for m in ms]
+    for item in (0, 1024, 3072, 65536):
+        for group in [[c] for c in chs] + [chs]:
+            arr = (ctypes.c_void_p * len(group))(*[c._h.value for c in group])
+            o, n, h = pb._BatchOpts(item, 0, 0, 0), ctypes.c_size_t(0), ctypes.c_void_p()
+            assert L.pb_batch_arena_bytes(arr, len(group), ctypes.byref(o), ctypes.byref(n)) == pb.PB_OK
+            a = aligned(n.value)
+            rc = L.pb_batch_create(arr, len(group), ctypes.byref(o), ctypes.c_void_p(a.ctypes.data), n, None, ctypes.byref(h))
+            assert rc == pb.PB_OK, L.pb_last_error().decode()
+            f = np.zeros(sum(c.nstate for c in group))
+            i, c, ms_ = ctypes.c_int32(0), ctypes.c_int32(0), ctypes.c_double(0)
+            rc = L.pb_batch_autotune(h, ctypes.c_void_p(f.ctypes.data), None, ctypes.byref(i), ctypes.byref(c), ctypes.byref(ms_))
+            assert rc == pb.PB_OK, L.pb_last_error().decode()
+            L.pb_batch_destroy(h)
+    """)
