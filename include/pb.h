@@ -275,7 +275,9 @@ int pb_dev_get_info(const pb_dev *dev, pb_dev_info *info);
  * use; the handle keeps its twelve most recent call graphs, shared with pb_scatter_rates,
  * pb_transport_iterate, the host-buffer calls, the RK4 adjoint steps and the transport solver's
  * passes); when `stream` is itself being captured, the launches are recorded into the caller's
- * capture. */
+ * capture.  A state whose f is not finite makes dfdt not finite in itself and in every state that it
+ * is coupled to (a pair with a nonzero coefficient); in other states that depends on the form, since
+ * pairs with zero coefficients may be left out or streamed.  The same holds for the other sweeps. */
 int pb_collision(pb_dev *dev, const double *f, double *dfdt, void *stream);
 
 /* Measurement aid (the paper has no counterpart): the average device duration of the

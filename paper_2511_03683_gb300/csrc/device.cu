@@ -187,8 +187,8 @@ double energy_reach_f32(const pb_channels *ch) {
 // pieces of at most `item` slots of npp (multiples of 8) and dealt to the 32 lanes of each; a lane's
 // partners within reach are a chain.  The row's chains, longest first, form bundles of 32, one work
 // item each: start = its first slot, len = steps, lane l's k-th pair at start + 32 k + l: its partner,
-// with the top bit of IDX set when partners out of reach follow it in the lane's order; all lower bits
-// set past the chain's end.
+// with the top bit of IDX set when partners out of reach follow it in the lane's order; past the chain's
+// end the row's own state with the next bit set.
 template <typename IDX>
 struct LanePlan {
   std::vector<Item> items;        // row = the list's state
@@ -243,8 +243,8 @@ void lane_plan(const double *eps, int64_t ns, int64_t npp, int64_t item, double 
   }
   P.item_ptr[ns] = (int32_t)P.items.size();
   if (!fill) return;
-  constexpr IDX kGap = (IDX)((IDX)1 << (8 * sizeof(IDX) - 1));
-  P.pidx.assign((size_t)P.slots, (IDX)(kGap - 1));
+  constexpr IDX kGap = (IDX)((IDX)1 << (8 * sizeof(IDX) - 1)), kPad = (IDX)(kGap >> 1);
+  P.pidx.resize((size_t)P.slots);
 #pragma omp parallel
   {
     std::vector<int32_t> cnt, rank, at, prev;
@@ -254,6 +254,8 @@ void lane_plan(const double *eps, int64_t ns, int64_t npp, int64_t item, double 
       at.assign(cnt.size(), -1);  // bundle and lane of every chain: 32 bundle + lane
       for (size_t q = 0; q < rank.size() && cnt[rank[q]] > 0; ++q) at[rank[q]] = (int32_t)q;
       std::fill(cnt.begin(), cnt.end(), 0);
+      for (int32_t i = P.item_ptr[r]; i < P.item_ptr[r + 1]; ++i)
+        std::fill_n(P.pidx.begin() + P.items[i].start, 32 * (int64_t)P.items[i].len, (IDX)(kPad | r));
       prev.assign(cnt.size(), 0);
       for (int64_t k = 0; k < np; ++k)
         for (int64_t p = p0[k]; p < std::min(p0[k + 1], ns); ++p)
@@ -286,7 +288,7 @@ GDense gdense_for(const pb_channels *ch, const pb_dev_opts &o, int sm, bool fill
   const bool mixed = o.variant == PB_VARIANT_G32 || o.variant == PB_VARIANT_G16 || o.variant == PB_VARIANT_H16;
   if (!mixed || (o.channel_per_lane != 0 && o.channel_per_lane != 5)) return g;
   const int64_t ns = ch->nstate, nm = ch->nmodes;
-  if (ns == 0 || nm == 0 || ns >= dev::kGapBit) return g;  // (more states than shared memory holds are refused later)
+  if (ns == 0 || nm == 0 || ns >= dev::kPadBit) return g;  // (more states than shared memory holds are refused later)
   const int64_t npp = (ns + 31) / 32 * 32;
   const double slots = (double)ns * (double)nm * (double)npp;
   if (o.channel_per_lane == 0 && (double)ch->row_ptr[ns] < 0.85 * slots) return g;

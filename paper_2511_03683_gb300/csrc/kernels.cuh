@@ -1378,12 +1378,13 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 3 : 1) k_stream_g_lane(const I
 // sums add the same terms in the same order as over all partners, where the pairs out of reach add
 // zeros (kGapBit of pidx: some follow this pair; the first zero may still move the compensation into
 // the sum, the others change nothing), while a bundle's lanes are busy for all of its I.len steps (lane l's slots are I.start + l
-// + 32 k).  Its partial goes to part[item].x.  Warp w takes the items order[wbeg[w]] ..
+// + 32 k; past its chain's end zero |g|^2 and, with kPadBit, the row's own state, so that a padding slot
+// reads no state that the row is not coupled to: 0 times a NaN is a NaN).  Its partial goes to part[item].x.  Warp w takes the items order[wbeg[w]] ..
 // order[wbeg[w + 1] - 1], longest first and about equal steps for every warp (a small system has
 // little more than one bundle per resident warp, three to eight steps long).  MODE_VJP: the FP32 adjoint's sum, the rate summands of each pair weighted by
 // lam_s - lam_p (lam in FP32 after the records in shared memory; see k_stream_g_vjp).
 constexpr int kDenseBranches = 6;  // branches whose loads a lane issues together (more: one at a time)
-constexpr int kGapBit = 0x8000;
+constexpr int kGapBit = 0x8000, kPadBit = 0x4000;
 constexpr int kDenseThreads = 1024;  // one CTA per SM (768 threads without spills measured slower)
 template <int MODE, typename G2T>
 __global__ void __launch_bounds__(kDenseThreads, 1) k_stream_g_dense(const Item *__restrict__ items,
@@ -1418,7 +1419,7 @@ __global__ void __launch_bounds__(kDenseThreads, 1) k_stream_g_dense(const Item 
     int pn = pr[0];  // the next pair's partner, loaded a step ahead
     for (int j = 0; j < I.len; ++j) {
       const bool gap = pn & kGapBit;
-      const int p = min(pn & (kGapBit - 1), ns - 1);  // past the end of the lane's chain: zero |g|^2
+      const int p = pn & (kPadBit - 1);
       if (j + 1 < I.len) pn = pr[32 * (j + 1)];
       const uint4 sp = gsd[p];
       const float dh = __fsub_rn(es, __uint_as_float(sp.x));
@@ -1504,8 +1505,8 @@ __global__ void k_slot_map(const Item *__restrict__ items, int nitems, const uin
     const Item I = items[it];
     for (int j = 0; j < I.len; ++j) {
       const long long slot = I.start + 32 * j + lane;
-      const int p = pidx[slot] & (kGapBit - 1);
-      if (p < ns) smap[(size_t)I.row * ns + p] = (uint32_t)slot;
+      const int p = pidx[slot];
+      if (!(p & kPadBit)) smap[(size_t)I.row * ns + (p & (kPadBit - 1))] = (uint32_t)slot;
     }
   }
 }
