@@ -107,7 +107,9 @@ __global__ void __launch_bounds__(512) k_stream_gbatch(const Item *__restrict__ 
 // chains of the global row I.row, its slots numbered within the instance (LanePlan); partner records
 // come through L1 (CTA b takes the items [cbeg[b], cbeg[b + 1]), ranges of about equal work, mostly
 // of one instance: rows differ tenfold in length over the instances).  The per-pair arithmetic is
-// k_stream_g_dense's (the bracket collected per pair).
+// k_stream_g_dense's (the bracket collected per pair).  pidx: as there, with 32-bit words (the top bit the
+// gap, the next the padding).
+constexpr uint32_t kPadBit32 = 0x40000000u;
 __global__ void __launch_bounds__(512, 2) k_stream_gbatch_dense(const Item *__restrict__ items,
                                                              const int *__restrict__ item_inst,
                                                              const int *__restrict__ cbeg,
@@ -134,7 +136,7 @@ __global__ void __launch_bounds__(512, 2) k_stream_gbatch_dense(const Item *__re
 #pragma unroll 1
     for (int left = I.len; left > 0; --left) {
       const bool gap = pn >> 31;
-      const int p = (int)min(pn & 0x7FFFFFFFu, (uint32_t)(B.ns - 1));  // past the chain's end: zero |g|^2
+      const int p = (int)(pn & (kPadBit32 - 1));
       pr += 32;
       if (left > 1) pn = pr[0];
       const uint4 sp = __ldg(gsi + p);
@@ -204,8 +206,8 @@ __global__ void __launch_bounds__(kBlock) k_slot_map_batch(const Item *__restric
     const BInst B = inst[item_inst[it]];
     for (int j = 0; j < I.len; ++j) {
       const long long slot = I.start + 32 * j + lane;
-      const uint32_t p = pidx[B.poff + slot] & 0x7FFFFFFFu;
-      if (p < (uint32_t)B.ns) smap[B.moff + (long long)(I.row - B.soff) * B.ns + p] = (uint32_t)slot;
+      const uint32_t p = pidx[B.poff + slot];
+      if (!(p & kPadBit32)) smap[B.moff + (long long)(I.row - B.soff) * B.ns + (p & (kPadBit32 - 1))] = (uint32_t)slot;
     }
   }
 }
@@ -1412,15 +1414,18 @@ extern "C" int pb_batch_autotune(pb_batch *b, const double *f, void *stream, int
   if (!b || !f) return set_error(PB_EINVAL, "pb_batch_autotune: null argument");
   cudaStream_t st = (cudaStream_t)stream;
   if (b->tiles) {
-    // the tile form: the launch shapes of the tile ring (stages x CTAs per SM)
-    const std::vector<int> shapes = b->prec == 2 ? std::vector<int>{2, 3, 4, 7, 8} : std::vector<int>{3, 2};
+    // the tile form: the launch shapes of the tile ring (stages x CTAs per SM).  A small float-float list
+    // takes no ring but one CTA per half-tile, three per SM whatever the shape.
+    static constexpr int kC32Shapes[] = {2, 3, 4, 7, 8}, kFFShapes[] = {3, 2};
+    const int *shapes = b->prec == 2 ? kC32Shapes : kFFShapes;
+    const int nshapes = b->prec == 2 ? 5 : chain_pdl(b->tnt, b->sm_count) ? 1 : 2;
     int bs = b->tshape;
     float best = 1e30f;
     cudaEvent_t e0, e1;
     PB_CUDA(cudaEventCreate(&e0));
     PB_CUDA(cudaEventCreate(&e1));
     int rc = batch_stage_input(b, f, st);
-    for (size_t a = 0; a < shapes.size() && rc == PB_OK; ++a) {
+    for (int a = 0; a < nshapes && rc == PB_OK; ++a) {
       b->tshape = shapes[a];
       if ((rc = batch_sweep(b, st))) break;  // warm-up
       cudaEventRecord(e0, st);

@@ -125,3 +125,29 @@ def test_dense_batch_plans_fit_the_arena(fake):
             assert rc == pb.PB_OK, L.pb_last_error().decode()
             L.pb_batch_destroy(h)
     """)
+
+
+def test_batch_autotune_times_the_shapes_that_run(fake):
+    """Two ring shapes for a float-float batch on the ring (4 x 69 tiles), one for a small list, whose
+    kernel has no ring, five for C32: one input launch, then a warm-up and three timed sweeps each."""
+    child(fake, """
+    def tune(chs, prec):
+        arr = (ctypes.c_void_p * len(chs))(*[c._h.value for c in chs])
+        o, n, h = pb._BatchOpts(0, 0, prec, 2), ctypes.c_size_t(0), ctypes.c_void_p()
+        assert L.pb_batch_arena_bytes(arr, len(chs), ctypes.byref(o), ctypes.byref(n)) == pb.PB_OK
+        a = aligned(n.value)
+        assert L.pb_batch_create(arr, len(chs), ctypes.byref(o), ctypes.c_void_p(a.ctypes.data), n, None, ctypes.byref(h)) == pb.PB_OK
+        f = np.zeros(sum(c.nstate for c in chs))
+        i, c, ms, before = ctypes.c_int32(0), ctypes.c_int32(0), ctypes.c_double(0), L.fake_count(0)
+        assert L.pb_batch_autotune(h, ctypes.c_void_p(f.ctypes.data), None, ctypes.byref(i), ctypes.byref(c), ctypes.byref(ms)) == pb.PB_OK
+        got, info = L.fake_count(0) - before, ctypes.c_int32(0)
+        assert L.pb_batch_get_info(h, None, None, None, None, ctypes.byref(info)) == pb.PB_OK
+        assert info.value == c.value
+        L.pb_batch_destroy(h)
+        return got, c.value
+
+    small, big = pb.Channels.from_model(synth.make_window4(16)), pb.Channels.from_model(synth.make_window4(24))
+    assert tune([small, small], 1) == (1 + 4, 3)
+    assert tune([big] * 4, 1)[0] == 1 + 2 * 4
+    assert tune([small], 2)[0] == 1 + 5 * 4
+    """)
