@@ -717,16 +717,14 @@ int batch_upload_dense(pb_batch *b, int item_ch, cudaStream_t st) {
 }
 
 int batch_upload_plan(pb_batch *b, int item_ch, cudaStream_t st) {
-  if (b->dense) {
-    try {
-      return batch_upload_dense(b, item_ch, st);
-    } catch (const std::bad_alloc &) {
-      return set_error(PB_ENOMEM, "pb_batch: out of host memory");
-    }
+  try {
+    if (b->dense) return batch_upload_dense(b, item_ch, st);
+    BatchPlan P;
+    batch_plan(b, item_ch, P);
+    return batch_upload_items(b, P, item_ch, st);
+  } catch (const std::bad_alloc &) {
+    return set_error(PB_ENOMEM, "pb_batch: out of host memory");
   }
-  BatchPlan P;
-  batch_plan(b, item_ch, P);
-  return batch_upload_items(b, P, item_ch, st);
 }
 
 // the tile sweep of every instance in one launch (the single-system kernels)

@@ -218,7 +218,12 @@ extern "C" int pb_build_channels(const pb_model *m, pb_g2_fn g2fn, void *user, c
         std::vector<int32_t> sb, pb_, vb;
 #pragma omp for schedule(dynamic, 4)
         for (int64_t r = 0; r < ns; ++r) {
-          int rc = fill_row(r, sb, pb_, vb);
+          int rc;
+          try {
+            rc = fill_row(r, sb, pb_, vb);
+          } catch (const std::bad_alloc &) {  // must not leave the parallel region
+            rc = 3;
+          }
           if (rc) {
 #pragma omp critical
             {
@@ -235,6 +240,7 @@ extern "C" int pb_build_channels(const pb_model *m, pb_g2_fn g2fn, void *user, c
         if (cb_status) bad = r;
       }
     }
+    if (cb_status == 3) throw std::bad_alloc();
     if (cb_status) {
       delete ch;
       return set_error(PB_ECALLBACK, cb_status == 1 ? "pb_build_channels: g2 callback failed on row %lld"

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstring>
 #include <memory>
@@ -196,6 +197,17 @@ struct LanePlan {
   std::vector<IDX> pidx;          // [slots] partner
   int64_t slots = 0;
 };
+// fn() inside a parallel region, which an exception must not leave: a failed allocation is noted, and
+// thrown after the region
+template <typename F>
+void guarded(std::atomic<bool> &failed, F &&fn) {
+  try {
+    fn();
+  } catch (const std::bad_alloc &) {
+    failed = true;
+  }
+}
+
 // the sizes of the pieces that a row of npp slots is cut into
 std::vector<int64_t> lane_pieces(int64_t npp, int64_t item) {
   const int64_t chunks = npp / kRowPad, np = std::max<int64_t>(1, (npp + item - 1) / item);
@@ -220,15 +232,18 @@ void lane_plan(const double *eps, int64_t ns, int64_t npp, int64_t item, double 
     std::iota(rank.begin(), rank.end(), 0);
     std::stable_sort(rank.begin(), rank.end(), [&](int32_t a, int32_t b) { return cnt[a] > cnt[b]; });
   };
+  std::atomic<bool> failed{false};
 #pragma omp parallel
   {
     std::vector<int32_t> cnt, rank;
 #pragma omp for schedule(dynamic, 16)
-    for (int64_t r = 0; r < ns; ++r) {
-      row(r, cnt, rank);
-      for (size_t q = 0; q < rank.size() && cnt[rank[q]] > 0; q += 32) steps[r].push_back(cnt[rank[q]]);
-    }
+    for (int64_t r = 0; r < ns; ++r)
+      guarded(failed, [&] {
+        row(r, cnt, rank);
+        for (size_t q = 0; q < rank.size() && cnt[rank[q]] > 0; q += 32) steps[r].push_back(cnt[rank[q]]);
+      });
   }
+  if (failed) throw std::bad_alloc();
   P.item_ptr.assign((size_t)ns + 1, 0);
   for (int64_t r = 0; r < ns; ++r) {
     P.item_ptr[r] = (int32_t)P.items.size();
@@ -249,7 +264,7 @@ void lane_plan(const double *eps, int64_t ns, int64_t npp, int64_t item, double 
   {
     std::vector<int32_t> cnt, rank, at, prev;
 #pragma omp for schedule(dynamic, 16)
-    for (int64_t r = 0; r < ns; ++r) {
+    for (int64_t r = 0; r < ns; ++r) guarded(failed, [&] {
       row(r, cnt, rank);
       at.assign(cnt.size(), -1);  // bundle and lane of every chain: 32 bundle + lane
       for (size_t q = 0; q < rank.size() && cnt[rank[q]] > 0; ++q) at[rank[q]] = (int32_t)q;
@@ -267,8 +282,9 @@ void lane_plan(const double *eps, int64_t ns, int64_t npp, int64_t item, double 
             if (cnt[c]++ > 0 && p - prev[c] > 32) P.pidx[slot - 32] |= kGap;
             prev[c] = (int32_t)p;
           }
-    }
+    });
   }
+  if (failed) throw std::bad_alloc();
 }
 
 // Dense pair-major form of the mixed-precision sweep (pb_dev_opts.channel_per_lane 5, or 0 when
@@ -1319,8 +1335,11 @@ extern "C" int pb_dev_create(const pb_channels *ch, const pb_dev_opts *opts, voi
   d->tnt = (int)T.tiles.size();
   d->nsp = T.nsp;
   GDense gd;
+  const TrRows trr = tr_rows_for(d->ns, sm, d->transport, merged, complete, o.variant, o);
   try {
     gd = gdense_for(ch, o, sm, true);
+    d->L = make_layout(ch, P, merged ? &S : nullptr, o.variant, d->transport, d->nfin_blocks, sym ? &T : nullptr, gd,
+                       o.adjoint != 0, c32 ? sizeof(float2) : sizeof(float4), trr.nseg, sm);
   } catch (const std::bad_alloc &) {
     delete d;
     return set_error(PB_ENOMEM, "pb_dev_create: out of host memory");
@@ -1329,11 +1348,8 @@ extern "C" int pb_dev_create(const pb_channels *ch, const pb_dev_opts *opts, voi
   d->gd_nitems = (int)(int64_t)gd.plan.items.size();
   d->gd_bytes = gd.bytes;
   d->gd_slots = (size_t)gd.plan.slots;
-  const TrRows trr = tr_rows_for(d->ns, sm, d->transport, merged, complete, o.variant, o);
   d->tr_nseg = trr.nseg;
   d->tr_seglen = trr.seglen;
-  d->L = make_layout(ch, P, merged ? &S : nullptr, o.variant, d->transport, d->nfin_blocks, sym ? &T : nullptr, gd,
-                     o.adjoint != 0, c32 ? sizeof(float2) : sizeof(float4), trr.nseg, sm);
   if (arena_bytes < d->L.total) {
     const size_t need = d->L.total;
     delete d;

@@ -151,3 +151,88 @@ def test_batch_autotune_times_the_shapes_that_run(fake):
     assert tune([big] * 4, 1)[0] == 1 + 2 * 4
     assert tune([small], 2)[0] == 1 + 5 * 4
     """)
+
+
+CREATE = {
+    "channels": "lambda: build(1)",
+    "channels, one callback at a time": "lambda: build(0)",
+    "tiles with transport": "lambda: dev(transport=1, adjoint=1)",
+    "rows": "lambda: dev(dense_rows=2, transport=1)",
+    "dense g32": "lambda: dev(variant=pb.VARIANTS['g32'], adjoint=1)",
+    "dense h16, cutoff list": "lambda: dev(cut, variant=pb.VARIANTS['h16'], channel_per_lane=5)",
+    "cutoff list, forced tiles": "lambda: dev(cut, dense_rows=3)",
+    "paper": "lambda: dev(variant=pb.VARIANTS['paper'])",
+    "batch fp32": "lambda: batch(0)",
+    "batch ff": "lambda: batch(1)",
+    "batch c32": "lambda: batch(2)",
+}
+
+
+@pytest.mark.parametrize("what", list(CREATE))
+def test_host_memory_that_runs_out_is_an_error_code(fake, what):
+    """The i-th allocation of the call fails, for every i up to the first hundred and then ever larger
+    steps: PB_ENOMEM (or success where the failed allocation has a fallback), never an exception through
+    the C interface or out of a parallel region."""
+    child(fake, f"""
+    import os
+    m = synth.make_window4(9)
+    ch = pb.Channels.from_model(m)
+    cut = pb.Channels.from_model(m, g2_min=1e-5, delta_nsigma=6.0)
+    rate = ctypes.CFUNCTYPE(ctypes.c_int, ctypes.c_int64, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p)
+
+    def g2(n, s, p, v, out, user):
+        ctypes.memset(out, 0, 8 * n)
+        return 0
+    g2c = rate(g2)
+
+    def build(threadsafe):
+        arrays = [np.ascontiguousarray(a, dtype=np.float64) for a in (m.eps, m.omega, m.win)]
+        M = pb._Model()
+        M.nk[:] = m.nk
+        M.nbands, M.nmodes = m.eps.shape[-1], m.omega.shape[-1]
+        M.eps, M.omega, M.win = (a.ctypes.data for a in arrays)
+        M.T, M.sigma = m.T, m.sigma
+        o = pb._BuildOpts(nthreads=1 if threadsafe else 0, callback_threadsafe=threadsafe, check_closure=1)
+        h = ctypes.c_void_p()
+        yield lambda: L.pb_build_channels(ctypes.byref(M), ctypes.cast(g2c, ctypes.c_void_p), None, ctypes.byref(o), ctypes.byref(h))
+        if h:
+            L.pb_channels_free(h)
+
+    def dev(c=ch, **kw):
+        o, n, h = opts(**kw), ctypes.c_size_t(0), ctypes.c_void_p()
+        assert L.pb_dev_arena_bytes(c._h, ctypes.byref(o), ctypes.byref(n)) == pb.PB_OK
+        a = aligned(n.value)
+        yield lambda: L.pb_dev_arena_bytes(c._h, ctypes.byref(o), ctypes.byref(n)) or L.pb_dev_create(
+            c._h, ctypes.byref(o), ctypes.c_void_p(a.ctypes.data), n, None, ctypes.byref(h))
+        if h:
+            L.pb_dev_destroy(h)
+
+    def batch(prec):
+        arr = (ctypes.c_void_p * 2)(ch._h.value, ch._h.value)
+        o, n, h = pb._BatchOpts(0, 0, prec, 0), ctypes.c_size_t(0), ctypes.c_void_p()
+        f = np.zeros(2 * ch.nstate)
+        assert L.pb_batch_arena_bytes(arr, 2, ctypes.byref(o), ctypes.byref(n)) == pb.PB_OK
+        a = aligned(n.value)
+        yield lambda: L.pb_batch_arena_bytes(arr, 2, ctypes.byref(o), ctypes.byref(n)) or L.pb_batch_create(
+            arr, 2, ctypes.byref(o), ctypes.c_void_p(a.ctypes.data), n, None, ctypes.byref(h)) or L.pb_batch_autotune(
+            h, ctypes.c_void_p(f.ctypes.data), None, None, None, None)
+        if h:
+            L.pb_batch_destroy(h)
+
+    i, failed = 0, 0
+    while True:
+        i += 1 + max(0, i - 100) // 20
+        it = ({CREATE[what]})()
+        call = next(it)
+        L.fake_fail_new(i)
+        rc = call()
+        done = L.fake_news() < i
+        L.fake_fail_new(0)
+        assert rc in (pb.PB_OK, pb.PB_ENOMEM), (i, rc, L.pb_last_error().decode())
+        failed += rc == pb.PB_ENOMEM
+        next(it, None)
+        if done:
+            assert rc == pb.PB_OK
+            break
+    assert failed >= 3, failed
+    """)
