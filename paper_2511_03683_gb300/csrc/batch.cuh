@@ -632,9 +632,9 @@ std::vector<int64_t> batch_lenp(const pb_channels *const *chs, int32_t n) {
   return lenp;
 }
 
-int batch_dense_grid(const pb_batch *b, int ctas) {
-  const int64_t need = (b->nitems * 32 + 511) / 512;
-  return (int)std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)b->sm_count * ctas));
+int batch_dense_grid(int64_t nitems, int sm_count, int ctas) {
+  const int64_t need = (nitems * 32 + 511) / 512;
+  return (int)std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)sm_count * ctas));
 }
 
 int batch_upload_items(pb_batch *b, const BatchPlan &P, int item_ch, cudaStream_t st) {
@@ -654,16 +654,18 @@ int batch_upload_items(pb_batch *b, const BatchPlan &P, int item_ch, cudaStream_
 }
 
 // The dense form's plan for an item size: the instances' lane plans, the slot map, the |g|^2 values
-// scattered into the slots from the channel list, and the CTAs' item ranges.
+// scattered into the slots from the channel list, and the CTAs' item ranges.  Everything that can fail
+// on the host comes before the first change on the device: after an error the plan before it is whole.
 int batch_upload_dense(pb_batch *b, int item_ch, cudaStream_t st) {
   BatchPlan D, C;
   std::vector<uint32_t> pidx;
+  std::vector<pb::dev::BInst> inst = b->hinst;
   int64_t values = 0, map = 0;
   for (int i = 0; i < b->n; ++i) {
     const int64_t s0 = b->soff[i], ns = b->soff[i + 1] - s0;
     LanePlan<uint32_t> P;
     lane_plan(b->heps.data() + s0, ns, batch_npp(ns), batch_dense_part(item_ch), b->reach[i], true, P);
-    auto &B = b->hinst[i];
+    auto &B = inst[i];
     B.doff = values;
     B.poff = (long long)pidx.size();
     B.moff = map;
@@ -680,6 +682,23 @@ int batch_upload_dense(pb_batch *b, int item_ch, cudaStream_t st) {
   D.item_ptr.push_back((int32_t)D.items.size());
   if ((int64_t)pidx.size() > b->slot_cap || values > b->value_cap)
     return set_error(PB_EINVAL, "pb_batch: item size %d needs more slots than the arena holds", item_ch);
+  batch_plan(b, 2048, C);  // the channel list's own items, for the scatter
+  const int64_t nitems = (int64_t)D.items.size();
+  if (std::max(nitems, (int64_t)C.items.size()) > b->nitems_cap)
+    return set_error(PB_EINVAL, "pb_batch: item size %d needs more items than the arena holds", item_ch);
+  // per CTAs-per-SM choice, item ranges of about equal work (steps times branches)
+  std::vector<int64_t> cost((size_t)nitems + 1, 0);
+  for (int64_t i = 0; i < nitems; ++i)
+    cost[i + 1] = cost[i] + (int64_t)D.items[i].len * (2 + inst[D.item_inst[i]].nm) + 4;
+  const int stride = b->sm_count * 4 + 1;
+  std::vector<int32_t> cb((size_t)4 * stride, (int32_t)nitems);
+  for (int c = 1; c <= 4; ++c) {
+    const int g = batch_dense_grid(nitems, b->sm_count, c);
+    for (int k = 0; k <= g; ++k)
+      cb[(size_t)(c - 1) * stride + k] =
+          (int32_t)(std::lower_bound(cost.begin(), cost.end(), cost[nitems] * k / g) - cost.begin());
+  }
+  b->hinst.swap(inst);
   int rc;
   PB_CUDA(cudaMemcpyAsync(b->inst, b->hinst.data(), sizeof(pb::dev::BInst) * b->hinst.size(), cudaMemcpyHostToDevice, st));
   PB_CUDA(cudaMemcpyAsync(b->pidx0, pidx.data(), sizeof(uint32_t) * pidx.size(), cudaMemcpyHostToDevice, st));
@@ -692,25 +711,12 @@ int batch_upload_dense(pb_batch *b, int item_ch, cudaStream_t st) {
   if ((rc = batch_upload_items(b, D, item_ch, st))) return rc;
   dev::k_slot_map_batch<<<grid(), dev::kBlock, 0, st>>>(b->items, b->item_inst, (int)b->nitems, b->inst, b->pidx0, b->smap);
   PB_LAUNCHED("k_slot_map_batch");
-  batch_plan(b, 2048, C);  // the channel list's own items, for the scatter
   if ((rc = batch_upload_items(b, C, 2048, st))) return rc;
   dev::k_dense_g2_batch<<<grid(), dev::kBlock, 0, st>>>(b->items, b->item_inst, (int)b->nitems, b->inst, b->col, b->g2,
                                                         b->smap, b->g2d);
   PB_LAUNCHED("k_dense_g2_batch");
   PB_CUDA(cudaStreamSynchronize(st));
   if ((rc = batch_upload_items(b, D, item_ch, st))) return rc;
-  // per CTAs-per-SM choice, item ranges of about equal work (steps times branches)
-  std::vector<int64_t> cost((size_t)b->nitems + 1, 0);
-  for (int64_t i = 0; i < b->nitems; ++i)
-    cost[i + 1] = cost[i] + (int64_t)D.items[i].len * (2 + b->hinst[D.item_inst[i]].nm) + 4;
-  const int stride = b->sm_count * 4 + 1;
-  std::vector<int32_t> cb((size_t)4 * stride, (int32_t)b->nitems);
-  for (int c = 1; c <= 4; ++c) {
-    const int g = batch_dense_grid(b, c);
-    for (int k = 0; k <= g; ++k)
-      cb[(size_t)(c - 1) * stride + k] =
-          (int32_t)(std::lower_bound(cost.begin(), cost.end(), cost[b->nitems] * k / g) - cost.begin());
-  }
   PB_CUDA(cudaMemcpyAsync(b->cbeg, cb.data(), sizeof(int32_t) * cb.size(), cudaMemcpyHostToDevice, st));
   PB_CUDA(cudaStreamSynchronize(st));
   return PB_OK;
@@ -771,7 +777,7 @@ int batch_sweep(pb_batch *b, cudaStream_t st) {
     PB_LAUNCHED("k_stream_ff (batch)");
     return PB_OK;
   }
-  const int grid = batch_dense_grid(b, b->ctas);  // of 512 threads
+  const int grid = batch_dense_grid(b->nitems, b->sm_count, b->ctas);  // of 512 threads
   if (b->dense) {
     pb::dev::k_stream_gbatch_dense<<<grid, 512, 0, st>>>(b->items, b->item_inst,
                                                           b->cbeg + (size_t)(b->ctas - 1) * (b->sm_count * 4 + 1),

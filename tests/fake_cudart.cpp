@@ -10,7 +10,7 @@
 #include <new>
 
 namespace {
-std::atomic<long> g_launches{0}, g_graph_launches{0}, g_instantiates{0}, g_fail{0}, g_fail_new{0}, g_news{0};
+std::atomic<long> g_launches{0}, g_graph_launches{0}, g_instantiates{0}, g_fail{0}, g_fail_new{0}, g_news{0}, g_copies{0};
 std::atomic<int> g_error{0};
 bool g_capturing = false;
 long g_nodes = 0;
@@ -40,7 +40,7 @@ void fake_fail_new(long i) {
   g_fail_new = i;
 }
 long fake_news(void) { return g_news; }
-long fake_count(int what) { return what == 0 ? g_launches : what == 1 ? g_graph_launches : g_instantiates; }
+long fake_count(int what) { return what == 0 ? g_launches : what == 1 ? g_graph_launches : what == 2 ? g_instantiates : g_copies; }
 
 void **__cudaRegisterFatBinary(void *) {
   static void *h;
@@ -152,10 +152,12 @@ cudaError_t cudaGraphLaunch(cudaGraphExec_t x, cudaStream_t) {
 }
 cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind, cudaStream_t) {
   if (n && !g_capturing) std::memcpy(d, s, n);
+  ++g_copies;
   return cudaSuccess;
 }
 cudaError_t cudaMemsetAsync(void *d, int v, size_t n, cudaStream_t) {
   if (n && !g_capturing) std::memset(d, v, n);
+  ++g_copies;
   return cudaSuccess;
 }
 cudaError_t cudaPointerGetAttributes(cudaPointerAttributes *a, const void *) {

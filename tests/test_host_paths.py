@@ -153,6 +153,44 @@ def test_batch_autotune_times_the_shapes_that_run(fake):
     """)
 
 
+def test_a_failed_batch_plan_leaves_the_one_before_it(fake):
+    """The autotuner's plans of the dense FP32 batch: wherever an allocation fails, no copy, clear or launch
+    of that plan has been made, so the items on the device still belong to its slots and ranges."""
+    child(fake, """
+    ch = pb.Channels.from_model(synth.make_window4(16))
+    arr = (ctypes.c_void_p * 2)(ch._h.value, ch._h.value)
+    o, n = pb._BatchOpts(0, 0, 0, 0), ctypes.c_size_t(0)
+    assert L.pb_batch_arena_bytes(arr, 2, ctypes.byref(o), ctypes.byref(n)) == pb.PB_OK
+    a, f = aligned(n.value), np.zeros(2 * ch.nstate)
+
+    def tune(i):
+        h = ctypes.c_void_p()
+        assert L.pb_batch_create(arr, 2, ctypes.byref(o), ctypes.c_void_p(a.ctypes.data), n, None, ctypes.byref(h)) == pb.PB_OK
+        before = L.fake_count(0) + L.fake_count(3)
+        L.fake_fail_new(i)
+        rc = L.pb_batch_autotune(h, ctypes.c_void_p(f.ctypes.data), None, None, None, None)
+        n_ = L.fake_news()
+        L.fake_fail_new(0)
+        L.pb_batch_destroy(h)
+        if not i:
+            global news
+            news = n_
+        return rc, L.fake_count(0) + L.fake_count(3) - before
+
+    rc, total = tune(0)
+    assert rc == pb.PB_OK
+    plan, rest = divmod(total - 1 - 3 * 12, 4)  # the input; three sizes' plans and 3 x 4 sweeps; the best's plan
+    assert rest == 0 and plan > 10
+    whole, failed = {1 + k * (plan + 12) for k in range(4)}, 0
+    for i in list(range(1, 40)) + list(range(news // 2, news, news // 60)) + list(range(news - 60, news + 20)):
+        rc, done = tune(i)
+        if rc != pb.PB_OK:
+            assert rc == pb.PB_ENOMEM and done in whole, (i, done, whole)
+            failed += 1
+    assert failed > 100
+    """)
+
+
 CREATE = {
     "channels": "lambda: build(1)",
     "channels, one callback at a time": "lambda: build(0)",
