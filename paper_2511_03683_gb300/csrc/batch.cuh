@@ -382,6 +382,7 @@ bool batch_dense_for(const pb_channels *const *chs, int32_t n, const pb_batch_op
   if (o.precision != 0 || o.layout != 0) return false;
   int64_t nch = 0, slots = 0;
   for (int i = 0; i < n; ++i) {
+    if (chs[i]->nstate > 60000) return false;  // slots (at most 1.1 per pair) are numbered in 32 bits
     nch += chs[i]->nch;
     slots += chs[i]->nstate * batch_npp(chs[i]->nstate) * chs[i]->nmodes;
   }
