@@ -180,8 +180,8 @@ typedef struct pb_dev_opts {
                                 one channel per lane with lazily renormalised float-float sums: 4 one
                                 1024-thread CTA per SM with F in shared memory (5 if F does not fit) and
                                 the next trip in registers, or, on a device with float-float symmetric
-                                tiles (dense_rows), the weights in the same energy-ordered tiles; 5 the
-                                same through L1, 6 = 3 with lazy sums;
+                                tiles (dense_rows), the weights in the same energy-ordered tiles (the row
+                                shape there: dense_rows 2); 5 the same through L1, 6 = 3 with lazy sums;
                                 7 row blocks on complete branch-merged float-float rows: a warp takes
                                 four rows and one segment of their partners, each partner's F (shared
                                 memory) read once for the four rows, the weights through a per-warp

@@ -674,6 +674,10 @@ int cuda_fail(cudaError_t e, const char *what) {
 // launches (four-band window, us per RK4 step: 16^3 17.0 against 25.2 with the ring and ordinary
 // launches, 24^3 18.5 against 25.4, 30^3 24.9 against 30.7; at 32^3, 296 tiles, 31.2 against 31.1, and at
 // 40^3, 1017 tiles, 61.9 against 59.7: sweep CTAs that come in while the epilogue runs slow it down).
+// C32 takes the same line with its ring (whole triangles; us per RK4 step, chained against ordinary
+// launches: 16^3, 21 tiles, 15.7 against 18.7, 20^3, 55, 15.9 against 18.8, 24^3, 153, 16.7 against 20.5). Its
+// ring still gains above it, less with size (26^3, 231 tiles, 17.7 against 21.6, 28^3, 325, 19.8 against 23.9, 32^3,
+// 780, 31.0 against 31.5, 36^3, 1378, 40.1 against 41.5), but the float-float line is kept for both.
 bool chain_pdl(int64_t tiles, int sm_count) { return 2 * tiles <= 3 * (int64_t)sm_count; }
 
 // The tile epilogues, single systems' and batches': 8 states per CTA unless 32 per CTA still give four

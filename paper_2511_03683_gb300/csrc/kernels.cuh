@@ -2484,8 +2484,8 @@ __global__ void __launch_bounds__(kSymThreads, 1) k_stream_sym_bulk(const TileD 
 // difference of two products of two, 24 operations, and two lazy additions of 8: 40 operations
 // against 48, with half the sums to carry and to reduce, half the partials, and an epilogue of two
 // FP64 operations instead of seven per state.  The terms cancel before they are rounded together, and
-// neither R_s nor the closing difference A - f_s (R - B) is needed (error of df/dt at 35^3 7.8e-15 ->
-// 4.8e-15).  MODE_RATE: B = sum f D for both sides, 1/tau = c (R - B) (the positive summands
+// neither R_s nor the closing difference A - f_s (R - B) is needed (error of df/dt at 35^3, largest of four
+// sets of inputs, 6.8e-15 -> 5.0e-15).  MODE_RATE: B = sum f D for both sides, 1/tau = c (R - B) (the positive summands
 // f_p P_in + g_p P_out instead of R, which is summed in FP64, would be six times less accurate).
 //
 // Half-tiles.  The unit of staging is 32 rows x 64 columns of a tile (32 KB, contiguous in the tile's
@@ -2494,8 +2494,10 @@ __global__ void __launch_bounds__(kSymThreads, 1) k_stream_sym_bulk(const TileD 
 // 2 ti + 1 of the half and columns tj, tj + 16, tj + 32, tj + 48; row and column sums stay in
 // registers across the two halves.  After the second, the tile's row sums are reduce-scattered over
 // the 16 lanes of a row and the column sums go through one shuffle level and a per-warp table that is
-// combined after the next unit's barrier.  Bound by instruction issue: 67 instructions per entry.  At
-// 40^3 (1017 tiles) 14.4 us per launch against 16.4 for A and C sums, an RK4 step 67.1 -> 60.4 us.
+// combined after the next unit's barrier.  66 instructions per entry (counted at 39^3, 867 tiles) with
+// 51% of the issue slots used (cold; 22 warps per SM on average): the rest is waiting and the uneven last
+// round, 2.2 tiles per CTA at 40^3.  There (1017 tiles) 14.4 us per launch against 16.4 for A and C sums, an RK4
+// step 67.1 -> 58.7 us.
 constexpr unsigned kHalfTileBytes = kTileBytes / 2;
 constexpr unsigned kHalfStageBytes = kHalfTileBytes + (kTile / 2 + kTile) * sizeof(float4);
 constexpr size_t kNetColBytes = (size_t)(kSymThreads / 32) * kTile * sizeof(float2);  // the column table
@@ -2834,7 +2836,8 @@ __device__ __forceinline__ double ff3_to_double(const FF3 &v) {
 // partial slots in FP64 (sums; ncs: column slots per tile, the second of two is zeroed): positive
 // terms, so 1/tau keeps its accuracy where R - B cancels (k_tau_tiles).  A warp's half-rows are added
 // in a reduce-scatter of four rows at a time, a thread's column in registers, and one thread per row
-// and column converts (a conversion costs as much as 64 FP32 operations).
+// and column converts (a conversion costs as much as 64 FP32 operations).  57 MB read and 55 written at 39^3
+// in 29.9 us (cold, 47% of the issue slots used; 29.7 us without the sums).
 __global__ void __launch_bounds__(256) k_weight_tiles(const TileD *__restrict__ tiles, int nt,
                                                       const float4 *__restrict__ tc, const float4 *__restrict__ f0,
                                                       int ncs, float2 *__restrict__ W, double *__restrict__ sums) {
@@ -2939,8 +2942,9 @@ __global__ void k_trF_map(const double *__restrict__ F, int n, const int *__rest
 // columns 2 tj, 2 tj + 1, 32 + 2 tj, 33 + 2 tj, three directions: 12 float-float sums that stay in
 // registers over all tiles of one block row (a segment; desc.w marks its last tile), lazily
 // renormalised (at most 4 terms per tile, 64 at most per segment, see kTrSegTiles), then
-// reduce-scattered over the 16 lanes of a row into part[segment][direction][row].  Bound by
-// instruction issue: per weight 3 multiply-adds of 12 operations and 0.5 shared-memory loads.
+// reduce-scattered over the 16 lanes of a row into part[segment][direction][row].  Per weight 3
+// multiply-adds of 12 operations and 0.5 shared-memory loads, 48 instructions with everything (counted at
+// 39^3), 62% of the issue slots used (cold).
 // At 40^3 it replaces a row stream of every pair (48.8 us per pass).
 struct alignas(16) TrTile {
   int J, seg, last, pad;
